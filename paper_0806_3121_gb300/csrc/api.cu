@@ -164,6 +164,10 @@ abft_status make_plan(const abft_desc* d, Plan* P) {
   L.nBblk = region((size_t)4 * p.nvc * 8);
   L.car_a = region((size_t)2 * p.nvr * 8);
   L.car_b = region((size_t)2 * p.nvc * 8);
+  size_t f64tc_bytes = 0;
+  p.tc64 = d->dtype == ABFT_F64 && plan_f64_tc(*d, p.R, p.Cc, &p.f64tc, &f64tc_bytes);
+  p.f64tc_hdr = region(p.tc64 ? 256 : 0);  // after car_b: cleared with it
+  p.f64tc_base = region(f64tc_bytes);
   L.E16 = region(lp ? (size_t)L.acs_rows * d->n * 4 : 0);
   L.F16 = region(lp ? (size_t)d->m * L.bcs_cols * 4 : 0);
   L.obs_col = region(p.fused ? (size_t)p.ntr_obs * 2 * d->n * 4 : 0);
@@ -199,6 +203,10 @@ abft_status make_plan(const abft_desc* d, Plan* P) {
   return ABFT_OK;
 }
 
+// Products with bounded waits: the tensor-core dtypes and the sliced binary64
+// product (whose status word the verify and the rebuild copy to kCntTimeout).
+bool has_status(const Plan& P) { return P.d.dtype != ABFT_F64 || P.tc64; }
+
 bool is_empty(const Plan& P) { return P.d.m == 0 || P.d.n == 0; }
 
 // A freshly encoded product carries no checksum deviation, and (tensor-core
@@ -206,8 +214,9 @@ bool is_empty(const Plan& P) { return P.d.m == 0 || P.d.n == 0; }
 // on it and no operand has been found inexact.
 cudaError_t clear_carry(const Plan& P, void* ws, cudaStream_t st) {
   char* w = static_cast<char*>(ws);
-  cudaError_t e = cudaMemsetAsync(w + P.L.car_a, 0, sizeof(double) * 2 * P.nvr, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w + P.L.car_b, 0, sizeof(double) * 2 * P.nvc, st);
+  // car_a, car_b and the sliced product's status words are adjacent regions
+  const size_t end = P.tc64 ? P.f64tc_hdr + 8 : P.L.car_b + sizeof(double) * 2 * P.nvc;
+  cudaError_t e = cudaMemsetAsync(w + P.L.car_a, 0, end - P.L.car_a, st);
   if (e == cudaSuccess && P.d.dtype != ABFT_F64)
     e = cudaMemsetAsync(w + P.L.scratch + sizeof(int32_t) * kCntTimeout, 0,
                         sizeof(int32_t) * (kCntFp8Inexact - kCntTimeout + 1), st);
@@ -472,7 +481,7 @@ abft_status abft_verify_correct(const abft_desc* desc, void* C, void* ws, int32_
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "abft_verify_correct");
   // status words of this workspace's last product and last encode
-  if (P.d.dtype != ABFT_F64 && cnt[kCntTimeout])
+  if (has_status(P) && cnt[kCntTimeout])
     return fail(ABFT_ERR_TIMEOUT,
                 "the tensor-core product on this workspace gave up waiting (bounded wait); C and "
                 "its checksums are incomplete and were not corrected");
@@ -583,7 +592,7 @@ abft_status abft_recover_blocks(const abft_desc* desc, void* C, void* ws, const 
     e = cudaMemcpyAsync(cnt, S.cnt, sizeof cnt, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "abft_recover_blocks");
-  if (P.d.dtype != ABFT_F64 && cnt[kCntTimeout])
+  if (has_status(P) && cnt[kCntTimeout])
     return fail(ABFT_ERR_TIMEOUT,
                 "the tensor-core product on this workspace gave up waiting (bounded wait); its "
                 "block checksums are incomplete and nothing was rebuilt");
@@ -643,7 +652,7 @@ abft_status abft_block_restore(const abft_desc* desc, void* C, void* ws, int32_t
   if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, S.cnt, sizeof cnt, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "abft_block_restore");
-  if (P.d.dtype != ABFT_F64 && cnt[kCntTimeout])
+  if (has_status(P) && cnt[kCntTimeout])
     return fail(ABFT_ERR_TIMEOUT,
                 "the tensor-core product on this workspace gave up waiting (bounded wait); "
                 "nothing was written");

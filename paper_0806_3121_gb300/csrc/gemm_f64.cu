@@ -1,4 +1,6 @@
-// Binary64 ABFT product (Eq. (1)): [A; acs] [B, bcs] on the FP64 FMA pipe.
+// Binary64 ABFT product (Eq. (1)): [A; acs] [B, bcs] on the FP64 FMA pipe, for
+// products below 128^3, checksum-free products without a workspace and the
+// tiles that the sliced product on the tensor cores (gemm_f64_tc.cu) leaves out.
 //
 // On GB300 the FP64 FMA pipe issues 2 DFMA per clock per SM (measured
 // 1.20 TFLOP/s over 152 SMs); mma.sync f64 runs slower (1.05 TFLOP/s) and
@@ -8,10 +10,13 @@
 // Memory traffic is ~(1/64 + 1/64) words per FMA, far below HBM and L2
 // bandwidth at this FMA rate.
 //
-// Tiles are scheduled as one 1-D grid in a grouped order (see decode_f64):
-// data tiles, whole tiles of checksum rows (acs, writing E) and checksum
-// columns (bcs, writing F); the corner (acs x bcs) is not computed.  Each output element is one FMA chain
-// over k in increasing order.
+// Tiles are scheduled as one 1-D grid in a grouped order (TileGrid): data tiles,
+// whole tiles of checksum rows (acs, writing E) and checksum columns (bcs,
+// writing F); the corner (acs x bcs) is not computed.  Each output element is one
+// FMA chain over k in increasing order.
+#include <algorithm>
+
+#include "gemm_f64.cuh"
 #include "internal.cuh"
 
 namespace abft {
@@ -21,74 +26,17 @@ constexpr int BM = 64, BN = 64, BK = 16, kThreads = 256;
 
 constexpr int GROUP_M = 16;  // tile rows per raster group
 
-struct GemmArgs {
-  const double* A;
-  const double* B;
-  const double* acs;
-  const double* bcs;
-  double* C;
-  double* E;
-  double* F;
-  int64_t lda, ldb, ldc, m, n, k, R, Cc;
-  int tm, tn;  // data tiles along rows / columns
-  int tr, tc;  // checksum tiles along rows / columns (0 for the plain product)
-};
-
-// Linear tile index -> (tile row, tile column), tile rows >= tm being checksum
-// rows and tile columns >= tn checksum columns.  Groups of GROUP_M data tile
-// rows run column by column; checksum tile rows are dealt round-robin to the
-// groups and checksum tile columns follow each group's data columns, so
-// consecutive CTAs share the A and B panels in L2.
-__device__ __forceinline__ void decode_f64(int64_t t, const GemmArgs& g, int& ty, int& tx) {
-  const int64_t ngr = (g.tm + GROUP_M - 1) / GROUP_M;
-  int64_t off = 0;
-  for (int64_t G = 0; G < ngr; ++G) {
-    const int64_t gd = min((int64_t)GROUP_M, (int64_t)g.tm - G * GROUP_M);
-    const int64_t nr = G < g.tr ? (g.tr - G + ngr - 1) / ngr : 0;
-    const int64_t part1 = (gd + nr) * g.tn, part2 = gd * g.tc;
-    if (t < off + part1 + part2) {
-      int64_t u = t - off;
-      if (u < part1) {
-        const int64_t ri = u % (gd + nr);
-        tx = (int)(u / (gd + nr));
-        ty = ri < gd ? (int)(G * GROUP_M + ri) : (int)(g.tm + G + (ri - gd) * ngr);
-      } else {
-        u -= part1;
-        tx = (int)(g.tn + u / gd);
-        ty = (int)(G * GROUP_M + u % gd);
-      }
-      return;
-    }
-    off += part1 + part2;
-  }
-  ty = tx = 0;
-}
-
-__global__ void __launch_bounds__(kThreads, 2) k_gemm_f64(const GemmArgs g) {
-  int ty_tile, tx_tile;
-  decode_f64(blockIdx.x, g, ty_tile, tx_tile);
-  const bool cs_row = ty_tile >= g.tm, cs_col = tx_tile >= g.tn;
-
+// The BM x BN tile at (row0, col0) of the data (cs_row = cs_col = false), of the
+// checksum rows (cs_row) or of the checksum columns (cs_col).
+__device__ __forceinline__ void tile_f64(const F64Args& g, bool cs_row, bool cs_col, int64_t row0,
+                                         int64_t col0) {
   // Source and destination of this tile.
-  const double* Asrc;
-  int64_t ldA, rlim, row0;
-  if (!cs_row) {
-    Asrc = g.A; ldA = g.lda; rlim = g.m; row0 = (int64_t)ty_tile * BM;
-  } else {
-    Asrc = g.acs; ldA = g.k; rlim = g.R; row0 = (int64_t)(ty_tile - g.tm) * BM;
-  }
-  const double* Bsrc;
-  int64_t ldB, clim, col0;
-  if (!cs_col) {
-    Bsrc = g.B; ldB = g.ldb; clim = g.n; col0 = (int64_t)tx_tile * BN;
-  } else {
-    Bsrc = g.bcs; ldB = g.Cc; clim = g.Cc; col0 = (int64_t)(tx_tile - g.tn) * BN;
-  }
-  double* Dst;
-  int64_t ldD;
-  if (!cs_row && !cs_col) { Dst = g.C; ldD = g.ldc; }
-  else if (cs_row) { Dst = g.E; ldD = g.n; }
-  else { Dst = g.F; ldD = g.Cc; }
+  const double* Asrc = cs_row ? g.acs : g.A;
+  const int64_t ldA = cs_row ? g.ldacs : g.lda, rlim = cs_row ? g.R : g.m;
+  const double* Bsrc = cs_col ? g.bcs : g.B;
+  const int64_t ldB = cs_col ? g.ldbcs : g.ldb, clim = cs_col ? g.Cc : g.n;
+  double* Dst = cs_row ? g.E : (cs_col ? g.F : g.C);
+  const int64_t ldD = cs_row ? g.lde : (cs_col ? g.ldf : g.ldc);
 
   __shared__ double As[2][BK][BM + 2];
   __shared__ double Bs[2][BK][BN];
@@ -97,9 +45,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_f64(const GemmArgs g) {
   const int tx = tid & 15, ty = tid >> 4;
   double acc[4][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 4; ++i) {
+    const int64_t row = row0 + ty + 16 * i;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < 4; ++j) {
+      const int64_t col = col0 + tx + 16 * j;
+      acc[i][j] = (g.accumulate && row < rlim && col < clim) ? Dst[row * ldD + col] : 0.0;
+    }
+  }
 
   double ra[4], rb[4];
   auto load = [&](int64_t k0) {
@@ -167,17 +120,54 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_f64(const GemmArgs g) {
   }
 }
 
+__global__ void __launch_bounds__(kThreads, 2) k_gemm_f64(const F64Args g, const TileGrid T) {
+  int ty, tx;
+  T.decode(blockIdx.x, ty, tx);
+  const bool cs_row = ty >= T.tm, cs_col = tx >= T.tn;
+  tile_f64(g, cs_row, cs_col, (int64_t)(cs_row ? ty - T.tm : ty) * BM,
+           (int64_t)(cs_col ? tx - T.tn : tx) * BN);
+}
+
+// The tiles (128 x 64 bpt) that the sliced product left out, as BM x BN tiles.
+__global__ void __launch_bounds__(kThreads, 2)
+    k_gemm_f64_bad(const F64Args g, const TileGrid T, int bpt, const int* any,
+                   const uint8_t* bad) {
+  if (*any == 0) return;
+  const int64_t total = T.total() * 2 * bpt;
+  for (int64_t u = blockIdx.x; u < total; u += gridDim.x) {
+    const int64_t t = u / (2 * bpt);
+    const int s = (int)(u - t * 2 * bpt);
+    if (!bad[t]) continue;
+    int ty, tx;
+    T.decode(t, ty, tx);
+    const bool cs_row = ty >= T.tm, cs_col = tx >= T.tn;
+    const int64_t row0 = (int64_t)(cs_row ? ty - T.tm : ty) * 2 * BM + (s & 1) * BM;
+    const int64_t col0 = ((int64_t)(cs_col ? tx - T.tn : tx) * bpt + (s >> 1)) * BN;
+    if (row0 >= (cs_row ? g.R : g.m) || col0 >= (cs_col ? g.Cc : g.n)) continue;
+    __syncthreads();  // the previous tile's shared memory has been read
+    tile_f64(g, cs_row, cs_col, row0, col0);
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_gemm_f64_bad(const F64Args& g, const TileGrid& tiles, int bpt, const int* any,
+                                const uint8_t* bad, cudaStream_t st) {
+  const int64_t total = tiles.total() * 2 * bpt;
+  const unsigned grid = (unsigned)std::min<int64_t>(total, 2 * num_sms());
+  k_gemm_f64_bad<<<grid, kThreads, 0, st>>>(g, tiles, bpt, any, bad);
+  count_launches(1);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_gemm_f64(const Plan& P, const double* A, const double* B, double* C, void* ws,
                             bool checksums, cudaStream_t st) {
   const abft_desc& d = P.d;
-  GemmArgs g{};
+  if (d.m == 0 || d.n == 0) return cudaSuccess;
+  F64Args g{};
   g.A = A; g.B = B; g.C = C;
   g.lda = d.lda; g.ldb = d.ldb; g.ldc = d.ldc;
   g.m = d.m; g.n = d.n; g.k = d.k;
-  g.tm = (int)cdiv(d.m, BM);
-  g.tn = (int)cdiv(d.n, BN);
   if (checksums) {
     char* w = static_cast<char*>(ws);
     g.acs = reinterpret_cast<const double*>(w + P.L.acs);
@@ -186,12 +176,14 @@ cudaError_t launch_gemm_f64(const Plan& P, const double* A, const double* B, dou
     g.F = reinterpret_cast<double*>(w + P.L.F);
     g.R = P.R;
     g.Cc = P.Cc;
-    g.tr = (int)cdiv(P.R, BM);
-    g.tc = (int)cdiv(P.Cc, BN);
+    g.ldacs = d.k;
+    g.ldbcs = g.ldf = P.Cc;
+    g.lde = d.n;
   }
-  if (d.m == 0 || d.n == 0) return cudaSuccess;
-  const int64_t tiles = (int64_t)g.tm * g.tn + (int64_t)g.tr * g.tn + (int64_t)g.tm * g.tc;
-  k_gemm_f64<<<(unsigned)tiles, kThreads, 0, st>>>(g);
+  if (P.tc64 && ws) return launch_gemm_f64_tc(P, g, ws, st);
+  const TileGrid T{(int)cdiv(d.m, BM), (int)cdiv(d.n, BN), (int)cdiv(g.R, BM), (int)cdiv(g.Cc, BN),
+                   GROUP_M};
+  k_gemm_f64<<<(unsigned)T.total(), kThreads, 0, st>>>(g, T);
   count_launches(1);
   return cudaGetLastError();
 }

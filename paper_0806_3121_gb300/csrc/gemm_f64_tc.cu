@@ -1,0 +1,907 @@
+// Binary64 product [A; acs] [B, bcs] on the tensor cores, by slicing the
+// operands into exact bf16 digits (the error-free splitting of Ozaki, Ogita,
+// Oishi and Rump, "Error-free transformations of matrix multiplication by using
+// fast routines of matrix multiplication and its applications", 2012).
+//
+// GB300's FP64 pipe issues 2 DFMA per clock and SM (1.2 TFLOP/s on the whole
+// chip); its tensor cores multiply bf16 at 1900 TFLOP/s.  Row i of A (column
+// j of B) is scaled by the power of two above its largest element and written
+// as eight signed radix-256 digits, d_0 2^-7 + d_1 2^-15 + ... + d_7 2^-63, each in
+// [-128, 128] and so exact in bf16.  Digit products of equal weight,
+//   L_s = sum_{i + j = s} D_i(A) D_j(B),
+// are integers; 1024 of them add up to at most 2^24, exact in the tensor cores'
+// binary32 accumulators, and the epilogue adds those partial sums as 32-bit
+// integers.  C_ij = 2^(eA_i + eB_j) sum_s L_s 2^(-14 - 8 s) is formed once, in
+// integers, and rounded to nearest once.
+//
+// How many levels.  What is left out is the digit products of the next level and
+// beyond: with levels 0..6 (28 products) a rms error of 2^-56.2 per term in units
+// of 2^(eA_i + eB_j), with levels 0..7 (36 products) 2^-64.2.  A DFMA chain's
+// rounding errors are about 0.38 2^-53 sqrt(k / 2) times the rms of the terms'
+// sum, at least 0.27 2^-53 M_ij with M_ij = sum_l |a_il b_lj| in the same units.
+// So levels 0..6 are as accurate as the chain where M_ij >= 0.405 sqrt(k), levels
+// 0..7 where M_ij >= 0.0016 sqrt(k).  M is one more product (plane 8: the
+// magnitudes as bf16, rounded towards zero), and every tile computes it first:
+// each element is checked, so rows of mixed scales, graded operands whose large
+// rows meet small columns, and sparse operands never lose accuracy.  An element
+// none of whose terms is cut (operands with few significant bits) needs no
+// check.  Tiles with an element below both lines, NaN or infinite operands, or
+// exponents outside [-440, 500] are left to the DFMA kernel (k_gemm_f64_bad).
+//
+// The tensor cores bound it: 29 or 37 products of 2 m n k bf16 flops each.
+// 128 x (64 bpt)-tiles, one CTA per SM: warps 0 / 10 copy A / B by TMA into a
+// shared-memory ring, warp 1 issues tcgen05.mma into two alternating TMEM
+// accumulators, warps 2-9 add each accumulator into 128 integer registers per
+// thread.  Level sums go to a per-CTA scratch (coalesced, mostly L2) because
+// eight levels do not fit the registers and the FP64 pipe is too narrow to fold
+// them as they come (8 folds of a 128 x 256 tile at 2 per clock would take 131 k
+// clocks of the tile's 1.9 M at k = 8192).
+//
+// Measured against the DFMA kernel alone (encode and product, and whole steps):
+// 8192^3 on a 16 x 16 grid 953.6 -> 27.4 ms, 4096^3 step 132.2 -> 7.0 ms, two chained
+// 2048^3 products 34.0 -> 2.5 ms, 1000 x 1501 x 777 step 2.92 -> 0.78 ms.  Relative
+// Frobenius error against the exact product, N(0,1): 4.5e-17 (DFMA 7.7e-16) at k =
+// 512, 2.8e-16 (2.0e-15) at k = 4096, 4.7e-16 (4.9e-15) at k = 20000.
+#include <cuda.h>
+
+#include <stdlib.h>
+
+#include <algorithm>
+
+#include "gemm_f64.cuh"
+#include "internal.cuh"
+#include "tc_ptx.cuh"
+
+namespace abft {
+namespace {
+
+constexpr int BM = 128, BK = 64;
+constexpr int kDigits = 8, kMagPlane = 8, kPlanes64 = 9;
+constexpr int kGroupSteps = 16;   // k-steps per accumulator: 1024 2^14 = 2^24
+constexpr int kLevels = 8;        // levels 0..6, and 7 where the magnitudes ask for it
+constexpr int kMaxPanel = 16320;  // 8 * 16320 * 2^14 < 2^31: a level sum fits 32 bits
+constexpr int kEpiWarps = 8;
+constexpr int kWarpProdB = 2 + kEpiWarps;
+constexpr int kThreads = 32 * (kWarpProdB + 1);
+constexpr uint32_t kABytes = BM * BK * 2, kBoxBytes = 64 * BK * 2;
+constexpr int kMaxStages = 8;
+constexpr int kMinExp = -440, kMaxExp = 500;
+constexpr int kNotExact = 100;    // digit index of an operand row that is cut or refused
+constexpr size_t kPlaneBudget = size_t(6) << 30;
+constexpr int kSms = 152;  // persistent CTAs the workspace is laid out for
+
+constexpr int stages(int bpt) { return bpt == 4 ? 4 : (bpt == 2 ? 6 : 8); }
+constexpr size_t smem_bytes(int bpt) {
+  return 1024 + (size_t)stages(bpt) * (kABytes + bpt * kBoxBytes) + 256;
+}
+static_assert(smem_bytes(4) <= 232448 && smem_bytes(2) <= 232448 && smem_bytes(1) <= 232448,
+              "shared memory per CTA");
+
+// ------------------------------------------------------------------ digits
+
+// Four binary64 values as the four elements of each plane.
+struct Digits4 {
+  uint2 plane[kPlanes64];
+};
+
+// x 2^(63 - e) rounded to a 64-bit integer (|x| < 2^e, e = efield - 1022 with
+// efield the biased exponent of the row's largest element); the bits cut off.
+__device__ __forceinline__ int64_t scaled(double x, int efield, bool& cut) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const int E = (int)(b >> 52) & 0x7ff;
+  const uint64_t mant = (b & 0xfffffffffffffull) | (E ? 0x10000000000000ull : 0ull);
+  const int s = 10 - (efield - max(E, 1));  // value = mant 2^(s) in units of 2^(e - 63)
+  uint64_t v;
+  if (s >= 0) {
+    v = mant << s;
+  } else if (s > -64) {
+    const int r = -s;
+    v = (mant + (1ull << (r - 1))) >> r;
+    cut |= (mant & ((1ull << r) - 1)) != 0;
+  } else {
+    v = 0;
+    cut |= mant != 0;
+  }
+  return (int64_t)(b >> 63 ? 0ull - v : v);
+}
+
+// |x| 2^-e as bf16, rounded towards zero (nonzero values at least 2^-60).
+__device__ __forceinline__ uint32_t magnitude(double x, int efield) {
+  const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  if ((hi | (uint32_t)__double2loint(x)) == 0) return 0;
+  const int ex = 126 - (efield - (int)(hi >> 20));  // bf16 exponent field
+  return ex < 67 ? 67u << 7 : ((uint32_t)ex << 7) | ((hi >> 13) & 0x7fu);
+}
+
+// Digits and magnitudes of four values; `bits` collects the integers' bits.
+__device__ __forceinline__ void slice4(const double (&x)[4], int efield, Digits4& D,
+                                       uint64_t& bits, bool& cut) {
+  // (X + 2^63) + sum_j 128 256^j has the bytes d + 128 of the digits below the
+  // top one, and the top digit (with the carry) in the last place
+  uint32_t w[4][2], top[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint64_t X = (uint64_t)scaled(x[q], efield, cut);
+    bits |= X;
+    const uint64_t u0 = X ^ 0x8000000000000000ull, u = u0 + 0x0080808080808080ull;
+    w[q][0] = (uint32_t)u;
+    w[q][1] = (uint32_t)(u >> 32);
+    top[q] = (w[q][1] >> 24) + (u < u0 ? 256u : 0u);
+  }
+#pragma unroll
+  for (int p = 0; p < kDigits; ++p) {
+    float f[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      // 2^23 + (d + 128) as binary32 bits, minus 2^23 + 128
+      const int byte = kDigits - 1 - p;
+      const uint32_t m =
+          p == 0 ? (0x4B000000u | top[q])
+                 : __byte_perm(w[q][byte >> 2], 0x4B000000u, 0x7440u | (uint32_t)(byte & 3));
+      f[q] = __uint_as_float(m) - 8388736.0f;
+    }
+    // bf16 holds a digit exactly: the upper halves of the binary32 words
+    D.plane[p].x = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632u);
+    D.plane[p].y = __byte_perm(__float_as_uint(f[2]), __float_as_uint(f[3]), 0x7632u);
+  }
+  D.plane[kMagPlane].x = magnitude(x[0], efield) | (magnitude(x[1], efield) << 16);
+  D.plane[kMagPlane].y = magnitude(x[2], efield) | (magnitude(x[3], efield) << 16);
+}
+
+// Four consecutive elements, zeros from element nv on.
+__device__ __forceinline__ void load4(const double* p, int64_t nv, double (&x)[4]) {
+  if (nv >= 4 && (reinterpret_cast<uintptr_t>(p) & 15) == 0) {
+    const double2 a = *reinterpret_cast<const double2*>(p);
+    const double2 b = *reinterpret_cast<const double2*>(p + 2);
+    x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q] = q < nv ? p[q] : 0.0;
+  }
+}
+
+// Largest high word and whether any element is nonzero, in one word pair.
+__device__ __forceinline__ void take_max(double x, uint32_t& hi, uint32_t& any) {
+  const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;
+  hi = max(hi, h);
+  any |= h | (uint32_t)__double2loint(x);
+}
+
+// The biased exponent that scales a row: 0 marks a row that the digits cannot
+// hold (NaN, infinite, exponent outside the range), 1023 - 1 a zero row.
+__device__ __forceinline__ int row_field(uint32_t hi, uint32_t any) {
+  const int E = (int)(hi >> 20);
+  if (any == 0) return 1022;
+  return (E - 1022 < kMinExp || E - 1022 > kMaxExp) ? 0 : E;
+}
+
+// {exponent e, index of the last digit that is used (kNotExact: some value is cut)}
+__device__ __forceinline__ int2 row_info(int efield, uint64_t bits, bool cut) {
+  if (efield == 0) return make_int2(0, kNotExact);
+  const int z = cut ? kNotExact : (bits ? kDigits - 1 - (__ffsll((long long)bits) - 1) / 8 : 0);
+  return make_int2(efield - 1022, z);
+}
+
+struct SliceArgs {
+  F64Args g;          // operands of this panel
+  int64_t kpad;       // panel length rounded up to 64
+  uint16_t* pa;       // planes of [A; acs]: [plane][rows_a][kpad]
+  uint16_t* pb;       // planes of [B, bcs]: [plane][kpad][cols_b]
+  int2* a_row;
+  int2* b_col;
+  int* hdr;           // {status, any bad tile}
+  int64_t rows_a, cols_b, row_cs, col_cs;
+  int tpr;            // threads per row of A
+  int64_t nb, nbc, na;  // CTAs: columns of B, of bcs, rows of A (the rest: acs)
+};
+
+constexpr int kSliceThreads = 256;
+
+// One row of A per tpr threads: the largest element, then (the row again, from
+// L1 / L2) its digits.
+__device__ __forceinline__ void slice_rows(const SliceArgs& a, const double* src, int64_t ld,
+                                           int64_t rows, int64_t row_out, int64_t blk,
+                                           uint32_t* sh) {
+  const int tpr = a.tpr, q = threadIdx.x & (tpr - 1), rib = threadIdx.x / tpr;
+  const int64_t r = blk * (kSliceThreads / tpr) + rib;
+  const bool rv = r < rows;
+  const double* p = src + (rv ? r : 0) * ld;
+  const int64_t k = rv ? a.g.k : 0;
+  uint32_t hi = 0, any = 0;
+#pragma unroll 2
+  for (int64_t l = 4 * q; l < k; l += 4 * tpr) {
+    double x[4];
+    load4(p + l, k - l, x);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) take_max(x[e], hi, any);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    any |= __shfl_xor_sync(0xffffffffu, any, o);
+  }
+  const int warp = threadIdx.x >> 5, wpr = tpr / 32, w0 = rib * wpr;
+  if ((threadIdx.x & 31) == 0) {
+    sh[2 * warp] = hi;
+    sh[2 * warp + 1] = any;
+  }
+  __syncthreads();
+  for (int w = w0; w < w0 + wpr; ++w) {
+    hi = max(hi, sh[2 * w]);
+    any |= sh[2 * w + 1];
+  }
+  const int ef = row_field(hi, any);
+  const int64_t out = row_out + r, plane = a.rows_a * a.kpad;
+  uint64_t bits = 0;
+  bool cut = false;
+  if (rv) {
+    for (int64_t l = 4 * q; l < a.kpad; l += 4 * tpr) {
+      double x[4] = {0.0, 0.0, 0.0, 0.0};
+      if (ef && l < k) load4(p + l, k - l, x);
+      Digits4 D;
+      slice4(x, ef ? ef : 1022, D, bits, cut);
+      if (!ef) D.plane[kMagPlane] = make_uint2(0x7fc07fc0u, 0x7fc07fc0u);  // NaN
+      uint16_t* o = a.pa + out * a.kpad + l;
+#pragma unroll
+      for (int pl = 0; pl < kPlanes64; ++pl)
+        *reinterpret_cast<uint2*>(o + pl * plane) = D.plane[pl];
+    }
+  }
+  uint32_t b0 = (uint32_t)bits, b1 = (uint32_t)(bits >> 32), c = cut ? 1u : 0u;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    b0 |= __shfl_xor_sync(0xffffffffu, b0, o);
+    b1 |= __shfl_xor_sync(0xffffffffu, b1, o);
+    c |= __shfl_xor_sync(0xffffffffu, c, o);
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) {
+    sh[3 * warp] = b0;
+    sh[3 * warp + 1] = b1;
+    sh[3 * warp + 2] = c;
+  }
+  __syncthreads();
+  if (q == 0 && rv) {
+    for (int w = w0; w < w0 + wpr; ++w) {
+      b0 |= sh[3 * w];
+      b1 |= sh[3 * w + 1];
+      c |= sh[3 * w + 2];
+    }
+    a.a_row[out] = row_info(ef, ((uint64_t)b1 << 32) | b0, c != 0);
+  }
+}
+
+// W columns of B per CTA (four per thread), all rows of the panel: the largest
+// elements, then the digits.
+template <int W>
+__device__ __forceinline__ void slice_cols(const SliceArgs& a, const double* src, int64_t ld,
+                                           int64_t cols, int64_t col_out, int64_t blk,
+                                           uint32_t* sh) {
+  constexpr int TW = W / 4, RG = kSliceThreads / TW;
+  const int tx = threadIdx.x % TW, rg = threadIdx.x / TW;
+  const int64_t c0 = blk * W + 4 * tx, nv = cols - c0;
+  const double* p = src + c0;
+  const int64_t k = a.g.k;
+  uint32_t hi[4] = {0, 0, 0, 0}, any[4] = {0, 0, 0, 0};
+  if (nv > 0) {
+#pragma unroll 4
+    for (int64_t l = rg; l < k; l += RG) {
+      double x[4];
+      load4(p + l * ld, nv, x);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) take_max(x[e], hi[e], any[e]);
+    }
+  }
+  // sh: [2][RG][W], then the columns' exponent fields [W]
+  uint32_t* sany = sh + RG * W;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    sh[rg * W + 4 * tx + e] = hi[e];
+    sany[rg * W + 4 * tx + e] = any[e];
+  }
+  __syncthreads();
+  int* sef = reinterpret_cast<int*>(sh + 2 * RG * W);
+  if (threadIdx.x < W) {
+    uint32_t h = 0, n = 0;
+    for (int g = 0; g < RG; ++g) {
+      h = max(h, sh[g * W + threadIdx.x]);
+      n |= sany[g * W + threadIdx.x];
+    }
+    sef[threadIdx.x] = row_field(h, n);
+  }
+  __syncthreads();
+  int ef[4];
+  uint64_t bits[4] = {0, 0, 0, 0};
+  bool cut[4] = {false, false, false, false};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) ef[e] = sef[4 * tx + e];
+  const int64_t plane = a.kpad * a.cols_b;
+#pragma unroll 2
+  for (int64_t l = rg; l < a.kpad; l += RG) {
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+    if (nv > 0 && l < k) load4(p + l * ld, nv, x);
+    // the four columns have scales of their own: one digit lane at a time
+    uint32_t lane[4][kPlanes64];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int f = ef[e];
+      const double v[4] = {f ? x[e] : 0.0, 0.0, 0.0, 0.0};
+      Digits4 D;
+      slice4(v, f ? f : 1022, D, bits[e], cut[e]);
+#pragma unroll
+      for (int pl = 0; pl < kPlanes64; ++pl) lane[e][pl] = D.plane[pl].x & 0xffffu;
+      if (!f) lane[e][kMagPlane] = 0x7fc0u;
+    }
+    uint16_t* o = a.pb + l * a.cols_b + col_out + c0;
+#pragma unroll
+    for (int pl = 0; pl < kPlanes64; ++pl)
+      *reinterpret_cast<uint2*>(o + pl * plane) = make_uint2(lane[0][pl] | (lane[1][pl] << 16),
+                                                             lane[2][pl] | (lane[3][pl] << 16));
+  }
+  __syncthreads();
+  // sh again: the columns' collected bits and cuts
+  if (threadIdx.x < W) sh[threadIdx.x] = sh[W + threadIdx.x] = sh[2 * W + threadIdx.x] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    atomicOr(&sh[4 * tx + e], (uint32_t)bits[e]);
+    atomicOr(&sh[W + 4 * tx + e], (uint32_t)(bits[e] >> 32));
+    if (cut[e]) atomicOr(&sh[2 * W + 4 * tx + e], 1u);
+  }
+  __syncthreads();
+  if (threadIdx.x < W && blk * W + threadIdx.x < cols)
+    a.b_col[col_out + blk * W + threadIdx.x] =
+        row_info(sef[threadIdx.x], ((uint64_t)sh[W + threadIdx.x] << 32) | sh[threadIdx.x],
+                 sh[2 * W + threadIdx.x] != 0);
+}
+
+template <int W>
+__global__ void __launch_bounds__(kSliceThreads) k_f64_slice(const SliceArgs a) {
+  __shared__ uint32_t sh[2 * 1024 + 64];
+  if (blockIdx.x == 0 && threadIdx.x < 2 && (threadIdx.x == 1 || !a.g.accumulate))
+    a.hdr[threadIdx.x] = 0;  // the status word covers every panel
+  int64_t b = blockIdx.x;
+  if (b < a.nb) return slice_cols<W>(a, a.g.B, a.g.ldb, a.g.n, 0, b, sh);
+  b -= a.nb;
+  if (b < a.nbc) return slice_cols<W>(a, a.g.bcs, a.g.ldbcs, a.g.Cc, a.col_cs, b, sh);
+  b -= a.nbc;
+  if (b < a.na) return slice_rows(a, a.g.A, a.g.lda, a.g.m, 0, b, sh);
+  slice_rows(a, a.g.acs, a.g.ldacs, a.g.R, a.row_cs, b - a.na, sh);
+}
+
+// ------------------------------------------------------------------ product
+
+struct Maps {
+  CUtensorMap a;   // (kpad, planes x rows_a): box 64 x 128
+  CUtensorMap bw;  // (64, planes x kpad, column boxes): box 64 x 64 x bpt
+  CUtensorMap b1;  // the same, one column box
+};
+
+struct ProdArgs {
+  F64Args g;
+  TileGrid T;
+  int nkb, bpt;                  // k-steps of a panel; boxes per tile
+  int kpad, rows_a, row_cs, col_cs;
+  const int2* a_row;
+  const int2* b_col;
+  uint8_t* bad;
+  int* hdr;                      // {status, any bad tile}
+  int4* scratch;                 // per CTA: [level][chunk][8][256 epilogue threads]
+  float line6, line7;            // magnitudes that levels 0..6 / 0..7 need
+  uint64_t wait_ns;
+  int stall_test;
+};
+
+// 16 consecutive fp32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// (H 2^32 + Lo) 2^e rounded to the nearest binary64 (ties to even; the result is
+// a normal number or zero), with integer instructions only.
+__device__ __forceinline__ double round_f64(int64_t H, int64_t Lo, int e) {
+  const int64_t h = H + (Lo >> 32);
+  const uint32_t w = (uint32_t)Lo;
+  const bool neg = h < 0;
+  const uint64_t mh = neg ? ~(uint64_t)h + (w == 0 ? 1ull : 0ull) : (uint64_t)h;
+  const uint32_t ml = neg ? 0u - w : w;
+  if ((mh | ml) == 0) return 0.0;
+  uint64_t top;
+  bool rest = false;
+  int pos;  // position of the leading bit
+  if (mh) {
+    const int z = __clzll((long long)mh);
+    const uint64_t lo64 = (uint64_t)ml << 32;
+    top = z ? (mh << z) | (lo64 >> (64 - z)) : mh;
+    rest = (lo64 << z) != 0;
+    pos = 95 - z;
+  } else {
+    const int z = __clz((int)ml);
+    top = (uint64_t)ml << (32 + z);
+    pos = 31 - z;
+  }
+  const uint64_t m = top >> 11;
+  const uint32_t r = (uint32_t)top & 0x7ffu;
+  const uint64_t up = (r > 0x400u || (r == 0x400u && (rest || (m & 1)))) ? 1 : 0;
+  const uint64_t bits = ((uint64_t)(pos + e + 1022) << 52) + m + up;
+  return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
+}
+
+struct TileView64 {
+  bool cs_row, cs_col;
+  int64_t row0, col0;     // in C / E / F
+  int arow, bcol;         // padded row of the A planes, column of the B planes
+  int nbox, ncols;        // boxes and valid columns
+  int64_t rlim;
+};
+
+__device__ __forceinline__ TileView64 view_tile(const ProdArgs& p, int64_t t) {
+  int ty, tx;
+  p.T.decode(t, ty, tx);
+  TileView64 V;
+  V.cs_row = ty >= p.T.tm;
+  V.cs_col = tx >= p.T.tn;
+  V.row0 = (int64_t)(V.cs_row ? ty - p.T.tm : ty) * BM;
+  V.col0 = (int64_t)(V.cs_col ? tx - p.T.tn : tx) * 64 * p.bpt;
+  V.arow = (int)V.row0 + (V.cs_row ? p.row_cs : 0);
+  V.bcol = (int)V.col0 + (V.cs_col ? p.col_cs : 0);
+  V.rlim = V.cs_row ? p.g.R : p.g.m;
+  V.ncols = (int)min((int64_t)64 * p.bpt, (V.cs_col ? p.g.Cc : p.g.n) - V.col0);
+  V.nbox = (V.ncols + 63) / 64;
+  return V;
+}
+
+// What a tile's magnitudes ask for.
+constexpr int kNeed7 = 1, kLeave = 2;
+
+__global__ void __launch_bounds__(kThreads, 1)
+    k_gemm_f64_tc(const __grid_constant__ Maps M, const ProdArgs p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  const int NS = stages(p.bpt);
+  const uint32_t stage = kABytes + p.bpt * kBoxBytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NS * stage);
+  // full [8], empty [8], tmem full [2], tmem empty [2], drain, decision
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 6);
+  volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* need = reinterpret_cast<volatile int*>(tmem_slot + 2);  // [2][kEpiWarps]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto full = [&](int s) { return tc::smem_addr(&bars[s]); };
+  auto empty = [&](int s) { return tc::smem_addr(&bars[kMaxStages + s]); };
+  auto tfull = [&](int a) { return tc::smem_addr(&bars[2 * kMaxStages + a]); };
+  auto tempty = [&](int a) { return tc::smem_addr(&bars[2 * kMaxStages + 2 + a]); };
+  const uint32_t drain = tc::smem_addr(&bars[2 * kMaxStages + 4]);
+  const uint32_t decided = tc::smem_addr(&bars[2 * kMaxStages + 5]);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NS; ++s) {
+      tc::mbar_init(full(s), 2);
+      tc::mbar_init(empty(s), 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      tc::mbar_init(tfull(a), 1);
+      tc::mbar_init(tempty(a), kEpiWarps);
+    }
+    tc::mbar_init(drain, 1);
+    tc::mbar_init(decided, kEpiWarps);
+    *abort = 0;
+    tc::wait_limit_ns() = p.wait_ns;
+    tc::fence_barrier_init();
+    tc::prefetch_tmap(&M.a);
+    tc::prefetch_tmap(&M.bw);
+    tc::prefetch_tmap(&M.b1);
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(tc::smem_addr(tmem_slot), 512);
+    tc::tmem_relinquish();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+  const int64_t total = p.T.total();
+  const int nkb = p.nkb;
+  // the tile's decision, known to every role before its level 7 (phase: tile parity)
+  auto decision = [&](uint32_t par) {
+    int f = 0;
+    for (int w = 0; w < kEpiWarps; ++w) f |= need[par * kEpiWarps + w];
+    return f;
+  };
+  auto last_level = [](int f) { return (f & kNeed7) && !(f & kLeave) ? 7 : 6; };
+
+  if (warp == 0 || warp == kWarpProdB) {
+    if (lane == 0) {
+      const bool pA = warp == 0;
+      int s = 0;
+      uint32_t ph = 0, par = 0;
+      int64_t issued = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < total && ok && !*abort; t += gridDim.x, par ^= 1) {
+        if (p.stall_test && t == 0) continue;
+        const TileView64 V = view_tile(p, t);
+        const uint32_t tx = pA ? kABytes : (uint32_t)V.nbox * kBoxBytes;
+        // one pair of planes: nkb k-steps
+        auto pair = [&](int pa, int pb) {
+          const int arow = pa * p.rows_a + V.arow, brow = pb * p.kpad, cb = V.bcol / 64;
+          for (int kb = 0; kb < nkb; ++kb) {
+            if (!tc::wait(empty(s), ph ^ 1, abort)) return false;
+            const uint32_t sa = tc::smem_addr(smem + s * stage);
+            tc::mbar_arrive_expect_tx(full(s), tx);
+            if (pA) {
+              tc::tma_load_2d(sa, &M.a, full(s), kb * BK, arow);
+            } else if (V.nbox == p.bpt) {
+              tc::tma_load_3d(sa + kABytes, &M.bw, full(s), 0, brow + kb * BK, cb);
+            } else {
+              for (int b = 0; b < V.nbox; ++b)
+                tc::tma_load_3d(sa + kABytes + b * kBoxBytes, &M.b1, full(s), 0, brow + kb * BK,
+                                cb + b);
+            }
+            ++issued;
+            if (++s == NS) { s = 0; ph ^= 1; }
+          }
+          return true;
+        };
+        ok = pair(kMagPlane, kMagPlane);
+        int top = 6;
+        for (int lev = 0; lev <= top && ok; ++lev) {
+          for (int i = 0; i <= lev && ok; ++i) ok = pair(i, lev - i);
+          if (lev == 6 && ok) {
+            ok = tc::wait(decided, par, abort);
+            if (ok) top = last_level(decision(par));
+          }
+        }
+      }
+      // no copies left in flight (bounded)
+      for (int q = 0; q < NS && issued > 0; ++q, --issued) {
+        if (--s < 0) { s = NS - 1; ph ^= 1; }
+        const uint64_t t0 = tc::globaltimer();
+        while (!tc::mbar_try_wait(full(s), ph) && tc::globaltimer() - t0 < tc::wait_limit_ns()) {
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int s = 0, acc = 0;
+      uint32_t ph = 0, aph = 0, par = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < total && ok && !*abort; t += gridDim.x, par ^= 1) {
+        const TileView64 V = view_tile(p, t);
+        const uint32_t idesc = tc::idesc_bf16(BM, (V.ncols + 15) / 16 * 16, 1);
+        // nk k-steps in accumulators of g each
+        auto level = [&](int nk, int g) {
+          for (int k0 = 0; k0 < nk; k0 += g) {
+            if (!tc::wait(tempty(acc), aph ^ 1, abort)) return false;
+            tc::fence_after_sync();
+            const uint32_t d = tmem + acc * 256;
+            const int k1 = min(k0 + g, nk);
+            for (int kb = k0; kb < k1; ++kb) {
+              if (!tc::wait(full(s), ph, abort)) return false;
+              tc::fence_after_sync();
+              const uint32_t sa = tc::smem_addr(smem + s * stage), sb = sa + kABytes;
+#pragma unroll
+              for (int kk = 0; kk < BK / 16; ++kk)
+                tc::mma_f16(d, tc::sdesc_sw128(sa + kk * 32, 16, 1024),
+                            tc::sdesc_sw128(sb + kk * 2048, kBoxBytes, 1024), idesc,
+                            (kb > k0 || kk > 0) ? 1u : 0u);
+              tc::commit(empty(s));
+              if (++s == NS) { s = 0; ph ^= 1; }
+            }
+            tc::commit(tfull(acc));
+            if (++acc == 2) { acc = 0; aph ^= 1; }
+          }
+          return true;
+        };
+        ok = level(nkb, nkb);
+        int top = 6;
+        for (int lev = 0; lev <= top && ok; ++lev) {
+          ok = level((lev + 1) * nkb, kGroupSteps);
+          if (lev == 6 && ok) {
+            ok = tc::wait(decided, par, abort);
+            if (ok) top = last_level(decision(par));
+          }
+        }
+      }
+      tc::commit(drain);  // every MMA has completed before TMEM is freed
+      const uint64_t t0 = tc::globaltimer();
+      while (!tc::mbar_try_wait(drain, 0) && tc::globaltimer() - t0 < tc::wait_limit_ns()) {
+      }
+    }
+    __syncwarp();
+  } else {
+    // epilogue: TMEM lane quarter q = warp % 4, column half (warp - 2) / 4
+    const int q = warp & 3, half = (warp - 2) >> 2, ew = warp - 2, et = ew * 32 + lane;
+    const int nch = p.bpt, c_lo = half * 32 * nch;  // 32-column chunks per warp
+    int4* const scr = p.scratch + (int64_t)blockIdx.x * kLevels * nch * 8 * 256 + et;
+    int acc = 0;
+    uint32_t aph = 0, par = 0;
+    bool ok = true;
+    const uint32_t lanes = (uint32_t)(q * 32) << 16;
+    // the same answer in every lane, and the warp converged after it
+    auto wait_all = [&](uint32_t bar, uint32_t ph) {
+      return __all_sync(0xffffffffu, tc::wait(bar, ph, abort)) != 0;
+    };
+    auto release = [&]() {
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(tempty(acc));
+      if (++acc == 2) { acc = 0; aph ^= 1; }
+    };
+    for (int64_t t = blockIdx.x; t < total && ok; t += gridDim.x, par ^= 1) {
+      const TileView64 V = view_tile(p, t);
+      const int64_t row = V.row0 + 32 * q + lane;
+      const bool rv = row < V.rlim;
+      const int2 ri = rv ? p.a_row[V.arow + 32 * q + lane] : make_int2(0, 0);
+      const int c_hi = min(c_lo + 32 * nch, V.ncols);  // this warp's valid columns
+      // ---- magnitudes: what the tile needs
+      int zr = ri.y, zc = 0;
+      for (int c = c_lo + lane; c < c_hi; c += 32) zc = max(zc, p.b_col[V.bcol + c].y);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        zr = max(zr, __shfl_xor_sync(0xffffffffu, zr, o));
+        zc = max(zc, __shfl_xor_sync(0xffffffffu, zc, o));
+      }
+      if (!wait_all(tfull(acc), aph)) { ok = false; break; }
+      tc::fence_after_sync();
+      int f = 0;
+      for (int c = c_lo; c < c_hi; c += 16) {
+        float v[16];
+        tmem_ld16(tmem + lanes + acc * 256 + c, v);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          if (rv && c + u < c_hi && v[u] != 0.0f) {  // NaN: neither line is reached
+            if (!(v[u] >= p.line6)) f |= kNeed7;
+            if (!(v[u] >= p.line7)) f |= kLeave;
+          }
+        }
+      }
+      release();
+      if (zr + zc <= 6) f = 0;               // no digit product is cut
+      else if (zr + zc <= 7) f = f ? kNeed7 : 0;
+      f = (__any_sync(0xffffffffu, f & kNeed7) ? kNeed7 : 0) |
+          (__any_sync(0xffffffffu, f & kLeave) ? kLeave : 0);
+      if (lane == 0) {
+        need[par * kEpiWarps + ew] = f;
+        __threadfence_block();
+        tc::mbar_arrive(decided);
+      }
+      // ---- levels
+      int top = 6;
+      f = 0;
+      for (int lev = 0; lev <= top && ok; ++lev) {
+        int sum[4][32];
+#pragma unroll
+        for (int ci = 0; ci < 4; ++ci)
+#pragma unroll
+          for (int u = 0; u < 32; ++u) sum[ci][u] = 0;
+        const int nk = (lev + 1) * nkb;
+        for (int k0 = 0; k0 < nk; k0 += kGroupSteps) {
+          if (!wait_all(tfull(acc), aph)) { ok = false; break; }
+          tc::fence_after_sync();
+          const uint32_t base = tmem + lanes + acc * 256 + c_lo;
+#pragma unroll
+          for (int ci = 0; ci < 4; ++ci) {
+            if (ci < nch && c_lo + 32 * ci < c_hi) {
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                float v[16];
+                tmem_ld16(base + 32 * ci + 16 * h, v);
+#pragma unroll
+                for (int u = 0; u < 16; ++u) sum[ci][16 * h + u] += __float2int_rn(v[u]);
+              }
+            }
+          }
+          release();
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int ci = 0; ci < 4; ++ci)
+          if (ci < nch && c_lo + 32 * ci < c_hi) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              scr[(int64_t)((lev * nch + ci) * 8 + j) * 256] =
+                  make_int4(sum[ci][4 * j], sum[ci][4 * j + 1], sum[ci][4 * j + 2],
+                            sum[ci][4 * j + 3]);
+          }
+        if (lev == 6) {
+          ok = wait_all(decided, par);
+          if (ok) {
+            f = decision(par);
+            top = last_level(f);
+          }
+        }
+      }
+      if (!ok) break;
+      if (ew == 0 && lane == 0) {
+        p.bad[t] = (f & kLeave) ? 1 : 0;
+        if (f & kLeave) atomicExch(&p.hdr[1], 1);
+      }
+      const int c_end = !(f & kLeave) && rv ? c_hi : 0;
+      // ---- the levels together, rounded once
+      double* const dst = (V.cs_row ? p.g.E : (V.cs_col ? p.g.F : p.g.C)) +
+                          row * (V.cs_row ? p.g.lde : (V.cs_col ? p.g.ldf : p.g.ldc)) + V.col0;
+#pragma unroll 1
+      for (int cj = 0; cj < 8 * nch; ++cj) {
+        const int c = c_lo + 4 * cj;
+        if (c >= c_end) break;
+        int L[kLevels][4];
+#pragma unroll
+        for (int s = 0; s < kLevels; ++s) {
+          const int4 x = s <= top ? scr[(int64_t)(s * nch * 8 + cj) * 256] : make_int4(0, 0, 0, 0);
+          L[s][0] = x.x; L[s][1] = x.y; L[s][2] = x.z; L[s][3] = x.w;
+        }
+        double o[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int64_t H = ((int64_t)L[0][u] << 24) + ((int64_t)L[1][u] << 16) +
+                            ((int64_t)L[2][u] << 8) + L[3][u];
+          const int64_t Lo = ((int64_t)L[4][u] << 24) + ((int64_t)L[5][u] << 16) +
+                             ((int64_t)L[6][u] << 8) + L[7][u];
+          const int eb = c + u < c_hi ? p.b_col[V.bcol + c + u].x : 0;
+          o[u] = round_f64(H, Lo, ri.x + eb - 70);
+        }
+        double* const d = dst + c;
+        if (p.g.accumulate) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (c + u < c_hi) o[u] += d[u];
+        }
+        if (c + 4 <= c_hi && (reinterpret_cast<uintptr_t>(d) & 15) == 0) {
+          *reinterpret_cast<double2*>(d) = make_double2(o[0], o[1]);
+          *reinterpret_cast<double2*>(d + 2) = make_double2(o[2], o[3]);
+        } else {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (c + u < c_hi) d[u] = o[u];
+        }
+      }
+      __syncwarp();
+    }
+  }
+
+  tc::fence_before_sync();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort) atomicExch(&p.hdr[0], 1);
+  if (warp == 1) {
+    tc::fence_after_sync();
+    tc::tmem_dealloc(tmem, 512);
+  }
+}
+
+size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+TileGrid tile_grid(int64_t m, int64_t n, int64_t R, int64_t Cc, int bpt) {
+  return TileGrid{(int)cdiv(m, BM), (int)cdiv(n, 64 * bpt), (int)cdiv(R, BM),
+                  (int)cdiv(Cc, 64 * bpt), 16};
+}
+
+}  // namespace
+
+bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, size_t* bytes) {
+  // Below 128^3 both paths are bound by their launches and latencies.
+  if (d.k < 1 || (double)d.m * (double)d.n * (double)d.k < 2097152.0) return false;
+  F64TcRegions& r = *rg;
+  r.row_cs = cdiv(d.m, BM) * BM;
+  r.rows_a = r.row_cs + cdiv(R, BM) * BM;
+  r.col_cs = cdiv(d.n, 256) * 256;
+  r.cols_b = r.col_cs + cdiv(Cc, 256) * 256;
+  // Panels of K: a level sum stays within 32 bits, the planes within a budget.
+  const int64_t per_k = (r.rows_a + r.cols_b) * kPlanes64 * 2;
+  const int64_t fit = (int64_t)(kPlaneBudget / per_k) / BK * BK;
+  r.kp = std::min<int64_t>({cdiv(d.k, BK) * BK, kMaxPanel, std::max<int64_t>(fit, BK)});
+  // Tile width: clocks per k-step (MMA 512 / 256 for four / two boxes; one box is
+  // bound by the 24 KiB that its operands read from shared memory) times waves.
+  const int clocks[3] = {192, 256, 512};
+  double best = 0;
+  for (int i = 2; i >= 0; --i) {
+    const int64_t t = tile_grid(d.m, d.n, R, Cc, 1 << i).total();
+    const double cost = (double)clocks[i] * cdiv(t, kSms);
+    if (i == 2 || cost < best) {
+      best = cost;
+      r.bpt = 1 << i;
+    }
+  }
+  const int64_t tiles = tile_grid(d.m, d.n, R, Cc, r.bpt).total();
+  const int64_t ctas = std::min<int64_t>(tiles, kSms);
+  size_t off = 0;
+  auto region = [&](size_t b) {
+    const size_t o = off;
+    off = align256(off + b);
+    return o;
+  };
+  r.a_planes = region((size_t)kPlanes64 * r.rows_a * r.kp * 2);
+  r.b_planes = region((size_t)kPlanes64 * r.cols_b * r.kp * 2);
+  r.a_row = region(sizeof(int2) * r.rows_a);
+  r.b_col = region(sizeof(int2) * r.cols_b);
+  r.bad = region((size_t)tiles);
+  r.scratch = region((size_t)ctas * kLevels * r.bpt * 8 * 256 * sizeof(int4));
+  *bytes = off;
+  return true;
+}
+
+cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaStream_t st) {
+  const F64TcRegions& r = P.f64tc;
+  char* w = static_cast<char*>(ws) + P.f64tc_base;
+  int* hdr = reinterpret_cast<int*>(static_cast<char*>(ws) + P.f64tc_hdr);
+  const TileGrid T = tile_grid(g.m, g.n, g.R, g.Cc, r.bpt);
+  const char* stall = getenv("ABFT_TEST_STALL_PRODUCER");
+  cudaError_t e = cudaFuncSetAttribute(k_gemm_f64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem_bytes(r.bpt));
+  for (int64_t k0 = 0; k0 < g.k && e == cudaSuccess; k0 += r.kp) {
+    F64Args gp = g;
+    gp.k = std::min(r.kp, g.k - k0);
+    gp.A += k0;
+    gp.B += k0 * g.ldb;
+    if (g.R) gp.acs += k0;
+    if (g.Cc) gp.bcs += k0 * g.ldbcs;
+    gp.accumulate = k0 > 0;
+    const int64_t kpad = cdiv(gp.k, BK) * BK;
+
+    SliceArgs a{};
+    a.g = gp;
+    a.kpad = kpad;
+    a.pa = reinterpret_cast<uint16_t*>(w + r.a_planes);
+    a.pb = reinterpret_cast<uint16_t*>(w + r.b_planes);
+    a.a_row = reinterpret_cast<int2*>(w + r.a_row);
+    a.b_col = reinterpret_cast<int2*>(w + r.b_col);
+    a.hdr = hdr;
+    a.rows_a = r.rows_a; a.cols_b = r.cols_b; a.row_cs = r.row_cs; a.col_cs = r.col_cs;
+    a.tpr = 32;
+    while (a.tpr < kSliceThreads && a.tpr * 8 < kpad) a.tpr *= 2;
+    const int rpc = kSliceThreads / a.tpr;
+    const int W = g.n <= 16 * kSms ? 16 : 32;
+    a.nb = cdiv(g.n, W);
+    a.nbc = cdiv(g.Cc, W);
+    a.na = cdiv(g.m, rpc);
+    const unsigned grid = (unsigned)(a.nb + a.nbc + a.na + cdiv(g.R, rpc));
+    if (W == 16)
+      k_f64_slice<16><<<grid, kSliceThreads, 0, st>>>(a);
+    else
+      k_f64_slice<32><<<grid, kSliceThreads, 0, st>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) break;
+
+    Maps M;
+    e = make_bf16_map(&M.a, a.pa, kPlanes64 * r.rows_a, kpad, kpad, BK, BM);
+    if (e == cudaSuccess)
+      e = make_bf16_map_boxes(&M.bw, a.pb, kPlanes64 * kpad, r.cols_b, r.cols_b, r.bpt);
+    if (e == cudaSuccess)
+      e = make_bf16_map_boxes(&M.b1, a.pb, kPlanes64 * kpad, r.cols_b, r.cols_b, 1);
+    if (e != cudaSuccess) break;
+    ProdArgs p{};
+    p.g = gp;
+    p.T = T;
+    p.nkb = (int)(kpad / BK);
+    p.bpt = r.bpt;
+    p.kpad = (int)kpad; p.rows_a = (int)r.rows_a; p.row_cs = (int)r.row_cs;
+    p.col_cs = (int)r.col_cs;
+    p.a_row = a.a_row;
+    p.b_col = a.b_col;
+    p.bad = reinterpret_cast<uint8_t*>(w + r.bad);
+    p.hdr = hdr;
+    p.scratch = reinterpret_cast<int4*>(w + r.scratch);
+    p.line6 = (float)(0.405 * sqrt((double)gp.k));
+    p.line7 = (float)(0.0016 * sqrt((double)gp.k));
+    p.stall_test = stall && stall[0] == '1';
+    p.wait_ns = p.stall_test ? 200000000ull : tc::kWaitLimitNs;
+    const unsigned ctas = (unsigned)std::min<int64_t>({T.total(), kSms, num_sms()});
+    k_gemm_f64_tc<<<ctas, kThreads, smem_bytes(r.bpt), st>>>(M, p);
+    if ((e = cudaGetLastError()) != cudaSuccess) break;
+    e = launch_gemm_f64_bad(gp, T, r.bpt, hdr + 1, p.bad, st);
+    count_launches(2);
+  }
+  return e;
+}
+
+}  // namespace abft

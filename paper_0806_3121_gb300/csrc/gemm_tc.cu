@@ -1541,7 +1541,6 @@ int64_t cs_stride(int64_t ncs, int64_t total, int grid) {
 // once: the persistent grid's size.  Clusters are placed within a GPC, so this
 // can be less than half the SM count.
 int g_pair_clusters[64] = {};
-int num_sms();
 int pair_clusters(const void* kernel, size_t smem) {
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1566,6 +1565,8 @@ int pair_clusters(const void* kernel, size_t smem) {
   return n;
 }
 
+}  // namespace
+
 int num_sms() {
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1577,8 +1578,6 @@ int num_sms() {
   }
   return g_num_sms[dev];
 }
-
-}  // namespace
 
 // Timeout word of checksum-free products run without a workspace.
 __device__ int g_tc_timeout_fallback = 0;

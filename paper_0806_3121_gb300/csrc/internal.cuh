@@ -71,6 +71,19 @@ struct Erased {
   int32_t bi[kMaxErased], bj[kMaxErased];
 };
 
+// Workspace regions of the sliced binary64 product (gemm_f64_tc.cu), byte
+// offsets from Plan::f64tc_base.
+struct F64TcRegions {
+  size_t a_planes, b_planes;  // bf16 digit planes of [A; acs] and [B, bcs], one panel of K
+  size_t a_row, b_col;        // int2 {exponent, last digit used} per row / column
+  size_t bad;                 // one byte per tile: left to the DFMA kernel
+  size_t scratch;             // per CTA: the level sums of its tile
+  int64_t kp;                 // longest panel of K
+  int64_t rows_a, cols_b;     // padded rows of [A; acs], columns of [B, bcs]
+  int64_t row_cs, col_cs;     // first padded checksum row / column
+  int bpt;                    // 64-column boxes per tile
+};
+
 // Everything the device code needs to know about one problem.
 struct Plan {
   abft_desc d;
@@ -86,6 +99,11 @@ struct Plan {
   // sums over column groups of g = min(vb_cols, 128) columns.
   int fused;
   int64_t g, ngrp, ntr_obs;
+  // Binary64: the product runs sliced on the tensor cores when a workspace is
+  // given; f64tc_hdr: its {status, any tile left to DFMA} words
+  int tc64;
+  F64TcRegions f64tc;
+  size_t f64tc_hdr, f64tc_base;
   abft_ws_layout L;
 };
 
@@ -111,6 +129,13 @@ Scratch scratch_view(const Plan& P, void* ws);
 size_t scratch_bytes(const Plan& P);
 
 __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// Multiprocessors of the current device.
+int num_sms();
+
+// Whether the binary64 product of d runs sliced on the tensor cores, and its
+// workspace regions.
+bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, size_t* bytes);
 
 // Host-side count of kernel launches (abft_kernel_launches()).
 void count_launches(int64_t n);

@@ -44,10 +44,13 @@ struct CheckArgs {
   int32_t* cnt;
   abft_fault* report;
   CandEntry* cand;
-  // status word of the workspace's last tensor-core product (nullptr for
-  // binary64): when that product timed out, C is incomplete and nothing is
+  // status word of the workspace's last tensor-core product (nullptr for a
+  // DFMA product): when that product timed out, C is incomplete and nothing is
   // located or corrected
   const int32_t* timeout;
+  // sliced binary64 product: the counter that the host reads it from (its own
+  // word lies outside the scratch)
+  int32_t* status_out;
 };
 
 template <typename TC>
@@ -209,6 +212,8 @@ __global__ void __launch_bounds__(kThreads) k_col_check(const CheckArgs a, int64
                                                         int64_t j_end, int64_t I_begin,
                                                         int64_t I_end, int mode) {
   const int64_t j = j_begin + (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (mode == 1 && a.status_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+    *a.status_out = *a.timeout;
   if (j >= j_end) return;
   for (int64_t I = I_begin + blockIdx.y; I < I_end; I += gridDim.y) {
     const int64_t i0 = I * a.vb_r, i1 = min(i0 + (int64_t)a.vb_r, a.m);
@@ -652,6 +657,7 @@ __device__ __forceinline__ void locate_body(const Pol& A, int32_t* cnt, const Fl
 
 template <typename TC>
 __global__ void __launch_bounds__(kLocThreads, 1) k_locate_correct(const CheckArgs a) {
+  if (a.status_out && threadIdx.x == 0) *a.status_out = *a.timeout;
   if (a.timeout && *a.timeout) return;  // an incomplete product: write nothing
   const SinglePol<TC> A{a};
   locate_body(A, a.cnt, a.colf, a.rowf, a.cand, a.report);
@@ -1076,7 +1082,12 @@ CheckArgs make_args(const Plan& P, void* C, void* ws) {
   a.nvr = P.nvr; a.nvc = P.nvc; a.Cc = P.Cc; a.bs = P.bs; a.bc = P.bc;
   a.s = P.s; a.f1c = P.f1_col; a.f2c = P.f2_col; a.f1r = P.f1_row; a.f2r = P.f2_row;
   a.colf = S.colf; a.rowf = S.rowf; a.cnt = S.cnt; a.report = S.report; a.cand = S.cand;
-  a.timeout = P.d.dtype == ABFT_F64 ? nullptr : S.cnt + kCntTimeout;
+  if (P.d.dtype != ABFT_F64) {
+    a.timeout = S.cnt + kCntTimeout;
+  } else if (P.tc64) {
+    a.timeout = reinterpret_cast<const int32_t*>(w + P.f64tc_hdr);
+    a.status_out = S.cnt + kCntTimeout;
+  }
   return a;
 }
 
