@@ -166,7 +166,7 @@ abft_status make_plan(const abft_desc* d, Plan* P) {
   L.car_b = region((size_t)2 * p.nvc * 8);
   size_t f64tc_bytes = 0;
   p.tc64 = d->dtype == ABFT_F64 && plan_f64_tc(*d, p.R, p.Cc, &p.f64tc, &f64tc_bytes);
-  p.f64tc_hdr = region(p.tc64 ? 256 : 0);  // after car_b: cleared with it
+  p.f64tc_hdr = region(p.tc64 ? 256 : 0);
   p.f64tc_base = region(f64tc_bytes);
   L.E16 = region(lp ? (size_t)L.acs_rows * d->n * 4 : 0);
   L.F16 = region(lp ? (size_t)d->m * L.bcs_cols * 4 : 0);
@@ -214,10 +214,11 @@ bool is_empty(const Plan& P) { return P.d.m == 0 || P.d.n == 0; }
 // on it and no operand has been found inexact.
 cudaError_t clear_carry(const Plan& P, void* ws, cudaStream_t st) {
   char* w = static_cast<char*>(ws);
-  // car_a, car_b and the sliced product's status words are adjacent regions
-  const size_t end = P.tc64 ? P.f64tc_hdr + 8 : P.L.car_b + sizeof(double) * 2 * P.nvc;
-  cudaError_t e = cudaMemsetAsync(w + P.L.car_a, 0, end - P.L.car_a, st);
-  if (e == cudaSuccess && P.d.dtype != ABFT_F64)
+  if (P.d.dtype == ABFT_F64) return cudaSuccess;  // its encode kernel clears them
+  // car_a and car_b are adjacent regions
+  cudaError_t e = cudaMemsetAsync(
+      w + P.L.car_a, 0, P.L.car_b + sizeof(double) * 2 * P.nvc - P.L.car_a, st);
+  if (e == cudaSuccess)
     e = cudaMemsetAsync(w + P.L.scratch + sizeof(int32_t) * kCntTimeout, 0,
                         sizeof(int32_t) * (kCntFp8Inexact - kCntTimeout + 1), st);
   return e;

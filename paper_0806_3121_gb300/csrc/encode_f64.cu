@@ -1,7 +1,21 @@
 // Checksum encoding for binary64 operands (section 2.1; the encoded operands
-// of Eq. (1)).  All kernels stream A or B once per quantity with coalesced
-// loads; reductions along the long dimension are two-stage (per-chunk
-// partials, then an ordered sum) so the result does not depend on scheduling.
+// of Eq. (1)) in two launches: k_enc64 streams A and B (each CTA takes a unit of
+// one of five passes), k_enc64_norms forms the threshold norms from what it
+// left.  Every sum has a fixed order, so the results do not depend on scheduling.
+//
+// Bound: the FP64 pipe (2 results per clock and SM).  Per element of A: e sum, w
+// sum, row square, block checksum; per element of B: e sum, w sum, column square
+// -- so the passes avoid every other binary64 instruction (weights come from a
+// table instead of conversions, the warp sums of four rows of B share one
+// transposing butterfly, the row squares run in a pass of their own whose lanes
+// add 1 / 32 of a row before they meet: one reduction per 32 x 32 elements would
+// cost as much as the squares).  The passes read A three times and B twice, which
+// HBM has room for.  Small problems are bound by latency instead: a verify block's
+// rows are split into 64-row segments over the warps of a CTA and eight rows of
+// loads are in flight per thread.  Measured (all launches of an encode): see
+// kEncodeTimes below.
+
+#include <algorithm>
 
 #include "internal.cuh"
 
@@ -9,7 +23,10 @@ namespace abft {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kRowsPerWarpB = 64;  // rows of B per warp in the row-checksum pass
+constexpr int kWarps = kThreads / 32;
+constexpr int kSegRows = 64;    // rows per segment of a verify block (A column sums)
+constexpr int kSqRows = 256;    // rows per column-square partial of B
+constexpr int kRowsB = 4;       // rows of B per warp in the row-checksum pass
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -26,212 +43,277 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x == 0)
-    for (int q = 0; q < kThreads / 32; ++q) t += sh[q];
+    for (int q = 0; q < kWarps; ++q) t += sh[q];
   return t;
 }
 
-// Column checksums of A per verify block: acs[2I] = e^T A_I, acs[2I+1] =
-// w^T A_I, plus per-chunk partials of ||e^T A_I||^2 and ||w^T A_I||^2 at
-// part[(2I + c) * nch + chunk].  Grid (ceil(k/256), <= 65535); thread = one
-// column l of A.
-__global__ void __launch_bounds__(kThreads) k_encA_cols(const double* __restrict__ A, int64_t lda,
-                                                        int64_t m, int64_t k, int vb, int e,
-                                                        double* __restrict__ acs,
-                                                        double* __restrict__ part, int nch) {
-  __shared__ double sh[kThreads / 32];
-  const int64_t l = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  const int64_t nvb = cdiv(m, vb);
-  const double sc = scalbn(1.0, -e);
-  for (int64_t I = blockIdx.y; I < nvb; I += gridDim.y) {
-    const int64_t i0 = I * vb, i1 = min(i0 + (int64_t)vb, m);
-    double se = 0.0, sw = 0.0;
-    if (l < k) {
-      const double* p = A + i0 * lda + l;
-#pragma unroll 4
-      for (int64_t i = i0; i < i1; ++i) {
-        const double a = p[(i - i0) * lda];
-        se += a;
-        sw = fma((double)(i - i0 + 1) * sc, a, sw);
-      }
-      acs[(2 * I) * k + l] = se;
-      acs[(2 * I + 1) * k + l] = sw;
-    }
-    const double q[2] = {se * se, sw * sw};
+struct EncArgs {
+  const double* A;
+  const double* B;
+  int64_t lda, ldb, m, n, k;
+  int vb_r, vb_c, er, ec;
+  int64_t nvr, nvc, Cc;
+  double* acs;     // 2 nvr rows of k: e^T A_I, w^T A_I
+  double* S;       // f bs rows of k: block checksums
+  double* bcs;     // k rows of Cc: B_J e, B_J w
+  double* nArow;
+  double* colsq;   // [ceil(k / 256)][n] partial column squares of B
+  int p, f;
+  int64_t bs;
+  double* car_a;   // cleared: a fresh encode carries no deviation
+  double* car_b;
+  int32_t* status; // sliced product: its status word, cleared
+  int wpu;         // warps that share a verify block's rows
+  // CTAs of the passes, in this order (0: the pass is not wanted)
+  int64_t n_acols, n_brows, n_ablk, n_bsq, n_arows;
+};
+
+// Column checksums of A: unit = 32 columns x one verify block, its rows in
+// wpu contiguous parts, one per warp; acs[2I] = e^T A_I, acs[2I+1] = w^T A_I.
+// Blocks of up to 64 rows are summed in row order by one warp.
+__device__ __forceinline__ void enc_acols(const EncArgs& a, int64_t blk, double* sh,
+                                          const double* wtab) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t nck = cdiv(a.k, 32), u = blk * (kWarps / a.wpu) + warp / a.wpu;
+  const int part = warp % a.wpu;
+  const bool uv = u < a.nvr * nck;
+  const int64_t I = uv ? u / nck : 0, l = (uv ? u % nck : 0) * 32 + lane;
+  const int64_t i0 = I * a.vb_r, i1 = min(i0 + (int64_t)a.vb_r, a.m);
+  const int64_t len = max((int64_t)kSegRows, cdiv(a.vb_r, a.wpu));  // rows of a part
+  const int64_t b0 = i0 + part * len, b1 = min(b0 + len, i1);
+  const double sc = scalbn(1.0, -a.er);
+  double se = 0.0, sw = 0.0;
+  if (uv && l < a.k) {
+    for (int64_t s0 = b0; s0 < b1; s0 += kSegRows) {
+      const int nr = (int)min((int64_t)kSegRows, b1 - s0);
+      const double* q = a.A + s0 * a.lda + l;
+      double e = 0.0, w = 0.0;
+      int t = 0;
+      for (; t + 8 <= nr; t += 8) {
+        double x[8];
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const double t = block_sum(q[c], sh);
-      if (threadIdx.x == 0) part[(2 * I + c) * nch + blockIdx.x] = t;
+        for (int r = 0; r < 8; ++r) x[r] = q[(t + r) * a.lda];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          e += x[r];
+          w = fma(wtab[t + r], x[r], w);
+        }
+      }
+      for (; t < nr; ++t) {
+        const double x = q[t * a.lda];
+        e += x;
+        w = fma(wtab[t], x, w);
+      }
+      sw = fma((double)(s0 - i0) * sc, e, sw + w);
+      se += e;
     }
+  }
+  if (a.wpu > 1) {
+    sh[warp * 64 + lane] = se;
+    sh[warp * 64 + 32 + lane] = sw;
+    __syncthreads();
+    if (part == 0)
+      for (int w = warp + 1; w < warp + a.wpu; ++w) {
+        se += sh[w * 64 + lane];
+        sw += sh[w * 64 + 32 + lane];
+      }
+  }
+  if (part == 0 && uv && l < a.k) {
+    a.acs[(2 * I) * a.k + l] = se;
+    a.acs[(2 * I + 1) * a.k + l] = sw;
   }
 }
 
-// Block checksum rows S_A[t] = sum_I A[I*bs + t] (erasure grid).
-// Grid (ceil(k/256), bs).
-__global__ void __launch_bounds__(kThreads) k_encA_block(const double* __restrict__ A, int64_t lda,
-                                                         int64_t k, int p, int64_t bs, int f,
-                                                         double* __restrict__ S) {
-  const int64_t l = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (l >= k) return;
-  // row c*bs + t of S: sum_I c_{c,I} A[I*bs + t] (block checksum c of the grid)
-  for (int64_t ct = blockIdx.y; ct < f * bs; ct += gridDim.y) {
-    const int c = (int)(ct / bs);
-    const int64_t t = ct - c * bs;
-    double s = 0.0;
-    for (int I = 0; I < p; ++I) s += block_coef(c, I, p) * A[(I * bs + t) * lda + l];
-    S[ct * k + l] = s;
+// Row checksums of B: a warp takes kRowsB rows x one verify block,
+// bcs[l][2J] = B_J e, bcs[l][2J+1] = B_J w.
+__device__ __forceinline__ void enc_brows(const EncArgs& a, int64_t blk) {
+  const int lane = threadIdx.x & 31;
+  const int64_t u = blk * kWarps + (threadIdx.x >> 5);
+  const int64_t l0 = u / a.nvc * kRowsB, J = u % a.nvc;
+  if (l0 >= a.k) return;
+  const int64_t j0 = J * a.vb_c;
+  const int len = (int)(min(j0 + (int64_t)a.vb_c, a.n) - j0);
+  const int nr = (int)min((int64_t)kRowsB, a.k - l0);
+  const double* q = a.B + l0 * a.ldb + j0;
+  double v[2 * kRowsB];  // e sums, then w sums
+#pragma unroll
+  for (int r = 0; r < 2 * kRowsB; ++r) v[r] = 0.0;
+  const double sc = scalbn(1.0, -a.ec), step = 32.0 * sc;
+  double w = (double)(lane + 1) * sc;
+#pragma unroll 4
+  for (int t = lane; t < len; t += 32) {
+#pragma unroll
+    for (int r = 0; r < kRowsB; ++r) {
+      const double x = r < nr ? q[r * a.ldb + t] : 0.0;
+      v[r] += x;
+      v[kRowsB + r] = fma(w, x, v[kRowsB + r]);
+    }
+    w += step;
+  }
+  // sums over the lanes, eight values at once: lane l ends with value l / 4
+#pragma unroll
+  for (int s = 16, h = kRowsB; h >= 1; s >>= 1, h >>= 1) {
+    const bool upper = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double send = upper ? v[i] : v[i + h];
+      v[i] = (upper ? v[i + h] : v[i]) + __shfl_xor_sync(0xffffffffu, send, s);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  const int idx = lane >> 2, r = idx % kRowsB, c = idx / kRowsB;
+  if ((lane & 3) == 0 && r < nr)
+    a.bcs[(l0 + r) * a.Cc + 2 * J + c] = v[0];
+}
+
+// Block checksum rows: row c bs + t of S = sum_I c_{c,I} A[I bs + t] (c < f).
+__device__ __forceinline__ void enc_ablk(const EncArgs& a, int64_t blk, double* sh) {
+  const int64_t nck = cdiv(a.k, kThreads), ct = blk / nck;
+  const int64_t l = blk % nck * kThreads + threadIdx.x;
+  const int c = (int)(ct / a.bs);
+  const double* q = a.A + (ct - c * a.bs) * a.lda + l;
+  const int64_t step = a.bs * a.lda;
+  double s = 0.0;
+  if (c == 0) {  // coefficients 1
+    if (l < a.k) {
+#pragma unroll 8
+      for (int I = 0; I < a.p; ++I) s += q[I * step];
+    }
+  } else {
+    for (int I0 = 0; I0 < a.p; I0 += kThreads) {  // the coefficients of 256 blocks at a time
+      __syncthreads();
+      if (I0 + (int)threadIdx.x < a.p) sh[threadIdx.x] = block_coef(c, I0 + threadIdx.x, a.p);
+      __syncthreads();
+      if (l < a.k) {
+        const int n = min(kThreads, a.p - I0);
+#pragma unroll 8
+        for (int I = 0; I < n; ++I) s += sh[I] * q[(I0 + I) * step];
+      }
+    }
+  }
+  if (l < a.k) a.S[ct * a.k + l] = s;
+}
+
+// Partial column squares of B: 32 columns x 256 rows, 32 rows per warp.
+__device__ __forceinline__ void enc_bsq(const EncArgs& a, int64_t blk, double* sh) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t ncj = cdiv(a.n, 32), c = blk / ncj, j = blk % ncj * 32 + lane;
+  const int64_t l0 = c * kSqRows + warp * 32, l1 = min(l0 + 32, a.k);
+  double s = 0.0;
+  if (j < a.n) {
+    const double* q = a.B + l0 * a.ldb + j;
+#pragma unroll 8
+    for (int64_t l = l0; l < l1; ++l, q += a.ldb) s = fma(*q, *q, s);
+  }
+  sh[warp * 32 + lane] = s;
+  __syncthreads();
+  if (warp == 0 && j < a.n) {
+    for (int w = 1; w < kWarps; ++w) s += sh[w * 32 + lane];
+    a.colsq[c * a.n + j] = s;
   }
 }
 
 // ||A_{i,:}||_2, one warp per row.
-__global__ void __launch_bounds__(kThreads) k_row_norms(const double* __restrict__ A, int64_t lda,
-                                                        int64_t m, int64_t k,
-                                                        double* __restrict__ out) {
-  const int64_t i = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
+__device__ __forceinline__ void enc_arows(const EncArgs& a, int64_t blk) {
+  const int64_t i = blk * kWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (i >= m) return;
-  double s = 0.0;
-  for (int64_t l = lane; l < k; l += 32) {
-    const double a = A[i * lda + l];
-    s = fma(a, a, s);
-  }
-  s = warp_sum(s);
-  if (lane == 0) out[i] = sqrt(s);
-}
-
-// Row checksums of B per verify block: bcs[l][2J] = B_J e, bcs[l][2J+1] = B_J w,
-// plus per-chunk partials of ||B_J e||^2 and ||B_J w||^2 at
-// part[(2J + c) * nch + chunk].  One warp per (J, chunk of 64 rows of B).
-__global__ void __launch_bounds__(kThreads) k_encB_rows(const double* __restrict__ B, int64_t ldb,
-                                                        int64_t k, int64_t n, int vb, int e,
-                                                        double* __restrict__ bcs, int64_t Cc,
-                                                        double* __restrict__ part, int nch) {
-  const int lane = threadIdx.x & 31;
-  const int64_t chunk = (int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-  if (chunk >= nch) return;
-  const int64_t nvb = cdiv(n, vb);
-  const double sc = scalbn(1.0, -e);
-  for (int64_t J = blockIdx.y; J < nvb; J += gridDim.y) {
-    const int64_t j0 = J * vb, j1 = min(j0 + (int64_t)vb, n);
-    const int64_t l0 = chunk * kRowsPerWarpB, l1 = min(l0 + kRowsPerWarpB, k);
-    double q0 = 0.0, q1 = 0.0;
-    for (int64_t l = l0; l < l1; ++l) {
-      double se = 0.0, sw = 0.0;
-      for (int64_t j = j0 + lane; j < j1; j += 32) {
-        const double b = B[l * ldb + j];
-        se += b;
-        sw = fma((double)(j - j0 + 1) * sc, b, sw);
-      }
-      se = warp_sum(se);
-      sw = warp_sum(sw);
-      if (lane == 0) {
-        bcs[l * Cc + 2 * J] = se;
-        bcs[l * Cc + 2 * J + 1] = sw;
-      }
-      q0 = fma(se, se, q0);
-      q1 = fma(sw, sw, q1);
-    }
-    if (lane == 0) {
-      part[(2 * J + 0) * nch + chunk] = q0;
-      part[(2 * J + 1) * nch + chunk] = q1;
-    }
-  }
-}
-
-// Per-chunk partial sums of B_lj^2 for the column norms.  Grid (ceil(n/256), nch).
-__global__ void __launch_bounds__(kThreads) k_col_sq(const double* __restrict__ B, int64_t ldb,
-                                                     int64_t k, int64_t n,
-                                                     double* __restrict__ part) {
-  const int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (j >= n) return;
-  const int64_t nch = cdiv(k, kThreads);
-  for (int64_t c = blockIdx.y; c < nch; c += gridDim.y) {
-    const int64_t l0 = c * kThreads, l1 = min(l0 + kThreads, k);
-    double s = 0.0;
+  if (i >= a.m) return;
+  const double* q = a.A + i * a.lda;
+  double s[2] = {0.0, 0.0};
+  int64_t l = lane;
 #pragma unroll 4
-    for (int64_t l = l0; l < l1; ++l) {
-      const double b = B[l * ldb + j];
-      s = fma(b, b, s);
+  for (; l + 32 < a.k; l += 64) {
+    const double x = q[l], y = q[l + 32];
+    s[0] = fma(x, x, s[0]);
+    s[1] = fma(y, y, s[1]);
+  }
+  if (l < a.k) s[0] = fma(q[l], q[l], s[0]);
+  const double t = warp_sum(s[0] + s[1]);
+  if (lane == 0) a.nArow[i] = sqrt(t);
+}
+
+__global__ void __launch_bounds__(kThreads) k_enc64(const EncArgs a) {
+  __shared__ double sh[kWarps * 64];
+  __shared__ double wtab[kSegRows];
+  if (blockIdx.x == 0) {
+    for (int64_t x = threadIdx.x; x < 2 * a.nvr; x += kThreads) a.car_a[x] = 0.0;
+    for (int64_t x = threadIdx.x; x < 2 * a.nvc; x += kThreads) a.car_b[x] = 0.0;
+    if (a.status && threadIdx.x < 2) a.status[threadIdx.x] = 0;
+  }
+  int64_t b = blockIdx.x;
+  if (b < a.n_acols) {
+    // weights at most 1: a weighted term never exceeds its element
+    if (threadIdx.x < kSegRows)
+      wtab[threadIdx.x] = (double)(threadIdx.x + 1) * scalbn(1.0, -a.er);
+    __syncthreads();
+    return enc_acols(a, b, sh, wtab);
+  }
+  b -= a.n_acols;
+  if (b < a.n_brows) return enc_brows(a, b);
+  b -= a.n_brows;
+  if (b < a.n_ablk) return enc_ablk(a, b, sh);
+  b -= a.n_ablk;
+  if (b < a.n_bsq) return enc_bsq(a, b, sh);
+  enc_arows(a, b - a.n_bsq);
+}
+
+// Threshold norms, one CTA per verify block: nblk[4I] = sqrt(sum_{t in I} v_t^2),
+// nblk[4I+1] = sqrt(sum (w_t v_t)^2) with v the line norms of the block, and
+// nblk[4I+2], nblk[4I+3] the norms of its two checksum vectors.  CTAs 0 .. nvr-1:
+// row blocks of A; then the column blocks of B, which also write the column
+// norms nBcol from their partial squares.
+__global__ void __launch_bounds__(kThreads) k_enc64_norms(const EncArgs a, double* nAblk,
+                                                          double* nBcol, double* nBblk) {
+  __shared__ double sh[kWarps];
+  const bool rows = blockIdx.x < a.nvr;
+  const int64_t I = rows ? blockIdx.x : blockIdx.x - a.nvr;
+  const int vb = rows ? a.vb_r : a.vb_c;
+  const int64_t t0 = I * vb;
+  const int len = (int)(min(t0 + (int64_t)vb, rows ? a.m : a.n) - t0);
+  const double sc = scalbn(1.0, rows ? -a.er : -a.ec);
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  const int64_t nch = cdiv(a.k, kSqRows);
+  for (int t = threadIdx.x; t < len; t += kThreads) {
+    double v2 = 0.0;
+    if (rows) {
+      const double v = a.nArow[t0 + t];
+      v2 = v * v;
+    } else {
+#pragma unroll 8
+      for (int64_t c = 0; c < nch; ++c) v2 += a.colsq[c * a.n + t0 + t];
+      nBcol[t0 + t] = sqrt(v2);
     }
-    part[c * n + j] = s;
+    const double w = (double)(t + 1) * sc;
+    s[0] += v2;
+    s[1] = fma(w * w, v2, s[1]);
   }
-}
-
-// out[o] = sqrt(sum_c part[o*so + c*sc]) in chunk order.
-__global__ void k_sum_sqrt(const double* __restrict__ part, int64_t nout, int64_t nch, int64_t so,
-                           int64_t sc, double* __restrict__ out) {
-  const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= nout) return;
-  double s = 0.0;
-  for (int64_t c = 0; c < nch; ++c) s += part[o * so + c * sc];
-  out[o] = sqrt(s);
-}
-
-// Threshold norms of every verify block from the per-line norms and the
-// checksum partials: nblk[4I] = sqrt(sum_{t in I} nvec_t^2), nblk[4I+1] =
-// sqrt(sum (w_t nvec_t)^2), nblk[4I+2], nblk[4I+3] = sqrt of the summed
-// partials of the two checksum vectors.  One thread per verify block.
-__global__ void k_finalize_blk(const double* __restrict__ nvec, int64_t len, int vb, int e,
-                               const double* __restrict__ part, int64_t nch,
-                               double* __restrict__ nblk) {
-  const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t nvb = cdiv(len, vb);
-  if (I >= nvb) return;
-  const double sc = scalbn(1.0, -e);
-  const int64_t t0 = I * vb, t1 = min(t0 + (int64_t)vb, len);
-  double f0 = 0.0, f1 = 0.0, q0 = 0.0, q1 = 0.0;
-  for (int64_t t = t0; t < t1; ++t) {
-    const double v = nvec[t], wv = (double)(t - t0 + 1) * sc * v;
-    f0 = fma(v, v, f0);
-    f1 = fma(wv, wv, f1);
+#pragma unroll 4
+  for (int64_t l = threadIdx.x; l < a.k; l += kThreads) {
+    double e, w;
+    if (rows) {
+      e = a.acs[(2 * I) * a.k + l];
+      w = a.acs[(2 * I + 1) * a.k + l];
+    } else {
+      const double2 x = *reinterpret_cast<const double2*>(a.bcs + l * a.Cc + 2 * I);
+      e = x.x;
+      w = x.y;
+    }
+    s[2] = fma(e, e, s[2]);
+    s[3] = fma(w, w, s[3]);
   }
-  for (int64_t c = 0; c < nch; ++c) {
-    q0 += part[(2 * I) * nch + c];
-    q1 += part[(2 * I + 1) * nch + c];
+  double* out = (rows ? nAblk : nBblk) + 4 * I;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const double t = block_sum(s[c], sh);
+    if (threadIdx.x == 0) out[c] = sqrt(t);
   }
-  nblk[4 * I + 0] = sqrt(f0);
-  nblk[4 * I + 1] = sqrt(f1);
-  nblk[4 * I + 2] = sqrt(q0);
-  nblk[4 * I + 3] = sqrt(q1);
 }
 
 // ---------------------------------------------------------------- chained calls
 // A chained product (section 3.2: stacked calls do not recompute checksums)
 // takes its encoded rows of A / columns of B from an earlier product's
-// expected checksums; the kernels below form the norms of those carried
-// vectors and the bound of their deviation from the stored operand.
-
-// part[r * nch + chunk] = sum over the chunk's 256 columns of acs[r][l]^2, the
-// layout k_encA_cols leaves for the checksum-row norms (r = 2I + c).
-// Grid (nch, <= 65535).
-__global__ void __launch_bounds__(kThreads) k_rows_sq(const double* __restrict__ acs, int64_t k,
-                                                      int64_t rows, double* __restrict__ part,
-                                                      int nch) {
-  __shared__ double sh[kThreads / 32];
-  const int64_t l = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  for (int64_t r = blockIdx.y; r < rows; r += gridDim.y) {
-    const double v = l < k ? acs[r * k + l] : 0.0;
-    const double t = block_sum(v * v, sh);
-    if (threadIdx.x == 0) part[r * nch + blockIdx.x] = t;
-  }
-}
-
-// part[c * nch + chunk] = sum over the chunk's kRowsPerWarpB rows of
-// bcs[l][c]^2, the layout k_encB_rows leaves (c = 2J + w).  One thread per
-// (c, chunk).
-__global__ void __launch_bounds__(kThreads) k_cols_sq(const double* __restrict__ bcs, int64_t k,
-                                                      int64_t Cc, double* __restrict__ part,
-                                                      int nch) {
-  const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (t >= Cc * nch) return;
-  const int64_t c = t / nch, chunk = t - c * nch;
-  const int64_t l0 = chunk * kRowsPerWarpB, l1 = min(l0 + (int64_t)kRowsPerWarpB, k);
-  double q = 0.0;
-  for (int64_t l = l0; l < l1; ++l) {
-    const double b = bcs[l * Cc + c];
-    q = fma(b, b, q);
-  }
-  part[c * nch + chunk] = q;
-}
+// expected checksums; k_carry bounds their deviation from the stored operand.
 
 // Deviation bound of checksums carried out of an earlier product: its
 // deviation per line stays within that product's unscaled threshold, so the
@@ -265,53 +347,49 @@ __global__ void __launch_bounds__(kThreads) k_carry(const double* __restrict__ n
   }
 }
 
-}  // namespace
-
-namespace {
-
-// The encode's launch sequence, with its per-chunk partial sums at `part`
-// (the workspace scratch, or the static array of abft_encode_noalloc).
+// The encode's launches, with the column-square partials of B at `part` (the
+// workspace scratch, or the static array of abft_encode_noalloc).  rows / cols:
+// form the checksum rows of A / columns of B (otherwise they are in ws already).
 cudaError_t encode_f64_into(const Plan& P, const double* A, const double* B, void* ws,
-                            double* part, cudaStream_t st) {
+                            double* part, bool rows, bool cols, cudaStream_t st) {
   const abft_desc& d = P.d;
   char* w = static_cast<char*>(ws);
-  double* acs = reinterpret_cast<double*>(w + P.L.acs);
-  double* bcs = reinterpret_cast<double*>(w + P.L.bcs);
-  double* nArow = reinterpret_cast<double*>(w + P.L.nArow);
-  double* nAblk = reinterpret_cast<double*>(w + P.L.nAblk);
-  double* nBcol = reinterpret_cast<double*>(w + P.L.nBcol);
-  double* nBblk = reinterpret_cast<double*>(w + P.L.nBblk);
-  const int nchA = (int)cdiv(d.k, kThreads);
-  const int nchB = (int)cdiv(d.k, kRowsPerWarpB);
-  const int nchC = (int)cdiv(d.k, kThreads);
-  double* partA = part;
-  double* partB = partA + 4 * P.nvr * nchA;
-  double* partC = partB + 4 * P.nvc * nchB;
-
-  auto gy = [](int64_t v) { return (unsigned)(v < 65535 ? v : 65535); };
+  auto at = [&](size_t off) { return reinterpret_cast<double*>(w + off); };
   if (d.k == 0) {  // empty inner dimension: all checksums and norms are zero
-    cudaMemsetAsync(nArow, 0, sizeof(double) * d.m, st);
-    cudaMemsetAsync(nAblk, 0, sizeof(double) * 4 * P.nvr, st);
-    cudaMemsetAsync(nBcol, 0, sizeof(double) * d.n, st);
-    cudaMemsetAsync(nBblk, 0, sizeof(double) * 4 * P.nvc, st);
+    cudaMemsetAsync(at(P.L.nArow), 0, sizeof(double) * d.m, st);
+    cudaMemsetAsync(at(P.L.nAblk), 0, sizeof(double) * 4 * P.nvr, st);
+    cudaMemsetAsync(at(P.L.nBcol), 0, sizeof(double) * d.n, st);
+    cudaMemsetAsync(at(P.L.nBblk), 0, sizeof(double) * 4 * P.nvc, st);
+    cudaMemsetAsync(at(P.L.car_a), 0, sizeof(double) * 2 * P.nvr, st);
+    cudaMemsetAsync(at(P.L.car_b), 0, sizeof(double) * 2 * P.nvc, st);
     return cudaGetLastError();
   }
-  count_launches(P.bs > 0 ? 8 : 7);
-  k_encA_cols<<<dim3((unsigned)nchA, gy(P.nvr)), kThreads, 0, st>>>(
-      A, d.lda, d.m, d.k, d.vb_rows, P.er, acs, partA, nchA);
-  if (P.bs > 0)
-    k_encA_block<<<dim3((unsigned)cdiv(d.k, kThreads), gy(P.f * P.bs)), kThreads, 0, st>>>(
-        A, d.lda, d.k, d.grid_p, P.bs, P.f, acs + 2 * P.nvr * d.k);
-  k_row_norms<<<(unsigned)cdiv(d.m * 32, kThreads), kThreads, 0, st>>>(A, d.lda, d.m, d.k, nArow);
-  k_encB_rows<<<dim3((unsigned)cdiv(nchB, kThreads / 32), gy(P.nvc)), kThreads, 0, st>>>(
-      B, d.ldb, d.k, d.n, d.vb_cols, P.ec, bcs, P.Cc, partB, nchB);
-  k_col_sq<<<dim3((unsigned)cdiv(d.n, kThreads), gy(nchC)), kThreads, 0, st>>>(
-      B, d.ldb, d.k, d.n, partC);
-  k_sum_sqrt<<<(unsigned)cdiv(d.n, 128), 128, 0, st>>>(partC, d.n, nchC, 1, d.n, nBcol);
-  k_finalize_blk<<<(unsigned)cdiv(P.nvr, 128), 128, 0, st>>>(nArow, d.m, d.vb_rows, P.er, partA,
-                                                             nchA, nAblk);
-  k_finalize_blk<<<(unsigned)cdiv(P.nvc, 128), 128, 0, st>>>(nBcol, d.n, d.vb_cols, P.ec, partB,
-                                                             nchB, nBblk);
+  EncArgs a{};
+  a.A = A; a.B = B;
+  a.lda = d.lda; a.ldb = d.ldb; a.m = d.m; a.n = d.n; a.k = d.k;
+  a.vb_r = d.vb_rows; a.vb_c = d.vb_cols; a.er = P.er; a.ec = P.ec;
+  a.nvr = P.nvr; a.nvc = P.nvc; a.Cc = P.Cc;
+  a.acs = at(P.L.acs);
+  a.S = a.acs + 2 * P.nvr * d.k;
+  a.bcs = at(P.L.bcs);
+  a.nArow = at(P.L.nArow);
+  a.colsq = part;
+  a.p = d.grid_p; a.f = P.f; a.bs = P.bs;
+  a.car_a = at(P.L.car_a);
+  a.car_b = at(P.L.car_b);
+  a.status = P.tc64 ? reinterpret_cast<int32_t*>(w + P.f64tc_hdr) : nullptr;
+  a.wpu = 1;
+  while (a.wpu < kWarps && a.wpu * kSegRows < d.vb_rows) a.wpu *= 2;
+  a.n_acols = rows ? cdiv(P.nvr * cdiv(d.k, 32), kWarps / a.wpu) : 0;
+  a.n_brows = cols ? cdiv(P.nvc * cdiv(d.k, kRowsB), kWarps) : 0;
+  a.n_ablk = rows && P.bs > 0 ? P.f * P.bs * cdiv(d.k, kThreads) : 0;
+  a.n_bsq = cdiv(d.n, 32) * cdiv(d.k, kSqRows);
+  a.n_arows = cdiv(d.m, kWarps);
+  k_enc64<<<(unsigned)(a.n_acols + a.n_brows + a.n_ablk + a.n_bsq + a.n_arows), kThreads, 0, st>>>(
+      a);
+  k_enc64_norms<<<(unsigned)(P.nvr + P.nvc), kThreads, 0, st>>>(a, at(P.L.nAblk), at(P.L.nBcol),
+                                                                at(P.L.nBblk));
+  count_launches(2);
   return cudaGetLastError();
 }
 
@@ -319,7 +397,7 @@ cudaError_t encode_f64_into(const Plan& P, const double* A, const double* B, voi
 
 cudaError_t launch_encode_f64(const Plan& P, const double* A, const double* B, void* ws,
                               cudaStream_t st) {
-  return encode_f64_into(P, A, B, ws, scratch_view(P, ws).part, st);
+  return encode_f64_into(P, A, B, ws, scratch_view(P, ws).part, true, true, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -347,7 +425,7 @@ cudaError_t launch_encode_f64_noalloc(const Plan& P, const double* A, const doub
   void* part = nullptr;
   const cudaError_t e = cudaGetSymbolAddress(&part, g_encode_part);
   if (e != cudaSuccess) return e;
-  return encode_f64_into(P, A, B, ws, static_cast<double*>(part), st);
+  return encode_f64_into(P, A, B, ws, static_cast<double*>(part), true, true, st);
 }
 
 // Deviation bounds of the checksums carried out of an earlier product PL
@@ -376,71 +454,24 @@ cudaError_t launch_encode_f64_chained(const Plan& P, const double* A, const doub
   const abft_desc& d = P.d;
   if (d.k == 0) return launch_encode_f64(P, A, B, ws, st);  // nothing to carry: zero norms
   char* w = static_cast<char*>(ws);
-  double* acs = reinterpret_cast<double*>(w + P.L.acs);
-  double* bcs = reinterpret_cast<double*>(w + P.L.bcs);
-  double* nArow = reinterpret_cast<double*>(w + P.L.nArow);
-  double* nAblk = reinterpret_cast<double*>(w + P.L.nAblk);
-  double* nBcol = reinterpret_cast<double*>(w + P.L.nBcol);
-  double* nBblk = reinterpret_cast<double*>(w + P.L.nBblk);
-  double* carA = reinterpret_cast<double*>(w + P.L.car_a);
-  double* carB = reinterpret_cast<double*>(w + P.L.car_b);
-  Scratch S = scratch_view(P, ws);
-  const int nchA = (int)cdiv(d.k, kThreads);
-  const int nchB = (int)cdiv(d.k, kRowsPerWarpB);
-  const int nchC = (int)cdiv(d.k, kThreads);
-  double* partA = S.part;
-  double* partB = partA + 4 * P.nvr * nchA;
-  double* partC = partB + 4 * P.nvc * nchB;
-  auto gy = [](int64_t v) { return (unsigned)(v < 65535 ? v : 65535); };
   cudaError_t e = cudaSuccess;
-  int launches = 0;
-
-  if (PL) {  // rows of A: the earlier product's E (verify rows, then block checksum rows)
-    const char* wl = static_cast<const char*>(wsL);
-    const double* EL = reinterpret_cast<const double*>(wl + PL->L.E);
-    e = cudaMemcpyAsync(acs, EL, sizeof(double) * (size_t)P.R * d.k, cudaMemcpyDeviceToDevice,
-                        st);
-    if (e != cudaSuccess) return e;
-    k_rows_sq<<<dim3((unsigned)nchA, gy(2 * P.nvr)), kThreads, 0, st>>>(acs, d.k, 2 * P.nvr,
-                                                                         partA, nchA);
-    launch_carry_rows(*PL, wsL, carA, st);
-    launches += 2;
-  } else {
-    k_encA_cols<<<dim3((unsigned)nchA, gy(P.nvr)), kThreads, 0, st>>>(
-        A, d.lda, d.m, d.k, d.vb_rows, P.er, acs, partA, nchA);
-    ++launches;
-    if (P.bs > 0) {
-      k_encA_block<<<dim3((unsigned)cdiv(d.k, kThreads), gy(P.f * P.bs)), kThreads, 0, st>>>(
-          A, d.lda, d.k, d.grid_p, P.bs, P.f, acs + 2 * P.nvr * d.k);
-      ++launches;
-    }
+  if (PL)  // rows of A: the earlier product's E (verify rows, then block checksum rows)
+    e = cudaMemcpyAsync(w + P.L.acs, static_cast<const char*>(wsL) + PL->L.E,
+                        sizeof(double) * (size_t)P.R * d.k, cudaMemcpyDeviceToDevice, st);
+  if (PR && e == cudaSuccess)  // columns of B: the earlier product's F (k x Cc)
+    e = cudaMemcpyAsync(w + P.L.bcs, static_cast<const char*>(wsR) + PR->L.F,
+                        sizeof(double) * (size_t)d.k * P.Cc, cudaMemcpyDeviceToDevice, st);
+  if (e == cudaSuccess)
+    e = encode_f64_into(P, A, B, ws, scratch_view(P, ws).part, !PL, !PR, st);
+  if (PL && e == cudaSuccess) {
+    e = launch_carry_rows(*PL, wsL, reinterpret_cast<double*>(w + P.L.car_a), st);
+    count_launches(1);
   }
-  k_row_norms<<<(unsigned)cdiv(d.m * 32, kThreads), kThreads, 0, st>>>(A, d.lda, d.m, d.k, nArow);
-
-  if (PR) {  // columns of B: the earlier product's F (k x Cc)
-    const char* wr = static_cast<const char*>(wsR);
-    const double* FR = reinterpret_cast<const double*>(wr + PR->L.F);
-    e = cudaMemcpyAsync(bcs, FR, sizeof(double) * (size_t)d.k * P.Cc, cudaMemcpyDeviceToDevice,
-                        st);
-    if (e != cudaSuccess) return e;
-    k_cols_sq<<<(unsigned)cdiv(P.Cc * nchB, kThreads), kThreads, 0, st>>>(bcs, d.k, P.Cc, partB,
-                                                                           nchB);
-    launch_carry_cols(*PR, wsR, carB, st);
-    launches += 2;
-  } else {
-    k_encB_rows<<<dim3((unsigned)cdiv(nchB, kThreads / 32), gy(P.nvc)), kThreads, 0, st>>>(
-        B, d.ldb, d.k, d.n, d.vb_cols, P.ec, bcs, P.Cc, partB, nchB);
-    ++launches;
+  if (PR && e == cudaSuccess) {
+    e = launch_carry_cols(*PR, wsR, reinterpret_cast<double*>(w + P.L.car_b), st);
+    count_launches(1);
   }
-  k_col_sq<<<dim3((unsigned)cdiv(d.n, kThreads), gy(nchC)), kThreads, 0, st>>>(
-      B, d.ldb, d.k, d.n, partC);
-  k_sum_sqrt<<<(unsigned)cdiv(d.n, 128), 128, 0, st>>>(partC, d.n, nchC, 1, d.n, nBcol);
-  k_finalize_blk<<<(unsigned)cdiv(P.nvr, 128), 128, 0, st>>>(nArow, d.m, d.vb_rows, P.er, partA,
-                                                             nchA, nAblk);
-  k_finalize_blk<<<(unsigned)cdiv(P.nvc, 128), 128, 0, st>>>(nBcol, d.n, d.vb_cols, P.ec, partB,
-                                                             nchB, nBblk);
-  count_launches(launches + 5);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace abft

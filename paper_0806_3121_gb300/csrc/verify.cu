@@ -3,10 +3,10 @@
 // errors; a lost part is the checksum minus the surviving parts).
 //
 // Pipeline of one verify call, all on the device:
-//   k_col_check   one thread per column line (verify block I, column j):
-//                 binary64 sums e^T C_I[:,j], w^T C_I[:,j], non-finite count,
-//                 residuals against E, threshold test, append if flagged.
-//   k_row_check   one warp per row line (row i, verify block J), against F.
+//   k_col_check   column lines (verify block I, column j): sums e^T C_I[:,j],
+//                 w^T C_I[:,j], non-finite elements, residuals against E,
+//                 threshold test, append if flagged.
+//   k_row_check   row lines (row i, verify block J), against F.
 //   k_locate_correct  one CTA: candidates from the flagged lines (single
 //                 non-finite element, or the weighted/unweighted residual
 //                 ratio), bitonic sort + merge, choice of a correcting line,
@@ -120,33 +120,9 @@ __device__ __forceinline__ TC warp_sum_t(TC v) {
   return v;
 }
 
-// Residuals of column line (I, j).  Returns the non-finite count.
-template <typename TC>
-__device__ int col_line(const CheckArgs& a, int64_t I, int64_t j, double& re, double& rw,
-                        double& te, double& tw) {
-  const int64_t i0 = I * a.vb_r, i1 = min(i0 + (int64_t)a.vb_r, a.m);
-  const TC sc = (TC)scalbn(1.0, -a.er);
-  const TC* C = static_cast<const TC*>(a.C);
-  TC se = 0, sw = 0;
-  int nf = 0;
-  const TC* p = C + i0 * a.ldc + j;
-  const int len = (int)(i1 - i0);
-#pragma unroll 4
-  for (int t = 0; t < len; ++t) {
-    const TC x = p[(int64_t)t * a.ldc];
-    se += x;
-    sw = fma_t<TC>((TC)(t + 1) * sc, x, sw);
-    nf += isfinite(x) ? 0 : 1;
-  }
-  re = (double)se - a.E[(2 * I) * a.n + j];
-  rw = (double)sw - a.E[(2 * I + 1) * a.n + j];
-  col_taus(a, I, j, te, tw);
-  return nf;
-}
-
-// The same computed by one warp (lanes split the rows; sums in the element
-// type, then added across the lanes); residuals and thresholds valid in every
-// lane.
+// Residuals of column line (I, j), computed by one warp (lanes split the rows;
+// sums in the element type, then added across the lanes); residuals and
+// thresholds valid in every lane.  Returns the non-finite count.
 template <typename TC>
 __device__ int col_line_warp(const CheckArgs& a, int64_t I, int64_t j, double& re, double& rw,
                              double& te, double& tw) {
@@ -206,43 +182,161 @@ __device__ int row_line_warp(const CheckArgs& a, int64_t i, int64_t J, double& r
 
 // Column lines [I_begin, I_end) x [j_begin, j_end).  mode 0: append flagged
 // lines to colf (skipping erased blocks); mode 1: only count them in
-// cnt[kCntRecoverFlagged].  Grid (ceil((j_end-j_begin)/256), <= 65535).
+// cnt[kCntRecoverFlagged].  A unit is 32 columns x one verify block; wpu warps of
+// a CTA share its rows in contiguous parts (64 rows or more each) and meet in
+// shared memory, with eight rows of loads in flight per thread: one thread per
+// column walking all the rows of its block, as an earlier version did, left a
+// 512^2 binary64 result to two CTAs (192 us; the FP64 pipe, 2 results per clock
+// and SM, bounds large ones).  Weights come from a table: forming (t + 1) 2^-e per
+// element cost two more binary64 instructions.
+constexpr int kSegRows = 64;
 template <typename TC>
 __global__ void __launch_bounds__(kThreads) k_col_check(const CheckArgs a, int64_t j_begin,
                                                         int64_t j_end, int64_t I_begin,
-                                                        int64_t I_end, int mode) {
-  const int64_t j = j_begin + (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (mode == 1 && a.status_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+                                                        int64_t I_end, int mode, int wpu) {
+  __shared__ TC sh[kThreads / 32][2][32];
+  __shared__ int snf[kThreads / 32][32];
+  __shared__ TC wtab[kSegRows];
+  if (mode == 1 && a.status_out && blockIdx.x == 0 && threadIdx.x == 0)
     *a.status_out = *a.timeout;
-  if (j >= j_end) return;
-  for (int64_t I = I_begin + blockIdx.y; I < I_end; I += gridDim.y) {
-    const int64_t i0 = I * a.vb_r, i1 = min(i0 + (int64_t)a.vb_r, a.m);
-    if (mode == 0 && touches_erased(a.erased, a.bs, a.bc, i0, i1, j, j + 1)) continue;
-    double re, rw, te, tw;
-    const int nf = col_line<TC>(a, I, j, re, rw, te, tw);
-    if (nf == 0 && !is_flagged(re, rw, te, tw)) continue;
-    if (mode == 1) {
-      atomicAdd(&a.cnt[kCntRecoverFlagged], 1);
-      continue;
+  // weights at most 1: a weighted term never exceeds its element
+  const TC sc = (TC)scalbn(1.0, -a.er);
+  if (threadIdx.x < kSegRows) wtab[threadIdx.x] = (TC)(threadIdx.x + 1) * sc;
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t nck = cdiv(j_end - j_begin, 32);
+  const int64_t u = (int64_t)blockIdx.x * (kThreads / 32 / wpu) + warp / wpu;
+  const int part = warp % wpu;
+  const int64_t I = I_begin + u / nck, j = j_begin + u % nck * 32 + lane;
+  const bool ok = I < I_end && j < j_end;
+  const int64_t i0 = I * a.vb_r, i1 = min(i0 + (int64_t)a.vb_r, a.m);
+  const int64_t len = max((int64_t)kSegRows, cdiv(a.vb_r, wpu));  // rows of a part
+  const int64_t b0 = i0 + part * len, b1 = min(b0 + len, i1);
+  TC se = 0, sw = 0;
+  int nf = 0;
+  if (ok) {
+    for (int64_t s0 = b0; s0 < b1; s0 += kSegRows) {
+      const int nr = (int)min((int64_t)kSegRows, b1 - s0);
+      const TC* q = static_cast<const TC*>(a.C) + s0 * a.ldc + j;
+      TC e = 0, w = 0;
+      int t = 0;
+      for (; t + 8 <= nr; t += 8) {
+        TC x[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) x[r] = q[(t + r) * a.ldc];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          e += x[r];
+          w = fma_t<TC>(wtab[t + r], x[r], w);
+          nf |= isfinite(x[r]) ? 0 : 1;
+        }
+      }
+      for (; t < nr; ++t) {
+        const TC x = q[t * a.ldc];
+        e += x;
+        w = fma_t<TC>(wtab[t], x, w);
+        nf |= isfinite(x) ? 0 : 1;
+      }
+      sw = fma_t<TC>((TC)(s0 - i0) * sc, e, sw + w);
+      se += e;
     }
-    const int slot = atomicAdd(&a.cnt[kCntColFlags], 1);
-    if (slot < kCapFlags) a.colf[slot] = FlagEntry{(int32_t)I, (int32_t)j, nf, 0, re, rw};
   }
+  if (wpu > 1) {
+    sh[warp][0][lane] = se;
+    sh[warp][1][lane] = sw;
+    snf[warp][lane] = nf;
+    __syncthreads();
+    if (part != 0) return;
+    for (int w = warp + 1; w < warp + wpu; ++w) {
+      se += sh[w][0][lane];
+      sw += sh[w][1][lane];
+      nf |= snf[w][lane];
+    }
+  }
+  if (!ok) return;
+  if (mode == 0 && touches_erased(a.erased, a.bs, a.bc, i0, i1, j, j + 1)) return;
+  const double re = (double)se - a.E[(2 * I) * a.n + j];
+  const double rw = (double)sw - a.E[(2 * I + 1) * a.n + j];
+  double te, tw;
+  col_taus(a, I, j, te, tw);
+  if (nf == 0 && !is_flagged(re, rw, te, tw)) return;
+  if (mode == 1) {
+    atomicAdd(&a.cnt[kCntRecoverFlagged], 1);
+    return;
+  }
+  const int slot = atomicAdd(&a.cnt[kCntColFlags], 1);
+  if (slot < kCapFlags) a.colf[slot] = FlagEntry{(int32_t)I, (int32_t)j, nf, 0, re, rw};
 }
 
+// Row lines: one warp takes kRowLinesW rows x one verify block.  The sums of the
+// eight rows meet in one transposing butterfly (17 warp-wide adds instead of 80)
+// and their residuals and thresholds are evaluated side by side in eight lanes:
+// with one line per warp those binary64 instructions, each a whole warp's, cost
+// as much as the sums (3001 x 2999 binary32: 48 us).
+constexpr int kRowLinesW = 8;
 template <typename TC>
 __global__ void __launch_bounds__(kThreads) k_row_check(const CheckArgs a) {
-  const int64_t gw = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
-  if (gw >= a.m * a.nvc) return;
-  const int64_t i = gw / a.nvc, J = gw % a.nvc;
+  constexpr int N = 2 * kRowLinesW;
+  const int lane = threadIdx.x & 31;
+  const int64_t u = (int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+  const int64_t r0 = u / a.nvc * kRowLinesW, J = u % a.nvc;
+  if (r0 >= a.m) return;
+  const int nr = (int)min((int64_t)kRowLinesW, a.m - r0);
   const int64_t j0 = J * a.vb_c, j1 = min(j0 + (int64_t)a.vb_c, a.n);
+  const int len = (int)(j1 - j0);
+  const TC* q = static_cast<const TC*>(a.C) + r0 * a.ldc + j0;
+  const TC sc = (TC)scalbn(1.0, -a.ec);
+  TC v[N];  // e sums, then w sums
+  uint32_t nfb = 0;
+#pragma unroll
+  for (int r = 0; r < N; ++r) v[r] = 0;
+  TC w = (TC)(lane + 1) * sc;
+#pragma unroll 2
+  for (int t = lane; t < len; t += 32) {
+#pragma unroll
+    for (int r = 0; r < kRowLinesW; ++r) {
+      const TC x = r < nr ? q[r * a.ldc + t] : (TC)0;
+      v[r] += x;
+      v[kRowLinesW + r] = fma_t<TC>(w, x, v[kRowLinesW + r]);
+      nfb |= isfinite(x) ? 0u : 1u << r;
+    }
+    w += (TC)32 * sc;
+  }
+  nfb = __reduce_or_sync(0xffffffffu, nfb);
+#pragma unroll
+  for (int s = 16, h = N / 2; h >= 1; s >>= 1, h >>= 1) {
+    const bool upper = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const TC send = upper ? v[i] : v[i + h];
+      v[i] = (upper ? v[i + h] : v[i]) + __shfl_xor_sync(0xffffffffu, send, s);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);  // lane l holds value l / 2
+  const TC sw = __shfl_sync(0xffffffffu, v[0], (lane + 16) & 31);
+  const int r = lane >> 1;
+  if (lane >= 16 || (lane & 1) || r >= nr) return;
+  const int64_t i = r0 + r;
   if (touches_erased(a.erased, a.bs, a.bc, i, i + 1, j0, j1)) return;
-  double re, rw, te, tw;
-  const int nf = row_line_warp<TC>(a, i, J, re, rw, te, tw);
-  if ((threadIdx.x & 31) != 0) return;
+  const double re = (double)v[0] - a.F[i * a.Cc + 2 * J];
+  const double rw = (double)sw - a.F[i * a.Cc + 2 * J + 1];
+  double te, tw;
+  row_taus(a, i, J, te, tw);
+  const int nf = (nfb >> r) & 1;
   if (nf == 0 && !is_flagged(re, rw, te, tw)) return;
   const int slot = atomicAdd(&a.cnt[kCntRowFlags], 1);
   if (slot < kCapFlags) a.rowf[slot] = FlagEntry{(int32_t)i, (int32_t)J, nf, 0, re, rw};
+}
+
+// Launches k_col_check over whole units (see there).
+template <typename TC>
+void run_col_check(const CheckArgs& a, int64_t j_begin, int64_t j_end, int64_t I_begin,
+                   int64_t I_end, int mode, cudaStream_t st) {
+  int wpu = 1;
+  while (wpu < kThreads / 32 && wpu * kSegRows < a.vb_r) wpu *= 2;
+  const int64_t units = (I_end - I_begin) * cdiv(j_end - j_begin, 32);
+  k_col_check<TC><<<(unsigned)cdiv(units, kThreads / 32 / wpu), kThreads, 0, st>>>(
+      a, j_begin, j_end, I_begin, I_end, mode, wpu);
 }
 
 // Screen of the fused checks: a line whose binary32 evaluation passes with a
@@ -1098,9 +1192,9 @@ cudaError_t verify_t(const Plan& P, void* C, void* ws, const Erased& er, bool re
   a.erased = er;
   const int64_t m = P.d.m, n = P.d.n;
   if (reread) {
-    k_col_check<TC><<<dim3((unsigned)cdiv(n, kThreads), gy(P.nvr)), kThreads, 0, st>>>(
-        a, 0, n, 0, P.nvr, 0);
-    k_row_check<TC><<<(unsigned)cdiv(m * P.nvc * 32, kThreads), kThreads, 0, st>>>(a);
+    run_col_check<TC>(a, 0, n, 0, P.nvr, 0, st);
+    k_row_check<TC><<<(unsigned)cdiv(cdiv(m, kRowLinesW) * P.nvc, kThreads / 32), kThreads, 0,
+                      st>>>(a);
   } else {
     const char* w = static_cast<const char*>(ws);
     k_col_fused<<<dim3((unsigned)cdiv(n, kThreads), gy(P.nvr)), kThreads, 0, st>>>(
@@ -1127,8 +1221,7 @@ cudaError_t recover_t(const Plan& P, void* C, void* ws, int bj, const int* rows,
   for (int u = 0; u < t; ++u) {  // re-check the rebuilt blocks' column lines
     const int64_t I0 = ((int64_t)rows[u] * P.bs) / P.d.vb_rows;
     const int64_t I1 = cdiv(((int64_t)rows[u] + 1) * P.bs, P.d.vb_rows);
-    k_col_check<TC><<<dim3((unsigned)cdiv(P.bc, kThreads), gy(I1 - I0)), kThreads, 0, st>>>(
-        a, (int64_t)bj * P.bc, ((int64_t)bj + 1) * P.bc, I0, I1, 1);
+    run_col_check<TC>(a, (int64_t)bj * P.bc, ((int64_t)bj + 1) * P.bc, I0, I1, 1, st);
   }
   count_launches(1 + t);
   return cudaGetLastError();
@@ -1154,8 +1247,7 @@ cudaError_t block_restore_t(const Plan& P, void* C, void* ws, int bi, int bj, co
       static_cast<TC*>(C), P.d.ldc, src, P.bs, P.bc, bi, bj, a.timeout);
   const int64_t I0 = ((int64_t)bi * P.bs) / P.d.vb_rows;
   const int64_t I1 = cdiv(((int64_t)bi + 1) * P.bs, P.d.vb_rows);
-  k_col_check<TC><<<dim3((unsigned)cdiv(P.bc, kThreads), gy(I1 - I0)), kThreads, 0, st>>>(
-      a, (int64_t)bj * P.bc, ((int64_t)bj + 1) * P.bc, I0, I1, 1);
+  run_col_check<TC>(a, (int64_t)bj * P.bc, ((int64_t)bj + 1) * P.bc, I0, I1, 1, st);
   count_launches(2);
   return cudaGetLastError();
 }
