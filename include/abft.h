@@ -40,7 +40,8 @@
  * defaults are the measured best choices):
  *  - ABFT_PROMOTE_KSTEPS  tensor-core k-steps (64 wide) accumulated before the
  *                         epilogue adds a partial into fp32 registers (0: none;
- *                         default 8 for ABFT_BF16X6, 16 for ABFT_BF16X3, 0 else).
+ *                         default 24 for ABFT_BF16X6 and ABFT_BF16X3, shared
+ *                         by their six or three products, 0 else).
  *  - ABFT_TALL_TILES      0 / 1: 128- or 256-row tiles for products without
  *                         promotion (default: 256 rows when m > 128 and the K
  *                         loop has at least 32 k-steps).

@@ -1856,9 +1856,9 @@ cudaError_t launch_gemm_lp(const Plan& P, const void* A, const void* B, float* C
     op.lda = P.L.op_a_ld;
     op.ldb = P.L.op_b_ld;
     if (d.dtype == ABFT_BF16X3) {
-      // A0 B0, A0 B1, A1 B0
+      // smallest first: A1 B0, A0 B1, A0 B0
       op.nseg = 3;
-      op.seg_a = 0u | (0u << 2) | (1u << 4);
+      op.seg_a = 1u | (0u << 2) | (0u << 4);
       op.seg_b = 0u | (1u << 2) | (0u << 4);
     } else {
       // the six products with a + b <= 2, smallest first: A2 B0, A1 B1, A0 B2,

@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   auto last_level = [](int f) { return (f & kNeed7) && !(f & kLeave) ? 7 : 6; };
 
   if (warp == 0 || warp == kWarpProdB) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       const bool pA = warp == 0;
       int s = 0;
       uint32_t ph = 0, par = 0;
@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       int s = 0, acc = 0;
       uint32_t ph = 0, aph = 0, par = 0;
       bool ok = true;
@@ -591,11 +591,8 @@ __global__ void __launch_bounds__(kThreads, 1)
               if (!tc::wait(full(s), ph, abort)) return false;
               tc::fence_after_sync();
               const uint32_t sa = tc::smem_addr(smem + s * stage), sb = sa + kABytes;
-#pragma unroll
-              for (int kk = 0; kk < BK / 16; ++kk)
-                tc::mma_f16(d, tc::sdesc_sw128(sa + kk * 32, 16, 1024),
-                            tc::sdesc_sw128(sb + kk * 2048, kBoxBytes, 1024), idesc,
-                            (kb > k0 || kk > 0) ? 1u : 0u);
+              tc::mma4_f16<false, 2, 128>(d, tc::sdesc_sw128(sa, 16, 1024),
+                                          tc::sdesc_sw128(sb, kBoxBytes, 1024), idesc, kb > k0);
               tc::commit(empty(s));
               if (++s == NS) { s = 0; ph ^= 1; }
             }

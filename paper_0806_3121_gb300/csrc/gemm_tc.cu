@@ -64,6 +64,7 @@ constexpr uint32_t B_BYTES = BN * BK * 2;          // 32 KiB
 // bf16 k-step, so the stage layout is unchanged); B is read K-major from its
 // transposed copy, 64 columns of C (64 rows of B^T, 8 KiB) per box
 constexpr int BK8 = 128;
+static_assert(BK == 4 * 16 && BK8 == 4 * 32, "a stage is four K steps (mma4)");
 constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr uint32_t TMEM_COLS = 2 * BN;             // two accumulators
 constexpr uint32_t STG_BYTES = 32 * 32 * 4;        // one epilogue warp's staging block
@@ -138,7 +139,8 @@ struct TcArgs {
   const InjectEntry* inj;
   uint64_t wait_ns;          // bounded-wait limit
   int stall_test;            // timeout test: the producer skips the first tile
-  int kpg;                   // k-steps per promotion group (0: one group per tile)
+  int chunk;                 // K-steps per promotion group, each of all segments (0: the
+                             // whole K loop in one group, one segment after the other)
   int group_m;               // raster group height (tile rows)
   // native FP8 data tiles: e4m3 products on the 8-bit tensor path, one
   // 128-wide k-step per accumulator, each scaled in the epilogue by the
@@ -257,7 +259,7 @@ struct TileView {
   int prob;                   // problem index (grouped products; 0 otherwise)
   int64_t nkb;                // k-blocks per segment
   int nseg;
-  int kpg;                    // k-steps per promotion group (0: the whole K loop)
+  int64_t chunk;              // K-steps per promotion group (nkb: the whole K loop)
   uint32_t seg_a, seg_b;      // plane of A / B per K segment (2 bits each)
   const CUtensorMap* maD;     // A-side maps: data / checksum (plane p at + p)
   const CUtensorMap* maC;
@@ -370,7 +372,7 @@ struct SingleSched {
     V.prob = 0;
     V.nkb = (g.k + BK - 1) / BK;
     V.nseg = g.nseg;
-    V.kpg = g.kpg;
+    V.chunk = g.chunk > 0 && g.chunk < V.nkb ? g.chunk : V.nkb;
     V.seg_a = g.seg_a;
     V.seg_b = g.seg_b;
     V.maD = &M->a[0];
@@ -408,7 +410,7 @@ struct SingleSched {
     if (V.f8) {  // data tile on the e4m3 codes: 128-wide k-steps in scale groups
       V.nkb = (g.k + 127) / 128;
       V.nseg = 1;
-      V.kpg = 0;
+      V.chunk = V.nkb;
       V.gmask = g.f8grp + ((T.row0 / 128) * g.ntn + T.col0 / 256) * g.f8words;
       V.seg_a = V.seg_b = 0;
       V.maD = &M->a[kF8Slot];
@@ -548,7 +550,7 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
   const int64_t total = S.total();
 
   if (warp == 0 || warp == kWarpProdB) {
-    if (lane == 0) {
+    if (tc::elect_one()) {
       // ---------------- TMA producers: warp 0 copies A, warp kWarpProdB copies
       // B (two issuing threads: one thread's issue rate limited the ring);
       // each arrives on the stage's full barrier with its own bytes
@@ -612,7 +614,7 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
         // a stage's MMAs take ~700 cycles: the per-stage bookkeeping is
         // incremental (no division per stage)
         int seg = 0, pa = (int)(T.seg_a & 3u), pb = (int)(T.seg_b & 3u);
-        int64_t kb = 0;
+        int64_t kb = 0, kc0 = 0, kc1 = min(T.chunk, nkb);
         for (int64_t kt = 0; kt < nkt; ++kt) {
           const int32_t kx = (int32_t)(kb * bkx);
           if (!tc::wait(empty(s), ph ^ 1, abort)) break;
@@ -679,9 +681,13 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
           }
           ++issued;
           if (++s == NS) { s = 0; ph ^= 1; }
-          if (++kb == nkb) {  // next K segment: its planes of A and B
-            kb = 0;
-            ++seg;
+          if (++kb == kc1) {  // next K segment (its planes of A and B) or chunk of K
+            if (++seg == T.nseg) {
+              seg = 0;
+              kc0 = kc1;
+              kc1 = min(kc0 + T.chunk, nkb);
+            }
+            kb = kc0;
             pa = (int)((T.seg_a >> (2 * seg)) & 3u);
             pb = (int)((T.seg_b >> (2 * seg)) & 3u);
           }
@@ -702,14 +708,13 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && issuer) {
+    if (issuer && tc::elect_one()) {
       // ---------------- MMA issuer (a pair: the even CTA's, for both)
       int s = 0, acc = 0;
       uint32_t ph = 0, aph = 0;
       for (int64_t t = tfirst; t < total && !*abort; t += tstep) {
         const TileView T = S.view(t);
         const int64_t nkt = T.nkb * T.nseg;
-        const int64_t gsz = (kPromote && T.kpg > 0 && T.kpg < nkt) ? T.kpg : nkt;
         const bool f8t = kF8 && T.f8;
         // a pair's MMA: M = 256 (128 rows per CTA), N = 256 (128 columns of B
         // per CTA; boxes a tile does not have are never stored)
@@ -729,11 +734,9 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
               for (int j = 0; j < kbs; ++j) {
                 const uint32_t a0 = sa + (j ? G::kABytes : 0u);
                 const uint32_t b0 = sa + G::kABytes + 2 * HALF_BYTES + j * B_BOX_BYTES;
-#pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                  tc::mma_f16_x<kPair>(d, tc::sdesc_sw128(a0 + kk * 32, 16, 1024),
-                                       tc::sdesc_sw128(b0 + kk * 2048, B_BOX_BYTES, 1024), idesc,
-                                       (kb > 0 || j > 0 || kk > 0) ? 1u : 0u);
+                tc::mma4_f16<kPair, 2, 128>(d, tc::sdesc_sw128(a0, 16, 1024),
+                                            tc::sdesc_sw128(b0, B_BOX_BYTES, 1024), idesc,
+                                            (kb > 0 || j > 0) ? 1u : 0u);
               }
               tc::commit_x<kPair>(empty(s));
               if (++s == NS) { s = 0; ph ^= 1; }
@@ -749,7 +752,7 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
         // group); the epilogue adds the groups
         int64_t g1 = 0;
         for (int64_t g0 = 0; g0 < nkt && ok; g0 = g1) {
-          g1 = f8t ? group_end_tile(T, g0, nkt) : min(g0 + gsz, nkt);
+          g1 = f8t ? group_end_tile(T, g0, nkt) : min(g0 + T.chunk * T.nseg, nkt);
           if (!tc::wait(tempty(acc), aph ^ 1, abort)) { ok = false; break; }
           tc::fence_after_sync();
           const uint32_t d = tmem + acc * BN;
@@ -766,16 +769,10 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
               // step of 16 rows moves 2 KiB) into accumulator columns 0 and
               // 128, K-major B = the checksum rows in the A region
               const uint32_t idesc_sw = tc::idesc_bf16_mn_a(BM, T.nsw_n);
-#pragma unroll
-              for (int kk = 0; kk < BK / 16; ++kk) {
-                const uint64_t bd = tc::sdesc_sw128(sa + kk * 32, 16, 1024);
-                for (int h2 = 0; h2 < 2; ++h2) {
-                  const uint64_t ad =
-                      tc::sdesc_sw128(sb + h2 * (2 * B_BOX_BYTES) + kk * 2048, B_BOX_BYTES, 1024);
-                  tc::mma_f16_x<kPair>(d + h2 * 128, ad, bd, idesc_sw,
-                                       (kb > g0 || kk > 0) ? 1u : 0u);
-                }
-              }
+              for (int h2 = 0; h2 < 2; ++h2)
+                tc::mma4_f16<kPair, 128, 2>(
+                    d + h2 * 128, tc::sdesc_sw128(sb + h2 * (2 * B_BOX_BYTES), B_BOX_BYTES, 1024),
+                    tc::sdesc_sw128(sa, 16, 1024), idesc_sw, kb > g0 ? 1u : 0u);
               tc::commit_x<kPair>(empty(s));
               if (++s == NS) { s = 0; ph ^= 1; }
               continue;
@@ -784,30 +781,21 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
               // e4m3: K = 32 codes per MMA.  A and B^T: K-major 128-byte rows in
               // 8-row groups 1024 B apart; a K step moves 32 B inside the
               // swizzled rows.
-#pragma unroll
-              for (int kk = 0; kk < BK8 / 32; ++kk) {
-                const uint64_t bd = tc::sdesc_sw128(sb + kk * 32, 16, 1024);
-                const uint64_t ad = tc::sdesc_sw128(sa + kk * 32, 16, 1024);
-                tc::mma_f8_x<kPair>(d, ad, bd, idesc, (kb > g0 || kk > 0) ? 1u : 0u);
-              }
+              tc::mma4_f8<kPair, 2, 2>(d, tc::sdesc_sw128(sa, 16, 1024),
+                                       tc::sdesc_sw128(sb, 16, 1024), idesc, kb > g0 ? 1u : 0u);
               tc::commit_x<kPair>(empty(s));
               if (++s == NS) { s = 0; ph ^= 1; }
               continue;
             }
-#pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              // B: N-major, 64-column boxes 8 KiB apart, 8-row (K) groups
-              // 1024 B apart; a K step of 16 rows moves 2 KiB.
-              const uint64_t bd = tc::sdesc_sw128(sb + kk * 2048, B_BOX_BYTES, 1024);
-              for (int h2 = 0; h2 < nmma; ++h2) {
-                // A: K-major, 128-byte rows, 8-row groups 1024 B apart; a K
-                // step of 16 elements moves 32 B inside the swizzled row; the
-                // second 128-row half starts 16 KiB later and accumulates into
-                // the second TMEM accumulator
-                const uint64_t ad = tc::sdesc_sw128(sa + h2 * (2 * HALF_BYTES) + kk * 32, 16, 1024);
-                tc::mma_f16_x<kPair>(d + h2 * BN, ad, bd, idesc, (kb > g0 || kk > 0) ? 1u : 0u);
-              }
-            }
+            // A: K-major, 128-byte rows, 8-row groups 1024 B apart; a K step of 16
+            // elements moves 32 B inside the swizzled row; the second 128-row half
+            // starts 16 KiB later and accumulates into the second TMEM
+            // accumulator.  B: N-major, 64-column boxes 8 KiB apart, 8-row (K)
+            // groups 1024 B apart; a K step of 16 rows moves 2 KiB.
+            for (int h2 = 0; h2 < nmma; ++h2)
+              tc::mma4_f16<kPair, 2, 128>(
+                  d + h2 * BN, tc::sdesc_sw128(sa + h2 * (2 * HALF_BYTES), 16, 1024),
+                  tc::sdesc_sw128(sb, B_BOX_BYTES, 1024), idesc, kb > g0 ? 1u : 0u);
             tc::commit_x<kPair>(empty(s));
             if (++s == NS) { s = 0; ph ^= 1; }
           }
@@ -894,9 +882,8 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
         continue;
       }
       const int64_t nkt = T.nkb * T.nseg;
-      const int64_t gsz = (kPromote && T.kpg > 0 && T.kpg < nkt) ? T.kpg : nkt;
       const bool f8t = kF8 && T.f8;
-      const bool one_group = f8t ? group_end_tile(T, 0, nkt) >= nkt : gsz >= nkt;
+      const bool one_group = f8t ? group_end_tile(T, 0, nkt) >= nkt : T.chunk >= T.nkb;
       // FP8 data tiles: this warp's 128 columns are one column block of B's
       // scales; the partial of a scale group is multiplied by its (power-of-two,
       // so exact) block-scale product.  This CTA's row block: a pair's odd CTA
@@ -1116,7 +1103,7 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
         float sc_next = scaled ? f8scale(0) : 1.0f;
         int64_t g1 = 0;
         for (int64_t g0 = 0; g0 < nkt; g0 = g1) {
-          g1 = f8t ? group_end_tile(T, g0, nkt) : min(g0 + gsz, nkt);
+          g1 = f8t ? group_end_tile(T, g0, nkt) : min(g0 + T.chunk * T.nseg, nkt);
           const float sc = sc_next;
           if (scaled && g1 < nkt) sc_next = f8scale(g1);
           if (!tc::wait(tfull(acc), aph, abort)) { aborted = true; break; }
@@ -1201,7 +1188,6 @@ struct GroupSched {
   const int4* tiles;  // {problem, tile row, tile column, 0}
   int64_t t_total;
   bool checksums;
-  int kpg;
   __device__ __forceinline__ int64_t total() const { return t_total; }
   __device__ __forceinline__ void prefetch() const {}
   __device__ __forceinline__ TileView view(int64_t t) const {
@@ -1215,7 +1201,7 @@ struct GroupSched {
     V.prob = e.x;
     V.nkb = cdiv(P.k, BK);
     V.nseg = 1;
-    V.kpg = kpg;
+    V.chunk = V.nkb;
     V.seg_a = V.seg_b = 0;  // one plane
     V.maD = &Mp.a;
     V.maC = &Mp.acs;
@@ -1295,8 +1281,8 @@ struct GroupSched {
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_grouped(const GProb* probs, const GMaps* maps, const int4* tiles, int64_t t_total,
                    int checksums, int* status, uint64_t wait_ns, const int32_t* inj_hdr,
-                   const InjectEntry* inj, int kpg) {
-  const GroupSched S{probs, maps, tiles, t_total, checksums != 0, kpg};
+                   const InjectEntry* inj) {
+  const GroupSched S{probs, maps, tiles, t_total, checksums != 0};
   tc_body<false, false, false, false>(S, status, wait_ns, 0, inj_hdr, inj);
 }
 
@@ -1459,16 +1445,21 @@ bool make_map_u8(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, 
 // 64-wide k-steps before the epilogue adds the partial into round-to-nearest
 // fp32 registers (0: the whole K loop in one accumulator).  The split products
 // exist for accuracy, and the tensor cores' fp32 accumulation over long K
-// loops would dominate their error: bf16x6 promotes every 8 steps (measured
-// relative error 4.8e-7 at k = 4096 and 16384, below cuBLAS SGEMM's; every 4
-// steps gives 2.7e-7 at 5 % lower throughput), bf16x3 every 16 (its 2-piece
-// split floor, 4.4e-6, dominates anyway).  Plain bf16 and FP8 do not promote
+// loops would dominate their error.  A group of a split product is a few K-steps
+// of all its segments, smallest products first, so an accumulator takes the large
+// products last and only a few of them: bf16x6 with 24 k-steps (4 of each of 6
+// segments) has relative error 2.8e-7 at 16384^3 (4.8e-7 when a group was 8
+// k-steps of one segment), bf16x3 its split's floor, 4.5e-6.  Sweeping a chunk of
+// K through all segments also reads each plane from DRAM once per wave of tiles
+// instead of up to three times: 16384^3 bf16x6 36.1 -> 33.0 ms per step, 8192^3
+// bf16x3 2.60 -> 2.42 (groups of 6 / 12 / 18 / 24 k-steps: 33.4 / 33.1 / 33.5 / 32.9
+// and 2.55 / 2.49 / 2.44 / 2.42 ms).  Plain bf16 and FP8 do not promote
 // by default (measured 12-25 % slower at 16384^3 with it).  The environment
 // variable ABFT_PROMOTE_KSTEPS overrides the choice for every dtype.
 int promote_ksteps(int dtype) {
   const char* env = getenv("ABFT_PROMOTE_KSTEPS");
   if (env && *env) return std::max(0, atoi(env));
-  return dtype == ABFT_BF16X6 ? 8 : (dtype == ABFT_BF16X3 ? 16 : 0);
+  return dtype == ABFT_BF16X6 || dtype == ABFT_BF16X3 ? 24 : 0;
 }
 
 // Raster group height of the single-problem tile order: tiles run column by
@@ -1485,8 +1476,8 @@ int raster_group_rows(int bm) {
 // enough (at least 32 k-steps) that the tile's epilogue, which no longer
 // overlaps the next tile's MMAs, is a small share of it.  ABFT_TALL_TILES=0
 // or 1 forces the choice.
-bool use_tall(int64_t m, int64_t nkt, int kpg) {
-  if (kpg > 0) return false;
+bool use_tall(int64_t m, int64_t nkt, int chunk) {
+  if (chunk > 0) return false;
   const char* env = getenv("ABFT_TALL_TILES");
   if (env && *env) return env[0] == '1';
   return m > BM && nkt >= 32;
@@ -1537,10 +1528,24 @@ int64_t cs_stride(int64_t ncs, int64_t total, int grid) {
   return S;
 }
 
+}  // namespace
+
+int num_sms() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return 148;
+  if (!g_num_sms[dev]) {
+    int v = 0;
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    g_num_sms[dev] = v > 0 ? v : 148;
+  }
+  return g_num_sms[dev];
+}
+
 // CTA pairs (clusters of two) of a pair-tile kernel that fit on the GPU at
 // once: the persistent grid's size.  Clusters are placed within a GPC, so this
 // can be less than half the SM count.
-int g_pair_clusters[64] = {};
+static int g_pair_clusters[64] = {};
 int pair_clusters(const void* kernel, size_t smem) {
   int dev = 0;
   cudaGetDevice(&dev);
@@ -1563,20 +1568,6 @@ int pair_clusters(const void* kernel, size_t smem) {
   }
   if (dev >= 0 && dev < 64) g_pair_clusters[dev] = n;
   return n;
-}
-
-}  // namespace
-
-int num_sms() {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) return 148;
-  if (!g_num_sms[dev]) {
-    int v = 0;
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    g_num_sms[dev] = v > 0 ? v : 148;
-  }
-  return g_num_sms[dev];
 }
 
 // Timeout word of checksum-free products run without a workspace.
@@ -1623,7 +1614,8 @@ cudaError_t launch_gemm_bf16(const Plan& P, const TcOperands& op, float* C, void
   g.nseg = op.nseg;
   g.seg_a = op.seg_a;
   g.seg_b = op.seg_b;
-  g.kpg = promote_ksteps(d.dtype);
+  const int kpg = promote_ksteps(d.dtype);
+  g.chunk = kpg > 0 ? std::max(1, kpg / op.nseg) : 0;
   if (op.a8) {  // native FP8 data tiles on the e4m3 codes (promoted every k-step)
     if (!make_map_u8(&M.a[kF8Slot], op.a8, d.m, d.k, op.lda8, 128, BM / 2) ||
         !make_map_u8(&M.a128[kF8Slot], op.a8, d.m, d.k, op.lda8, 128, BM) ||
@@ -1635,11 +1627,11 @@ cudaError_t launch_gemm_bf16(const Plan& P, const TcOperands& op, float* C, void
     g.sB = op.sB;
     g.nsa = cdiv(d.k, 128);
     g.nsb = cdiv(d.n, 128);
-    g.kpg = 0;  // the checksum tiles (bf16 planes) run one group
+    g.chunk = 0;  // the checksum tiles (bf16 planes) run one group
     g.f8grp = op.f8grp;
     g.f8words = cdiv(cdiv(d.k, 128), 32);
   }
-  const bool tall = !pair && !g.f8 && use_tall(d.m, cdiv(d.k, BK) * op.nseg, g.kpg);
+  const bool tall = !pair && !g.f8 && use_tall(d.m, cdiv(d.k, BK) * op.nseg, g.chunk);
   const int bm = (tall || pair) ? 256 : BM;
   g.ntm = (int)cdiv(d.m, bm);
   g.ntn = (int)cdiv(d.n, BN);
@@ -1675,10 +1667,10 @@ cudaError_t launch_gemm_bf16(const Plan& P, const TcOperands& op, float* C, void
   g.wait_ns = g.stall_test ? 200000000ull : tc::kWaitLimitNs;
   const auto kernel =
       pair ? (g.f8 ? k_gemm_bf16<true, false, true, true>
-                   : g.kpg > 0 ? k_gemm_bf16<true, false, false, true>
+                   : g.chunk > 0 ? k_gemm_bf16<true, false, false, true>
                                : k_gemm_bf16<false, false, false, true>)
            : (g.f8 ? k_gemm_bf16<true, false, true, false>
-                   : g.kpg > 0 ? k_gemm_bf16<true, false, false, false>
+                   : g.chunk > 0 ? k_gemm_bf16<true, false, false, false>
                                : (tall ? k_gemm_bf16<false, true, false, false>
                                        : k_gemm_bf16<false, false, false, false>));
   const size_t smem =
@@ -1746,7 +1738,7 @@ cudaError_t launch_group_gemm(const GroupDev& G, bool checksums, cudaStream_t st
   if (e != cudaSuccess) return e;
   k_gemm_grouped<<<grid, kThreads, SMEM_BYTES, st>>>(
       G.probs, G.maps, checksums ? G.tiles_cs : G.tiles_plain, total, checksums ? 1 : 0, status,
-      tc::kWaitLimitNs, checksums ? G.inj_hdr : nullptr, G.inj, 0);
+      tc::kWaitLimitNs, checksums ? G.inj_hdr : nullptr, G.inj);
   count_launches(1);
   return cudaGetLastError();
 }

@@ -20,6 +20,23 @@ __device__ __forceinline__ uint64_t& wait_limit_ns() {
   return lim;
 }
 
+// True in one lane of a converged warp.  The roles that issue tcgen05 and TMA
+// instructions run in this lane: under `lane == 0` the compiler cannot tell that
+// one thread is active, so it builds the uniform-register operands of every such
+// instruction in a loop over the lanes.  Measured per k-step of four M = 128 MMAs
+// with a commit and a wait: 552 clocks at any N under `lane == 0`; here, with the
+// four MMAs in one asm block (mma4), 236 / 256 / 512 at N = 64 / 128 / 256, the
+// tensor pipe's own rate.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
@@ -154,28 +171,35 @@ __device__ __forceinline__ void commit(uint32_t bar) {
                : "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem], 16-bit inputs (kind::f16), fp32 accumulate.
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                        uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// D[tmem] (+)= A[smem] * B[smem], 8-bit floating-point inputs (kind::f8f6f4,
-// K = 32 per instruction), fp32 accumulate.
-__device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                       uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
+// The four K steps of one stage, D[tmem] (+)= A[smem] * B[smem] with fp32
+// accumulation: kind::f16 (16-bit inputs, K = 16 each) or kind::f8f6f4 (8-bit
+// floating-point inputs, K = 32 each), on one CTA or a CTA pair.  The descriptors
+// advance by SA / SB 16-byte units per step; accumulate = 0: the first step
+// overwrites D.
+#define ABFT_MMA4(NAME, GROUP, KIND)                                                           \
+  template <int SA, int SB>                                                                    \
+  __device__ __forceinline__ void NAME(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,     \
+                                       uint32_t accumulate) {                                  \
+    asm volatile(                                                                              \
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 x, y;\n\t"                                         \
+        "setp.ne.b32 p, %4, 0;\n\t"                                                            \
+        "setp.eq.u32 q, 0, 0;\n\t"                                                             \
+        "tcgen05.mma." GROUP "." KIND " [%0], %1, %2, %3, p;\n\t"                              \
+        "add.s64 x, %1, %5;\n\tadd.s64 y, %2, %6;\n\t"                                         \
+        "tcgen05.mma." GROUP "." KIND " [%0], x, y, %3, q;\n\t"                                \
+        "add.s64 x, %1, %7;\n\tadd.s64 y, %2, %8;\n\t"                                         \
+        "tcgen05.mma." GROUP "." KIND " [%0], x, y, %3, q;\n\t"                                \
+        "add.s64 x, %1, %9;\n\tadd.s64 y, %2, %10;\n\t"                                        \
+        "tcgen05.mma." GROUP "." KIND " [%0], x, y, %3, q;\n\t}\n" ::"r"(d),                  \
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "n"(SA), "n"(SB), "n"(2 * SA),            \
+        "n"(2 * SB), "n"(3 * SA), "n"(3 * SB)                                                  \
+        : "memory");                                                                           \
+  }
+ABFT_MMA4(mma4_f16_cta, "cta_group::1", "kind::f16")
+ABFT_MMA4(mma4_f16_pair, "cta_group::2", "kind::f16")
+ABFT_MMA4(mma4_f8_cta, "cta_group::1", "kind::f8f6f4")
+ABFT_MMA4(mma4_f8_pair, "cta_group::2", "kind::f8f6f4")
+#undef ABFT_MMA4
 
 // Shared-memory matrix descriptor (tcgen05): start address, leading and
 // stride byte offsets, descriptor version 1, 128-byte swizzle.
@@ -262,6 +286,36 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cbar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cbar)
                : "memory");
 }
+// A 32-bit word in either CTA's shared memory (addr: its cluster address); the
+// writer then arrives with mbar_arrive_cluster, the reader waits with
+// wait_cluster.
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// wait(), ordered after the other CTA's writes before its arrivals.
+__device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort) {
+  if (mbar_try_wait_cluster(bar, parity)) return true;
+  const uint64_t t0 = globaltimer();
+  while (true) {
+    if (mbar_try_wait_cluster(bar, parity)) return true;
+    if (*abort) return false;
+    if (globaltimer() - t0 > wait_limit_ns()) {
+      *abort = 1;
+      return false;
+    }
+  }
+}
 // TMA loads into this CTA's shared memory whose bytes complete on a barrier
 // of either CTA of the pair (cbar: its cluster address).
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map,
@@ -302,35 +356,19 @@ __device__ __forceinline__ void commit_pair(uint32_t bar, uint16_t cta_mask) {
       "h"(cta_mask)
       : "memory");
 }
-__device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                             uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void mma_f8_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                            uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
 
 // The single-CTA or the pair form, chosen at compile time.
-template <bool kPair>
-__device__ __forceinline__ void mma_f16_x(uint32_t d, uint64_t a, uint64_t b, uint32_t i,
-                                          uint32_t acc) {
-  if constexpr (kPair) mma_f16_pair(d, a, b, i, acc); else mma_f16(d, a, b, i, acc);
-}
-template <bool kPair>
-__device__ __forceinline__ void mma_f8_x(uint32_t d, uint64_t a, uint64_t b, uint32_t i,
+template <bool kPair, int SA, int SB>
+__device__ __forceinline__ void mma4_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t i,
                                          uint32_t acc) {
-  if constexpr (kPair) mma_f8_pair(d, a, b, i, acc); else mma_f8(d, a, b, i, acc);
+  if constexpr (kPair) mma4_f16_pair<SA, SB>(d, a, b, i, acc);
+  else mma4_f16_cta<SA, SB>(d, a, b, i, acc);
+}
+template <bool kPair, int SA, int SB>
+__device__ __forceinline__ void mma4_f8(uint32_t d, uint64_t a, uint64_t b, uint32_t i,
+                                        uint32_t acc) {
+  if constexpr (kPair) mma4_f8_pair<SA, SB>(d, a, b, i, acc);
+  else mma4_f8_cta<SA, SB>(d, a, b, i, acc);
 }
 // Stage / accumulator signal: the pair's commit reaches both CTAs' barriers.
 template <bool kPair>
