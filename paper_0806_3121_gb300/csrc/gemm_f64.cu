@@ -128,21 +128,21 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_f64(const F64Args g, const
            (int64_t)(cs_col ? tx - T.tn : tx) * BN);
 }
 
-// The tiles (128 x 64 bpt) that the sliced product left out, as BM x BN tiles.
+// The tiles (64 hpt x 64 bpt) that the sliced product left out, as BM x BN tiles.
 __global__ void __launch_bounds__(kThreads, 2)
-    k_gemm_f64_bad(const F64Args g, const TileGrid T, int bpt, const int* any,
+    k_gemm_f64_bad(const F64Args g, const TileGrid T, int hpt, int bpt, const int* any,
                    const uint8_t* bad) {
   if (*any == 0) return;
-  const int64_t total = T.total() * 2 * bpt;
+  const int64_t total = T.total() * hpt * bpt;
   for (int64_t u = blockIdx.x; u < total; u += gridDim.x) {
-    const int64_t t = u / (2 * bpt);
-    const int s = (int)(u - t * 2 * bpt);
+    const int64_t t = u / (hpt * bpt);
+    const int s = (int)(u - t * hpt * bpt);
     if (!bad[t]) continue;
     int ty, tx;
     T.decode(t, ty, tx);
     const bool cs_row = ty >= T.tm, cs_col = tx >= T.tn;
-    const int64_t row0 = (int64_t)(cs_row ? ty - T.tm : ty) * 2 * BM + (s & 1) * BM;
-    const int64_t col0 = ((int64_t)(cs_col ? tx - T.tn : tx) * bpt + (s >> 1)) * BN;
+    const int64_t row0 = ((int64_t)(cs_row ? ty - T.tm : ty) * hpt + s % hpt) * BM;
+    const int64_t col0 = ((int64_t)(cs_col ? tx - T.tn : tx) * bpt + s / hpt) * BN;
     if (row0 >= (cs_row ? g.R : g.m) || col0 >= (cs_col ? g.Cc : g.n)) continue;
     __syncthreads();  // the previous tile's shared memory has been read
     tile_f64(g, cs_row, cs_col, row0, col0);
@@ -151,11 +151,11 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 }  // namespace
 
-cudaError_t launch_gemm_f64_bad(const F64Args& g, const TileGrid& tiles, int bpt, const int* any,
-                                const uint8_t* bad, cudaStream_t st) {
-  const int64_t total = tiles.total() * 2 * bpt;
+cudaError_t launch_gemm_f64_bad(const F64Args& g, const TileGrid& tiles, int hpt, int bpt,
+                                const int* any, const uint8_t* bad, cudaStream_t st) {
+  const int64_t total = tiles.total() * hpt * bpt;
   const unsigned grid = (unsigned)std::min<int64_t>(total, 2 * num_sms());
-  k_gemm_f64_bad<<<grid, kThreads, 0, st>>>(g, tiles, bpt, any, bad);
+  k_gemm_f64_bad<<<grid, kThreads, 0, st>>>(g, tiles, hpt, bpt, any, bad);
   count_launches(1);
   return cudaGetLastError();
 }

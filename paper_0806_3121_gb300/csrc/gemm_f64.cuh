@@ -58,10 +58,10 @@ struct F64Args {
   int accumulate;  // 1: add to C, E, F (a later panel of K) instead of writing them
 };
 
-// The DFMA kernel on the tiles (128 x 64 bpt) of the sliced product whose byte
+// The DFMA kernel on the tiles (64 hpt x 64 bpt) of the sliced product whose byte
 // in `bad` is set; returns at once when *any is zero.
-cudaError_t launch_gemm_f64_bad(const F64Args& g, const TileGrid& tiles, int bpt, const int* any,
-                                const uint8_t* bad, cudaStream_t st);
+cudaError_t launch_gemm_f64_bad(const F64Args& g, const TileGrid& tiles, int hpt, int bpt,
+                                const int* any, const uint8_t* bad, cudaStream_t st);
 
 // The sliced product in the workspace regions of P.f64tc.
 cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaStream_t st);

@@ -29,17 +29,17 @@
 // exponents outside [-440, 500] are left to the DFMA kernel (k_gemm_f64_bad).
 //
 // The tensor cores bound it: 29 or 37 products of 2 m n k bf16 flops each.
-// 128 x (64 bpt)-tiles, one CTA per SM: warps 0 / 10 copy A / B by TMA into a
-// shared-memory ring, warp 1 issues tcgen05.mma into two alternating TMEM
+// 128 x (64 bpt)-tiles on one CTA or 256 x 256 tiles on a pair, one CTA per SM:
+// warps 0 / 10 copy A / B by TMA into a shared-memory ring, warp 1 issues tcgen05.mma into two alternating TMEM
 // accumulators, warps 2-9 add each accumulator into 128 integer registers per
 // thread.  Level sums go to a per-CTA scratch (coalesced, mostly L2) because
 // eight levels do not fit the registers and the FP64 pipe is too narrow to fold
 // them as they come (8 folds of a 128 x 256 tile at 2 per clock would take 131 k
 // clocks of the tile's 1.9 M at k = 8192).
 //
-// Measured against the DFMA kernel alone (encode and product, and whole steps):
-// 8192^3 on a 16 x 16 grid 953.6 -> 27.4 ms, 4096^3 step 132.2 -> 7.0 ms, two chained
-// 2048^3 products 34.0 -> 2.5 ms, 1000 x 1501 x 777 step 2.92 -> 0.78 ms.  Relative
+// Measured, product kernels alone: 8192^3 on a 16 x 16 grid 949 ms on the FP64 pipe,
+// 22 here; 4096^3 on an 8 x 8 grid 130 -> 2.9; 2048^3 16.3 -> 0.38 .. 0.47; 1000 x 1501
+// x 777 2.36 -> 0.13; 512^3 0.53 -> 0.06.  Relative
 // Frobenius error against the exact product, N(0,1): 4.5e-17 (DFMA 7.7e-16) at k =
 // 512, 2.8e-16 (2.0e-15) at k = 4096, 4.7e-16 (4.9e-15) at k = 20000.
 #include <cuda.h>
@@ -70,9 +70,13 @@ constexpr int kNotExact = 100;    // digit index of an operand row that is cut o
 constexpr size_t kPlaneBudget = size_t(6) << 30;
 constexpr int kSms = 152;  // persistent CTAs the workspace is laid out for
 
-constexpr int stages(int bpt) { return bpt == 4 ? 4 : (bpt == 2 ? 6 : 8); }
-constexpr size_t smem_bytes(int bpt) {
-  return 1024 + (size_t)stages(bpt) * (kABytes + bpt * kBoxBytes) + 256;
+// Tile kinds.  One CTA: 128 rows x bpt 64-column boxes.  CTA pair (bpt = 4): 256
+// x 256, one cta_group::2 MMA per K step reads 128 rows of A and 128 columns of B
+// from each CTA's shared memory.
+constexpr int cta_boxes(int bpt, bool pair) { return pair ? bpt / 2 : bpt; }
+constexpr int stages(int boxes) { return boxes == 4 ? 4 : (boxes == 2 ? 6 : 8); }
+constexpr size_t smem_bytes(int boxes) {
+  return 1024 + (size_t)stages(boxes) * (kABytes + boxes * kBoxBytes) + 320;
 }
 static_assert(smem_bytes(4) <= 232448 && smem_bytes(2) <= 232448 && smem_bytes(1) <= 232448,
               "shared memory per CTA");
@@ -373,8 +377,8 @@ __global__ void __launch_bounds__(kSliceThreads) k_f64_slice(const SliceArgs a) 
 
 struct Maps {
   CUtensorMap a;   // (kpad, planes x rows_a): box 64 x 128
-  CUtensorMap bw;  // (64, planes x kpad, column boxes): box 64 x 64 x bpt
-  CUtensorMap b1;  // the same, one column box
+  CUtensorMap bw;  // (64, planes x kpad, column boxes): box 64 x 64 x a CTA's boxes
+  CUtensorMap b1;  // (cols_b, planes x kpad): box 64 x 64
 };
 
 struct ProdArgs {
@@ -440,43 +444,55 @@ __device__ __forceinline__ double round_f64(int64_t H, int64_t Lo, int e) {
 
 struct TileView64 {
   bool cs_row, cs_col;
-  int64_t row0, col0;     // in C / E / F
+  int64_t row0, col0;     // this CTA's first row, the tile's first column, in C / E / F
   int arow, bcol;         // padded row of the A planes, column of the B planes
-  int nbox, ncols;        // boxes and valid columns
+  int ncols, nmma;        // valid columns; the MMA's N
+  int bx, nbox;           // this CTA's first column of the B planes and its boxes
+  bool full;              // all boxes of a full tile (one copy)
   int64_t rlim;
 };
 
-__device__ __forceinline__ TileView64 view_tile(const ProdArgs& p, int64_t t) {
+template <bool kPair>
+__device__ __forceinline__ TileView64 view_tile(const ProdArgs& p, int64_t t, int rank) {
   int ty, tx;
   p.T.decode(t, ty, tx);
   TileView64 V;
   V.cs_row = ty >= p.T.tm;
   V.cs_col = tx >= p.T.tn;
-  V.row0 = (int64_t)(V.cs_row ? ty - p.T.tm : ty) * BM;
+  V.row0 = (int64_t)(V.cs_row ? ty - p.T.tm : ty) * (kPair ? 2 * BM : BM) + BM * rank;
   V.col0 = (int64_t)(V.cs_col ? tx - p.T.tn : tx) * 64 * p.bpt;
   V.arow = (int)V.row0 + (V.cs_row ? p.row_cs : 0);
   V.bcol = (int)V.col0 + (V.cs_col ? p.col_cs : 0);
   V.rlim = V.cs_row ? p.g.R : p.g.m;
   V.ncols = (int)min((int64_t)64 * p.bpt, (V.cs_col ? p.g.Cc : p.g.n) - V.col0);
-  V.nbox = (V.ncols + 63) / 64;
+  // a pair's MMA takes half of its N columns from each CTA
+  V.nmma = kPair ? (V.ncols + 31) / 32 * 32 : (V.ncols + 15) / 16 * 16;
+  V.bx = V.bcol + (kPair ? V.nmma / 2 * rank : 0);
+  V.nbox = ((kPair ? V.nmma / 2 : V.ncols) + 63) / 64;
+  V.full = kPair ? V.nmma == 64 * p.bpt : V.nbox == p.bpt;
   return V;
 }
 
 // What a tile's magnitudes ask for.
 constexpr int kNeed7 = 1, kLeave = 2;
 
+template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_f64_tc(const __grid_constant__ Maps M, const ProdArgs p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  const int NS = stages(p.bpt);
-  const uint32_t stage = kABytes + p.bpt * kBoxBytes;
+  const int boxes = cta_boxes(p.bpt, kPair);  // this CTA's boxes of a full tile
+  const int NS = stages(boxes);
+  const uint32_t stage = kABytes + boxes * kBoxBytes;
+  constexpr int kWarpsAll = kPair ? 2 * kEpiWarps : kEpiWarps;  // epilogue warps of a tile
+  const int rank = kPair ? (int)tc::cluster_ctarank() : 0;
+  const bool issuer = rank == 0;  // its MMA warp issues for both CTAs of a pair
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NS * stage);
   // full [8], empty [8], tmem full [2], tmem empty [2], drain, decision
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 6);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* need = reinterpret_cast<volatile int*>(tmem_slot + 2);  // [2][kEpiWarps]
+  volatile int* need = reinterpret_cast<volatile int*>(tmem_slot + 2);  // [2][kWarpsAll]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   auto full = [&](int s) { return tc::smem_addr(&bars[s]); };
   auto empty = [&](int s) { return tc::smem_addr(&bars[kMaxStages + s]); };
@@ -492,10 +508,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int a = 0; a < 2; ++a) {
       tc::mbar_init(tfull(a), 1);
-      tc::mbar_init(tempty(a), kEpiWarps);
+      tc::mbar_init(tempty(a), kWarpsAll);
     }
     tc::mbar_init(drain, 1);
-    tc::mbar_init(decided, kEpiWarps);
+    tc::mbar_init(decided, kWarpsAll);
     *abort = 0;
     tc::wait_limit_ns() = p.wait_ns;
     tc::fence_barrier_init();
@@ -504,20 +520,33 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc::prefetch_tmap(&M.b1);
   }
   if (warp == 1) {
-    tc::tmem_alloc(tc::smem_addr(tmem_slot), 512);
-    tc::tmem_relinquish();
+    if constexpr (kPair) {
+      tc::tmem_alloc_pair(tc::smem_addr(tmem_slot), 512);
+      tc::tmem_relinquish_pair();
+    } else {
+      tc::tmem_alloc(tc::smem_addr(tmem_slot), 512);
+      tc::tmem_relinquish();
+    }
   }
   tc::fence_before_sync();
-  __syncthreads();
+  if constexpr (kPair)
+    tc::cluster_sync();
+  else
+    __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
   const int64_t total = p.T.total();
+  const int64_t tfirst = kPair ? (int64_t)tc::cluster_id() : (int64_t)blockIdx.x;
+  const int64_t tstep = kPair ? (int64_t)tc::num_clusters() : (int64_t)gridDim.x;
   const int nkb = p.nkb;
   // the tile's decision, known to every role before its level 7 (phase: tile parity)
   auto decision = [&](uint32_t par) {
     int f = 0;
-    for (int w = 0; w < kEpiWarps; ++w) f |= need[par * kEpiWarps + w];
+    for (int w = 0; w < kWarpsAll; ++w) f |= need[par * kWarpsAll + w];
     return f;
+  };
+  auto wait_decided = [&](uint32_t par) {
+    return kPair ? tc::wait_cluster(decided, par, abort) : tc::wait(decided, par, abort);
   };
   auto last_level = [](int f) { return (f & kNeed7) && !(f & kLeave) ? 7 : 6; };
 
@@ -528,25 +557,39 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t ph = 0, par = 0;
       int64_t issued = 0;
       bool ok = true;
-      for (int64_t t = blockIdx.x; t < total && ok && !*abort; t += gridDim.x, par ^= 1) {
+      for (int64_t t = tfirst; t < total && ok && !*abort; t += tstep, par ^= 1) {
         if (p.stall_test && t == 0) continue;
-        const TileView64 V = view_tile(p, t);
-        const uint32_t tx = pA ? kABytes : (uint32_t)V.nbox * kBoxBytes;
+        const TileView64 V = view_tile<kPair>(p, t, rank);
+        // a pair's bytes (both CTAs') land on the issuer's barrier, which the
+        // issuer's producers expect
+        const uint32_t tx = (pA ? kABytes : (uint32_t)V.nbox * kBoxBytes) * (kPair ? 2 : 1);
         // one pair of planes: nkb k-steps
         auto pair = [&](int pa, int pb) {
-          const int arow = pa * p.rows_a + V.arow, brow = pb * p.kpad, cb = V.bcol / 64;
+          const int arow = pa * p.rows_a + V.arow, brow = pb * p.kpad;
           for (int kb = 0; kb < nkb; ++kb) {
             if (!tc::wait(empty(s), ph ^ 1, abort)) return false;
             const uint32_t sa = tc::smem_addr(smem + s * stage);
-            tc::mbar_arrive_expect_tx(full(s), tx);
+            if (issuer) tc::mbar_arrive_expect_tx(full(s), tx);
+            const uint32_t fb = kPair ? tc::mapa(full(s), 0) : full(s);
             if (pA) {
-              tc::tma_load_2d(sa, &M.a, full(s), kb * BK, arow);
-            } else if (V.nbox == p.bpt) {
-              tc::tma_load_3d(sa + kABytes, &M.bw, full(s), 0, brow + kb * BK, cb);
+              if constexpr (kPair)
+                tc::tma_load_2d_pair(sa, &M.a, fb, kb * BK, arow);
+              else
+                tc::tma_load_2d(sa, &M.a, fb, kb * BK, arow);
+            } else if (V.full) {
+              if constexpr (kPair)
+                tc::tma_load_3d_pair(sa + kABytes, &M.bw, fb, 0, brow + kb * BK, V.bx / 64);
+              else
+                tc::tma_load_3d(sa + kABytes, &M.bw, fb, 0, brow + kb * BK, V.bx / 64);
             } else {
-              for (int b = 0; b < V.nbox; ++b)
-                tc::tma_load_3d(sa + kABytes + b * kBoxBytes, &M.b1, full(s), 0, brow + kb * BK,
-                                cb + b);
+              for (int b = 0; b < V.nbox; ++b) {
+                if constexpr (kPair)
+                  tc::tma_load_2d_pair(sa + kABytes + b * kBoxBytes, &M.b1, fb, V.bx + 64 * b,
+                                       brow + kb * BK);
+                else
+                  tc::tma_load_2d(sa + kABytes + b * kBoxBytes, &M.b1, fb, V.bx + 64 * b,
+                                  brow + kb * BK);
+              }
             }
             ++issued;
             if (++s == NS) { s = 0; ph ^= 1; }
@@ -558,28 +601,30 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int lev = 0; lev <= top && ok; ++lev) {
           for (int i = 0; i <= lev && ok; ++i) ok = pair(i, lev - i);
           if (lev == 6 && ok) {
-            ok = tc::wait(decided, par, abort);
+            ok = wait_decided(par);
             if (ok) top = last_level(decision(par));
           }
         }
       }
-      // no copies left in flight (bounded)
+      // no copies left in flight (bounded): a pair's complete on the issuer's
+      // barriers, so its CTAs wait until the MMAs have consumed the stages
       for (int q = 0; q < NS && issued > 0; ++q, --issued) {
         if (--s < 0) { s = NS - 1; ph ^= 1; }
         const uint64_t t0 = tc::globaltimer();
-        while (!tc::mbar_try_wait(full(s), ph) && tc::globaltimer() - t0 < tc::wait_limit_ns()) {
+        const uint32_t bar = kPair ? empty(s) : full(s);
+        while (!tc::mbar_try_wait(bar, ph) && tc::globaltimer() - t0 < tc::wait_limit_ns()) {
         }
       }
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (tc::elect_one()) {
+    if (issuer && tc::elect_one()) {
       int s = 0, acc = 0;
       uint32_t ph = 0, aph = 0, par = 0;
       bool ok = true;
-      for (int64_t t = blockIdx.x; t < total && ok && !*abort; t += gridDim.x, par ^= 1) {
-        const TileView64 V = view_tile(p, t);
-        const uint32_t idesc = tc::idesc_bf16(BM, (V.ncols + 15) / 16 * 16, 1);
+      for (int64_t t = tfirst; t < total && ok && !*abort; t += tstep, par ^= 1) {
+        const TileView64 V = view_tile<kPair>(p, t, rank);
+        const uint32_t idesc = tc::idesc_bf16(kPair ? 2 * BM : BM, V.nmma, 1);
         // nk k-steps in accumulators of g each
         auto level = [&](int nk, int g) {
           for (int k0 = 0; k0 < nk; k0 += g) {
@@ -591,12 +636,12 @@ __global__ void __launch_bounds__(kThreads, 1)
               if (!tc::wait(full(s), ph, abort)) return false;
               tc::fence_after_sync();
               const uint32_t sa = tc::smem_addr(smem + s * stage), sb = sa + kABytes;
-              tc::mma4_f16<false, 2, 128>(d, tc::sdesc_sw128(sa, 16, 1024),
+              tc::mma4_f16<kPair, 2, 128>(d, tc::sdesc_sw128(sa, 16, 1024),
                                           tc::sdesc_sw128(sb, kBoxBytes, 1024), idesc, kb > k0);
-              tc::commit(empty(s));
+              tc::commit_x<kPair>(empty(s));
               if (++s == NS) { s = 0; ph ^= 1; }
             }
-            tc::commit(tfull(acc));
+            tc::commit_x<kPair>(tfull(acc));
             if (++acc == 2) { acc = 0; aph ^= 1; }
           }
           return true;
@@ -606,12 +651,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int lev = 0; lev <= top && ok; ++lev) {
           ok = level((lev + 1) * nkb, kGroupSteps);
           if (lev == 6 && ok) {
-            ok = tc::wait(decided, par, abort);
+            ok = wait_decided(par);
             if (ok) top = last_level(decision(par));
           }
         }
       }
-      tc::commit(drain);  // every MMA has completed before TMEM is freed
+      // every MMA has completed before TMEM is freed
+      if constexpr (kPair)
+        tc::commit_pair(drain, 1);
+      else
+        tc::commit(drain);
       const uint64_t t0 = tc::globaltimer();
       while (!tc::mbar_try_wait(drain, 0) && tc::globaltimer() - t0 < tc::wait_limit_ns()) {
       }
@@ -633,11 +682,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto release = [&]() {
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(tempty(acc));
+      if (lane == 0) {
+        if constexpr (kPair)
+          tc::mbar_arrive_cluster(tc::mapa(tempty(acc), 0));
+        else
+          tc::mbar_arrive(tempty(acc));
+      }
       if (++acc == 2) { acc = 0; aph ^= 1; }
     };
-    for (int64_t t = blockIdx.x; t < total && ok; t += gridDim.x, par ^= 1) {
-      const TileView64 V = view_tile(p, t);
+    for (int64_t t = tfirst; t < total && ok; t += tstep, par ^= 1) {
+      const TileView64 V = view_tile<kPair>(p, t, rank);
       const int64_t row = V.row0 + 32 * q + lane;
       const bool rv = row < V.rlim;
       const int2 ri = rv ? p.a_row[V.arow + 32 * q + lane] : make_int2(0, 0);
@@ -669,10 +723,19 @@ __global__ void __launch_bounds__(kThreads, 1)
       else if (zr + zc <= 7) f = f ? kNeed7 : 0;
       f = (__any_sync(0xffffffffu, f & kNeed7) ? kNeed7 : 0) |
           (__any_sync(0xffffffffu, f & kLeave) ? kLeave : 0);
+      // every warp of the tile tells every CTA of it
       if (lane == 0) {
-        need[par * kEpiWarps + ew] = f;
-        __threadfence_block();
-        tc::mbar_arrive(decided);
+        if constexpr (kPair) {
+          const uint32_t at = tc::smem_addr(const_cast<int*>(&need[par * kWarpsAll])) +
+                              4 * (rank * kEpiWarps + ew);
+          for (int r = 0; r < 2; ++r) {
+            tc::st_cluster(tc::mapa(at, r), (uint32_t)f);
+            tc::mbar_arrive_cluster(tc::mapa(decided, r));
+          }
+        } else {
+          need[par * kWarpsAll + ew] = f;
+          tc::mbar_arrive(decided);
+        }
       }
       // ---- levels
       int top = 6;
@@ -713,7 +776,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             sum[ci][4 * j + 3]);
           }
         if (lev == 6) {
-          ok = wait_all(decided, par);
+          ok = __all_sync(0xffffffffu, wait_decided(par)) != 0;
           if (ok) {
             f = decision(par);
             top = last_level(f);
@@ -721,7 +784,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       if (!ok) break;
-      if (ew == 0 && lane == 0) {
+      if (issuer && ew == 0 && lane == 0) {
         p.bad[t] = (f & kLeave) ? 1 : 0;
         if (f & kLeave) atomicExch(&p.hdr[1], 1);
       }
@@ -769,19 +832,29 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   tc::fence_before_sync();
-  __syncthreads();
+  // a pair: neither CTA frees TMEM or exits while the other may still signal its
+  // barriers or the issuer's MMAs read its shared memory
+  if constexpr (kPair)
+    tc::cluster_sync();
+  else
+    __syncthreads();
   if (threadIdx.x == 0 && *abort) atomicExch(&p.hdr[0], 1);
   if (warp == 1) {
     tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, 512);
+    if constexpr (kPair)
+      tc::tmem_dealloc_pair(tmem, 512);
+    else
+      tc::tmem_dealloc(tmem, 512);
   }
+  if constexpr (kPair) tc::cluster_sync();
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-TileGrid tile_grid(int64_t m, int64_t n, int64_t R, int64_t Cc, int bpt) {
-  return TileGrid{(int)cdiv(m, BM), (int)cdiv(n, 64 * bpt), (int)cdiv(R, BM),
-                  (int)cdiv(Cc, 64 * bpt), 16};
+TileGrid tile_grid(int64_t m, int64_t n, int64_t R, int64_t Cc, int bpt, bool pair) {
+  const int bm = pair ? 2 * BM : BM;
+  return TileGrid{(int)cdiv(m, bm), (int)cdiv(n, 64 * bpt), (int)cdiv(R, bm),
+                  (int)cdiv(Cc, 64 * bpt), 2048 / bm};
 }
 
 }  // namespace
@@ -790,28 +863,40 @@ bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, si
   // Below 128^3 both paths are bound by their launches and latencies.
   if (d.k < 1 || (double)d.m * (double)d.n * (double)d.k < 2097152.0) return false;
   F64TcRegions& r = *rg;
-  r.row_cs = cdiv(d.m, BM) * BM;
-  r.rows_a = r.row_cs + cdiv(R, BM) * BM;
+  r.row_cs = cdiv(d.m, 2 * BM) * 2 * BM;
+  r.rows_a = r.row_cs + cdiv(R, 2 * BM) * 2 * BM;
   r.col_cs = cdiv(d.n, 256) * 256;
   r.cols_b = r.col_cs + cdiv(Cc, 256) * 256;
   // Panels of K: a level sum stays within 32 bits, the planes within a budget.
   const int64_t per_k = (r.rows_a + r.cols_b) * kPlanes64 * 2;
   const int64_t fit = (int64_t)(kPlaneBudget / per_k) / BK * BK;
   r.kp = std::min<int64_t>({cdiv(d.k, BK) * BK, kMaxPanel, std::max<int64_t>(fit, BK)});
-  // Tile width: clocks per k-step (MMA 512 / 256 for four / two boxes; one box is
-  // bound by the 24 KiB that its operands read from shared memory) times waves.
-  const int clocks[3] = {192, 256, 512};
+  // Tile kind: clocks per k-step times waves.  The copies bind the one-CTA tiles
+  // (L2 delivers about 75 bytes per clock and SM; a k-step of four, two, one boxes
+  // is 48, 32, 24 KiB: 640, 420, 360 clocks at 4096^3, where the MMAs take 512,
+  // 256, 192); a pair's CTAs copy 32 KiB per 512-clock k-step (590).  Whole steps
+  // with pairs / four / two / one boxes: 512^3 292 / 300 / 248 / 234 us, 1000 x 1501
+  // x 777 374 / 381 / 301 / 376, 2048 chain 1.68 / 1.42 / 1.56 / 2.04 ms, 4096^3
+  // 4.09 / 4.21 / 4.45 / 6.52, 8192^3 encode + product 26.1 / 27.5 / 36.2 / 46.0:
+  // the rule takes the best of each.
+  struct Kind {
+    int bpt;
+    bool pair;
+    int clocks;
+  };
+  const Kind kinds[] = {{4, true, 590}, {4, false, 640}, {2, false, 420}, {1, false, 360}};
   double best = 0;
-  for (int i = 2; i >= 0; --i) {
-    const int64_t t = tile_grid(d.m, d.n, R, Cc, 1 << i).total();
-    const double cost = (double)clocks[i] * cdiv(t, kSms);
-    if (i == 2 || cost < best) {
+  for (const Kind& kd : kinds) {
+    const int64_t t = tile_grid(d.m, d.n, R, Cc, kd.bpt, kd.pair).total();
+    const double cost = (double)kd.clocks * cdiv(t, kd.pair ? kSms / 2 : kSms);
+    if (best == 0 || cost < best) {
       best = cost;
-      r.bpt = 1 << i;
+      r.bpt = kd.bpt;
+      r.pair = kd.pair;
     }
   }
-  const int64_t tiles = tile_grid(d.m, d.n, R, Cc, r.bpt).total();
-  const int64_t ctas = std::min<int64_t>(tiles, kSms);
+  const int64_t tiles = tile_grid(d.m, d.n, R, Cc, r.bpt, r.pair).total();
+  const int64_t ctas = std::min<int64_t>(r.pair ? 2 * tiles : tiles, kSms);
   size_t off = 0;
   auto region = [&](size_t b) {
     const size_t o = off;
@@ -832,10 +917,13 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
   const F64TcRegions& r = P.f64tc;
   char* w = static_cast<char*>(ws) + P.f64tc_base;
   int* hdr = reinterpret_cast<int*>(static_cast<char*>(ws) + P.f64tc_hdr);
-  const TileGrid T = tile_grid(g.m, g.n, g.R, g.Cc, r.bpt);
+  const TileGrid T = tile_grid(g.m, g.n, g.R, g.Cc, r.bpt, r.pair);
   const char* stall = getenv("ABFT_TEST_STALL_PRODUCER");
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_f64_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem_bytes(r.bpt));
+  const auto kernel = r.pair ? k_gemm_f64_tc<true> : k_gemm_f64_tc<false>;
+  const int boxes = cta_boxes(r.bpt, r.pair);
+  const size_t smem = smem_bytes(boxes);
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   for (int64_t k0 = 0; k0 < g.k && e == cudaSuccess; k0 += r.kp) {
     F64Args gp = g;
     gp.k = std::min(r.kp, g.k - k0);
@@ -872,9 +960,9 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     Maps M;
     e = make_bf16_map(&M.a, a.pa, kPlanes64 * r.rows_a, kpad, kpad, BK, BM);
     if (e == cudaSuccess)
-      e = make_bf16_map_boxes(&M.bw, a.pb, kPlanes64 * kpad, r.cols_b, r.cols_b, r.bpt);
+      e = make_bf16_map_boxes(&M.bw, a.pb, kPlanes64 * kpad, r.cols_b, r.cols_b, boxes);
     if (e == cudaSuccess)
-      e = make_bf16_map_boxes(&M.b1, a.pb, kPlanes64 * kpad, r.cols_b, r.cols_b, 1);
+      e = make_bf16_map(&M.b1, a.pb, kPlanes64 * kpad, r.cols_b, r.cols_b, BK, BK);
     if (e != cudaSuccess) break;
     ProdArgs p{};
     p.g = gp;
@@ -892,10 +980,23 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     p.line7 = (float)(0.0016 * sqrt((double)gp.k));
     p.stall_test = stall && stall[0] == '1';
     p.wait_ns = p.stall_test ? 200000000ull : tc::kWaitLimitNs;
-    const unsigned ctas = (unsigned)std::min<int64_t>({T.total(), kSms, num_sms()});
-    k_gemm_f64_tc<<<ctas, kThreads, smem_bytes(r.bpt), st>>>(M, p);
-    if ((e = cudaGetLastError()) != cudaSuccess) break;
-    e = launch_gemm_f64_bad(gp, T, r.bpt, hdr + 1, p.bad, st);
+    const int workers = r.pair ? pair_clusters(reinterpret_cast<const void*>(kernel), smem)
+                               : num_sms();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    const unsigned per = r.pair ? 2 : 1;  // CTAs per worker
+    cfg.gridDim =
+        dim3(per * (unsigned)std::min<int64_t>({T.total(), kSms / per, workers}), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = r.pair ? 1 : 0;
+    if ((e = cudaLaunchKernelEx(&cfg, kernel, M, p)) != cudaSuccess) break;
+    e = launch_gemm_f64_bad(gp, T, r.pair ? 4 : 2, r.bpt, hdr + 1, p.bad, st);
     count_launches(2);
   }
   return e;

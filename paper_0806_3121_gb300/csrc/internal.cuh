@@ -82,6 +82,7 @@ struct F64TcRegions {
   int64_t rows_a, cols_b;     // padded rows of [A; acs], columns of [B, bcs]
   int64_t row_cs, col_cs;     // first padded checksum row / column
   int bpt;                    // 64-column boxes per tile
+  bool pair;                  // 256-row tiles on CTA pairs
 };
 
 // Everything the device code needs to know about one problem.
@@ -132,6 +133,9 @@ __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 
 
 // Multiprocessors of the current device.
 int num_sms();
+// CTA pairs (clusters of two) of a kernel with `smem` dynamic shared memory that
+// run at once on the current device.
+int pair_clusters(const void* kernel, size_t smem);
 
 // Whether the binary64 product of d runs sliced on the tensor cores, and its
 // workspace regions.
