@@ -236,7 +236,7 @@ size_t part_elems(const Plan& P) {
 void count_launches(int64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 size_t scratch_bytes(const Plan& P) {
-  size_t b = 256;  // counters
+  size_t b = kReportAfterCounters;
   b += align256(sizeof(FlagEntry) * kCapFlags) * 2;
   b += align256(sizeof(CandEntry) * kCapCands);
   b += align256(sizeof(abft_fault) * kCapReport);
@@ -249,18 +249,40 @@ Scratch scratch_view(const Plan& P, void* ws) {
   Scratch S;
   size_t o = 0;
   S.cnt = reinterpret_cast<int32_t*>(base + o);
-  o += 256;
+  o += kReportAfterCounters;
+  S.report = reinterpret_cast<abft_fault*>(base + o);
+  o += align256(sizeof(abft_fault) * kCapReport);
   S.colf = reinterpret_cast<FlagEntry*>(base + o);
   o += align256(sizeof(FlagEntry) * kCapFlags);
   S.rowf = reinterpret_cast<FlagEntry*>(base + o);
   o += align256(sizeof(FlagEntry) * kCapFlags);
   S.cand = reinterpret_cast<CandEntry*>(base + o);
   o += align256(sizeof(CandEntry) * kCapCands);
-  S.report = reinterpret_cast<abft_fault*>(base + o);
-  o += align256(sizeof(abft_fault) * kCapReport);
   S.part = reinterpret_cast<double*>(base + o);
   S.part_elems = part_elems(P);
   return S;
+}
+
+cudaError_t fetch_report(const int32_t* dev, int32_t (&cnt)[kNumCounters],
+                         std::vector<abft_fault>& rep, cudaStream_t st) {
+  constexpr int kFirst = 16;  // entries copied with the counters
+  alignas(abft_fault) char buf[kReportAfterCounters + kFirst * sizeof(abft_fault)];
+  cudaError_t e = cudaMemcpyAsync(buf, dev, sizeof buf, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return e;
+  memcpy(cnt, buf, sizeof cnt);
+  const int stored = std::max(0, std::min(cnt[kCntReport], kCapReport));
+  rep.resize((size_t)stored);
+  const int first = std::min(stored, kFirst);
+  if (first > 0) memcpy(rep.data(), buf + kReportAfterCounters, sizeof(abft_fault) * first);
+  if (stored > first) {
+    e = cudaMemcpyAsync(rep.data() + first,
+                        reinterpret_cast<const char*>(dev) + kReportAfterCounters +
+                            sizeof(abft_fault) * first,
+                        sizeof(abft_fault) * (stored - first), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  }
+  return e;
 }
 
 }  // namespace abft
@@ -478,8 +500,8 @@ abft_status abft_verify_correct(const abft_desc* desc, void* C, void* ws, int32_
   e = launch_verify(P, C, ws, er, reread_C != 0 || !P.fused, s);
   if (e != cudaSuccess) return cuda_fail(e, "abft_verify_correct launch");
   int32_t cnt[kNumCounters];
-  e = cudaMemcpyAsync(cnt, S.cnt, sizeof cnt, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  std::vector<abft_fault> rep;
+  e = fetch_report(S.cnt, cnt, rep, s);
   if (e != cudaSuccess) return cuda_fail(e, "abft_verify_correct");
   // status words of this workspace's last product and last encode
   if (has_status(P) && cnt[kCntTimeout])
@@ -490,15 +512,7 @@ abft_status abft_verify_correct(const abft_desc* desc, void* C, void* ws, int32_
     return fail(ABFT_ERR_INVALID,
                 "an e4m3 value times its block scale is not exact in bf16: the block scales "
                 "must be powers of two (and the operands finite)");
-  const int total = cnt[kCntReport];
-  const int stored = std::min(total, kCapReport);
-  std::vector<abft_fault> rep((size_t)stored);
-  if (stored > 0) {
-    e = cudaMemcpyAsync(rep.data(), S.report, sizeof(abft_fault) * stored, cudaMemcpyDeviceToHost,
-                        s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "abft_verify_correct report");
-  }
+  const int total = cnt[kCntReport], stored = (int)rep.size();
   std::sort(rep.begin(), rep.end(), [](const abft_fault& x, const abft_fault& y) {
     if (x.row != y.row) return x.row < y.row;
     if (x.col != y.col) return x.col < y.col;

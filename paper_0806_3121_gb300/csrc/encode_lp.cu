@@ -964,17 +964,33 @@ __global__ void __launch_bounds__(kThreads) k_lp_col_sq(const __nv_bfloat16* __r
 }
 
 // The line norms and the threshold norms of their verify blocks in one pass:
-// CTA I (256 threads) takes the lines of verify block I, each line's norm
+// a CTA (256 threads) takes the lines of one verify block, each line's norm
 // sqrt(sum_c part[t so + c sc]) from its fp32 partials (summed in fp32: the
 // norms scale the thresholds, a few u32 of relative error is immaterial), then
 // the block's norms: sqrt of the sums of squares of its line norms, unweighted
 // and weighted (the weights of the block's lines), and of its checksum partials.
-__global__ void __launch_bounds__(kThreads) k_lp_norms_blk(
-    const float* __restrict__ part, int64_t nout, int64_t nch, int64_t so, int64_t sc,
-    double* __restrict__ nvec, int vb, int e, const double* __restrict__ cpart, int64_t cnch,
-    double* __restrict__ nblk) {
+// CTAs 0 .. nvr-1 take the row blocks of A, the others the column blocks of B.
+struct NormSide {
+  const float* part;
+  int64_t nout, nch, so, sc;
+  double* nvec;
+  int vb, e;
+  const double* cpart;
+  int64_t cnch;
+  double* nblk;
+};
+__global__ void __launch_bounds__(kThreads) k_lp_norms_blk(const NormSide sa, const NormSide sb,
+                                                           int64_t nvr) {
   __shared__ float sh[kThreads / 32];
-  const int64_t I = blockIdx.x;
+  const bool rows = blockIdx.x < nvr;
+  const NormSide& q = rows ? sa : sb;
+  const int64_t I = rows ? blockIdx.x : blockIdx.x - nvr;
+  const float* const part = q.part;
+  const int64_t nout = q.nout, nch = q.nch, so = q.so, sc = q.sc, cnch = q.cnch;
+  double* const nvec = q.nvec;
+  double* const nblk = q.nblk;
+  const double* const cpart = q.cpart;
+  const int vb = q.vb, e = q.e;
   const int64_t t0 = I * vb, t1 = min(t0 + (int64_t)vb, nout);
   const float scw = scalbnf(1.0f, -e);
   float f0 = 0.f, f1 = 0.f;
@@ -1267,24 +1283,26 @@ __global__ void __launch_bounds__(kThreads) k_x3B_rows_any(const float* __restri
   }
 }
 
-// E[r][j] = sum_{p < npc} E16[npc r + p][j]: the products of the npc pieces of
-// each checksum row (bf16: hi and lo rows, npc = 2; split bf16x3: npc = 1),
-// added in binary64.
-__global__ void k_fold_E(const float* __restrict__ E16, int64_t R, int npc, int64_t n,
-                         double* __restrict__ E) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  for (int64_t r = blockIdx.y; r < R; r += gridDim.y) {
-    double v = 0.0;
-    for (int p = 0; p < npc; ++p) v += (double)E16[(npc * r + p) * n + j];
-    E[r * n + j] = v;
+// The product's checksum pieces folded in binary64, one launch: CTAs 0 ..
+// ncx * ncy - 1: E[r][j] = sum_{p < npc} E16[npc r + p][j] (ncx CTAs of 256 columns
+// per row), then F[i][c] = sum_{p < npc} F16[i][npc c + p].
+__global__ void __launch_bounds__(256) k_fold(const float* __restrict__ E16, int64_t R, int npc,
+                                              int64_t n, double* __restrict__ E, int64_t ncx,
+                                              int64_t ncy, const float* __restrict__ F16,
+                                              int64_t m, int64_t Cc, int64_t C16,
+                                              double* __restrict__ F) {
+  const int64_t b = blockIdx.x;
+  if (b < ncx * ncy) {
+    const int64_t j = b % ncx * 256 + threadIdx.x;
+    if (j >= n) return;
+    for (int64_t r = b / ncx; r < R; r += ncy) {
+      double v = 0.0;
+      for (int p = 0; p < npc; ++p) v += (double)E16[(npc * r + p) * n + j];
+      E[r * n + j] = v;
+    }
+    return;
   }
-}
-
-// F[i][c] = sum_{p < npc} F16[i][npc c + p]   (binary64)
-__global__ void k_fold_F(const float* __restrict__ F16, int64_t m, int64_t Cc, int64_t C16,
-                         int npc, double* __restrict__ F) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t = (b - ncx * ncy) * 256 + threadIdx.x;
   if (t >= m * Cc) return;
   const int64_t i = t / Cc, c = t % Cc;
   double v = 0.0;
@@ -1596,6 +1614,12 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
   float* rowpart = reinterpret_cast<float*>(partB + 2 * P.nvc * nchB);
   float* colpart = rowpart + d.m * nchr;
   const bool fastB = d.vb_cols >= 8 && d.vb_cols <= 256 && (d.vb_cols & (d.vb_cols - 1)) == 0;
+  // the norms of both sides (ncA: checksum-norm partials per row of acs)
+  auto norms = [&](int64_t ncA) {
+    const NormSide sa{rowpart, d.m, nchr, nchr, 1, nArow, d.vb_rows, P.er, partA, ncA, nAblk};
+    const NormSide sb{colpart, d.n, nchB, 1, d.n, nBcol, d.vb_cols, P.ec, partB, nchB, nBblk};
+    k_lp_norms_blk<<<(unsigned)(P.nvr + P.nvc), kThreads, 0, st>>>(sa, sb, P.nvr);
+  };
   for (int pl = 0; pl < P.L.planes; ++pl)
     if (P.L.bcs_ld > P.L.bcs_cols)
       cudaMemset2DAsync(reinterpret_cast<char*>(bcs) + pl * P.L.bcs_plane + P.L.bcs_cols * 2,
@@ -1621,8 +1645,6 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
       k_x3A_block<<<dim3((unsigned)cdiv(d.k, kThreads), gy(P.f * P.bs)), kThreads, 0, st>>>(
           Af, d.lda, d.k, d.grid_p, P.bs, P.f, sp, P.L.acs_ld);
     }
-    k_lp_norms_blk<<<(unsigned)P.nvr, kThreads, 0, st>>>(rowpart, d.m, nchr, nchr, 1, nArow,
-                                                       d.vb_rows, P.er, partA, nchA, nAblk);
     if (fastB) {
       k_x3B_rows<<<dim3((unsigned)cdiv(P.L.op_b_ld, kColsPerCta), (unsigned)nchB), kThreads, 0,
                    st>>>(
@@ -1634,9 +1656,8 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
       k_x3B_rows_any<<<dim3((unsigned)cdiv(nchB, kThreads / 32), gy(P.nvc)), kThreads, 0, st>>>(
           Bf, d.ldb, d.k, d.n, d.vb_cols, P.ec, bcsp, P.L.bcs_ld, partB, nchB);
     }
-    k_lp_norms_blk<<<(unsigned)P.nvc, kThreads, 0, st>>>(colpart, d.n, nchB, 1, d.n, nBcol,
-                                                       d.vb_cols, P.ec, partB, nchB, nBblk);
-    count_launches(4 + (P.bs > 0 ? 1 : 0) + (fastB ? 0 : 1));
+    norms(nchA);
+    count_launches(3 + (P.bs > 0 ? 1 : 0) + (fastB ? 0 : 1));
     return cudaGetLastError();
   }
   // FP8: the exact dequantised values go to bf16 operand planes, which the
@@ -1717,8 +1738,6 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
   if (P.bs > 0)
     k_lpA_block<<<dim3((unsigned)cdiv(d.k, kThreads), gy(P.f * P.bs)), kThreads, 0, st>>>(
         A, lda, d.k, d.grid_p, P.bs, P.f, acs + 4 * P.nvr * P.L.acs_ld, P.L.acs_ld);
-  k_lp_norms_blk<<<(unsigned)P.nvr, kThreads, 0, st>>>(rowpart, d.m, nchr, nchr, 1, nArow,
-                                                     d.vb_rows, P.er, partA, nchr, nAblk);
   if (f8B || (fastB && rows_aligned(B, ldb))) {
     SingleBUnits U{};
     U.base = EncBUnit{B, ldb, d.k, d.n, d.vb_cols, P.ec, bcs, P.L.bcs_ld, colpart, partB, nchB,
@@ -1737,9 +1756,8 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
     k_lp_col_sq<<<dim3((unsigned)cdiv(d.n, kThreads), gy(nchB)), kThreads, 0, st>>>(
         B, ldb, d.k, d.n, colpart);
   }
-  k_lp_norms_blk<<<(unsigned)P.nvc, kThreads, 0, st>>>(colpart, d.n, nchB, 1, d.n, nBcol,
-                                                     d.vb_cols, P.ec, partB, nchB, nBblk);
-  count_launches(nlaunch + 2 + (P.bs > 0 ? 1 : 0) + (fastB ? 0 : 2));
+  norms(nchr);
+  count_launches(nlaunch + 1 + (P.bs > 0 ? 1 : 0) + (fastB ? 0 : 2));
   return cudaGetLastError();
 }
 
@@ -1764,6 +1782,12 @@ cudaError_t launch_encode_lp_chained(const Plan& P, const void* Av, const void* 
   float* rowpart = reinterpret_cast<float*>(partB + 2 * P.nvc * nchB);
   float* colpart = rowpart + d.m * nchr;
   const bool fastB = d.vb_cols >= 8 && d.vb_cols <= 256 && (d.vb_cols & (d.vb_cols - 1)) == 0;
+  // the norms of both sides (ncA: checksum-norm partials per row of acs)
+  auto norms = [&](int64_t ncA) {
+    const NormSide sa{rowpart, d.m, nchr, nchr, 1, nArow, d.vb_rows, P.er, partA, ncA, nAblk};
+    const NormSide sb{colpart, d.n, nchB, 1, d.n, nBcol, d.vb_cols, P.ec, partB, nchB, nBblk};
+    k_lp_norms_blk<<<(unsigned)(P.nvr + P.nvc), kThreads, 0, st>>>(sa, sb, P.nvr);
+  };
   const float* Af = static_cast<const float*>(Av);
   const float* Bf = static_cast<const float*>(Bv);
   const int np = P.L.planes;
@@ -1800,9 +1824,6 @@ cudaError_t launch_encode_lp_chained(const Plan& P, const void* Av, const void* 
         Af, d.lda, d.k, d.grid_p, P.bs, P.f, sp, P.L.acs_ld);
     ++launches;
   }
-  k_lp_norms_blk<<<(unsigned)P.nvr, kThreads, 0, st>>>(rowpart, d.m, nchr, nchr, 1, nArow,
-                                                     d.vb_rows, P.er, partA, nchA, nAblk);
-  ++launches;
   // B: operand planes and column norms from B; checksum columns carried (F of
   // the earlier product) or formed
   if (PR) {
@@ -1825,8 +1846,7 @@ cudaError_t launch_encode_lp_chained(const Plan& P, const void* Av, const void* 
         Bf, d.ldb, d.k, d.n, d.vb_cols, P.ec, bcsp, P.L.bcs_ld, partB, nchB);
     launches += 2;
   }
-  k_lp_norms_blk<<<(unsigned)P.nvc, kThreads, 0, st>>>(colpart, d.n, nchB, 1, d.n, nBcol,
-                                                     d.vb_cols, P.ec, partB, nchB, nBblk);
+  norms(nchA);
   ++launches;
   count_launches(launches);
   return cudaGetLastError();
@@ -1905,9 +1925,10 @@ cudaError_t launch_gemm_lp(const Plan& P, const void* A, const void* B, float* C
   const float* F16 = reinterpret_cast<const float*>(w + P.L.F16);
   double* E = reinterpret_cast<double*>(w + P.L.E);
   double* F = reinterpret_cast<double*>(w + P.L.F);
-  k_fold_E<<<dim3((unsigned)cdiv(d.n, 256), gy(P.R)), 256, 0, st>>>(E16, P.R, npc, d.n, E);
-  k_fold_F<<<(unsigned)cdiv(d.m * P.Cc, 256), 256, 0, st>>>(F16, d.m, P.Cc, P.L.bcs_cols, npc, F);
-  count_launches(2);
+  const int64_t ncx = cdiv(d.n, 256), ncy = gy(P.R);
+  k_fold<<<(unsigned)(ncx * ncy + cdiv(d.m * P.Cc, 256)), 256, 0, st>>>(
+      E16, P.R, npc, d.n, E, ncx, ncy, F16, d.m, P.Cc, P.L.bcs_cols, F);
+  count_launches(1);
   return cudaGetLastError();
 }
 

@@ -333,11 +333,12 @@ abft_status abft_group_create(const abft_problem* problems, int32_t count, int32
     off = al256(off + bytes);
     return o;
   };
+  static_assert(kReportAfterCounters == 256, "the report follows the counters");
   G->off_cnt = region(256);
+  G->off_report = region(sizeof(abft_fault) * kCapReport);
   G->off_colf = region(sizeof(FlagEntry) * kCapFlags);
   G->off_rowf = region(sizeof(FlagEntry) * kCapFlags);
   G->off_cand = region(sizeof(CandEntry) * kCapCands);
-  G->off_report = region(sizeof(abft_fault) * kCapReport);
   G->off_inject = region(16 + sizeof(InjectEntry) * kMaxInject);
   G->off_probs = region(sizeof(GProb) * count);
   G->off_maps = region(sizeof(GMaps) * count);
@@ -482,22 +483,14 @@ abft_status abft_group_report(abft_group g, abft_fault* report, int32_t max_repo
     return fail(ABFT_ERR_INVALID, "bad report buffer");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   int32_t cnt[kNumCounters];
-  cudaError_t e = cudaMemcpyAsync(cnt, g->dev.cnt, sizeof cnt, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  std::vector<abft_fault> rep;
+  const cudaError_t e = fetch_report(g->dev.cnt, cnt, rep, st);
   if (e != cudaSuccess) return cuda_fail(e, "abft_group_report");
   if (cnt[kCntTimeout])  // the group's status word of its last product
     return fail(ABFT_ERR_TIMEOUT,
                 "the group's product gave up waiting (bounded wait); results are incomplete and "
                 "were not corrected");
-  const int total = cnt[kCntReport];
-  const int stored = std::min(total, kCapReport);
-  std::vector<abft_fault> rep((size_t)stored);
-  if (stored > 0) {
-    e = cudaMemcpyAsync(rep.data(), g->dev.report, sizeof(abft_fault) * stored,
-                        cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(e, "abft_group_report");
-  }
+  const int total = cnt[kCntReport], stored = (int)rep.size();
   std::sort(rep.begin(), rep.end(), [](const abft_fault& x, const abft_fault& y) {
     if (x.problem != y.problem) return x.problem < y.problem;
     if (x.row != y.row) return x.row < y.row;

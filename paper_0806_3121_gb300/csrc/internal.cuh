@@ -7,6 +7,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/abft.h"
 
 namespace abft {
@@ -125,6 +127,13 @@ struct Scratch {
   double* part;  // partial reductions of encode
   size_t part_elems;
 };
+
+// The report entries follow the counters, so one copy brings both.
+constexpr size_t kReportAfterCounters = 256;
+// Counters and report entries (at `dev`) to the host: one copy, and a second one
+// when there are more than 16 entries.  Synchronises the stream.
+cudaError_t fetch_report(const int32_t* dev, int32_t (&cnt)[kNumCounters],
+                         std::vector<abft_fault>& rep, cudaStream_t st);
 
 Scratch scratch_view(const Plan& P, void* ws);
 size_t scratch_bytes(const Plan& P);

@@ -3,20 +3,24 @@
 // errors; a lost part is the checksum minus the surviving parts).
 //
 // Pipeline of one verify call, all on the device:
-//   k_col_check   column lines (verify block I, column j): sums e^T C_I[:,j],
+//   k_check       column lines (verify block I, column j): sums e^T C_I[:,j],
 //                 w^T C_I[:,j], non-finite elements, residuals against E,
-//                 threshold test, append if flagged.
-//   k_row_check   row lines (row i, verify block J), against F.
+//                 threshold test, append if flagged; row lines (row i, verify
+//                 block J) against F.  k_fused: the same from the sums that the
+//                 product's epilogue observed.
 //   k_locate_correct  one CTA: candidates from the flagged lines (single
 //                 non-finite element, or the weighted/unweighted residual
 //                 ratio), bitonic sort + merge, choice of a correcting line,
 //                 recomputation in binary64, re-check of the touched lines,
 //                 report entries.
 // Recovery: k_recover rebuilds an erased block from S = sum_I C_I, then
-// k_col_check (count mode) re-checks the rebuilt block.
+// k_check (count mode) re-checks the rebuilt block.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace abft {
 namespace {
@@ -180,37 +184,45 @@ __device__ int row_line_warp(const CheckArgs& a, int64_t i, int64_t J, double& r
   return nf;
 }
 
-// Column lines [I_begin, I_end) x [j_begin, j_end).  mode 0: append flagged
-// lines to colf (skipping erased blocks); mode 1: only count them in
-// cnt[kCntRecoverFlagged].  A unit is 32 columns x one verify block; wpu warps of
-// a CTA share its rows in contiguous parts (64 rows or more each) and meet in
-// shared memory, with eight rows of loads in flight per thread: one thread per
-// column walking all the rows of its block, as an earlier version did, left a
-// 512^2 binary64 result to two CTAs (192 us; the FP64 pipe, 2 results per clock
-// and SM, bounds large ones).  Weights come from a table: forming (t + 1) 2^-e per
-// element cost two more binary64 instructions.
+// The column lines of one launch: [I_begin, I_end) x [j_begin, j_end).  mode 0:
+// append flagged lines to colf (skipping erased blocks); mode 1: only count them in
+// cnt[kCntRecoverFlagged].  wpu warps share a unit (32 columns x one verify
+// block); blocks: the CTAs of the column lines (row lines take the CTAs after).
+struct ColLines {
+  int64_t j_begin, j_end, I_begin, I_end;
+  int mode, wpu;
+  int64_t blocks;
+};
 constexpr int kSegRows = 64;
-template <typename TC>
-__global__ void __launch_bounds__(kThreads) k_col_check(const CheckArgs a, int64_t j_begin,
-                                                        int64_t j_end, int64_t I_begin,
-                                                        int64_t I_end, int mode, int wpu) {
+
+// The warps of a unit take contiguous parts of the verify block's rows (64 rows or
+// more each) and meet in shared memory, with eight rows of loads in flight per
+// thread: one thread per column walking all the rows of its block left a 512^2
+// binary64 result to two CTAs (192 us).  Binary64 sums are bound by the FP64 pipe
+// (2 results per clock and SM), so on small results the warps of a unit are spread
+// over the CTAs of a cluster (kCluster: two warps per CTA), each on an SM of its
+// own.  Weights come from a table: forming (t + 1) 2^-e per element cost two more
+// binary64 instructions.
+template <typename TC, bool kCluster>
+__device__ __forceinline__ void col_lines(const CheckArgs& a, const ColLines& c) {
   __shared__ TC sh[kThreads / 32][2][32];
   __shared__ int snf[kThreads / 32][32];
   __shared__ TC wtab[kSegRows];
-  if (mode == 1 && a.status_out && blockIdx.x == 0 && threadIdx.x == 0)
+  if (c.mode == 1 && a.status_out && blockIdx.x == 0 && threadIdx.x == 0)
     *a.status_out = *a.timeout;
   // weights at most 1: a weighted term never exceeds its element
   const TC sc = (TC)scalbn(1.0, -a.er);
   if (threadIdx.x < kSegRows) wtab[threadIdx.x] = (TC)(threadIdx.x + 1) * sc;
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t nck = cdiv(j_end - j_begin, 32);
-  const int64_t u = (int64_t)blockIdx.x * (kThreads / 32 / wpu) + warp / wpu;
-  const int part = warp % wpu;
-  const int64_t I = I_begin + u / nck, j = j_begin + u % nck * 32 + lane;
-  const bool ok = I < I_end && j < j_end;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int64_t nck = cdiv(c.j_end - c.j_begin, 32);
+  const int64_t gw = (int64_t)blockIdx.x * nw + warp;
+  const int64_t u = gw / c.wpu;
+  const int part = (int)(gw - u * c.wpu);
+  const int64_t I = c.I_begin + u / nck, j = c.j_begin + u % nck * 32 + lane;
+  const bool ok = I < c.I_end && j < c.j_end;
   const int64_t i0 = I * a.vb_r, i1 = min(i0 + (int64_t)a.vb_r, a.m);
-  const int64_t len = max((int64_t)kSegRows, cdiv(a.vb_r, wpu));  // rows of a part
+  const int64_t len = max((int64_t)kSegRows, cdiv(a.vb_r, c.wpu));  // rows of a part
   const int64_t b0 = i0 + part * len, b1 = min(b0 + len, i1);
   TC se = 0, sw = 0;
   int nf = 0;
@@ -241,26 +253,41 @@ __global__ void __launch_bounds__(kThreads) k_col_check(const CheckArgs a, int64
       se += e;
     }
   }
-  if (wpu > 1) {
+  if (c.wpu > 1) {
     sh[warp][0][lane] = se;
     sh[warp][1][lane] = sw;
     snf[warp][lane] = nf;
-    __syncthreads();
-    if (part != 0) return;
-    for (int w = warp + 1; w < warp + wpu; ++w) {
-      se += sh[w][0][lane];
-      sw += sh[w][1][lane];
-      nf |= snf[w][lane];
+    if constexpr (kCluster) {
+      // part p of the unit: warp p % nw of the cluster's CTA p / nw
+      cg::cluster_group cl = cg::this_cluster();
+      cl.sync();
+      if (part == 0)
+        for (int p = 1; p < c.wpu; ++p) {
+          const auto* rs = cl.map_shared_rank(&sh[0], p / nw);
+          const auto* rn = cl.map_shared_rank(&snf[0], p / nw);
+          se += rs[p % nw][0][lane];
+          sw += rs[p % nw][1][lane];
+          nf |= rn[p % nw][lane];
+        }
+      cl.sync();  // the sums have been read
+    } else {
+      __syncthreads();
+      if (part == 0)
+        for (int w = warp + 1; w < warp + c.wpu; ++w) {
+          se += sh[w][0][lane];
+          sw += sh[w][1][lane];
+          nf |= snf[w][lane];
+        }
     }
   }
-  if (!ok) return;
-  if (mode == 0 && touches_erased(a.erased, a.bs, a.bc, i0, i1, j, j + 1)) return;
+  if (!ok || part != 0) return;
+  if (c.mode == 0 && touches_erased(a.erased, a.bs, a.bc, i0, i1, j, j + 1)) return;
   const double re = (double)se - a.E[(2 * I) * a.n + j];
   const double rw = (double)sw - a.E[(2 * I + 1) * a.n + j];
   double te, tw;
   col_taus(a, I, j, te, tw);
   if (nf == 0 && !is_flagged(re, rw, te, tw)) return;
-  if (mode == 1) {
+  if (c.mode == 1) {
     atomicAdd(&a.cnt[kCntRecoverFlagged], 1);
     return;
   }
@@ -268,20 +295,20 @@ __global__ void __launch_bounds__(kThreads) k_col_check(const CheckArgs a, int64
   if (slot < kCapFlags) a.colf[slot] = FlagEntry{(int32_t)I, (int32_t)j, nf, 0, re, rw};
 }
 
-// Row lines: one warp takes kRowLinesW rows x one verify block.  The sums of the
-// eight rows meet in one transposing butterfly (17 warp-wide adds instead of 80)
-// and their residuals and thresholds are evaluated side by side in eight lanes:
-// with one line per warp those binary64 instructions, each a whole warp's, cost
-// as much as the sums (3001 x 2999 binary32: 48 us).
-constexpr int kRowLinesW = 8;
-template <typename TC>
-__global__ void __launch_bounds__(kThreads) k_row_check(const CheckArgs a) {
-  constexpr int N = 2 * kRowLinesW;
+// Row lines: one warp takes R rows x one verify block.  The sums of its rows meet
+// in one transposing butterfly (17 warp-wide adds for eight rows instead of 80)
+// and their residuals and thresholds are evaluated side by side: with one line
+// per warp those binary64 instructions, each a whole warp's, cost as much as the
+// sums (3001 x 2999 binary32: 48 us).  R = 8; two on small results, to occupy
+// every SM.
+template <typename TC, int R>
+__device__ __forceinline__ void row_lines(const CheckArgs& a, int64_t block) {
+  constexpr int N = 2 * R, kPer = 32 / N;  // lanes per value after the butterfly
   const int lane = threadIdx.x & 31;
-  const int64_t u = (int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-  const int64_t r0 = u / a.nvc * kRowLinesW, J = u % a.nvc;
+  const int64_t u = block * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int64_t r0 = u / a.nvc * R, J = u % a.nvc;
   if (r0 >= a.m) return;
-  const int nr = (int)min((int64_t)kRowLinesW, a.m - r0);
+  const int nr = (int)min((int64_t)R, a.m - r0);
   const int64_t j0 = J * a.vb_c, j1 = min(j0 + (int64_t)a.vb_c, a.n);
   const int len = (int)(j1 - j0);
   const TC* q = static_cast<const TC*>(a.C) + r0 * a.ldc + j0;
@@ -291,13 +318,13 @@ __global__ void __launch_bounds__(kThreads) k_row_check(const CheckArgs a) {
 #pragma unroll
   for (int r = 0; r < N; ++r) v[r] = 0;
   TC w = (TC)(lane + 1) * sc;
-#pragma unroll 2
+#pragma unroll(16 / R)
   for (int t = lane; t < len; t += 32) {
 #pragma unroll
-    for (int r = 0; r < kRowLinesW; ++r) {
+    for (int r = 0; r < R; ++r) {
       const TC x = r < nr ? q[r * a.ldc + t] : (TC)0;
       v[r] += x;
-      v[kRowLinesW + r] = fma_t<TC>(w, x, v[kRowLinesW + r]);
+      v[R + r] = fma_t<TC>(w, x, v[R + r]);
       nfb |= isfinite(x) ? 0u : 1u << r;
     }
     w += (TC)32 * sc;
@@ -312,10 +339,12 @@ __global__ void __launch_bounds__(kThreads) k_row_check(const CheckArgs a) {
       v[i] = (upper ? v[i + h] : v[i]) + __shfl_xor_sync(0xffffffffu, send, s);
     }
   }
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);  // lane l holds value l / 2
+#pragma unroll
+  for (int o = kPer / 2; o >= 1; o >>= 1)  // lane l holds value l / kPer
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
   const TC sw = __shfl_sync(0xffffffffu, v[0], (lane + 16) & 31);
-  const int r = lane >> 1;
-  if (lane >= 16 || (lane & 1) || r >= nr) return;
+  const int r = lane / kPer;
+  if (lane >= 16 || lane % kPer || r >= nr) return;
   const int64_t i = r0 + r;
   if (touches_erased(a.erased, a.bs, a.bc, i, i + 1, j0, j1)) return;
   const double re = (double)v[0] - a.F[i * a.Cc + 2 * J];
@@ -328,15 +357,45 @@ __global__ void __launch_bounds__(kThreads) k_row_check(const CheckArgs a) {
   if (slot < kCapFlags) a.rowf[slot] = FlagEntry{(int32_t)i, (int32_t)J, nf, 0, re, rw};
 }
 
-// Launches k_col_check over whole units (see there).
+// Both checks in one launch: the column lines' CTAs, then the row lines'.
+template <typename TC, int R, bool kCluster>
+__global__ void __launch_bounds__(kThreads) k_check(const CheckArgs a, const ColLines c) {
+  if (blockIdx.x < c.blocks)
+    col_lines<TC, kCluster>(a, c);
+  else
+    row_lines<TC, R>(a, blockIdx.x - c.blocks);
+}
+
+// Launches k_check on the column lines of `c` (wpu and blocks are set here) and,
+// with rows, on every row line.  Small results (fewer column warps than two CTAs
+// per SM would hold) take 64-thread CTAs, clusters and two rows per warp: 512^2
+// binary64 checks 59 -> 12 us; large ones gain nothing from it.
 template <typename TC>
-void run_col_check(const CheckArgs& a, int64_t j_begin, int64_t j_end, int64_t I_begin,
-                   int64_t I_end, int mode, cudaStream_t st) {
-  int wpu = 1;
-  while (wpu < kThreads / 32 && wpu * kSegRows < a.vb_r) wpu *= 2;
-  const int64_t units = (I_end - I_begin) * cdiv(j_end - j_begin, 32);
-  k_col_check<TC><<<(unsigned)cdiv(units, kThreads / 32 / wpu), kThreads, 0, st>>>(
-      a, j_begin, j_end, I_begin, I_end, mode, wpu);
+cudaError_t run_check(const CheckArgs& a, ColLines c, bool rows, cudaStream_t st) {
+  c.wpu = 1;
+  while (c.wpu < kThreads / 32 && c.wpu * kSegRows < a.vb_r) c.wpu *= 2;
+  const int64_t units = (c.I_end - c.I_begin) * cdiv(c.j_end - c.j_begin, 32);
+  const bool small = units * c.wpu < 2 * (int64_t)num_sms() * (kThreads / 32);
+  const int nw = small ? 2 : kThreads / 32;
+  const unsigned cluster = small && c.wpu > nw ? (unsigned)(c.wpu / nw) : 1;
+  auto whole = [&](int64_t b) { return (b + cluster - 1) / cluster * cluster; };
+  c.blocks = whole(cdiv(units * c.wpu, nw));
+  const int64_t rblocks =
+      rows ? whole(cdiv(cdiv(a.m, (int64_t)(small ? 2 : 8)) * a.nvc, nw)) : 0;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(c.blocks + rblocks), 1, 1);
+  cfg.blockDim = dim3(32 * nw, 1, 1);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  count_launches(1);
+  if (cluster > 1) return cudaLaunchKernelEx(&cfg, k_check<TC, 2, true>, a, c);
+  if (small) return cudaLaunchKernelEx(&cfg, k_check<TC, 2, false>, a, c);
+  return cudaLaunchKernelEx(&cfg, k_check<TC, 8, false>, a, c);
 }
 
 // Screen of the fused checks: a line whose binary32 evaluation passes with a
@@ -362,15 +421,15 @@ constexpr float kU32 = 5.9604645e-8f;  // 2^-24
 // 32-row blocks.  A non-finite observed sum marks the line non-finite (the
 // locate step then scans C for it).  The lines that pass the binary32 screen
 // are done; the others are decided by the binary64 rule.
-__global__ void __launch_bounds__(kThreads) k_col_fused(const CheckArgs a, const float* obs,
-                                                        int64_t ntr) {
+__device__ __forceinline__ void col_fused(const CheckArgs& a, const float* obs, int64_t ntr,
+                                          int64_t bx, int64_t by, int64_t ny) {
   __shared__ float tI[2];  // the verify block's threshold factors (binary32)
-  const int64_t j = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const int64_t j = bx * kThreads + threadIdx.x;
   const bool jv = j < a.n;
   const int64_t tpb = a.vb_r / 32;  // 32-row blocks per verify block
   const float nbj = jv ? (float)a.nBcol[j] : 0.f;
   const float slack = (float)(tpb + 2) * kU32;
-  for (int64_t I = blockIdx.y; I < a.nvr; I += gridDim.y) {
+  for (int64_t I = by; I < a.nvr; I += ny) {
     __syncthreads();  // every thread has read the previous tI
     if (threadIdx.x == 0) {
       tI[0] = (float)(a.s * (a.f1c * a.nAblk[4 * I + 0] + a.f2c * a.nAblk[4 * I + 2] + a.carA[2 * I]));
@@ -414,8 +473,8 @@ __global__ void __launch_bounds__(kThreads) k_col_fused(const CheckArgs a, const
 // verify blocks' threshold factors in binary32 in shared memory (up to
 // kRowTauSmem blocks; more: computed per line), then the same screen.
 constexpr int kRowTauSmem = 2048;
-__global__ void __launch_bounds__(kThreads) k_row_fused(const CheckArgs a, const float* obs,
-                                                        int64_t g, int64_t ngrp) {
+__device__ __forceinline__ void row_fused(const CheckArgs& a, const float* obs, int64_t g,
+                                          int64_t ngrp, int64_t block) {
   __shared__ float tJ[2 * kRowTauSmem];
   const bool smem_tau = a.nvc <= kRowTauSmem;
   if (smem_tau) {
@@ -427,7 +486,7 @@ __global__ void __launch_bounds__(kThreads) k_row_fused(const CheckArgs a, const
     }
     __syncthreads();
   }
-  const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  const int64_t t = block * kThreads + threadIdx.x;
   if (t >= a.m * a.nvc) return;
   const int64_t i = t / a.nvc, J = t % a.nvc;
   const int64_t j0 = J * a.vb_c, j1 = min(j0 + (int64_t)a.vb_c, a.n);
@@ -460,6 +519,19 @@ __global__ void __launch_bounds__(kThreads) k_row_fused(const CheckArgs a, const
   if (nf == 0 && !is_flagged(re, rw, te, tw)) return;
   const int slot = atomicAdd(&a.cnt[kCntRowFlags], 1);
   if (slot < kCapFlags) a.rowf[slot] = FlagEntry{(int32_t)i, (int32_t)J, nf, 0, re, rw};
+}
+
+// Both fused checks in one launch: the column lines' CTAs (ncx per verify block
+// row, ncy of those), then the row lines'.
+__global__ void __launch_bounds__(kThreads) k_fused(const CheckArgs a, const float* obs_col,
+                                                    int64_t ntr, int64_t ncx, int64_t ncy,
+                                                    const float* obs_row, int64_t g,
+                                                    int64_t ngrp) {
+  const int64_t b = blockIdx.x;
+  if (b < ncx * ncy)
+    col_fused(a, obs_col, ntr, b % ncx, b / ncx, ncy);
+  else
+    row_fused(a, obs_row, g, ngrp, b - ncx * ncy);
 }
 
 // Position (0-based) of a single error inside a line of len elements from
@@ -727,25 +799,30 @@ __device__ __forceinline__ void locate_body(const Pol& A, int32_t* cnt, const Fl
   }
   __syncthreads();
 
-  // 7. re-check both lines of every corrected element (each line once)
-  for (int t = warp; t < nc; t += nwarps) {
+  // 7. re-check both lines of every corrected element (each line once), a warp
+  //    per line
+  for (int t2 = warp; t2 < 2 * nc; t2 += nwarps) {
+    const int t = t2 >> 1;
+    const bool colside = (t2 & 1) == 0;
     if (how[t] < 0) continue;
     const int p = A.kp(keys[t]);
     const Geo G = A.geo(p);
     const int32_t r = A.kr(keys[t]), c = A.kc(keys[t]);
     const int64_t I = r / G.vb_r, J = c / G.vb_c;
-    bool dup_c = false, dup_r = false;
-    for (int u = 0; u < t; ++u) {
+    bool dup = false;
+    for (int u = 0; u < t && !dup; ++u) {
       if (how[u] < 0 || A.kp(keys[u]) != p) continue;
       const int32_t r2 = A.kr(keys[u]), c2 = A.kc(keys[u]);
-      if (c2 == c && r2 / G.vb_r == I) dup_c = true;
-      if (r2 == r && c2 / G.vb_c == J) dup_r = true;
+      dup = colside ? c2 == c && r2 / G.vb_r == I : r2 == r && c2 / G.vb_c == J;
     }
+    if (dup) continue;
     double re, rw;
-    if (!dup_c && A.recheck_col(p, I, c, re, rw) && lane == 0)  // warp-wide
-      push_report(report, cnt, p, -1, c, ABFT_KIND_UNCORRECTABLE, 0, 0.0, re, rw);
-    if (!dup_r && A.recheck_row(p, r, J, re, rw))
+    if (colside) {
+      if (A.recheck_col(p, I, c, re, rw) && lane == 0)  // warp-wide
+        push_report(report, cnt, p, -1, c, ABFT_KIND_UNCORRECTABLE, 0, 0.0, re, rw);
+    } else if (A.recheck_row(p, r, J, re, rw)) {
       push_report(report, cnt, p, r, -1, ABFT_KIND_UNCORRECTABLE, 1, 0.0, re, rw);
+    }
   }
 }
 
@@ -1192,18 +1269,18 @@ cudaError_t verify_t(const Plan& P, void* C, void* ws, const Erased& er, bool re
   a.erased = er;
   const int64_t m = P.d.m, n = P.d.n;
   if (reread) {
-    run_col_check<TC>(a, 0, n, 0, P.nvr, 0, st);
-    k_row_check<TC><<<(unsigned)cdiv(cdiv(m, kRowLinesW) * P.nvc, kThreads / 32), kThreads, 0,
-                      st>>>(a);
+    const cudaError_t e = run_check<TC>(a, ColLines{0, n, 0, P.nvr, 0, 0, 0}, true, st);
+    if (e != cudaSuccess) return e;
   } else {
     const char* w = static_cast<const char*>(ws);
-    k_col_fused<<<dim3((unsigned)cdiv(n, kThreads), gy(P.nvr)), kThreads, 0, st>>>(
-        a, reinterpret_cast<const float*>(w + P.L.obs_col), P.ntr_obs);
-    k_row_fused<<<(unsigned)cdiv(m * P.nvc, kThreads), kThreads, 0, st>>>(
-        a, reinterpret_cast<const float*>(w + P.L.obs_row), P.g, P.ngrp);
+    const int64_t ncx = cdiv(n, kThreads), ncy = gy(P.nvr);
+    k_fused<<<(unsigned)(ncx * ncy + cdiv(m * P.nvc, kThreads)), kThreads, 0, st>>>(
+        a, reinterpret_cast<const float*>(w + P.L.obs_col), P.ntr_obs, ncx, ncy,
+        reinterpret_cast<const float*>(w + P.L.obs_row), P.g, P.ngrp);
+    count_launches(1);
   }
   k_locate_correct<TC><<<1, kLocThreads, 0, st>>>(a);
-  count_launches(3);
+  count_launches(1);
   return cudaGetLastError();
 }
 
@@ -1221,9 +1298,11 @@ cudaError_t recover_t(const Plan& P, void* C, void* ws, int bj, const int* rows,
   for (int u = 0; u < t; ++u) {  // re-check the rebuilt blocks' column lines
     const int64_t I0 = ((int64_t)rows[u] * P.bs) / P.d.vb_rows;
     const int64_t I1 = cdiv(((int64_t)rows[u] + 1) * P.bs, P.d.vb_rows);
-    run_col_check<TC>(a, (int64_t)bj * P.bc, ((int64_t)bj + 1) * P.bc, I0, I1, 1, st);
+    const cudaError_t e = run_check<TC>(
+        a, ColLines{(int64_t)bj * P.bc, ((int64_t)bj + 1) * P.bc, I0, I1, 1, 0, 0}, false, st);
+    if (e != cudaSuccess) return e;
   }
-  count_launches(1 + t);
+  count_launches(1);
   return cudaGetLastError();
 }
 
@@ -1247,9 +1326,9 @@ cudaError_t block_restore_t(const Plan& P, void* C, void* ws, int bi, int bj, co
       static_cast<TC*>(C), P.d.ldc, src, P.bs, P.bc, bi, bj, a.timeout);
   const int64_t I0 = ((int64_t)bi * P.bs) / P.d.vb_rows;
   const int64_t I1 = cdiv(((int64_t)bi + 1) * P.bs, P.d.vb_rows);
-  run_col_check<TC>(a, (int64_t)bj * P.bc, ((int64_t)bj + 1) * P.bc, I0, I1, 1, st);
-  count_launches(2);
-  return cudaGetLastError();
+  count_launches(1);
+  return run_check<TC>(
+      a, ColLines{(int64_t)bj * P.bc, ((int64_t)bj + 1) * P.bc, I0, I1, 1, 0, 0}, false, st);
 }
 
 }  // namespace
