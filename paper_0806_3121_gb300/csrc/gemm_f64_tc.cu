@@ -83,30 +83,22 @@ static_assert(smem_bytes(4) <= 232448 && smem_bytes(2) <= 232448 && smem_bytes(1
 
 // ------------------------------------------------------------------ digits
 
-// Four binary64 values as the four elements of each plane.
-struct Digits4 {
-  uint2 plane[kPlanes64];
-};
-
 // x 2^(63 - e) rounded to a 64-bit integer (|x| < 2^e, e = efield - 1022 with
 // efield the biased exponent of the row's largest element); the bits cut off.
-__device__ __forceinline__ int64_t scaled(double x, int efield, bool& cut) {
+__device__ __forceinline__ uint64_t scaled(double x, int efield, bool& cut) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
   const int E = (int)(b >> 52) & 0x7ff;
-  const uint64_t mant = (b & 0xfffffffffffffull) | (E ? 0x10000000000000ull : 0ull);
-  const int s = 10 - (efield - max(E, 1));  // value = mant 2^(s) in units of 2^(e - 63)
-  uint64_t v;
-  if (s >= 0) {
-    v = mant << s;
-  } else if (s > -64) {
-    const int r = -s;
-    v = (mant + (1ull << (r - 1))) >> r;
-    cut |= (mant & ((1ull << r) - 1)) != 0;
+  const uint64_t m =
+      ((b & 0xfffffffffffffull) | (E ? 0x10000000000000ull : 0ull)) << 10;  // below 2^63
+  const int r = efield - max(E, 1);
+  uint64_t v = 0;
+  if (r < 64) {
+    v = (m + ((1ull << r) >> 1)) >> r;
+    cut |= (v << r) != m;
   } else {
-    v = 0;
-    cut |= mant != 0;
+    cut |= m != 0;
   }
-  return (int64_t)(b >> 63 ? 0ull - v : v);
+  return b >> 63 ? 0ull - v : v;
 }
 
 // |x| 2^-e as bf16, rounded towards zero (nonzero values at least 2^-60).
@@ -117,23 +109,29 @@ __device__ __forceinline__ uint32_t magnitude(double x, int efield) {
   return ex < 67 ? 67u << 7 : ((uint32_t)ex << 7) | ((hi >> 13) & 0x7fu);
 }
 
-// Digits and magnitudes of four values; `bits` collects the integers' bits.
-__device__ __forceinline__ void slice4(const double (&x)[4], int efield, Digits4& D,
-                                       uint64_t& bits, bool& cut) {
+// Four consecutive elements of every plane, at o (planes `plane` elements apart),
+// from four values with scales ef (0: a line that the digits cannot hold, whose
+// digits are zero and whose magnitudes are NaN); bits / cut collect the integers'
+// bits and whether any were cut off.
+__device__ __forceinline__ void slice4(const double (&x)[4], const int (&ef)[4], uint16_t* o,
+                                       int64_t plane, uint64_t (&bits)[4], bool (&cut)[4]) {
   // (X + 2^63) + sum_j 128 256^j has the bytes d + 128 of the digits below the
   // top one, and the top digit (with the carry) in the last place
-  uint32_t w[4][2], top[4];
+  uint32_t w[4][2], top[4], mag[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const uint64_t X = (uint64_t)scaled(x[q], efield, cut);
-    bits |= X;
+    const int f = ef[q] ? ef[q] : 1022;
+    const double v = ef[q] ? x[q] : 0.0;
+    const uint64_t X = scaled(v, f, cut[q]);
+    bits[q] |= X;
     const uint64_t u0 = X ^ 0x8000000000000000ull, u = u0 + 0x0080808080808080ull;
     w[q][0] = (uint32_t)u;
     w[q][1] = (uint32_t)(u >> 32);
     top[q] = (w[q][1] >> 24) + (u < u0 ? 256u : 0u);
+    mag[q] = ef[q] ? magnitude(v, f) : 0x7fc0u;
   }
 #pragma unroll
-  for (int p = 0; p < kDigits; ++p) {
+  for (int p = 0; p < kDigits; ++p, o += plane) {
     float f[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -145,11 +143,11 @@ __device__ __forceinline__ void slice4(const double (&x)[4], int efield, Digits4
       f[q] = __uint_as_float(m) - 8388736.0f;
     }
     // bf16 holds a digit exactly: the upper halves of the binary32 words
-    D.plane[p].x = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632u);
-    D.plane[p].y = __byte_perm(__float_as_uint(f[2]), __float_as_uint(f[3]), 0x7632u);
+    *reinterpret_cast<uint2*>(o) =
+        make_uint2(__byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632u),
+                   __byte_perm(__float_as_uint(f[2]), __float_as_uint(f[3]), 0x7632u));
   }
-  D.plane[kMagPlane].x = magnitude(x[0], efield) | (magnitude(x[1], efield) << 16);
-  D.plane[kMagPlane].y = magnitude(x[2], efield) | (magnitude(x[3], efield) << 16);
+  *reinterpret_cast<uint2*>(o) = make_uint2(mag[0] | (mag[1] << 16), mag[2] | (mag[3] << 16));
 }
 
 // Four consecutive elements, zeros from element nv on.
@@ -164,26 +162,24 @@ __device__ __forceinline__ void load4(const double* p, int64_t nv, double (&x)[4
   }
 }
 
-// Largest high word and whether any element is nonzero, in one word pair.
-__device__ __forceinline__ void take_max(double x, uint32_t& hi, uint32_t& any) {
-  const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;
-  hi = max(hi, h);
-  any |= h | (uint32_t)__double2loint(x);
+// A value's key for the maximum: its high word (whose upper bits are the
+// exponent), with the last bit set when any lower bit is, so that 0 means zero.
+__device__ __forceinline__ uint32_t max_key(double x) {
+  return ((uint32_t)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
 }
 
-// The biased exponent that scales a row: 0 marks a row that the digits cannot
-// hold (NaN, infinite, exponent outside the range), 1023 - 1 a zero row.
-__device__ __forceinline__ int row_field(uint32_t hi, uint32_t any) {
-  const int E = (int)(hi >> 20);
-  if (any == 0) return 1022;
+// The biased exponent that scales a line with that maximal key: 0 marks a line
+// that the digits cannot hold (NaN, infinite, exponent outside the range).
+__device__ __forceinline__ int line_field(uint32_t key) {
+  const int E = (int)(key >> 20);
+  if (key == 0) return 1022;
   return (E - 1022 < kMinExp || E - 1022 > kMaxExp) ? 0 : E;
 }
 
-// {exponent e, index of the last digit that is used (kNotExact: some value is cut)}
-__device__ __forceinline__ int2 row_info(int efield, uint64_t bits, bool cut) {
-  if (efield == 0) return make_int2(0, kNotExact);
-  const int z = cut ? kNotExact : (bits ? kDigits - 1 - (__ffsll((long long)bits) - 1) / 8 : 0);
-  return make_int2(efield - 1022, z);
+// Index of the last digit that a line uses; kNotExact when values are cut.
+__device__ __forceinline__ int last_digit(int field, uint64_t bits, bool cut) {
+  if (field == 0 || cut) return kNotExact;
+  return bits ? kDigits - 1 - (__ffsll((long long)bits) - 1) / 8 : 0;
 }
 
 struct SliceArgs {
@@ -191,186 +187,166 @@ struct SliceArgs {
   int64_t kpad;       // panel length rounded up to 64
   uint16_t* pa;       // planes of [A; acs]: [plane][rows_a][kpad]
   uint16_t* pb;       // planes of [B, bcs]: [plane][kpad][cols_b]
-  int2* a_row;
+  int2* a_row;        // {exponent, last digit} per row / column
   int2* b_col;
+  uint32_t* cmax;     // [ceil(kpad / 256)][cols_b] maximal keys of 256 rows of B
   int* hdr;           // {status, any bad tile}
   int64_t rows_a, cols_b, row_cs, col_cs;
-  int tpr;            // threads per row of A
-  int64_t nb, nbc, na;  // CTAs: columns of B, of bcs, rows of A (the rest: acs)
+  int tpr;            // threads per row of A in the maximum pass
+  int64_t n0, n1, n2; // CTAs: A or B data, then their checksums (see the kernels)
 };
 
 constexpr int kSliceThreads = 256;
+constexpr int kMaxRows = 256;     // rows of B per partial maximum
+constexpr int kSliceCols = 256;   // columns and rows of a slicing CTA
+constexpr int kSliceRows = 16;
 
-// One row of A per tpr threads: the largest element, then (the row again, from
-// L1 / L2) its digits.
-__device__ __forceinline__ void slice_rows(const SliceArgs& a, const double* src, int64_t ld,
-                                           int64_t rows, int64_t row_out, int64_t blk,
-                                           uint32_t* sh) {
+// The maximal keys: rows of [A; acs] (tpr threads per row), columns of [B, bcs]
+// (32 columns x 256 rows per CTA).  Two passes over the operands in two launches
+// (here and k_f64_slice) instead of one CTA that walks a strip of columns twice:
+// 512^3 31 -> 21 us, 8192^3 1.60 -> 0.82 ms (the planes are 18 bytes per element,
+// 2.6 GB at 8192^3; with two reads 4.9 GB, 0.72 ms at the copy rate).
+__device__ __forceinline__ void max_rows(const SliceArgs& a, const double* src, int64_t ld,
+                                         int64_t rows, int64_t row_out, int64_t blk,
+                                         uint32_t* sh) {
   const int tpr = a.tpr, q = threadIdx.x & (tpr - 1), rib = threadIdx.x / tpr;
   const int64_t r = blk * (kSliceThreads / tpr) + rib;
-  const bool rv = r < rows;
-  const double* p = src + (rv ? r : 0) * ld;
-  const int64_t k = rv ? a.g.k : 0;
-  uint32_t hi = 0, any = 0;
-#pragma unroll 2
+  const double* p = src + (r < rows ? r : 0) * ld;
+  const int64_t k = r < rows ? a.g.k : 0;
+  uint32_t key = 0;
+#pragma unroll 4
   for (int64_t l = 4 * q; l < k; l += 4 * tpr) {
     double x[4];
     load4(p + l, k - l, x);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) take_max(x[e], hi, any);
+    for (int e = 0; e < 4; ++e) key = max(key, max_key(x[e]));
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    any |= __shfl_xor_sync(0xffffffffu, any, o);
-  }
-  const int warp = threadIdx.x >> 5, wpr = tpr / 32, w0 = rib * wpr;
-  if ((threadIdx.x & 31) == 0) {
-    sh[2 * warp] = hi;
-    sh[2 * warp + 1] = any;
-  }
+  key = __reduce_max_sync(0xffffffffu, key);
+  const int warp = threadIdx.x >> 5, wpr = tpr / 32;
+  if ((threadIdx.x & 31) == 0) sh[warp] = key;
   __syncthreads();
-  for (int w = w0; w < w0 + wpr; ++w) {
-    hi = max(hi, sh[2 * w]);
-    any |= sh[2 * w + 1];
-  }
-  const int ef = row_field(hi, any);
-  const int64_t out = row_out + r, plane = a.rows_a * a.kpad;
-  uint64_t bits = 0;
-  bool cut = false;
-  if (rv) {
-    for (int64_t l = 4 * q; l < a.kpad; l += 4 * tpr) {
-      double x[4] = {0.0, 0.0, 0.0, 0.0};
-      if (ef && l < k) load4(p + l, k - l, x);
-      Digits4 D;
-      slice4(x, ef ? ef : 1022, D, bits, cut);
-      if (!ef) D.plane[kMagPlane] = make_uint2(0x7fc07fc0u, 0x7fc07fc0u);  // NaN
-      uint16_t* o = a.pa + out * a.kpad + l;
-#pragma unroll
-      for (int pl = 0; pl < kPlanes64; ++pl)
-        *reinterpret_cast<uint2*>(o + pl * plane) = D.plane[pl];
-    }
-  }
-  uint32_t b0 = (uint32_t)bits, b1 = (uint32_t)(bits >> 32), c = cut ? 1u : 0u;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    b0 |= __shfl_xor_sync(0xffffffffu, b0, o);
-    b1 |= __shfl_xor_sync(0xffffffffu, b1, o);
-    c |= __shfl_xor_sync(0xffffffffu, c, o);
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) {
-    sh[3 * warp] = b0;
-    sh[3 * warp + 1] = b1;
-    sh[3 * warp + 2] = c;
-  }
-  __syncthreads();
-  if (q == 0 && rv) {
-    for (int w = w0; w < w0 + wpr; ++w) {
-      b0 |= sh[3 * w];
-      b1 |= sh[3 * w + 1];
-      c |= sh[3 * w + 2];
-    }
-    a.a_row[out] = row_info(ef, ((uint64_t)b1 << 32) | b0, c != 0);
+  if (q == 0 && r < rows) {
+    for (int w = 1; w < wpr; ++w) key = max(key, sh[warp + w]);
+    const int f = line_field(key);
+    a.a_row[row_out + r] = make_int2(f ? f - 1022 : kMinExp - 1, 0);
   }
 }
 
-// W columns of B per CTA (four per thread), all rows of the panel: the largest
-// elements, then the digits.
-template <int W>
-__device__ __forceinline__ void slice_cols(const SliceArgs& a, const double* src, int64_t ld,
-                                           int64_t cols, int64_t col_out, int64_t blk,
-                                           uint32_t* sh) {
-  constexpr int TW = W / 4, RG = kSliceThreads / TW;
-  const int tx = threadIdx.x % TW, rg = threadIdx.x / TW;
-  const int64_t c0 = blk * W + 4 * tx, nv = cols - c0;
-  const double* p = src + c0;
-  const int64_t k = a.g.k;
-  uint32_t hi[4] = {0, 0, 0, 0}, any[4] = {0, 0, 0, 0};
-  if (nv > 0) {
-#pragma unroll 4
-    for (int64_t l = rg; l < k; l += RG) {
-      double x[4];
-      load4(p + l * ld, nv, x);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) take_max(x[e], hi[e], any[e]);
-    }
+__device__ __forceinline__ void max_cols(const SliceArgs& a, const double* src, int64_t ld,
+                                         int64_t cols, int64_t col_out, int64_t blk,
+                                         uint32_t* sh) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t ncj = cdiv(cols, 32), c = blk / ncj, j = blk % ncj * 32 + lane;
+  const int64_t l0 = c * kMaxRows + warp * 32, l1 = min(l0 + 32, a.g.k);
+  uint32_t key = 0;
+  if (j < cols) {
+    const double* p = src + l0 * ld + j;
+#pragma unroll 8
+    for (int64_t l = l0; l < l1; ++l, p += ld) key = max(key, max_key(*p));
   }
-  // sh: [2][RG][W], then the columns' exponent fields [W]
-  uint32_t* sany = sh + RG * W;
+  sh[warp * 32 + lane] = key;
+  __syncthreads();
+  if (warp == 0 && j < cols) {
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    sh[rg * W + 4 * tx + e] = hi[e];
-    sany[rg * W + 4 * tx + e] = any[e];
+    for (int w = 1; w < kSliceThreads / 32; ++w) key = max(key, sh[w * 32 + lane]);
+    a.cmax[c * a.cols_b + col_out + j] = key;
+    if (c == 0) a.b_col[col_out + j] = make_int2(0, 0);
   }
-  __syncthreads();
-  int* sef = reinterpret_cast<int*>(sh + 2 * RG * W);
-  if (threadIdx.x < W) {
-    uint32_t h = 0, n = 0;
-    for (int g = 0; g < RG; ++g) {
-      h = max(h, sh[g * W + threadIdx.x]);
-      n |= sany[g * W + threadIdx.x];
-    }
-    sef[threadIdx.x] = row_field(h, n);
-  }
-  __syncthreads();
-  int ef[4];
-  uint64_t bits[4] = {0, 0, 0, 0};
-  bool cut[4] = {false, false, false, false};
-#pragma unroll
-  for (int e = 0; e < 4; ++e) ef[e] = sef[4 * tx + e];
-  const int64_t plane = a.kpad * a.cols_b;
-#pragma unroll 2
-  for (int64_t l = rg; l < a.kpad; l += RG) {
-    double x[4] = {0.0, 0.0, 0.0, 0.0};
-    if (nv > 0 && l < k) load4(p + l * ld, nv, x);
-    // the four columns have scales of their own: one digit lane at a time
-    uint32_t lane[4][kPlanes64];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int f = ef[e];
-      const double v[4] = {f ? x[e] : 0.0, 0.0, 0.0, 0.0};
-      Digits4 D;
-      slice4(v, f ? f : 1022, D, bits[e], cut[e]);
-#pragma unroll
-      for (int pl = 0; pl < kPlanes64; ++pl) lane[e][pl] = D.plane[pl].x & 0xffffu;
-      if (!f) lane[e][kMagPlane] = 0x7fc0u;
-    }
-    uint16_t* o = a.pb + l * a.cols_b + col_out + c0;
-#pragma unroll
-    for (int pl = 0; pl < kPlanes64; ++pl)
-      *reinterpret_cast<uint2*>(o + pl * plane) = make_uint2(lane[0][pl] | (lane[1][pl] << 16),
-                                                             lane[2][pl] | (lane[3][pl] << 16));
-  }
-  __syncthreads();
-  // sh again: the columns' collected bits and cuts
-  if (threadIdx.x < W) sh[threadIdx.x] = sh[W + threadIdx.x] = sh[2 * W + threadIdx.x] = 0;
-  __syncthreads();
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    atomicOr(&sh[4 * tx + e], (uint32_t)bits[e]);
-    atomicOr(&sh[W + 4 * tx + e], (uint32_t)(bits[e] >> 32));
-    if (cut[e]) atomicOr(&sh[2 * W + 4 * tx + e], 1u);
-  }
-  __syncthreads();
-  if (threadIdx.x < W && blk * W + threadIdx.x < cols)
-    a.b_col[col_out + blk * W + threadIdx.x] =
-        row_info(sef[threadIdx.x], ((uint64_t)sh[W + threadIdx.x] << 32) | sh[threadIdx.x],
-                 sh[2 * W + threadIdx.x] != 0);
 }
 
-template <int W>
-__global__ void __launch_bounds__(kSliceThreads) k_f64_slice(const SliceArgs a) {
-  __shared__ uint32_t sh[2 * 1024 + 64];
+__global__ void __launch_bounds__(kSliceThreads) k_f64_max(const SliceArgs a) {
+  __shared__ uint32_t sh[kSliceThreads];
   if (blockIdx.x == 0 && threadIdx.x < 2 && (threadIdx.x == 1 || !a.g.accumulate))
     a.hdr[threadIdx.x] = 0;  // the status word covers every panel
   int64_t b = blockIdx.x;
-  if (b < a.nb) return slice_cols<W>(a, a.g.B, a.g.ldb, a.g.n, 0, b, sh);
-  b -= a.nb;
-  if (b < a.nbc) return slice_cols<W>(a, a.g.bcs, a.g.ldbcs, a.g.Cc, a.col_cs, b, sh);
-  b -= a.nbc;
-  if (b < a.na) return slice_rows(a, a.g.A, a.g.lda, a.g.m, 0, b, sh);
-  slice_rows(a, a.g.acs, a.g.ldacs, a.g.R, a.row_cs, b - a.na, sh);
+  if (b < a.n0) return max_cols(a, a.g.B, a.g.ldb, a.g.n, 0, b, sh);
+  b -= a.n0;
+  if (b < a.n1) return max_cols(a, a.g.bcs, a.g.ldbcs, a.g.Cc, a.col_cs, b, sh);
+  b -= a.n1;
+  if (b < a.n2) return max_rows(a, a.g.A, a.g.lda, a.g.m, 0, b, sh);
+  max_rows(a, a.g.acs, a.g.ldacs, a.g.R, a.row_cs, b - a.n2, sh);
+}
+
+// The digits of 16 rows x 256 columns of A (one scale per row) or B (one per
+// column): a thread takes four columns of every fourth row.
+template <bool kRowsScaled>
+__device__ __forceinline__ void slice_tile(const SliceArgs& a, const double* src, int64_t ld,
+                                           int64_t rows, int64_t cols, int64_t prow,
+                                           int64_t pcol, int64_t blk, int* sef) {
+  const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6, lane = threadIdx.x & 31;
+  const int64_t pw = kRowsScaled ? a.kpad : cdiv(cols, 64) * 64;  // padded columns
+  const int64_t ph = kRowsScaled ? rows : a.kpad;                 // padded rows
+  const int64_t nbx = cdiv(pw, kSliceCols);
+  const int64_t r0 = blk / nbx * kSliceRows, c0 = blk % nbx * kSliceCols + 4 * tx;
+  const int64_t ldp = kRowsScaled ? a.kpad : a.cols_b;
+  const int64_t plane = (kRowsScaled ? a.rows_a : a.kpad) * ldp;
+  uint16_t* const out = kRowsScaled ? a.pa : a.pb;
+  if constexpr (!kRowsScaled) {  // the columns' scales from their partial maxima
+    const int64_t j = blk % nbx * kSliceCols + threadIdx.x;
+    uint32_t key = 0;
+    if (j < cols)
+      for (int64_t c = 0; c < cdiv(a.g.k, kMaxRows); ++c)
+        key = max(key, a.cmax[c * a.cols_b + pcol + j]);
+    const int f = line_field(key);
+    sef[threadIdx.x] = f;
+    if (r0 == 0 && j < cols) a.b_col[pcol + j].x = f ? f - 1022 : 0;
+    __syncthreads();
+  }
+  int ef[4];
+  uint64_t bits[4] = {0, 0, 0, 0};
+  bool cut[4] = {false, false, false, false};
+  if constexpr (!kRowsScaled) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ef[q] = sef[4 * tx + q];
+  }
+  const bool in = c0 < pw;
+#pragma unroll 2
+  for (int i = 0; i < kSliceRows / 4; ++i) {
+    const int64_t r = r0 + ty + 4 * i;
+    if (r >= ph) break;  // the whole warp: a row belongs to one
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+    if (in && r < rows) load4(src + r * ld + c0, cols - c0, x);
+    if constexpr (kRowsScaled) {
+      const int e = a.a_row[prow + r].x;
+      const int f = e < kMinExp ? 0 : e + 1022;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        ef[q] = f;
+        bits[q] = 0;
+        cut[q] = false;
+      }
+    }
+    if (in) slice4(x, ef, out + (prow + r) * ldp + pcol + c0, plane, bits, cut);
+    if constexpr (kRowsScaled) {
+      const uint64_t b = bits[0] | bits[1] | bits[2] | bits[3];
+      const uint32_t b0 = __reduce_or_sync(0xffffffffu, (uint32_t)b);
+      const uint32_t b1 = __reduce_or_sync(0xffffffffu, (uint32_t)(b >> 32));
+      const bool c = __any_sync(0xffffffffu, cut[0] | cut[1] | cut[2] | cut[3]);
+      const int z = last_digit(ef[0], ((uint64_t)b1 << 32) | b0, c);
+      if (lane == 0 && a.a_row[prow + r].y < z) atomicMax(&a.a_row[prow + r].y, z);
+    }
+  }
+  if constexpr (!kRowsScaled) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (c0 + q >= cols) break;
+      const int z = last_digit(ef[q], bits[q], cut[q]);
+      int2* const at = a.b_col + pcol + c0 + q;
+      if (at->y < z) atomicMax(&at->y, z);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kSliceThreads) k_f64_slice(const SliceArgs a) {
+  __shared__ int sef[kSliceCols];
+  int64_t b = blockIdx.x;
+  if (b < a.n0) return slice_tile<false>(a, a.g.B, a.g.ldb, a.g.k, a.g.n, 0, 0, b, sef);
+  b -= a.n0;
+  if (b < a.n1)
+    return slice_tile<false>(a, a.g.bcs, a.g.ldbcs, a.g.k, a.g.Cc, 0, a.col_cs, b, sef);
+  b -= a.n1;
+  if (b < a.n2) return slice_tile<true>(a, a.g.A, a.g.lda, a.g.m, a.g.k, 0, 0, b, sef);
+  slice_tile<true>(a, a.g.acs, a.g.ldacs, a.g.R, a.g.k, a.row_cs, 0, b - a.n2, sef);
 }
 
 // ------------------------------------------------------------------ product
@@ -907,6 +883,7 @@ bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, si
   r.b_planes = region((size_t)kPlanes64 * r.cols_b * r.kp * 2);
   r.a_row = region(sizeof(int2) * r.rows_a);
   r.b_col = region(sizeof(int2) * r.cols_b);
+  r.cmax = region(sizeof(uint32_t) * cdiv(r.kp, kMaxRows) * r.cols_b);
   r.bad = region((size_t)tiles);
   r.scratch = region((size_t)ctas * kLevels * r.bpt * 8 * 256 * sizeof(int4));
   *bytes = off;
@@ -943,18 +920,22 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     a.b_col = reinterpret_cast<int2*>(w + r.b_col);
     a.hdr = hdr;
     a.rows_a = r.rows_a; a.cols_b = r.cols_b; a.row_cs = r.row_cs; a.col_cs = r.col_cs;
+    a.cmax = reinterpret_cast<uint32_t*>(w + r.cmax);
     a.tpr = 32;
     while (a.tpr < kSliceThreads && a.tpr * 8 < kpad) a.tpr *= 2;
     const int rpc = kSliceThreads / a.tpr;
-    const int W = g.n <= 16 * kSms ? 16 : 32;
-    a.nb = cdiv(g.n, W);
-    a.nbc = cdiv(g.Cc, W);
-    a.na = cdiv(g.m, rpc);
-    const unsigned grid = (unsigned)(a.nb + a.nbc + a.na + cdiv(g.R, rpc));
-    if (W == 16)
-      k_f64_slice<16><<<grid, kSliceThreads, 0, st>>>(a);
-    else
-      k_f64_slice<32><<<grid, kSliceThreads, 0, st>>>(a);
+    const int64_t nch = cdiv(gp.k, kMaxRows);
+    a.n0 = cdiv(g.n, 32) * nch;
+    a.n1 = cdiv(g.Cc, 32) * nch;
+    a.n2 = cdiv(g.m, rpc);
+    k_f64_max<<<(unsigned)(a.n0 + a.n1 + a.n2 + cdiv(g.R, rpc)), kSliceThreads, 0, st>>>(a);
+    auto tiles = [&](int64_t rows, int64_t cols) {
+      return cdiv(rows, kSliceRows) * cdiv(cdiv(cols, BK) * BK, kSliceCols);
+    };
+    a.n0 = tiles(kpad, g.n);
+    a.n1 = tiles(kpad, g.Cc);
+    a.n2 = tiles(g.m, kpad);
+    k_f64_slice<<<(unsigned)(a.n0 + a.n1 + a.n2 + tiles(g.R, kpad)), kSliceThreads, 0, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) break;
 
     Maps M;
@@ -997,7 +978,7 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     cfg.numAttrs = r.pair ? 1 : 0;
     if ((e = cudaLaunchKernelEx(&cfg, kernel, M, p)) != cudaSuccess) break;
     e = launch_gemm_f64_bad(gp, T, r.pair ? 4 : 2, r.bpt, hdr + 1, p.bad, st);
-    count_launches(2);
+    count_launches(3);
   }
   return e;
 }

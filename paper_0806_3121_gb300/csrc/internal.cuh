@@ -78,6 +78,7 @@ struct Erased {
 struct F64TcRegions {
   size_t a_planes, b_planes;  // bf16 digit planes of [A; acs] and [B, bcs], one panel of K
   size_t a_row, b_col;        // int2 {exponent, last digit used} per row / column
+  size_t cmax;                // maximal keys of 256 rows of each column of [B, bcs]
   size_t bad;                 // one byte per tile: left to the DFMA kernel
   size_t scratch;             // per CTA: the level sums of its tile
   int64_t kp;                 // longest panel of K
