@@ -84,8 +84,8 @@ typedef enum {
 
 typedef enum {
   ABFT_F64 = 0,     /* A, B, C binary64, binary64 checksums; the product runs on
-                       the tensor cores in exact bf16 digits (from 128^3 up, with a
-                       workspace) or on the FP64 pipe: never less accurate than a
+                       the tensor cores in exact bf16 residues (from 128^3 up, with
+                       a workspace) or on the FP64 pipe: never less accurate than a
                        chain of binary64 multiply-adds                              */
   ABFT_BF16 = 1,    /* A, B bfloat16; C binary32; tensor-core product, fp32 accum.  */
   ABFT_BF16X3 = 2,  /* A, B binary32 split into bf16 hi+lo planes by abft_encode;
@@ -262,11 +262,11 @@ abft_status abft_encode_chained(const abft_desc* desc, const void* A, const void
 /* The ABFT product (Eq. (1)): [A; C_C^T A] [B, B C_R] on the GPU.  Writes the
  * data block A B into C and the checksum blocks into ws (E and F).  Requires a
  * preceding abft_encode on the same ws and operands.  ABFT_F64 with m n k of at
- * least 2^21: the operands are sliced into exact bf16 digits (in ws, below
- * layout.scratch) and multiplied on the tensor cores; the tiles whose operands
- * would lose accuracy that way (NaN, infinities, exponents outside [-440, 500],
- * elements far below their row's and column's scales) run on the FP64 pipe, as
- * all smaller products do.  ABFT_BF16X3 and
+ * least 2^21: the operands become integers whose residues modulo 17 small
+ * numbers (bf16, in ws below layout.scratch) are multiplied on the tensor cores;
+ * the elements that would lose accuracy that way (NaN, infinities, exponents
+ * outside [-440, 500], terms far below their row's and column's scales) run on
+ * the FP64 pipe, as all smaller products do.  ABFT_BF16X3 and
  * ABFT_BF16X6 multiply the bf16 operand planes that encode wrote.
  * ABFT_FP8_E4M3: the data block multiplies the e4m3 codes of A and the
  * transposed codes of B that encode wrote, on the 8-bit tensor path
@@ -292,7 +292,7 @@ abft_status abft_set_epilogue_faults(const abft_desc* desc, void* ws, const int6
 
 /* The same GEMM kernel with no checksum tiles: C = A B only.  This is the
  * checksum-free baseline the ABFT overhead is measured against.  ABFT_F64: with
- * ws the kernel of abft_gemm (it writes ws's digit planes and status word, not
+ * ws the kernel of abft_gemm (it writes ws's residue planes and status word, not
  * its checksums), without ws always the FP64 pipe.  ws may be NULL except for ABFT_BF16X3, ABFT_BF16X6 and ABFT_FP8_E4M3, whose products read the bf16
  * operand planes a preceding abft_encode wrote into ws.  A bounded wait that
  * gives up is recorded in ws's status word (as for abft_gemm); without ws it

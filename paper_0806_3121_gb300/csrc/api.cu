@@ -203,8 +203,8 @@ abft_status make_plan(const abft_desc* d, Plan* P) {
   return ABFT_OK;
 }
 
-// Products with bounded waits: the tensor-core dtypes and the sliced binary64
-// product (whose status word the verify and the rebuild copy to kCntTimeout).
+// Products with bounded waits: the tensor-core dtypes and the binary64
+// product on them (whose status word the verify and the rebuild copy to kCntTimeout).
 bool has_status(const Plan& P) { return P.d.dtype != ABFT_F64 || P.tc64; }
 
 bool is_empty(const Plan& P) { return P.d.m == 0 || P.d.n == 0; }

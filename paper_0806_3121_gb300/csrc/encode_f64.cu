@@ -62,7 +62,7 @@ struct EncArgs {
   int64_t bs;
   double* car_a;   // cleared: a fresh encode carries no deviation
   double* car_b;
-  int32_t* status; // sliced product: its status word, cleared
+  int32_t* status; // tensor-core product: its status word, cleared
   int wpu;         // warps that share a verify block's rows
   // CTAs of the passes, in this order (0: the pass is not wanted)
   int64_t n_acols, n_brows, n_ablk, n_bsq, n_arows;

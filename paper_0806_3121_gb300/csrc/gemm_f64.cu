@@ -1,6 +1,6 @@
 // Binary64 ABFT product (Eq. (1)): [A; acs] [B, bcs] on the FP64 FMA pipe, for
 // products below 128^3, checksum-free products without a workspace and the
-// tiles that the sliced product on the tensor cores (gemm_f64_tc.cu) leaves out.
+// chunks that the product on the tensor cores (gemm_f64_tc.cu) leaves out.
 //
 // On GB300 the FP64 FMA pipe issues 2 DFMA per clock per SM (measured
 // 1.20 TFLOP/s over 152 SMs); mma.sync f64 runs slower (1.05 TFLOP/s) and
@@ -27,9 +27,10 @@ constexpr int BM = 64, BN = 64, BK = 16, kThreads = 256;
 constexpr int GROUP_M = 16;  // tile rows per raster group
 
 // The BM x BN tile at (row0, col0) of the data (cs_row = cs_col = false), of the
-// checksum rows (cs_row) or of the checksum columns (cs_col).
+// checksum rows (cs_row) or of the checksum columns (cs_col); bit 2 r + c of mask:
+// write its 32 x 32 quarter (r, c).
 __device__ __forceinline__ void tile_f64(const F64Args& g, bool cs_row, bool cs_col, int64_t row0,
-                                         int64_t col0) {
+                                         int64_t col0, int mask) {
   // Source and destination of this tile.
   const double* Asrc = cs_row ? g.acs : g.A;
   const int64_t ldA = cs_row ? g.ldacs : g.lda, rlim = cs_row ? g.R : g.m;
@@ -115,7 +116,7 @@ __device__ __forceinline__ void tile_f64(const F64Args& g, bool cs_row, bool cs_
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int64_t col = col0 + tx + 16 * j;
-      if (col < clim) Dst[row * ldD + col] = acc[i][j];
+      if (col < clim && (mask >> ((i >> 1) * 2 + (j >> 1)) & 1)) Dst[row * ldD + col] = acc[i][j];
     }
   }
 }
@@ -125,10 +126,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemm_f64(const F64Args g, const
   T.decode(blockIdx.x, ty, tx);
   const bool cs_row = ty >= T.tm, cs_col = tx >= T.tn;
   tile_f64(g, cs_row, cs_col, (int64_t)(cs_row ? ty - T.tm : ty) * BM,
-           (int64_t)(cs_col ? tx - T.tn : tx) * BN);
+           (int64_t)(cs_col ? tx - T.tn : tx) * BN, 15);
 }
 
-// The tiles (64 hpt x 64 bpt) that the sliced product left out, as BM x BN tiles.
+// The 32 x 32 chunks that the product on the tensor cores left out (tiles of 64 hpt x
+// 64 bpt; bad: per tile [chunk row][chunk column]), each with the BM x BN tile it is
+// a quarter of.
 __global__ void __launch_bounds__(kThreads, 2)
     k_gemm_f64_bad(const F64Args g, const TileGrid T, int hpt, int bpt, const int* any,
                    const uint8_t* bad) {
@@ -136,16 +139,19 @@ __global__ void __launch_bounds__(kThreads, 2)
   const int64_t total = T.total() * hpt * bpt;
   for (int64_t u = blockIdx.x; u < total; u += gridDim.x) {
     const int64_t t = u / (hpt * bpt);
-    const int s = (int)(u - t * hpt * bpt);
-    if (!bad[t]) continue;
+    const int s = (int)(u - t * hpt * bpt), sr = s % hpt, sc = s / hpt;
+    const uint8_t* const b = bad + t * (4 * hpt * bpt) + 2 * sr * (2 * bpt) + 2 * sc;
+    const int mask = (b[0] ? 1 : 0) | (b[1] ? 2 : 0) | (b[2 * bpt] ? 4 : 0) |
+                     (b[2 * bpt + 1] ? 8 : 0);
+    if (!mask) continue;
     int ty, tx;
     T.decode(t, ty, tx);
     const bool cs_row = ty >= T.tm, cs_col = tx >= T.tn;
-    const int64_t row0 = ((int64_t)(cs_row ? ty - T.tm : ty) * hpt + s % hpt) * BM;
-    const int64_t col0 = ((int64_t)(cs_col ? tx - T.tn : tx) * bpt + s / hpt) * BN;
+    const int64_t row0 = ((int64_t)(cs_row ? ty - T.tm : ty) * hpt + sr) * BM;
+    const int64_t col0 = ((int64_t)(cs_col ? tx - T.tn : tx) * bpt + sc) * BN;
     if (row0 >= (cs_row ? g.R : g.m) || col0 >= (cs_col ? g.Cc : g.n)) continue;
     __syncthreads();  // the previous tile's shared memory has been read
-    tile_f64(g, cs_row, cs_col, row0, col0);
+    tile_f64(g, cs_row, cs_col, row0, col0, mask);
   }
 }
 

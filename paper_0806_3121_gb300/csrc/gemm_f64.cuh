@@ -1,5 +1,5 @@
 // Shared by the two binary64 products: the DFMA kernel (gemm_f64.cu) and the
-// sliced product on the tensor cores (gemm_f64_tc.cu).
+// product on the tensor cores (gemm_f64_tc.cu).
 #pragma once
 
 #include "internal.cuh"
@@ -58,12 +58,12 @@ struct F64Args {
   int accumulate;  // 1: add to C, E, F (a later panel of K) instead of writing them
 };
 
-// The DFMA kernel on the tiles (64 hpt x 64 bpt) of the sliced product whose byte
-// in `bad` is set; returns at once when *any is zero.
+// The DFMA kernel on the 32 x 32 chunks of the tiles (64 hpt x 64 bpt) of the product
+// on the tensor cores whose byte in `bad` is set; returns at once when *any is zero.
 cudaError_t launch_gemm_f64_bad(const F64Args& g, const TileGrid& tiles, int hpt, int bpt,
                                 const int* any, const uint8_t* bad, cudaStream_t st);
 
-// The sliced product in the workspace regions of P.f64tc.
+// The product on the tensor cores in the workspace regions of P.f64tc.
 cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaStream_t st);
 
 }  // namespace abft

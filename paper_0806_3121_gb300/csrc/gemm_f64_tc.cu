@@ -1,47 +1,47 @@
-// Binary64 product [A; acs] [B, bcs] on the tensor cores, by slicing the
-// operands into exact bf16 digits (the error-free splitting of Ozaki, Ogita,
-// Oishi and Rump, "Error-free transformations of matrix multiplication by using
-// fast routines of matrix multiplication and its applications", 2012).
+// Binary64 product [A; acs] [B, bcs] on the tensor cores, by integer arithmetic
+// modulo small numbers (the scheme of Ozaki, Uchino and Imamura, "Ozaki scheme II: a
+// GEMM-oriented emulation of floating-point matrix multiplication using an integer
+// modular technique", 2025, with bf16 residues instead of 8-bit integers).
 //
 // GB300's FP64 pipe issues 2 DFMA per clock and SM (1.2 TFLOP/s on the whole
 // chip); its tensor cores multiply bf16 at 1900 TFLOP/s.  Row i of A (column
-// j of B) is scaled by the power of two above its largest element and written
-// as eight signed radix-256 digits, d_0 2^-7 + d_1 2^-15 + ... + d_7 2^-63, each in
-// [-128, 128] and so exact in bf16.  Digit products of equal weight,
-//   L_s = sum_{i + j = s} D_i(A) D_j(B),
-// are integers; 1024 of them add up to at most 2^24, exact in the tensor cores'
-// binary32 accumulators, and the epilogue adds those partial sums as 32-bit
-// integers.  C_ij = 2^(eA_i + eB_j) sum_s L_s 2^(-14 - 8 s) is formed once, in
-// integers, and rounded to nearest once.
+// j of B) is scaled by the power of two above its largest element and rounded to
+// an integer a' of b = 58 or 59 bits.  The exact integer C' = sum_l a'_il b'_lj is
+// below half of P, the product of 17 coprime moduli up to 256 (133 bits), so it
+// follows from its residues.  A residue is at most 128 in magnitude: exact in bf16,
+// and 1024 products of two add up to at most 2^24, exact in the tensor cores'
+// binary32 accumulators.  One bf16 product per modulus gives C' mod p (the epilogue
+// reduces each accumulator modulo p), the Chinese remainder theorem C' itself, and
+// C_ij = 2^(eA_i + eB_j - 2 b) C' is rounded to nearest once: all in integer and
+// exact binary32 arithmetic.
 //
-// How many levels.  What is left out is the digit products of the next level and
-// beyond: with levels 0..6 (28 products) a rms error of 2^-56.2 per term in units
-// of 2^(eA_i + eB_j), with levels 0..7 (36 products) 2^-64.2.  A DFMA chain's
-// rounding errors are about 0.38 2^-53 sqrt(k / 2) times the rms of the terms'
-// sum, at least 0.27 2^-53 M_ij with M_ij = sum_l |a_il b_lj| in the same units.
-// So levels 0..6 are as accurate as the chain where M_ij >= 0.405 sqrt(k), levels
-// 0..7 where M_ij >= 0.0016 sqrt(k).  M is one more product (plane 8: the
-// magnitudes as bf16, rounded towards zero), and every tile computes it first:
-// each element is checked, so rows of mixed scales, graded operands whose large
-// rows meet small columns, and sparse operands never lose accuracy.  An element
-// none of whose terms is cut (operands with few significant bits) needs no
-// check.  Tiles with an element below both lines, NaN or infinite operands, or
-// exponents outside [-440, 500] are left to the DFMA kernel (k_gemm_f64_bad).
+// Accuracy.  What is lost is the rounding of a and b to 59 bits below their row's
+// and column's scale: a rms error of at most 2^-60.3 (b = 59) per term in units of
+// 2^(eA_i + eB_j).  A DFMA chain's rounding errors are about 0.38 2^-53 sqrt(k / 2)
+// times the rms of the terms' sum, at least 0.27 2^-53 M_ij with M_ij = sum_l |a_il
+// b_lj| in the same units.  So the product is as accurate as the chain where M_ij >=
+// 2^(53 - b - 1.3) / 0.27 sqrt(k) = 0.0235 sqrt(k) (b = 59).  M is one more product
+// (plane 17: the magnitudes as bf16, rounded towards zero), and every tile computes
+// it first: each element is checked, so rows of mixed scales, graded operands whose
+// large rows meet small columns, and sparse operands never lose accuracy.  Elements
+// of rows and columns that are integers as they are need no check.  The 32 x 32
+// chunks that hold an element below the line, NaN or infinite operands or exponents
+// outside [-440, 500] are left to the DFMA kernel (k_gemm_f64_bad).
 //
-// The tensor cores bound it: 29 or 37 products of 2 m n k bf16 flops each.
-// 128 x (64 bpt)-tiles on one CTA or 256 x 256 tiles on a pair, one CTA per SM:
-// warps 0 / 10 copy A / B by TMA into a shared-memory ring, warp 1 issues tcgen05.mma into two alternating TMEM
-// accumulators, warps 2-9 add each accumulator into 128 integer registers per
-// thread.  Level sums go to a per-CTA scratch (coalesced, mostly L2) because
-// eight levels do not fit the registers and the FP64 pipe is too narrow to fold
-// them as they come (8 folds of a 128 x 256 tile at 2 per clock would take 131 k
-// clocks of the tile's 1.9 M at k = 8192).
+// The tensor cores bound it: 18 products of 2 m n k bf16 flops each.  (Exact digits
+// in radix 256 instead of residues take 29 to 37 products for the same accuracy,
+// a level sum in 32-bit integers per thread and a copy of every level: 8192^3 21.6
+// ms, 4096^3 2.93, 2048^3 0.38 .. 0.47, 512^3 59 us.)  128 x (64 bpt)-tiles on one
+// CTA or 256 x 256 tiles on a pair, one CTA per SM: warps 0 / 10 copy A / B by TMA
+// into a shared-memory ring, warp 1 issues tcgen05.mma into two alternating TMEM
+// accumulators, warps 2-9 reduce each accumulator modulo p and keep the residues of
+// a finished modulus, one byte each, in a per-CTA scratch (coalesced, mostly L2).
 //
 // Measured, product kernels alone: 8192^3 on a 16 x 16 grid 949 ms on the FP64 pipe,
-// 22 here; 4096^3 on an 8 x 8 grid 130 -> 2.9; 2048^3 16.3 -> 0.38 .. 0.47; 1000 x 1501
-// x 777 2.36 -> 0.13; 512^3 0.53 -> 0.06.  Relative
-// Frobenius error against the exact product, N(0,1): 4.5e-17 (DFMA 7.7e-16) at k =
-// 512, 2.8e-16 (2.0e-15) at k = 4096, 4.7e-16 (4.9e-15) at k = 20000.
+// 11.7 .. 15 here (with the clock); 4096^3 on an 8 x 8 grid 130 -> 1.95; 2048^3 16.3 ->
+// 0.28; 1000 x 1501 x 777 2.36 -> 0.093; 512^3 0.53 -> 0.053.  Relative Frobenius error
+// against the exact product, N(0,1): 4.5e-17 (DFMA 7.7e-16) at k = 512, 4.7e-17 (2.0e-15)
+// at k = 4096, 7.0e-17 (4.9e-15) at k = 20000 in two panels of K.
 #include <cuda.h>
 
 #include <stdlib.h>
@@ -56,18 +56,18 @@ namespace abft {
 namespace {
 
 constexpr int BM = 128, BK = 64;
-constexpr int kDigits = 8, kMagPlane = 8, kPlanes64 = 9;
-constexpr int kGroupSteps = 16;   // k-steps per accumulator: 1024 2^14 = 2^24
-constexpr int kLevels = 8;        // levels 0..6, and 7 where the magnitudes ask for it
-constexpr int kMaxPanel = 16320;  // 8 * 16320 * 2^14 < 2^31: a level sum fits 32 bits
+constexpr int kModuli = 17, kMagPlane = kModuli, kPlanes64 = kModuli + 1;
+constexpr int kGroupSteps = 16;   // k-steps per accumulator: 1024 products of at most 2^14
+constexpr int kMaxPanel = 16320;  // K of a pass: 255 k-steps, 16 partial residues per thread
+constexpr int kMaxBits = 59;      // of an operand's integers (four 15-bit limbs hold them)
 constexpr int kEpiWarps = 8;
 constexpr int kWarpProdB = 2 + kEpiWarps;
 constexpr int kThreads = 32 * (kWarpProdB + 1);
 constexpr uint32_t kABytes = BM * BK * 2, kBoxBytes = 64 * BK * 2;
 constexpr int kMaxStages = 8;
 constexpr int kMinExp = -440, kMaxExp = 500;
-constexpr int kNotExact = 100;    // digit index of an operand row that is cut or refused
-constexpr size_t kPlaneBudget = size_t(6) << 30;
+constexpr int kCut = 1, kRefused = 2;  // operand lines that were rounded / cannot be held
+constexpr size_t kPlaneBudget = size_t(12) << 30;
 constexpr int kSms = 152;  // persistent CTAs the workspace is laid out for
 
 // Tile kinds.  One CTA: 128 rows x bpt 64-column boxes.  CTA pair (bpt = 4): 256
@@ -81,16 +81,114 @@ constexpr size_t smem_bytes(int boxes) {
 static_assert(smem_bytes(4) <= 232448 && smem_bytes(2) <= 232448 && smem_bytes(1) <= 232448,
               "shared memory per CTA");
 
-// ------------------------------------------------------------------ digits
+// ------------------------------------------------------------------ residues
 
-// x 2^(63 - e) rounded to a 64-bit integer (|x| < 2^e, e = efield - 1022 with
-// efield the biased exponent of the row's largest element); the bits cut off.
-__device__ __forceinline__ uint64_t scaled(double x, int efield, bool& cut) {
+// The moduli (pairwise coprime) and what the device needs of them.  Residues are
+// signed and smallest in magnitude.  Signed limbs: x = sum_i limb_i 2^(32 i), each in
+// [-2^31, 2^31).
+struct Moduli {
+  int p[kModuli] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197,
+                    193, 191};
+  float pf[kModuli] = {}, inv[kModuli] = {};
+  // weights of the 15-bit limbs of an integer in its residue, for B; for A times
+  // (P / p)^-1 mod p, so the product's residue x_t has C' = sum_t x_t P / p_t mod P
+  float ca[kModuli][4] = {}, cb[kModuli][4] = {};
+  // reconstruction in groups of three moduli (the last of two): y = sum x_t g_t, the
+  // product of the group's other moduli; C' = sum_j y_j P / (group's product) - n P
+  int g[kModuli] = {};
+  int limb[6][4] = {};  // P / (group's product)
+  int frac[6] = {};     // 2^40 / (group's product)
+  int P[5] = {};
+};
+constexpr double kLog2P = 132.95;  // P = 2^132.953
+
+constexpr int centred(int64_t x, int p) {
+  int64_t r = x % p;
+  if (r < 0) r += p;
+  return (int)(2 * r > p ? r - p : r);
+}
+
+constexpr Moduli make_moduli() {
+  Moduli M;
+  for (int t = 0; t < kModuli; ++t) {
+    const int p = M.p[t];
+    M.pf[t] = (float)p;
+    M.inv[t] = 1.0f / (float)p;
+    int64_t q = 1;  // P / p mod p
+    for (int u = 0; u < kModuli; ++u)
+      if (u != t) q = q * M.p[u] % p;
+    int64_t w = 1;
+    while (q * w % p != 1) ++w;
+    int64_t c = 1;
+    for (int i = 0; i < 4; ++i) {
+      M.cb[t][i] = (float)centred(c, p);
+      M.ca[t][i] = (float)centred(c * w, p);
+      c = c * 32768 % p;
+    }
+    const int j0 = t / 3 * 3;
+    M.g[t] = 1;
+    for (int u = j0; u < j0 + 3 && u < kModuli; ++u)
+      if (u != t) M.g[t] *= M.p[u];
+  }
+  for (int j = 0; j <= 6; ++j) {  // j = 6: P itself
+    uint64_t v[6] = {1, 0, 0, 0, 0, 0};  // 32-bit limbs
+    int64_t group = 1;
+    for (int u = 0; u < kModuli; ++u) {
+      if (u / 3 == j) {
+        group *= M.p[u];
+        continue;
+      }
+      uint64_t carry = 0;
+      for (int i = 0; i < 6; ++i) {
+        const uint64_t x = v[i] * (uint64_t)M.p[u] + carry;
+        v[i] = x & 0xffffffffull;
+        carry = x >> 32;
+      }
+    }
+    int64_t carry = 0;
+    for (int i = 0; i < 5; ++i) {
+      int64_t x = (int64_t)v[i] + carry;
+      carry = 0;
+      if (x >= 2147483648ll) {
+        x -= 4294967296ll;
+        carry = 1;
+      }
+      if (j == 6)
+        M.P[i] = (int)x;
+      else if (i < 4)
+        M.limb[j][i] = (int)x;
+    }
+    if (j < 6) M.frac[j] = (int)(((1ll << 40) + group / 2) / group);
+  }
+  return M;
+}
+
+// Compile-time: as instruction operands they cost nothing, where a constant bank's
+// cold misses cost a small product 10 us.
+constexpr Moduli kM = make_moduli();
+
+// {p, 1 / p} where the modulus is a loop variable.
+struct ModulusTable {
+  float2 m[kModuli];
+};
+constexpr ModulusTable make_table() {
+  ModulusTable T{};
+  for (int t = 0; t < kModuli; ++t) {
+    T.m[t].x = kM.pf[t];
+    T.m[t].y = kM.inv[t];
+  }
+  return T;
+}
+__constant__ ModulusTable kModulus = make_table();
+
+// x 2^(bits - e) rounded to the nearest integer (|x| < 2^e, e = efield - 1022 with
+// efield the biased exponent of the line's largest element; bits <= 59).
+__device__ __forceinline__ int64_t scaled(double x, int efield, int bits, bool& cut) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
   const int E = (int)(b >> 52) & 0x7ff;
   const uint64_t m =
       ((b & 0xfffffffffffffull) | (E ? 0x10000000000000ull : 0ull)) << 10;  // below 2^63
-  const int r = efield - max(E, 1);
+  const int r = efield - max(E, 1) + (63 - bits);
   uint64_t v = 0;
   if (r < 64) {
     v = (m + ((1ull << r) >> 1)) >> r;
@@ -98,7 +196,7 @@ __device__ __forceinline__ uint64_t scaled(double x, int efield, bool& cut) {
   } else {
     cut |= m != 0;
   }
-  return b >> 63 ? 0ull - v : v;
+  return (int64_t)(b >> 63 ? 0ull - v : v);
 }
 
 // |x| 2^-e as bf16, rounded towards zero (nonzero values at least 2^-60).
@@ -109,45 +207,53 @@ __device__ __forceinline__ uint32_t magnitude(double x, int efield) {
   return ex < 67 ? 67u << 7 : ((uint32_t)ex << 7) | ((hi >> 13) & 0x7fu);
 }
 
+constexpr float kRound = 12582912.0f;  // 1.5 2^23: x + kRound - kRound rounds x, |x| <= 2^22
+
+// The smallest residue of the integer s (|s| <= 2^24) modulo p.
+__device__ __forceinline__ float residue(float s, float p, float inv) {
+  return fmaf(-(fmaf(s, inv, kRound) - kRound), p, s);
+}
+
+// The residues modulo p_t and all later moduli of four integers, from their limbs.
+template <bool kA, int t>
+__device__ __forceinline__ void residues4(const float (&l)[4][4], uint16_t* o, int64_t plane) {
+  constexpr float c0 = kA ? kM.ca[t][0] : kM.cb[t][0], c1 = kA ? kM.ca[t][1] : kM.cb[t][1],
+                  c2 = kA ? kM.ca[t][2] : kM.cb[t][2], c3 = kA ? kM.ca[t][3] : kM.cb[t][3],
+                  p = kM.pf[t], inv = kM.inv[t];
+  float r[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)  // the sum is at most 4 2^14 2^7: exact
+    r[q] = residue(fmaf(l[q][3], c3, fmaf(l[q][2], c2, fmaf(l[q][1], c1, l[q][0] * c0))), p, inv);
+  // bf16 holds a residue exactly: the upper halves of the binary32 words
+  *reinterpret_cast<uint2*>(o) =
+      make_uint2(__byte_perm(__float_as_uint(r[0]), __float_as_uint(r[1]), 0x7632u),
+                 __byte_perm(__float_as_uint(r[2]), __float_as_uint(r[3]), 0x7632u));
+  if constexpr (t + 1 < kModuli) residues4<kA, t + 1>(l, o + plane, plane);
+}
+
 // Four consecutive elements of every plane, at o (planes `plane` elements apart),
-// from four values with scales ef (0: a line that the digits cannot hold, whose
-// digits are zero and whose magnitudes are NaN); bits / cut collect the integers'
-// bits and whether any were cut off.
-__device__ __forceinline__ void slice4(const double (&x)[4], const int (&ef)[4], uint16_t* o,
-                                       int64_t plane, uint64_t (&bits)[4], bool (&cut)[4]) {
-  // (X + 2^63) + sum_j 128 256^j has the bytes d + 128 of the digits below the
-  // top one, and the top digit (with the carry) in the last place
-  uint32_t w[4][2], top[4], mag[4];
+// from four values with scales ef (0: a line that cannot be held, whose residues are
+// zero and whose magnitudes are NaN); cut: whether any bits were cut off.
+template <bool kA>
+__device__ __forceinline__ void slice4(const double (&x)[4], const int (&ef)[4], int bits,
+                                       uint16_t* o, int64_t plane, bool (&cut)[4]) {
+  float l[4][4];  // 15-bit signed limbs of the integers
+  uint32_t mag[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int f = ef[q] ? ef[q] : 1022;
     const double v = ef[q] ? x[q] : 0.0;
-    const uint64_t X = scaled(v, f, cut[q]);
-    bits[q] |= X;
-    const uint64_t u0 = X ^ 0x8000000000000000ull, u = u0 + 0x0080808080808080ull;
-    w[q][0] = (uint32_t)u;
-    w[q][1] = (uint32_t)(u >> 32);
-    top[q] = (w[q][1] >> 24) + (u < u0 ? 256u : 0u);
+    // with 2^14 added in every limb but the top one, the limbs are bit fields
+    const int64_t u = scaled(v, f, bits, cut[q]) + 0x100020004000ll;
     mag[q] = ef[q] ? magnitude(v, f) : 0x7fc0u;
-  }
 #pragma unroll
-  for (int p = 0; p < kDigits; ++p, o += plane) {
-    float f[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      // 2^23 + (d + 128) as binary32 bits, minus 2^23 + 128
-      const int byte = kDigits - 1 - p;
-      const uint32_t m =
-          p == 0 ? (0x4B000000u | top[q])
-                 : __byte_perm(w[q][byte >> 2], 0x4B000000u, 0x7440u | (uint32_t)(byte & 3));
-      f[q] = __uint_as_float(m) - 8388736.0f;
-    }
-    // bf16 holds a digit exactly: the upper halves of the binary32 words
-    *reinterpret_cast<uint2*>(o) =
-        make_uint2(__byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632u),
-                   __byte_perm(__float_as_uint(f[2]), __float_as_uint(f[3]), 0x7632u));
+    for (int i = 0; i < 3; ++i)  // 2^23 + field as binary32 bits, minus 2^23 + 2^14
+      l[q][i] = __uint_as_float(0x4B000000u | ((uint32_t)(u >> (15 * i)) & 0x7fffu)) - 8404992.0f;
+    l[q][3] = __uint_as_float(0x4B000000u | (uint32_t)((int)(u >> 45) + 32768)) - 8421376.0f;
   }
-  *reinterpret_cast<uint2*>(o) = make_uint2(mag[0] | (mag[1] << 16), mag[2] | (mag[3] << 16));
+  residues4<kA, 0>(l, o, plane);
+  *reinterpret_cast<uint2*>(o + kMagPlane * plane) =
+      make_uint2(mag[0] | (mag[1] << 16), mag[2] | (mag[3] << 16));
 }
 
 // Four consecutive elements, zeros from element nv on.
@@ -169,43 +275,40 @@ __device__ __forceinline__ uint32_t max_key(double x) {
 }
 
 // The biased exponent that scales a line with that maximal key: 0 marks a line
-// that the digits cannot hold (NaN, infinite, exponent outside the range).
+// that the integers cannot hold (NaN, infinite, exponent outside the range).
 __device__ __forceinline__ int line_field(uint32_t key) {
   const int E = (int)(key >> 20);
   if (key == 0) return 1022;
   return (E - 1022 < kMinExp || E - 1022 > kMaxExp) ? 0 : E;
 }
 
-// Index of the last digit that a line uses; kNotExact when values are cut.
-__device__ __forceinline__ int last_digit(int field, uint64_t bits, bool cut) {
-  if (field == 0 || cut) return kNotExact;
-  return bits ? kDigits - 1 - (__ffsll((long long)bits) - 1) / 8 : 0;
-}
-
 struct SliceArgs {
   F64Args g;          // operands of this panel
   int64_t kpad;       // panel length rounded up to 64
+  int bits;           // of the integers
   uint16_t* pa;       // planes of [A; acs]: [plane][rows_a][kpad]
   uint16_t* pb;       // planes of [B, bcs]: [plane][kpad][cols_b]
-  int2* a_row;        // {exponent, last digit} per row / column
+  int2* a_row;        // {exponent, kCut / kRefused} per row / column
   int2* b_col;
   uint32_t* cmax;     // [ceil(kpad / 256)][cols_b] maximal keys of 256 rows of B
   int* hdr;           // {status, any bad tile}
   int64_t rows_a, cols_b, row_cs, col_cs;
   int tpr;            // threads per row of A in the maximum pass
+  int rows;           // rows of a slicing CTA
   int64_t n0, n1, n2; // CTAs: A or B data, then their checksums (see the kernels)
 };
 
 constexpr int kSliceThreads = 256;
 constexpr int kMaxRows = 256;     // rows of B per partial maximum
 constexpr int kSliceCols = 256;   // columns and rows of a slicing CTA
-constexpr int kSliceRows = 16;
+constexpr int kSliceRows = 16;    // 4 where 16 would leave SMs idle
 
 // The maximal keys: rows of [A; acs] (tpr threads per row), columns of [B, bcs]
 // (32 columns x 256 rows per CTA).  Two passes over the operands in two launches
 // (here and k_f64_slice) instead of one CTA that walks a strip of columns twice:
-// 512^3 31 -> 21 us, 8192^3 1.60 -> 0.82 ms (the planes are 18 bytes per element,
-// 2.6 GB at 8192^3; with two reads 4.9 GB, 0.72 ms at the copy rate).
+// 512^3 31 -> 21 us, 8192^3 1.60 -> 0.82 ms with nine planes of radix-256 digits.  The
+// 18 planes are 36 bytes per element: 1.07 ms at 8192^3 for 6.3 GB, 0.87 of the copy
+// rate.
 __device__ __forceinline__ void max_rows(const SliceArgs& a, const double* src, int64_t ld,
                                          int64_t rows, int64_t row_out, int64_t blk,
                                          uint32_t* sh) {
@@ -267,7 +370,7 @@ __global__ void __launch_bounds__(kSliceThreads) k_f64_max(const SliceArgs a) {
   max_rows(a, a.g.acs, a.g.ldacs, a.g.R, a.row_cs, b - a.n2, sh);
 }
 
-// The digits of 16 rows x 256 columns of A (one scale per row) or B (one per
+// The residues of a.rows rows x 256 columns of A (one scale per row) or B (one per
 // column): a thread takes four columns of every fourth row.
 template <bool kRowsScaled>
 __device__ __forceinline__ void slice_tile(const SliceArgs& a, const double* src, int64_t ld,
@@ -277,7 +380,7 @@ __device__ __forceinline__ void slice_tile(const SliceArgs& a, const double* src
   const int64_t pw = kRowsScaled ? a.kpad : cdiv(cols, 64) * 64;  // padded columns
   const int64_t ph = kRowsScaled ? rows : a.kpad;                 // padded rows
   const int64_t nbx = cdiv(pw, kSliceCols);
-  const int64_t r0 = blk / nbx * kSliceRows, c0 = blk % nbx * kSliceCols + 4 * tx;
+  const int64_t r0 = blk / nbx * a.rows, c0 = blk % nbx * kSliceCols + 4 * tx;
   const int64_t ldp = kRowsScaled ? a.kpad : a.cols_b;
   const int64_t plane = (kRowsScaled ? a.rows_a : a.kpad) * ldp;
   uint16_t* const out = kRowsScaled ? a.pa : a.pb;
@@ -293,7 +396,6 @@ __device__ __forceinline__ void slice_tile(const SliceArgs& a, const double* src
     __syncthreads();
   }
   int ef[4];
-  uint64_t bits[4] = {0, 0, 0, 0};
   bool cut[4] = {false, false, false, false};
   if constexpr (!kRowsScaled) {
 #pragma unroll
@@ -301,7 +403,7 @@ __device__ __forceinline__ void slice_tile(const SliceArgs& a, const double* src
   }
   const bool in = c0 < pw;
 #pragma unroll 2
-  for (int i = 0; i < kSliceRows / 4; ++i) {
+  for (int i = 0; i < a.rows / 4; ++i) {
     const int64_t r = r0 + ty + 4 * i;
     if (r >= ph) break;  // the whole warp: a row belongs to one
     double x[4] = {0.0, 0.0, 0.0, 0.0};
@@ -312,17 +414,14 @@ __device__ __forceinline__ void slice_tile(const SliceArgs& a, const double* src
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         ef[q] = f;
-        bits[q] = 0;
         cut[q] = false;
       }
     }
-    if (in) slice4(x, ef, out + (prow + r) * ldp + pcol + c0, plane, bits, cut);
+    if (in)
+      slice4<kRowsScaled>(x, ef, a.bits, out + (prow + r) * ldp + pcol + c0, plane, cut);
     if constexpr (kRowsScaled) {
-      const uint64_t b = bits[0] | bits[1] | bits[2] | bits[3];
-      const uint32_t b0 = __reduce_or_sync(0xffffffffu, (uint32_t)b);
-      const uint32_t b1 = __reduce_or_sync(0xffffffffu, (uint32_t)(b >> 32));
       const bool c = __any_sync(0xffffffffu, cut[0] | cut[1] | cut[2] | cut[3]);
-      const int z = last_digit(ef[0], ((uint64_t)b1 << 32) | b0, c);
+      const int z = ef[0] == 0 ? kRefused : (c ? kCut : 0);
       if (lane == 0 && a.a_row[prow + r].y < z) atomicMax(&a.a_row[prow + r].y, z);
     }
   }
@@ -330,7 +429,7 @@ __device__ __forceinline__ void slice_tile(const SliceArgs& a, const double* src
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (c0 + q >= cols) break;
-      const int z = last_digit(ef[q], bits[q], cut[q]);
+      const int z = ef[q] == 0 ? kRefused : (cut[q] ? kCut : 0);
       int2* const at = a.b_col + pcol + c0 + q;
       if (at->y < z) atomicMax(&at->y, z);
     }
@@ -366,8 +465,10 @@ struct ProdArgs {
   const int2* b_col;
   uint8_t* bad;
   int* hdr;                      // {status, any bad tile}
-  int4* scratch;                 // per CTA: [level][chunk][8][256 epilogue threads]
-  float line6, line7;            // magnitudes that levels 0..6 / 0..7 need
+  uint32_t* scratch;             // per CTA: [modulus][chunk][8][256 epilogue threads], four
+                                 // residues of a thread's row each
+  int bits;                      // of the operands' integers
+  float line;                    // the magnitude that an element needs
   uint64_t wait_ns;
   int stall_test;
 };
@@ -388,33 +489,86 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// (H 2^32 + Lo) 2^e rounded to the nearest binary64 (ties to even; the result is
-// a normal number or zero), with integer instructions only.
-__device__ __forceinline__ double round_f64(int64_t H, int64_t Lo, int e) {
-  const int64_t h = H + (Lo >> 32);
-  const uint32_t w = (uint32_t)Lo;
-  const bool neg = h < 0;
-  const uint64_t mh = neg ? ~(uint64_t)h + (w == 0 ? 1ull : 0ull) : (uint64_t)h;
-  const uint32_t ml = neg ? 0u - w : w;
-  if ((mh | ml) == 0) return 0.0;
-  uint64_t top;
-  bool rest = false;
-  int pos;  // position of the leading bit
-  if (mh) {
-    const int z = __clzll((long long)mh);
-    const uint64_t lo64 = (uint64_t)ml << 32;
-    top = z ? (mh << z) | (lo64 >> (64 - z)) : mh;
-    rest = (lo64 << z) != 0;
-    pos = 95 - z;
-  } else {
-    const int z = __clz((int)ml);
-    top = (uint64_t)ml << (32 + z);
-    pos = 31 - z;
+// Byte u of x as a signed number.
+__device__ __forceinline__ int signed_byte(uint32_t x, int u) {
+  return (int)(x << (24 - 8 * u)) >> 24;
+}
+
+// Group j and all later ones: y_j P / (group's product) added to acc, in limbs, and
+// y_j / (group's product) to nf, in 2^-40.
+template <int j>
+__device__ __forceinline__ void add_groups(const uint32_t (&x)[kModuli], int u,
+                                           int64_t (&acc)[4], int64_t& nf) {
+  constexpr int g0 = kM.g[3 * j], g1 = kM.g[3 * j + 1],
+                g2 = 3 * j + 2 < kModuli ? kM.g[3 * j + 2 < kModuli ? 3 * j + 2 : 0] : 0,
+                l0 = kM.limb[j][0], l1 = kM.limb[j][1], l2 = kM.limb[j][2], l3 = kM.limb[j][3],
+                f = kM.frac[j];
+  int y = signed_byte(x[3 * j], u) * g0 + signed_byte(x[3 * j + 1], u) * g1;
+  if constexpr (3 * j + 2 < kModuli) y += signed_byte(x[3 * j + 2], u) * g2;
+  acc[0] += (int64_t)y * l0;
+  acc[1] += (int64_t)y * l1;
+  acc[2] += (int64_t)y * l2;
+  acc[3] += (int64_t)y * l3;
+  nf += (int64_t)y * f;
+  if constexpr (j + 1 < 6) add_groups<j + 1>(x, u, acc, nf);
+}
+
+// C' 2^e rounded to the nearest binary64 (ties to even; the result is a normal
+// number or zero), with C' from its residues: byte u of x[t].  Integer instructions
+// only: y_j of each group of three moduli, n = round(sum_j y_j / (group's product))
+// in 40-bit fixed point (within 1e-4 of the exact sum; 2 |C'| < P keeps it away from
+// a half by far more), C' = sum_j y_j P / (group's product) - n P in 32-bit limbs.
+__device__ __forceinline__ double crt_f64(const uint32_t (&x)[kModuli], int u, int e) {
+  int64_t acc[4] = {0, 0, 0, 0}, nf = 0;
+  add_groups<0>(x, u, acc, nf);
+  const int n = (int)((nf + (1ll << 39)) >> 40);
+  constexpr int P0 = kM.P[0], P1 = kM.P[1], P2 = kM.P[2], P3 = kM.P[3], P4 = kM.P[4];
+  acc[0] -= (int64_t)n * P0;
+  acc[1] -= (int64_t)n * P1;
+  acc[2] -= (int64_t)n * P2;
+  acc[3] -= (int64_t)n * P3;
+  acc[1] += acc[0] >> 32;
+  acc[2] += acc[1] >> 32;
+  acc[3] += acc[2] >> 32;
+  const int top = (int)(acc[3] >> 32) - n * P4;  // the fifth limb
+  uint32_t w[5] = {(uint32_t)acc[0], (uint32_t)acc[1], (uint32_t)acc[2], (uint32_t)acc[3],
+                   (uint32_t)top};
+  const bool neg = top < 0;
+  if (neg) {
+    uint32_t carry = 1;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      w[i] = ~w[i] + carry;
+      carry = carry & (w[i] == 0 ? 1u : 0u);
+    }
   }
-  const uint64_t m = top >> 11;
-  const uint32_t r = (uint32_t)top & 0x7ffu;
-  const uint64_t up = (r > 0x400u || (r == 0x400u && (rest || (m & 1)))) ? 1 : 0;
-  const uint64_t bits = ((uint64_t)(pos + e + 1022) << 52) + m + up;
+  // the leading three words hi, mid, lo (hi: word idx, not zero) and what is below
+  int idx = 4;
+  uint32_t hi = w[4], mid = w[3], lo = w[2], rest = w[0] | w[1];
+#pragma unroll
+  for (int i = 1; i >= 0; --i)
+    if (hi == 0) {
+      hi = mid;
+      mid = lo;
+      lo = w[i];
+      rest = i == 1 ? w[0] : 0u;
+      --idx;
+    }
+  if (hi == 0) {  // below 2^64
+    if ((mid | lo) == 0) return 0.0;
+    idx = mid ? 1 : 0;
+    hi = mid ? mid : lo;
+    mid = idx ? lo : 0u;
+    lo = 0u;
+  }
+  const int z = __clz((int)hi);
+  const uint64_t t64 =
+      ((uint64_t)__funnelshift_l(mid, hi, z) << 32) | __funnelshift_l(lo, mid, z);
+  const uint64_t m = t64 >> 11;
+  const uint32_t r = (uint32_t)t64 & 0x7ffu;
+  const bool below = ((lo << z) | rest) != 0;
+  const uint64_t up = (r > 0x400u || (r == 0x400u && (below || (m & 1)))) ? 1 : 0;
+  const uint64_t bits = ((uint64_t)(32 * idx + 31 - z + e + 1022) << 52) + m + up;
   return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
@@ -449,9 +603,6 @@ __device__ __forceinline__ TileView64 view_tile(const ProdArgs& p, int64_t t, in
   return V;
 }
 
-// What a tile's magnitudes ask for.
-constexpr int kNeed7 = 1, kLeave = 2;
-
 template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_f64_tc(const __grid_constant__ Maps M, const ProdArgs p) {
@@ -465,17 +616,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int rank = kPair ? (int)tc::cluster_ctarank() : 0;
   const bool issuer = rank == 0;  // its MMA warp issues for both CTAs of a pair
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NS * stage);
-  // full [8], empty [8], tmem full [2], tmem empty [2], drain, decision
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 6);
+  // full [8], empty [8], tmem full [2], tmem empty [2], drain
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 5);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* need = reinterpret_cast<volatile int*>(tmem_slot + 2);  // [2][kWarpsAll]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   auto full = [&](int s) { return tc::smem_addr(&bars[s]); };
   auto empty = [&](int s) { return tc::smem_addr(&bars[kMaxStages + s]); };
   auto tfull = [&](int a) { return tc::smem_addr(&bars[2 * kMaxStages + a]); };
   auto tempty = [&](int a) { return tc::smem_addr(&bars[2 * kMaxStages + 2 + a]); };
   const uint32_t drain = tc::smem_addr(&bars[2 * kMaxStages + 4]);
-  const uint32_t decided = tc::smem_addr(&bars[2 * kMaxStages + 5]);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -487,7 +636,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc::mbar_init(tempty(a), kWarpsAll);
     }
     tc::mbar_init(drain, 1);
-    tc::mbar_init(decided, kWarpsAll);
     *abort = 0;
     tc::wait_limit_ns() = p.wait_ns;
     tc::fence_barrier_init();
@@ -515,35 +663,25 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int64_t tfirst = kPair ? (int64_t)tc::cluster_id() : (int64_t)blockIdx.x;
   const int64_t tstep = kPair ? (int64_t)tc::num_clusters() : (int64_t)gridDim.x;
   const int nkb = p.nkb;
-  // the tile's decision, known to every role before its level 7 (phase: tile parity)
-  auto decision = [&](uint32_t par) {
-    int f = 0;
-    for (int w = 0; w < kWarpsAll; ++w) f |= need[par * kWarpsAll + w];
-    return f;
-  };
-  auto wait_decided = [&](uint32_t par) {
-    return kPair ? tc::wait_cluster(decided, par, abort) : tc::wait(decided, par, abort);
-  };
-  auto last_level = [](int f) { return (f & kNeed7) && !(f & kLeave) ? 7 : 6; };
-
   if (warp == 0 || warp == kWarpProdB) {
     if (tc::elect_one()) {
       const bool pA = warp == 0;
       int s = 0;
-      uint32_t ph = 0, par = 0;
+      uint32_t ph = 0;
       int64_t issued = 0;
       bool ok = true;
-      for (int64_t t = tfirst; t < total && ok && !*abort; t += tstep, par ^= 1) {
+      for (int64_t t = tfirst; t < total && ok && !*abort; t += tstep) {
         if (p.stall_test && t == 0) continue;
         const TileView64 V = view_tile<kPair>(p, t, rank);
         // a pair's bytes (both CTAs') land on the issuer's barrier, which the
         // issuer's producers expect
         const uint32_t tx = (pA ? kABytes : (uint32_t)V.nbox * kBoxBytes) * (kPair ? 2 : 1);
-        // one pair of planes: nkb k-steps
-        auto pair = [&](int pa, int pb) {
-          const int arow = pa * p.rows_a + V.arow, brow = pb * p.kpad;
+        // a plane of A and of B: the magnitudes, then the residues
+        for (int i = 0; i < kPlanes64 && ok; ++i) {
+          const int plane = i == 0 ? kMagPlane : i - 1;
+          const int arow = plane * p.rows_a + V.arow, brow = plane * p.kpad;
           for (int kb = 0; kb < nkb; ++kb) {
-            if (!tc::wait(empty(s), ph ^ 1, abort)) return false;
+            if (!tc::wait(empty(s), ph ^ 1, abort)) { ok = false; break; }
             const uint32_t sa = tc::smem_addr(smem + s * stage);
             if (issuer) tc::mbar_arrive_expect_tx(full(s), tx);
             const uint32_t fb = kPair ? tc::mapa(full(s), 0) : full(s);
@@ -570,16 +708,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             ++issued;
             if (++s == NS) { s = 0; ph ^= 1; }
           }
-          return true;
-        };
-        ok = pair(kMagPlane, kMagPlane);
-        int top = 6;
-        for (int lev = 0; lev <= top && ok; ++lev) {
-          for (int i = 0; i <= lev && ok; ++i) ok = pair(i, lev - i);
-          if (lev == 6 && ok) {
-            ok = wait_decided(par);
-            if (ok) top = last_level(decision(par));
-          }
         }
       }
       // no copies left in flight (bounded): a pair's complete on the issuer's
@@ -596,9 +724,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     if (issuer && tc::elect_one()) {
       int s = 0, acc = 0;
-      uint32_t ph = 0, aph = 0, par = 0;
+      uint32_t ph = 0, aph = 0;
       bool ok = true;
-      for (int64_t t = tfirst; t < total && ok && !*abort; t += tstep, par ^= 1) {
+      for (int64_t t = tfirst; t < total && ok && !*abort; t += tstep) {
         const TileView64 V = view_tile<kPair>(p, t, rank);
         const uint32_t idesc = tc::idesc_bf16(kPair ? 2 * BM : BM, V.nmma, 1);
         // nk k-steps in accumulators of g each
@@ -622,15 +750,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           return true;
         };
-        ok = level(nkb, nkb);
-        int top = 6;
-        for (int lev = 0; lev <= top && ok; ++lev) {
-          ok = level((lev + 1) * nkb, kGroupSteps);
-          if (lev == 6 && ok) {
-            ok = wait_decided(par);
-            if (ok) top = last_level(decision(par));
-          }
-        }
+        ok = level(nkb, nkb);  // magnitudes
+        for (int i = 0; i < kModuli && ok; ++i) ok = level(nkb, kGroupSteps);
       }
       // every MMA has completed before TMEM is freed
       if constexpr (kPair)
@@ -646,9 +767,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     // epilogue: TMEM lane quarter q = warp % 4, column half (warp - 2) / 4
     const int q = warp & 3, half = (warp - 2) >> 2, ew = warp - 2, et = ew * 32 + lane;
     const int nch = p.bpt, c_lo = half * 32 * nch;  // 32-column chunks per warp
-    int4* const scr = p.scratch + (int64_t)blockIdx.x * kLevels * nch * 8 * 256 + et;
+    uint32_t* const scr = p.scratch + (int64_t)blockIdx.x * kModuli * nch * 8 * 256 + et;
     int acc = 0;
-    uint32_t aph = 0, par = 0;
+    uint32_t aph = 0;
     bool ok = true;
     const uint32_t lanes = (uint32_t)(q * 32) << 16;
     // the same answer in every lane, and the warp converged after it
@@ -666,64 +787,48 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (++acc == 2) { acc = 0; aph ^= 1; }
     };
-    for (int64_t t = tfirst; t < total && ok; t += tstep, par ^= 1) {
+    for (int64_t t = tfirst; t < total && ok; t += tstep) {
       const TileView64 V = view_tile<kPair>(p, t, rank);
       const int64_t row = V.row0 + 32 * q + lane;
       const bool rv = row < V.rlim;
       const int2 ri = rv ? p.a_row[V.arow + 32 * q + lane] : make_int2(0, 0);
       const int c_hi = min(c_lo + 32 * nch, V.ncols);  // this warp's valid columns
-      // ---- magnitudes: what the tile needs
-      int zr = ri.y, zc = 0;
-      for (int c = c_lo + lane; c < c_hi; c += 32) zc = max(zc, p.b_col[V.bcol + c].y);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        zr = max(zr, __shfl_xor_sync(0xffffffffu, zr, o));
-        zc = max(zc, __shfl_xor_sync(0xffffffffu, zc, o));
-      }
+      // ---- magnitudes: the chunks with an element below the line are left out
       if (!wait_all(tfull(acc), aph)) { ok = false; break; }
       tc::fence_after_sync();
-      int f = 0;
-      for (int c = c_lo; c < c_hi; c += 16) {
-        float v[16];
-        tmem_ld16(tmem + lanes + acc * 256 + c, v);
+      const bool cut_rows = __any_sync(0xffffffffu, ri.y != 0);
+      uint32_t leave = 0;  // bit ci: chunk ci
+      for (int ci = 0; ci < nch; ++ci) {
+        const int c = c_lo + 32 * ci;
+        if (c >= c_hi) break;
+        const bool cut =
+            cut_rows | __any_sync(0xffffffffu, c + lane < c_hi && p.b_col[V.bcol + c + lane].y != 0);
+        bool low = false;
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          if (rv && c + u < c_hi && v[u] != 0.0f) {  // NaN: neither line is reached
-            if (!(v[u] >= p.line6)) f |= kNeed7;
-            if (!(v[u] >= p.line7)) f |= kLeave;
-          }
+        for (int h = 0; h < 2; ++h) {
+          float v[16];
+          tmem_ld16(tmem + lanes + acc * 256 + c + 16 * h, v);
+#pragma unroll
+          for (int u = 0; u < 16; ++u)  // NaN is below the line
+            low |= c + 16 * h + u < c_hi && v[u] != 0.0f && !(v[u] >= p.line);
         }
+        // zero: every term is zero; nothing cut: the integers are exact
+        if (__any_sync(0xffffffffu, low && rv) && cut) leave |= 1u << ci;
       }
       release();
-      if (zr + zc <= 6) f = 0;               // no digit product is cut
-      else if (zr + zc <= 7) f = f ? kNeed7 : 0;
-      f = (__any_sync(0xffffffffu, f & kNeed7) ? kNeed7 : 0) |
-          (__any_sync(0xffffffffu, f & kLeave) ? kLeave : 0);
-      // every warp of the tile tells every CTA of it
-      if (lane == 0) {
-        if constexpr (kPair) {
-          const uint32_t at = tc::smem_addr(const_cast<int*>(&need[par * kWarpsAll])) +
-                              4 * (rank * kEpiWarps + ew);
-          for (int r = 0; r < 2; ++r) {
-            tc::st_cluster(tc::mapa(at, r), (uint32_t)f);
-            tc::mbar_arrive_cluster(tc::mapa(decided, r));
-          }
-        } else {
-          need[par * kWarpsAll + ew] = f;
-          tc::mbar_arrive(decided);
-        }
-      }
-      // ---- levels
-      int top = 6;
-      f = 0;
-      for (int lev = 0; lev <= top && ok; ++lev) {
-        int sum[4][32];
+      if (lane < nch)
+        p.bad[((t * (kPair ? 8 : 4)) + 4 * rank + q) * (2 * p.bpt) + half * nch + lane] =
+            (uint8_t)((leave >> lane) & 1);
+      if (leave && lane == 0) atomicExch(&p.hdr[1], 1);
+      // ---- residues
+      for (int t = 0; t < kModuli; ++t) {
+        const float pm = kModulus.m[t].x, inv = kModulus.m[t].y;
+        float sum[4][32];
 #pragma unroll
         for (int ci = 0; ci < 4; ++ci)
 #pragma unroll
-          for (int u = 0; u < 32; ++u) sum[ci][u] = 0;
-        const int nk = (lev + 1) * nkb;
-        for (int k0 = 0; k0 < nk; k0 += kGroupSteps) {
+          for (int u = 0; u < 32; ++u) sum[ci][u] = 0.0f;
+        for (int k0 = 0; k0 < nkb; k0 += kGroupSteps) {
           if (!wait_all(tfull(acc), aph)) { ok = false; break; }
           tc::fence_after_sync();
           const uint32_t base = tmem + lanes + acc * 256 + c_lo;
@@ -735,7 +840,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 float v[16];
                 tmem_ld16(base + 32 * ci + 16 * h, v);
 #pragma unroll
-                for (int u = 0; u < 16; ++u) sum[ci][16 * h + u] += __float2int_rn(v[u]);
+                for (int u = 0; u < 16; ++u) sum[ci][16 * h + u] += residue(v[u], pm, inv);
               }
             }
           }
@@ -746,47 +851,40 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int ci = 0; ci < 4; ++ci)
           if (ci < nch && c_lo + 32 * ci < c_hi) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-              scr[(int64_t)((lev * nch + ci) * 8 + j) * 256] =
-                  make_int4(sum[ci][4 * j], sum[ci][4 * j + 1], sum[ci][4 * j + 2],
-                            sum[ci][4 * j + 3]);
+            for (int j = 0; j < 8; ++j) {
+              uint32_t r[4];  // the residue is the low byte
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                r[u] = __float_as_uint(residue(sum[ci][4 * j + u], pm, inv) + kRound);
+              scr[(int64_t)((t * nch + ci) * 8 + j) * 256] = __byte_perm(
+                  __byte_perm(r[0], r[1], 0x0040u), __byte_perm(r[2], r[3], 0x0040u), 0x5410u);
+            }
           }
-        if (lev == 6) {
-          ok = __all_sync(0xffffffffu, wait_decided(par)) != 0;
-          if (ok) {
-            f = decision(par);
-            top = last_level(f);
-          }
-        }
       }
       if (!ok) break;
-      if (issuer && ew == 0 && lane == 0) {
-        p.bad[t] = (f & kLeave) ? 1 : 0;
-        if (f & kLeave) atomicExch(&p.hdr[1], 1);
-      }
-      const int c_end = !(f & kLeave) && rv ? c_hi : 0;
-      // ---- the levels together, rounded once
+      // ---- the residues together, rounded once; the next four columns' residues are
+      // in flight while these are put together
       double* const dst = (V.cs_row ? p.g.E : (V.cs_col ? p.g.F : p.g.C)) +
                           row * (V.cs_row ? p.g.lde : (V.cs_col ? p.g.ldf : p.g.ldc)) + V.col0;
-#pragma unroll 1
-      for (int cj = 0; cj < 8 * nch; ++cj) {
-        const int c = c_lo + 4 * cj;
-        if (c >= c_end) break;
-        int L[kLevels][4];
+      const int ncj = (min(c_hi, c_lo + 32 * nch) - c_lo + 3) / 4;  // groups of four columns
+      uint32_t x[kModuli], y[kModuli];
+      auto fetch = [&](int cj) {
 #pragma unroll
-        for (int s = 0; s < kLevels; ++s) {
-          const int4 x = s <= top ? scr[(int64_t)(s * nch * 8 + cj) * 256] : make_int4(0, 0, 0, 0);
-          L[s][0] = x.x; L[s][1] = x.y; L[s][2] = x.z; L[s][3] = x.w;
-        }
+        for (int t = 0; t < kModuli; ++t) y[t] = scr[(int64_t)(t * nch * 8 + cj) * 256];
+      };
+      if (ncj > 0) fetch(0);
+#pragma unroll 1
+      for (int cj = 0; cj < ncj; ++cj) {
+#pragma unroll
+        for (int t = 0; t < kModuli; ++t) x[t] = y[t];
+        if (cj + 1 < ncj) fetch(cj + 1);
+        if (!rv || ((leave >> (cj >> 3)) & 1)) continue;
+        const int c = c_lo + 4 * cj;
         double o[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int64_t H = ((int64_t)L[0][u] << 24) + ((int64_t)L[1][u] << 16) +
-                            ((int64_t)L[2][u] << 8) + L[3][u];
-          const int64_t Lo = ((int64_t)L[4][u] << 24) + ((int64_t)L[5][u] << 16) +
-                             ((int64_t)L[6][u] << 8) + L[7][u];
           const int eb = c + u < c_hi ? p.b_col[V.bcol + c + u].x : 0;
-          o[u] = round_f64(H, Lo, ri.x + eb - 70);
+          o[u] = crt_f64(x, u, ri.x + eb - 2 * p.bits);
         }
         double* const d = dst + c;
         if (p.g.accumulate) {
@@ -836,14 +934,16 @@ TileGrid tile_grid(int64_t m, int64_t n, int64_t R, int64_t Cc, int bpt, bool pa
 }  // namespace
 
 bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, size_t* bytes) {
-  // Below 128^3 both paths are bound by their launches and latencies.
+  // 128^3: 136 us on the FP64 pipe (one 64 x 64 tile's chain of k), 59 here; below,
+  // both are bound by latency and the FP64 pipe needs one launch instead of four
+  // (1024 x 1024 x 64: 134 and 64 us, 100000 x 3 x 300: 3.34 and 0.65 ms).
   if (d.k < 1 || (double)d.m * (double)d.n * (double)d.k < 2097152.0) return false;
   F64TcRegions& r = *rg;
   r.row_cs = cdiv(d.m, 2 * BM) * 2 * BM;
   r.rows_a = r.row_cs + cdiv(R, 2 * BM) * 2 * BM;
   r.col_cs = cdiv(d.n, 256) * 256;
   r.cols_b = r.col_cs + cdiv(Cc, 256) * 256;
-  // Panels of K: a level sum stays within 32 bits, the planes within a budget.
+  // Panels of K: the planes stay within a budget.
   const int64_t per_k = (r.rows_a + r.cols_b) * kPlanes64 * 2;
   const int64_t fit = (int64_t)(kPlaneBudget / per_k) / BK * BK;
   r.kp = std::min<int64_t>({cdiv(d.k, BK) * BK, kMaxPanel, std::max<int64_t>(fit, BK)});
@@ -851,9 +951,9 @@ bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, si
   // (L2 delivers about 75 bytes per clock and SM; a k-step of four, two, one boxes
   // is 48, 32, 24 KiB: 640, 420, 360 clocks at 4096^3, where the MMAs take 512,
   // 256, 192); a pair's CTAs copy 32 KiB per 512-clock k-step (590).  Whole steps
-  // with pairs / four / two / one boxes: 512^3 292 / 300 / 248 / 234 us, 1000 x 1501
-  // x 777 374 / 381 / 301 / 376, 2048 chain 1.68 / 1.42 / 1.56 / 2.04 ms, 4096^3
-  // 4.09 / 4.21 / 4.45 / 6.52, 8192^3 encode + product 26.1 / 27.5 / 36.2 / 46.0:
+  // with pairs / four / two / one boxes: 512^3 241 / 237 / 190 / 170 us, 1000 x 1501
+  // x 777 313 / 327 / 265 / 300, 2048 chain 1.32 / 1.16 / 1.25 / 1.58 ms, 4096^3
+  // 3.03 / 3.11 / 3.24 / 4.61, 8192^3 encode + product 16.7 / 17.0 / 19.8 / 28.4:
   // the rule takes the best of each.
   struct Kind {
     int bpt;
@@ -884,8 +984,8 @@ bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, si
   r.a_row = region(sizeof(int2) * r.rows_a);
   r.b_col = region(sizeof(int2) * r.cols_b);
   r.cmax = region(sizeof(uint32_t) * cdiv(r.kp, kMaxRows) * r.cols_b);
-  r.bad = region((size_t)tiles);
-  r.scratch = region((size_t)ctas * kLevels * r.bpt * 8 * 256 * sizeof(int4));
+  r.bad = region((size_t)tiles * (r.pair ? 8 : 4) * 2 * r.bpt);
+  r.scratch = region((size_t)ctas * kModuli * r.bpt * 8 * 256 * sizeof(uint32_t));
   *bytes = off;
   return true;
 }
@@ -914,6 +1014,9 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     SliceArgs a{};
     a.g = gp;
     a.kpad = kpad;
+    // 2 k 2^(2 bits) < P
+    const int bits = std::min(kMaxBits, (int)floor((kLog2P - 1 - log2((double)gp.k)) / 2));
+    a.bits = bits;
     a.pa = reinterpret_cast<uint16_t*>(w + r.a_planes);
     a.pb = reinterpret_cast<uint16_t*>(w + r.b_planes);
     a.a_row = reinterpret_cast<int2*>(w + r.a_row);
@@ -930,8 +1033,10 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     a.n2 = cdiv(g.m, rpc);
     k_f64_max<<<(unsigned)(a.n0 + a.n1 + a.n2 + cdiv(g.R, rpc)), kSliceThreads, 0, st>>>(a);
     auto tiles = [&](int64_t rows, int64_t cols) {
-      return cdiv(rows, kSliceRows) * cdiv(cdiv(cols, BK) * BK, kSliceCols);
+      return cdiv(rows, a.rows) * cdiv(cdiv(cols, BK) * BK, kSliceCols);
     };
+    a.rows = kSliceRows;
+    if (tiles(kpad, g.n) + tiles(g.m, kpad) < 8 * num_sms()) a.rows = 4;
     a.n0 = tiles(kpad, g.n);
     a.n1 = tiles(kpad, g.Cc);
     a.n2 = tiles(g.m, kpad);
@@ -956,9 +1061,9 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     p.b_col = a.b_col;
     p.bad = reinterpret_cast<uint8_t*>(w + r.bad);
     p.hdr = hdr;
-    p.scratch = reinterpret_cast<int4*>(w + r.scratch);
-    p.line6 = (float)(0.405 * sqrt((double)gp.k));
-    p.line7 = (float)(0.0016 * sqrt((double)gp.k));
+    p.scratch = reinterpret_cast<uint32_t*>(w + r.scratch);
+    p.bits = bits;
+    p.line = (float)(1.52 * ldexp(1.0, 53 - bits) * sqrt((double)gp.k));
     p.stall_test = stall && stall[0] == '1';
     p.wait_ns = p.stall_test ? 200000000ull : tc::kWaitLimitNs;
     const int workers = r.pair ? pair_clusters(reinterpret_cast<const void*>(kernel), smem)

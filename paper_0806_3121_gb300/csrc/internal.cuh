@@ -73,14 +73,14 @@ struct Erased {
   int32_t bi[kMaxErased], bj[kMaxErased];
 };
 
-// Workspace regions of the sliced binary64 product (gemm_f64_tc.cu), byte
+// Workspace regions of the binary64 product on the tensor cores (gemm_f64_tc.cu), byte
 // offsets from Plan::f64tc_base.
 struct F64TcRegions {
-  size_t a_planes, b_planes;  // bf16 digit planes of [A; acs] and [B, bcs], one panel of K
-  size_t a_row, b_col;        // int2 {exponent, last digit used} per row / column
+  size_t a_planes, b_planes;  // bf16 residue planes of [A; acs] and [B, bcs], one panel of K
+  size_t a_row, b_col;        // int2 {exponent, cut or refused} per row / column
   size_t cmax;                // maximal keys of 256 rows of each column of [B, bcs]
-  size_t bad;                 // one byte per tile: left to the DFMA kernel
-  size_t scratch;             // per CTA: the level sums of its tile
+  size_t bad;                 // one byte per 32 x 32 chunk: left to the DFMA kernel
+  size_t scratch;             // per CTA: the residues of its tile
   int64_t kp;                 // longest panel of K
   int64_t rows_a, cols_b;     // padded rows of [A; acs], columns of [B, bcs]
   int64_t row_cs, col_cs;     // first padded checksum row / column
@@ -103,7 +103,7 @@ struct Plan {
   // sums over column groups of g = min(vb_cols, 128) columns.
   int fused;
   int64_t g, ngrp, ntr_obs;
-  // Binary64: the product runs sliced on the tensor cores when a workspace is
+  // Binary64: the product runs on the tensor cores when a workspace is
   // given; f64tc_hdr: its {status, any tile left to DFMA} words
   int tc64;
   F64TcRegions f64tc;
@@ -147,7 +147,7 @@ int num_sms();
 // run at once on the current device.
 int pair_clusters(const void* kernel, size_t smem);
 
-// Whether the binary64 product of d runs sliced on the tensor cores, and its
+// Whether the binary64 product of d runs on the tensor cores, and its
 // workspace regions.
 bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, size_t* bytes);
 

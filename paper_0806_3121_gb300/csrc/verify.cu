@@ -52,7 +52,7 @@ struct CheckArgs {
   // DFMA product): when that product timed out, C is incomplete and nothing is
   // located or corrected
   const int32_t* timeout;
-  // sliced binary64 product: the counter that the host reads it from (its own
+  // binary64 product on the tensor cores: the counter that the host reads it from (its own
   // word lies outside the scratch)
   int32_t* status_out;
 };

@@ -1,12 +1,13 @@
-"""The sliced binary64 product on the tensor cores (abft_gemm / abft_gemm_plain with a
+"""The binary64 product on the tensor cores (abft_gemm / abft_gemm_plain with a
 workspace) against the exact product of sampled rows and columns in extended precision.
 
 Tolerance: elementwise 2 k u (|A||B|), u = 2^-53, the rounding bound of any order of k
-multiply-adds.  The sliced product meets it by construction: where levels 0..6 are used,
-the digit products left out are at most 8.1 2^-56 per term in units of the row and column
-scales, and |A||B| is at least 0.405 sqrt(k) in those units, so the error is at most
-2.6 sqrt(k) u (|A||B|).  Its Frobenius error is also at most that of the DFMA kernel (the
-same call without a workspace) or one rounding."""
+multiply-adds.  The product meets it by construction: the operands are rounded at most
+2^-(b+1) of their row's and column's scale (b = 58 or 59), so a term errs by at most
+2^-b + 2^-2b in those units, and an element is only taken where |A||B| is at least
+1.52 2^(53-b) sqrt(k) of them: the error is at most 0.7 sqrt(k) u (|A||B|).  Its Frobenius
+error is also at most that of the DFMA kernel (the same call without a workspace) or one
+rounding."""
 import numpy as np
 import pytest
 
@@ -45,9 +46,9 @@ def operands(kind, m, n, k):
     elif kind == "sparse":
         A *= r.random((m, k)) < 0.01
         B *= r.random((k, n)) < 0.01
-    elif kind == "digits":   # every digit is -128: the accumulators reach 2^24
+    elif kind == "equal":    # one value everywhere: residues add up with one sign
         A[:] = B[:] = -(128 * (256 ** 8 - 1) // 255) / 2.0 ** 63
-    elif kind == "wide":     # exponents outside the range of the digits' scales
+    elif kind == "wide":     # exponents outside the range of the lines' scales
         A *= 10.0 ** r.uniform(-200, -100, (m, 1))
     elif kind == "zero":
         A[::2] = 0
@@ -93,9 +94,9 @@ def check(A, B, C, C0=None):
 
 
 # edges of the 128-row tiles, the 64-column boxes, the 64-wide k-steps, the 1024-term
-# accumulators and the 16320-wide panels; one, two and four boxes per tile
+# accumulators and the 16320-wide panels; one, two and four boxes per tile, CTA pairs
 SHAPES = [(128, 128, 128), (129, 127, 129), (1, 2500, 1000), (300, 3, 3000), (257, 65, 1023),
-          (127, 193, 1025), (640, 2600, 64), (2000, 2100, 100), (130, 200, 16321)]
+          (127, 193, 1025), (640, 2600, 64), (2000, 2100, 100), (130, 200, 16321), (2800, 3000, 130)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
@@ -107,7 +108,7 @@ def test_edges(shape):
     assert np.array_equal(product(A, B, pad=1)[0], A @ B)
 
 
-@pytest.mark.parametrize("kind", ["rows", "graded", "outlier", "eye", "sparse", "digits", "wide",
+@pytest.mark.parametrize("kind", ["rows", "graded", "outlier", "eye", "sparse", "equal", "wide",
                                   "zero"])
 def test_operand_kinds(kind):
     A, B = operands(kind, 300, 330, 1100)
