@@ -63,6 +63,43 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// Two binary32 values in one 64-bit register pair and their packed arithmetic (each
+// half rounded to nearest as the scalar instruction): the streaming passes are bound
+// by instruction issue (issue active 64 - 75 % with DRAM at 28 - 53 %), and a packed
+// instruction does two elements.
+struct F2 {
+  uint64_t v;
+};
+__device__ __forceinline__ F2 pack2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(F2 x) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(x.v));
+  return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ float sum2(F2 x) {
+  const float2 f = unpack2(x);
+  return f.x + f.y;
+}
+
 __device__ __forceinline__ float warp_sumf(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -125,14 +162,11 @@ __device__ __forceinline__ uint4 load8raw(const __nv_bfloat16* row, int64_t c, i
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-__device__ __forceinline__ void unpack8(const uint4& u, float (&v)[8]) {
-  const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+__device__ __forceinline__ void unpack8(const uint4& u, F2 (&v)[4]) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const float2 f = __bfloat1622float2(h[q]);
-    v[2 * q] = f.x;
-    v[2 * q + 1] = f.y;
-  }
+  for (int q = 0; q < 4; ++q)
+    v[q] = pack2(__uint_as_float(w[q] << 16), __uint_as_float(w[q] & 0xffff0000u));
 }
 
 __device__ __forceinline__ void store8(__nv_bfloat16* dst, const __nv_bfloat16 (&v)[8]) {
@@ -149,24 +183,43 @@ __device__ __forceinline__ void store8(__nv_bfloat16* dst, const __nv_bfloat16 (
 // checksum pieces and norm partials.
 // A lane's 8 consecutive floats to shared memory as two 16-byte stores (dst
 // 16-byte aligned).
-__device__ __forceinline__ void st_shared8(float* dst, const float (&v)[8]) {
-  reinterpret_cast<float4*>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
-  reinterpret_cast<float4*>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
+__device__ __forceinline__ void st_shared8(float* dst, const F2 (&v)[4]) {
+  const float2 a = unpack2(v[0]), b = unpack2(v[1]), c = unpack2(v[2]), d = unpack2(v[3]);
+  reinterpret_cast<float4*>(dst)[0] = make_float4(a.x, a.y, b.x, b.y);
+  reinterpret_cast<float4*>(dst)[1] = make_float4(c.x, c.y, d.x, d.y);
 }
 
-__device__ __forceinline__ void lpA_rows(const float (&v)[8], int t, float sc, float (&se)[8],
-                                         float (&sw)[8], float& sq) {
+__device__ __forceinline__ void lpA_rows(const F2 (&v)[4], int t, float sc, F2 (&se)[4],
+                                         F2 (&sw)[4], float& sq) {
+  const float w = (float)(t + 1) * sc;
+  const F2 w2 = pack2(w, w);
+  F2 s2 = mul2(v[0], v[0]);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    se[q] = add2(se[q], v[q]);
+    sw[q] = fma2(w2, v[q], sw[q]);
+    if (q > 0) s2 = fma2(v[q], v[q], s2);
+  }
+  sq = sum2(s2);
+}
+
+// The same from scalar values (e4m3: the conversions leave them in single registers,
+// and packing them first made the passes 8 - 20 % slower).
+__device__ __forceinline__ void lpA_rows(const float (&v)[8], int t, float sc, F2 (&se)[4],
+                                         F2 (&sw)[4], float& sq) {
   const float w = (float)(t + 1) * sc;
   sq = 0.f;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    se[q] += v[q];
-    sw[q] = fmaf(w, v[q], sw[q]);
-    sq = fmaf(v[q], v[q], sq);
+  for (int q = 0; q < 4; ++q) {
+    const float a = v[2 * q], b = v[2 * q + 1];
+    const float2 e = unpack2(se[q]), x = unpack2(sw[q]);
+    se[q] = pack2(e.x + a, e.y + b);
+    sw[q] = pack2(fmaf(w, a, x.x), fmaf(w, b, x.y));
+    sq = fmaf(b, b, fmaf(a, a, sq));
   }
 }
 
-__device__ __forceinline__ void lpA_finish(const float (&se)[8], const float (&sw)[8],
+__device__ __forceinline__ void lpA_finish(const F2 (&se)[4], const F2 (&sw)[4],
                                            __nv_bfloat16* __restrict__ acs, int64_t ldk,
                                            double* __restrict__ part, int64_t nchr, int64_t cx,
                                            int64_t I, float* red, float* sh) {
@@ -197,11 +250,21 @@ __device__ __forceinline__ void lpA_finish(const float (&se)[8], const float (&s
     q0 = te * te;
     q1 = tw * tw;
   }
-  const float t0 = block_sumf(q0, sh);
-  if (threadIdx.x == 0) part[(2 * I) * nchr + cx] = (double)t0;
-  const float t1 = block_sumf(q1, sh);
-  if (threadIdx.x == 0) part[(2 * I + 1) * nchr + cx] = (double)t1;
-  __syncthreads();  // red is reused by the next unit
+  // both norm partials behind one barrier, after which red may be written again
+  // (sh is written again only behind the next unit's first barrier)
+  q0 = warp_sumf(q0);
+  q1 = warp_sumf(q1);
+  if (lane == 0) {
+    sh[warp] = q0;
+    sh[kEncWarps + warp] = q1;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < kEncWarps; ++w) t += sh[threadIdx.x * kEncWarps + w];
+    part[(2 * I + threadIdx.x) * nchr + cx] = (double)t;
+  }
 }
 
 // One unit with register loads (any alignment): kRowBatch rows of loads in
@@ -218,9 +281,9 @@ __device__ __forceinline__ void lpA_unit(const __nv_bfloat16* __restrict__ A, in
   const int64_t i0 = I * vb, i1 = min(i0 + (int64_t)vb, m);
   const int nrow = (int)(i1 - i0);
   const __nv_bfloat16* Ab = A + i0 * lda;
-  float se[8], sw[8];
+  F2 se[4], sw[4];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) se[q] = sw[q] = 0.f;
+  for (int q = 0; q < 4; ++q) se[q] = sw[q] = pack2(0.f, 0.f);
   constexpr int kLanesPerRow = 32 / kRowBatch;
   for (int rb = warp; rb < nrow; rb += kEncWarps * kRowBatch) {
     uint4 raw[kRowBatch];
@@ -232,7 +295,7 @@ __device__ __forceinline__ void lpA_unit(const __nv_bfloat16* __restrict__ A, in
     float sq[kRowBatch];
 #pragma unroll
     for (int r = 0; r < kRowBatch; ++r) {
-      float v[8];
+      F2 v[4];
       unpack8(raw[r], v);
       lpA_rows(v, rb + kEncWarps * r, sc, se, sw, sq[r]);
     }
@@ -249,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_lpA_cols(const __nv_bfloat16* _
                                                        int64_t ldk, float* __restrict__ rowpart,
                                                        int64_t nchr, double* __restrict__ part) {
   __shared__ __align__(16) float red[kEncWarps * kEncCols * 2];
-  __shared__ float sh[kThreads / 32];
+  __shared__ float sh[2 * kEncWarps];
   const int64_t nvb = cdiv(m, vb);
   for (int64_t I = blockIdx.y; I < nvb; I += gridDim.y)
     lpA_unit(A, lda, m, k, vb, e, acs, ldk, rowpart, nchr, part, blockIdx.x, I, red, sh);
@@ -283,7 +346,7 @@ __global__ void __launch_bounds__(kThreads) k_lpA_block(const __nv_bfloat16* __r
 // (chunk cx) x 128 rows (chunk ry): lane = 8 consecutive columns, warp w = rows
 // l0 + w + 8 t; the warps' column squares and block partials meet in shared
 // memory (red: [8][256] floats, redq: [8][32][2] floats) in lpB_finish.
-__device__ __forceinline__ void lpB_finish(const float (&cs)[8], float q0, float q1, int64_t n,
+__device__ __forceinline__ void lpB_finish(const F2 (&cs)[4], float q0, float q1, int64_t n,
                                            int vb, float* __restrict__ colpart,
                                            double* __restrict__ part, int64_t nch, int64_t cx,
                                            int64_t ry, float* red, float* redq) {
@@ -313,15 +376,32 @@ __device__ __forceinline__ void lpB_finish(const float (&cs)[8], float q0, float
 
 // One row of B in a lane's 8 columns: its (e, w) partial sums (reduced over
 // the verify block by the caller) and the column squares.
-__device__ __forceinline__ void lpB_row(const float (&v)[8], const float (&wq)[8], float (&cs)[8],
+__device__ __forceinline__ void lpB_row(const F2 (&v)[4], const F2 (&wq)[4], F2 (&cs)[4],
+                                        float& se, float& sw) {
+  F2 e = v[0], w = mul2(wq[0], v[0]);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (q > 0) {
+      e = add2(e, v[q]);
+      w = fma2(wq[q], v[q], w);
+    }
+    cs[q] = fma2(v[q], v[q], cs[q]);
+  }
+  se = sum2(e);
+  sw = sum2(w);
+}
+
+__device__ __forceinline__ void lpB_row(const float (&v)[8], const F2 (&wq)[4], F2 (&cs)[4],
                                         float& se, float& sw) {
   se = 0.f;
   sw = 0.f;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    se += v[q];
-    sw = fmaf(wq[q], v[q], sw);
-    cs[q] = fmaf(v[q], v[q], cs[q]);
+  for (int q = 0; q < 4; ++q) {
+    const float a = v[2 * q], b = v[2 * q + 1];
+    const float2 w = unpack2(wq[q]), c = unpack2(cs[q]);
+    se = (se + a) + b;
+    sw = fmaf(w.y, b, fmaf(w.x, a, sw));
+    cs[q] = pack2(fmaf(a, a, c.x), fmaf(b, b, c.y));
   }
 }
 
@@ -358,12 +438,13 @@ __device__ __forceinline__ void lpB_unit(const __nv_bfloat16* __restrict__ B, in
   const bool leader = (lane % seg) == 0 && c0 < n;
   const int64_t J = c0 / vb;
   const float sc = scalbnf(1.0f, -e);
-  float wq[8];
+  F2 wq[4], cs[4];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) wq[q] = (float)((int)((c0 + q) % vb) + 1) * sc;
-  float cs[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) cs[q] = 0.f;
+  for (int q = 0; q < 4; ++q) {  // a verify block holds a lane's 8 columns
+    const int w = (int)((c0 + 2 * q) % vb) + 1;
+    wq[q] = pack2((float)w * sc, (float)(w + 1) * sc);
+    cs[q] = pack2(0.f, 0.f);
+  }
   float q0 = 0.f, q1 = 0.f;
   const int nrow = (int)(l1 - l0);
   const __nv_bfloat16* Bb = B + l0 * ldb;
@@ -377,7 +458,8 @@ __device__ __forceinline__ void lpB_unit(const __nv_bfloat16* __restrict__ B, in
 #pragma unroll
     for (int r = 0; r < kRowBatchB; ++r) {
       const int64_t l = l0 + rb + kEncWarps * r;
-      float v[8], se, sw;
+      F2 v[4];
+      float se, sw;
       unpack8(raw[r], v);
       lpB_row(v, wq, cs, se, sw);
       lpB_store_shfl(se, sw, seg, leader, l < l1, bcs + l * ldcs + 4 * J, q0, q1);
@@ -731,28 +813,38 @@ struct F8Batch {
 // dequantised with their block scale, and their bf16 values written to the
 // operand plane.
 template <bool kF8>
+struct Row8;  // a lane's eight values of a row
+template <>
+struct Row8<false> {
+  F2 v[4];
+};
+template <>
+struct Row8<true> {
+  float v[8];
+};
+template <bool kF8>
 __device__ __forceinline__ void ring_row(const typename Ring<kF8>::Slot& raw, const Fp8Src& f8,
                                          const F8Batch* fb, int r, bool valid, int64_t c0,
-                                         int64_t cols, float (&v)[8], bool& bad) {
+                                         int64_t cols, Row8<kF8>& v, bool& bad) {
   if constexpr (kF8) {
     const bool in = valid && c0 < cols;
     const int64_t si = fb->sidx + (fb->rin + kEncWarps * r >= 128 ? f8.sld : 0);
     const float scl = in ? f8.sc[si] : 0.f;
     __nv_bfloat16 o[8];
-    dequant8(raw.x, raw.y, scl, c0 + 8 <= cols, c0, cols, v, o);
+    dequant8(raw.x, raw.y, scl, c0 + 8 <= cols, c0, cols, v.v, o);
     // a value that is not exact in bf16 (scale not a power of two in range)
     // or a NaN code (bytes past cols are zero-filled by the copy)
     bad |= in && (!scale_exact(scl) || nan_code4(raw.x) || nan_code4(raw.y));
     if (valid && c0 < f8.pld) store8(fb->plane + (int64_t)(kEncWarps * r) * f8.pld, o);
   } else {
-    unpack8(raw, v);
+    unpack8(raw, v.v);
   }
 }
 
 template <class Units, bool kF8>
 __global__ void __launch_bounds__(kThreads, 2) k_encA_stream(const Units U, const Fp8Src f8) {
   __shared__ __align__(16) float red[kEncWarps * kEncCols * 2];
-  __shared__ float sh[kThreads / 32];
+  __shared__ float sh[2 * kEncWarps];
   using R = Ring<kF8>;
   extern __shared__ uint4 ring_s[];  // R::kBytes
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -771,9 +863,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_encA_stream(const Units U, cons
     const RowSrc src = rows_of(X);
     const int nbat = warp_batches(src.nrow, warp);
     const float sc = scalbnf(1.0f, -X.e);
-    float se[8], sw[8];
+    F2 se[4], sw[4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) se[q] = sw[q] = 0.f;
+    for (int q = 0; q < 4; ++q) se[q] = sw[q] = pack2(0.f, 0.f);
     for (int b = 0; b < nbat; ++b) {
       cp_async_wait<R::kBatches - 1>();  // this warp's oldest batch has landed
       const typename R::Slot* slot = ring + (consumed % R::kBatches) * kRowBatch * 32;
@@ -784,9 +876,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_encA_stream(const Units U, cons
 #pragma unroll
       for (int r = 0; r < kRowBatch; ++r) {
         const int t = tb + kEncWarps * r;
-        float v[8];
+        Row8<kF8> v;
         ring_row<kF8>(slot[r * 32 + lane], f8, &fb, r, t < src.nrow, c0, src.cols, v, bad);
-        lpA_rows(v, t, sc, se, sw, sq[r]);
+        lpA_rows(v.v, t, sc, se, sw, sq[r]);
       }
       ++consumed;
       is.next();  // refills the slot just read (each lane reads only its own copies)
@@ -828,11 +920,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_encB_stream(const Units U, cons
     const bool leader = (lane % seg) == 0 && c0 < X.n;
     const int64_t J = c0 / X.vb;
     const float sc = scalbnf(1.0f, -X.e);
-    float wq[8], cs[8];
+    F2 wq[4], cs[4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      wq[q] = (float)((int)((c0 + q) % X.vb) + 1) * sc;
-      cs[q] = 0.f;
+    for (int q = 0; q < 4; ++q) {
+      const int w = (int)((c0 + 2 * q) % X.vb) + 1;
+      wq[q] = pack2((float)w * sc, (float)(w + 1) * sc);
+      cs[q] = pack2(0.f, 0.f);
     }
     float q0 = 0.f, q1 = 0.f;
     for (int b = 0; b < nbat; ++b) {
@@ -848,11 +941,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_encB_stream(const Units U, cons
 #pragma unroll
         for (int r = 0; r < kRowBatch; ++r) {
           const int t = tb + kEncWarps * r;
-          float v[8];
+          Row8<kF8> v;
           ring_row<kF8>(slot[r * 32 + lane], f8, &fb, r, t < src.nrow, c0, X.n, v, bad);
           if constexpr (kF8)
             if (wbt) bt_store_row(tileT, t, lane, slot[r * 32 + lane]);
-          lpB_row(v, wq, cs, sums[2 * r], sums[2 * r + 1]);
+          lpB_row(v.v, wq, cs, sums[2 * r], sums[2 * r + 1]);
         }
         ++consumed;
         is.next();
@@ -874,11 +967,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_encB_stream(const Units U, cons
 #pragma unroll
         for (int r = 0; r < kRowBatch; ++r) {
           const int t = tb + kEncWarps * r;
-          float v[8], se, sw;
+          Row8<kF8> v;
+          float se, sw;
           ring_row<kF8>(slot[r * 32 + lane], f8, &fb, r, t < src.nrow, c0, X.n, v, bad);
           if constexpr (kF8)
             if (wbt) bt_store_row(tileT, t, lane, slot[r * 32 + lane]);
-          lpB_row(v, wq, cs, se, sw);
+          lpB_row(v.v, wq, cs, se, sw);
           lpB_store_shfl(se, sw, seg, leader, t < src.nrow, X.bcs + (l0 + t) * X.ldcs + 4 * J,
                          q0, q1);
         }
