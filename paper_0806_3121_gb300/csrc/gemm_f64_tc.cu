@@ -467,6 +467,7 @@ struct ProdArgs {
   int* hdr;                      // {status, any bad tile}
   uint32_t* scratch;             // per CTA: [modulus][chunk][8][256 epilogue threads], four
                                  // residues of a thread's row each
+  int split;                     // CTAs that share a tile's planes
   int bits;                      // of the operands' integers
   float line;                    // the magnitude that an element needs
   uint64_t wait_ns;
@@ -603,7 +604,11 @@ __device__ __forceinline__ TileView64 view_tile(const ProdArgs& p, int64_t t, in
   return V;
 }
 
-template <bool kPair>
+// kSplit: the planes of a tile (magnitudes, then the moduli) are dealt to the p.split
+// CTAs of a cluster, each takes them like a whole tile, the residues meet in the
+// cluster's scratch and every CTA puts a share of the columns together: a small
+// product then occupies p.split times as many SMs.
+template <bool kPair, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_f64_tc(const __grid_constant__ Maps M, const ProdArgs p) {
   extern __shared__ uint8_t smem_raw[];
@@ -613,11 +618,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int NS = stages(boxes);
   const uint32_t stage = kABytes + boxes * kBoxBytes;
   constexpr int kWarpsAll = kPair ? 2 * kEpiWarps : kEpiWarps;  // epilogue warps of a tile
+  static_assert(!(kPair && kSplit), "pairs do not split");
   const int rank = kPair ? (int)tc::cluster_ctarank() : 0;
+  const int part = kSplit ? (int)tc::cluster_ctarank() : 0, nparts = kSplit ? p.split : 1;
+  const int plane0 = kPlanes64 * part / nparts, plane1 = kPlanes64 * (part + 1) / nparts;
   const bool issuer = rank == 0;  // its MMA warp issues for both CTAs of a pair
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NS * stage);
-  // full [8], empty [8], tmem full [2], tmem empty [2], drain
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 5);
+  // full [8], empty [8], tmem full [2], tmem empty [2], drain, residues done
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 6);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   auto full = [&](int s) { return tc::smem_addr(&bars[s]); };
@@ -625,6 +633,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   auto tfull = [&](int a) { return tc::smem_addr(&bars[2 * kMaxStages + a]); };
   auto tempty = [&](int a) { return tc::smem_addr(&bars[2 * kMaxStages + 2 + a]); };
   const uint32_t drain = tc::smem_addr(&bars[2 * kMaxStages + 4]);
+  const uint32_t done = tc::smem_addr(&bars[2 * kMaxStages + 5]);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -636,6 +645,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc::mbar_init(tempty(a), kWarpsAll);
     }
     tc::mbar_init(drain, 1);
+    tc::mbar_init(done, kEpiWarps * nparts);
     *abort = 0;
     tc::wait_limit_ns() = p.wait_ns;
     tc::fence_barrier_init();
@@ -653,15 +663,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   tc::fence_before_sync();
-  if constexpr (kPair)
+  if constexpr (kPair || kSplit)
     tc::cluster_sync();
   else
     __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tmem_slot;
   const int64_t total = p.T.total();
-  const int64_t tfirst = kPair ? (int64_t)tc::cluster_id() : (int64_t)blockIdx.x;
-  const int64_t tstep = kPair ? (int64_t)tc::num_clusters() : (int64_t)gridDim.x;
+  constexpr bool kCluster = kPair || kSplit;
+  const int64_t tfirst = kCluster ? (int64_t)tc::cluster_id() : (int64_t)blockIdx.x;
+  const int64_t tstep = kCluster ? (int64_t)tc::num_clusters() : (int64_t)gridDim.x;
   const int nkb = p.nkb;
   if (warp == 0 || warp == kWarpProdB) {
     if (tc::elect_one()) {
@@ -677,7 +688,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // issuer's producers expect
         const uint32_t tx = (pA ? kABytes : (uint32_t)V.nbox * kBoxBytes) * (kPair ? 2 : 1);
         // a plane of A and of B: the magnitudes, then the residues
-        for (int i = 0; i < kPlanes64 && ok; ++i) {
+        for (int i = plane0; i < plane1 && ok; ++i) {
           const int plane = i == 0 ? kMagPlane : i - 1;
           const int arow = plane * p.rows_a + V.arow, brow = plane * p.kpad;
           for (int kb = 0; kb < nkb; ++kb) {
@@ -750,8 +761,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           return true;
         };
-        ok = level(nkb, nkb);  // magnitudes
-        for (int i = 0; i < kModuli && ok; ++i) ok = level(nkb, kGroupSteps);
+        for (int i = plane0; i < plane1 && ok; ++i)
+          ok = level(nkb, i == 0 ? nkb : kGroupSteps);  // magnitudes: one accumulator
       }
       // every MMA has completed before TMEM is freed
       if constexpr (kPair)
@@ -767,7 +778,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     // epilogue: TMEM lane quarter q = warp % 4, column half (warp - 2) / 4
     const int q = warp & 3, half = (warp - 2) >> 2, ew = warp - 2, et = ew * 32 + lane;
     const int nch = p.bpt, c_lo = half * 32 * nch;  // 32-column chunks per warp
-    uint32_t* const scr = p.scratch + (int64_t)blockIdx.x * kModuli * nch * 8 * 256 + et;
+    // a cluster's scratch alternates between two slots (one while others still read the
+    // other)
+    const int64_t slot = (int64_t)kModuli * nch * 8 * 256;
+    uint32_t* scr = p.scratch + (kSplit ? 2 * tfirst : (int64_t)blockIdx.x) * slot + et;
+    uint32_t par = 0;
     int acc = 0;
     uint32_t aph = 0;
     bool ok = true;
@@ -794,34 +809,36 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int2 ri = rv ? p.a_row[V.arow + 32 * q + lane] : make_int2(0, 0);
       const int c_hi = min(c_lo + 32 * nch, V.ncols);  // this warp's valid columns
       // ---- magnitudes: the chunks with an element below the line are left out
-      if (!wait_all(tfull(acc), aph)) { ok = false; break; }
-      tc::fence_after_sync();
-      const bool cut_rows = __any_sync(0xffffffffu, ri.y != 0);
+      uint8_t* const bad =
+          p.bad + (t * (kPair ? 8 : 4) + 4 * rank + q) * (2 * p.bpt) + half * nch;
       uint32_t leave = 0;  // bit ci: chunk ci
-      for (int ci = 0; ci < nch; ++ci) {
-        const int c = c_lo + 32 * ci;
-        if (c >= c_hi) break;
-        const bool cut =
-            cut_rows | __any_sync(0xffffffffu, c + lane < c_hi && p.b_col[V.bcol + c + lane].y != 0);
-        bool low = false;
+      if (plane0 == 0) {
+        if (!wait_all(tfull(acc), aph)) { ok = false; break; }
+        tc::fence_after_sync();
+        const bool cut_rows = __any_sync(0xffffffffu, ri.y != 0);
+        for (int ci = 0; ci < nch; ++ci) {
+          const int c = c_lo + 32 * ci;
+          if (c >= c_hi) break;
+          const bool cut = cut_rows | __any_sync(0xffffffffu, c + lane < c_hi &&
+                                                                  p.b_col[V.bcol + c + lane].y != 0);
+          bool low = false;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float v[16];
-          tmem_ld16(tmem + lanes + acc * 256 + c + 16 * h, v);
+          for (int h = 0; h < 2; ++h) {
+            float v[16];
+            tmem_ld16(tmem + lanes + acc * 256 + c + 16 * h, v);
 #pragma unroll
-          for (int u = 0; u < 16; ++u)  // NaN is below the line
-            low |= c + 16 * h + u < c_hi && v[u] != 0.0f && !(v[u] >= p.line);
+            for (int u = 0; u < 16; ++u)  // NaN is below the line
+              low |= c + 16 * h + u < c_hi && v[u] != 0.0f && !(v[u] >= p.line);
+          }
+          // zero: every term is zero; nothing cut: the integers are exact
+          if (__any_sync(0xffffffffu, low && rv) && cut) leave |= 1u << ci;
         }
-        // zero: every term is zero; nothing cut: the integers are exact
-        if (__any_sync(0xffffffffu, low && rv) && cut) leave |= 1u << ci;
+        release();
+        if (lane < nch) bad[lane] = (uint8_t)((leave >> lane) & 1);
+        if (leave && lane == 0) atomicExch(&p.hdr[1], 1);
       }
-      release();
-      if (lane < nch)
-        p.bad[((t * (kPair ? 8 : 4)) + 4 * rank + q) * (2 * p.bpt) + half * nch + lane] =
-            (uint8_t)((leave >> lane) & 1);
-      if (leave && lane == 0) atomicExch(&p.hdr[1], 1);
       // ---- residues
-      for (int t = 0; t < kModuli; ++t) {
+      for (int t = max(plane0, 1) - 1; t < plane1 - 1; ++t) {
         const float pm = kModulus.m[t].x, inv = kModulus.m[t].y;
         float sum[4][32];
 #pragma unroll
@@ -862,19 +879,29 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
       }
       if (!ok) break;
+      if constexpr (kSplit) {  // every CTA's residues and the left-out chunks are written
+        __syncwarp();
+        if (lane == 0) {
+          __threadfence();
+          for (int r = 0; r < nparts; ++r) tc::mbar_arrive_cluster(tc::mapa(done, r));
+        }
+        if (!__all_sync(0xffffffffu, tc::wait_cluster(done, par, abort))) { ok = false; break; }
+        leave = __ballot_sync(0xffffffffu, lane < nch && __ldcg(&bad[lane]) != 0);
+      }
       // ---- the residues together, rounded once; the next four columns' residues are
       // in flight while these are put together
       double* const dst = (V.cs_row ? p.g.E : (V.cs_col ? p.g.F : p.g.C)) +
                           row * (V.cs_row ? p.g.lde : (V.cs_col ? p.g.ldf : p.g.ldc)) + V.col0;
-      const int ncj = (min(c_hi, c_lo + 32 * nch) - c_lo + 3) / 4;  // groups of four columns
+      const int ncj0 = (min(c_hi, c_lo + 32 * nch) - c_lo + 3) / 4;  // groups of four columns
+      const int first = ncj0 * part / nparts, ncj = ncj0 * (part + 1) / nparts;
       uint32_t x[kModuli], y[kModuli];
       auto fetch = [&](int cj) {
 #pragma unroll
-        for (int t = 0; t < kModuli; ++t) y[t] = scr[(int64_t)(t * nch * 8 + cj) * 256];
+        for (int t = 0; t < kModuli; ++t) y[t] = __ldcg(&scr[(int64_t)(t * nch * 8 + cj) * 256]);
       };
-      if (ncj > 0) fetch(0);
+      if (first < ncj) fetch(first);
 #pragma unroll 1
-      for (int cj = 0; cj < ncj; ++cj) {
+      for (int cj = first; cj < ncj; ++cj) {
 #pragma unroll
         for (int t = 0; t < kModuli; ++t) x[t] = y[t];
         if (cj + 1 < ncj) fetch(cj + 1);
@@ -902,13 +929,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       __syncwarp();
+      if constexpr (kSplit) {
+        scr += par ? -slot : slot;
+        par ^= 1;
+      }
     }
   }
 
   tc::fence_before_sync();
-  // a pair: neither CTA frees TMEM or exits while the other may still signal its
-  // barriers or the issuer's MMAs read its shared memory
-  if constexpr (kPair)
+  // a cluster: no CTA frees TMEM or exits while another may still signal its barriers
+  // or (pairs) the issuer's MMAs read its shared memory
+  if constexpr (kCluster)
     tc::cluster_sync();
   else
     __syncthreads();
@@ -933,6 +964,12 @@ TileGrid tile_grid(int64_t m, int64_t n, int64_t R, int64_t Cc, int bpt, bool pa
 
 }  // namespace
 
+// Clusters of `split` CTAs that run at once (of six: 23, since a cluster stays within a
+// GPC; the others with the same margin).
+static int64_t split_workers(int split) {
+  return split == 1 ? kSms : (split == 2 ? 74 : (split == 3 ? 46 : 22));
+}
+
 bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, size_t* bytes) {
   // 128^3: 136 us on the FP64 pipe (one 64 x 64 tile's chain of k), 59 here; below,
   // both are bound by latency and the FP64 pipe needs one launch instead of four
@@ -955,22 +992,34 @@ bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, si
   // x 777 313 / 327 / 265 / 300, 2048 chain 1.32 / 1.16 / 1.25 / 1.58 ms, 4096^3
   // 3.03 / 3.11 / 3.24 / 4.61, 8192^3 encode + product 16.7 / 17.0 / 19.8 / 28.4:
   // the rule takes the best of each.
+  // Few tiles leave SMs idle: their planes are split over clusters of 2, 3 or 6 CTAs
+  // (the residues are put together in about 8000 clocks per box).  512^3 step with one /
+  // two / three / six CTAs per tile of one box 171 / 157 / 149 / 156 us, of two boxes 193 /
+  // 164 / 158 / 155; 1000 x 1501 x 777 with two boxes 259 / 261 / 273 / 281, four 322 / 250 /
+  // 275 / 266.
   struct Kind {
     int bpt;
     bool pair;
     int clocks;
   };
   const Kind kinds[] = {{4, true, 590}, {4, false, 640}, {2, false, 420}, {1, false, 360}};
+  const int64_t nkb = cdiv(std::min(d.k, r.kp), BK);
   double best = 0;
-  for (const Kind& kd : kinds) {
-    const int64_t t = tile_grid(d.m, d.n, R, Cc, kd.bpt, kd.pair).total();
-    const double cost = (double)kd.clocks * cdiv(t, kd.pair ? kSms / 2 : kSms);
-    if (best == 0 || cost < best) {
-      best = cost;
-      r.bpt = kd.bpt;
-      r.pair = kd.pair;
+  for (const Kind& kd : kinds)
+    for (int split : {1, 2, 3, 6}) {
+      if (kd.pair && split > 1) continue;
+      const int64_t t = tile_grid(d.m, d.n, R, Cc, kd.bpt, kd.pair).total();
+      const int64_t workers = kd.pair ? kSms / 2 : split_workers(split);
+      if (split > 1 && t > workers) continue;
+      const double cost = ((double)kd.clocks * nkb * kPlanes64 + 8000.0 * kd.bpt) / split *
+                          cdiv(t, workers);
+      if (best == 0 || cost < best) {
+        best = cost;
+        r.bpt = kd.bpt;
+        r.pair = kd.pair;
+        r.split = split;
+      }
     }
-  }
   const int64_t tiles = tile_grid(d.m, d.n, R, Cc, r.bpt, r.pair).total();
   const int64_t ctas = std::min<int64_t>(r.pair ? 2 * tiles : tiles, kSms);
   size_t off = 0;
@@ -985,7 +1034,8 @@ bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, si
   r.b_col = region(sizeof(int2) * r.cols_b);
   r.cmax = region(sizeof(uint32_t) * cdiv(r.kp, kMaxRows) * r.cols_b);
   r.bad = region((size_t)tiles * (r.pair ? 8 : 4) * 2 * r.bpt);
-  r.scratch = region((size_t)ctas * kModuli * r.bpt * 8 * 256 * sizeof(uint32_t));
+  r.scratch = region((size_t)ctas * (r.split > 1 ? 2 : 1) * kModuli * r.bpt * 8 * 256 *
+                     sizeof(uint32_t));
   *bytes = off;
   return true;
 }
@@ -996,7 +1046,9 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
   int* hdr = reinterpret_cast<int*>(static_cast<char*>(ws) + P.f64tc_hdr);
   const TileGrid T = tile_grid(g.m, g.n, g.R, g.Cc, r.bpt, r.pair);
   const char* stall = getenv("ABFT_TEST_STALL_PRODUCER");
-  const auto kernel = r.pair ? k_gemm_f64_tc<true> : k_gemm_f64_tc<false>;
+  const auto kernel = r.pair      ? k_gemm_f64_tc<true, false>
+                      : r.split > 1 ? k_gemm_f64_tc<false, true>
+                                    : k_gemm_f64_tc<false, false>;
   const int boxes = cta_boxes(r.bpt, r.pair);
   const size_t smem = smem_bytes(boxes);
   cudaError_t e =
@@ -1066,21 +1118,23 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     p.line = (float)(1.52 * ldexp(1.0, 53 - bits) * sqrt((double)gp.k));
     p.stall_test = stall && stall[0] == '1';
     p.wait_ns = p.stall_test ? 200000000ull : tc::kWaitLimitNs;
-    const int workers = r.pair ? pair_clusters(reinterpret_cast<const void*>(kernel), smem)
-                               : num_sms();
+    const int per = r.pair ? 2 : r.split;  // CTAs per worker
+    const int workers =
+        per > 1 ? max_clusters(reinterpret_cast<const void*>(kernel), smem, per, kThreads)
+                : num_sms();
+    p.split = r.split;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.x = per;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    const unsigned per = r.pair ? 2 : 1;  // CTAs per worker
     cfg.gridDim =
-        dim3(per * (unsigned)std::min<int64_t>({T.total(), kSms / per, workers}), 1, 1);
+        dim3((unsigned)(per * std::min<int64_t>({T.total(), kSms / per, workers})), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = at;
-    cfg.numAttrs = r.pair ? 1 : 0;
+    cfg.numAttrs = per > 1 ? 1 : 0;
     if ((e = cudaLaunchKernelEx(&cfg, kernel, M, p)) != cudaSuccess) break;
     e = launch_gemm_f64_bad(gp, T, r.pair ? 4 : 2, r.bpt, hdr + 1, p.bad, st);
     count_launches(3);

@@ -32,6 +32,7 @@
 
 #include <stdlib.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "internal.cuh"
@@ -1546,31 +1547,33 @@ int num_sms() {
   return g_num_sms[dev];
 }
 
-// CTA pairs (clusters of two) of a pair-tile kernel that fit on the GPU at
-// once: the persistent grid's size.  Clusters are placed within a GPC, so this
-// can be less than half the SM count.
-static int g_pair_clusters[64] = {};
-int pair_clusters(const void* kernel, size_t smem) {
+// Clusters are placed within a GPC, so fewer than num_sms() / size may fit: the
+// persistent grid's size.  Looked up once per device and size (every caller's CTA
+// fills an SM).
+static std::atomic<int> g_max_clusters[64][9];
+int max_clusters(const void* kernel, size_t smem, int size, int threads) {
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && g_pair_clusters[dev]) return g_pair_clusters[dev];
+  std::atomic<int>* const kept =
+      dev >= 0 && dev < 64 && size >= 1 && size <= 8 ? &g_max_clusters[dev][size] : nullptr;
+  if (kept && kept->load(std::memory_order_relaxed)) return kept->load(std::memory_order_relaxed);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.x = size;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(2 * (num_sms() / 2), 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.gridDim = dim3(size * (num_sms() / size), 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) {
     cudaGetLastError();
-    n = num_sms() / 2;
+    n = std::max(1, num_sms() / size / 2);
   }
-  if (dev >= 0 && dev < 64) g_pair_clusters[dev] = n;
+  if (kept) kept->store(n, std::memory_order_relaxed);
   return n;
 }
 
@@ -1683,7 +1686,8 @@ cudaError_t launch_gemm_bf16(const Plan& P, const TcOperands& op, float* C, void
   if (e != cudaSuccess) return e;
   // tile workers: CTAs, or CTA pairs
   const int workers = (int)std::min<int64_t>(
-      g.t_total, pair ? pair_clusters(reinterpret_cast<const void*>(kernel), smem) : num_sms());
+      g.t_total, pair ? max_clusters(reinterpret_cast<const void*>(kernel), smem, 2, kThreads)
+                      : num_sms());
   if (workers == 0) return cudaSuccess;
   if (g.f8) g.cs_stride = cs_stride(g.t_total - g.t_data, g.t_total, workers);  // 1 unless set
   e = cudaMemsetAsync(status, 0, sizeof(int), st);  // the status of this product

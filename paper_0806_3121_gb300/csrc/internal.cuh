@@ -86,6 +86,7 @@ struct F64TcRegions {
   int64_t row_cs, col_cs;     // first padded checksum row / column
   int bpt;                    // 64-column boxes per tile
   bool pair;                  // 256-row tiles on CTA pairs
+  int split;                  // CTAs of a cluster that share a tile's planes
 };
 
 // Everything the device code needs to know about one problem.
@@ -143,9 +144,9 @@ __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 
 
 // Multiprocessors of the current device.
 int num_sms();
-// CTA pairs (clusters of two) of a kernel with `smem` dynamic shared memory that
-// run at once on the current device.
-int pair_clusters(const void* kernel, size_t smem);
+// Clusters of `size` CTAs (of `threads` threads and `smem` bytes of dynamic shared
+// memory, one CTA per SM) of a kernel that run at once on the current device.
+int max_clusters(const void* kernel, size_t smem, int size, int threads);
 
 // Whether the binary64 product of d runs on the tensor cores, and its
 // workspace regions.
