@@ -12,8 +12,9 @@
 // cost as much as the squares).  The passes read A three times and B twice, which
 // HBM has room for.  Small problems are bound by latency instead: a verify block's
 // rows are split into 64-row segments over the warps of a CTA and eight rows of
-// loads are in flight per thread.  Measured (all launches of an encode): see
-// kEncodeTimes below.
+// loads are in flight per thread.  Measured, both launches against the eight kernels
+// before them: 512^3 902 -> 21 us, 2048^3 557 -> 66, 4096^3 on an 8 x 8 grid 1152 -> 252,
+// 8192^3 on a 16 x 16 grid 2604 -> 935 (FP64 pipe: 850).
 
 #include <algorithm>
 
@@ -32,19 +33,6 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// Sum of v over the 256 threads of the block; valid in thread 0.
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int q = 0; q < kWarps; ++q) t += sh[q];
-  return t;
 }
 
 struct EncArgs {
@@ -261,11 +249,25 @@ __global__ void __launch_bounds__(kThreads) k_enc64(const EncArgs a) {
 // Threshold norms, one CTA per verify block: nblk[4I] = sqrt(sum_{t in I} v_t^2),
 // nblk[4I+1] = sqrt(sum (w_t v_t)^2) with v the line norms of the block, and
 // nblk[4I+2], nblk[4I+3] the norms of its two checksum vectors.  CTAs 0 .. nvr-1:
-// row blocks of A; then the column blocks of B, which also write the column
-// norms nBcol from their partial squares.
-__global__ void __launch_bounds__(kThreads) k_enc64_norms(const EncArgs a, double* nAblk,
-                                                          double* nBcol, double* nBblk) {
-  __shared__ double sh[kWarps];
+// row blocks of A; then the column blocks of B; then the column norms nBcol from their
+// partial squares, 512 columns per CTA (a square root is some twenty instructions of
+// the FP64 pipe, 16 clocks each per warp, so they are spread over CTAs of their own).
+constexpr int kNormThreads = 512;
+__global__ void __launch_bounds__(kNormThreads) k_enc64_norms(const EncArgs a, double* nAblk,
+                                                              double* nBcol, double* nBblk) {
+  __shared__ double sh[4][kNormThreads / 32];
+  const int64_t nch = cdiv(a.k, kSqRows);
+  auto column_square = [&](int64_t j) {
+    double v = 0.0;
+#pragma unroll 8
+    for (int64_t c = 0; c < nch; ++c) v += a.colsq[c * a.n + j];
+    return v;
+  };
+  if (blockIdx.x >= a.nvr + a.nvc) {
+    const int64_t j = (blockIdx.x - a.nvr - a.nvc) * kNormThreads + threadIdx.x;
+    if (j < a.n) nBcol[j] = sqrt(column_square(j));
+    return;
+  }
   const bool rows = blockIdx.x < a.nvr;
   const int64_t I = rows ? blockIdx.x : blockIdx.x - a.nvr;
   const int vb = rows ? a.vb_r : a.vb_c;
@@ -273,23 +275,8 @@ __global__ void __launch_bounds__(kThreads) k_enc64_norms(const EncArgs a, doubl
   const int len = (int)(min(t0 + (int64_t)vb, rows ? a.m : a.n) - t0);
   const double sc = scalbn(1.0, rows ? -a.er : -a.ec);
   double s[4] = {0.0, 0.0, 0.0, 0.0};
-  const int64_t nch = cdiv(a.k, kSqRows);
-  for (int t = threadIdx.x; t < len; t += kThreads) {
-    double v2 = 0.0;
-    if (rows) {
-      const double v = a.nArow[t0 + t];
-      v2 = v * v;
-    } else {
-#pragma unroll 8
-      for (int64_t c = 0; c < nch; ++c) v2 += a.colsq[c * a.n + t0 + t];
-      nBcol[t0 + t] = sqrt(v2);
-    }
-    const double w = (double)(t + 1) * sc;
-    s[0] += v2;
-    s[1] = fma(w * w, v2, s[1]);
-  }
 #pragma unroll 4
-  for (int64_t l = threadIdx.x; l < a.k; l += kThreads) {
+  for (int64_t l = threadIdx.x; l < a.k; l += kNormThreads) {
     double e, w;
     if (rows) {
       e = a.acs[(2 * I) * a.k + l];
@@ -302,11 +289,37 @@ __global__ void __launch_bounds__(kThreads) k_enc64_norms(const EncArgs a, doubl
     s[2] = fma(e, e, s[2]);
     s[3] = fma(w, w, s[3]);
   }
-  double* out = (rows ? nAblk : nBblk) + 4 * I;
+  for (int t = threadIdx.x; t < len; t += kNormThreads) {
+    double v2;
+    if (rows) {
+      const double v = a.nArow[t0 + t];
+      v2 = v * v;
+    } else {
+      v2 = column_square(t0 + t);
+    }
+    const double w = (double)(t + 1) * sc;
+    s[0] += v2;
+    s[1] = fma(w * w, v2, s[1]);
+  }
+  // the four sums together, in a transposing butterfly (lane l: sum l / 8), the warps'
+  // in shared memory, one warp per sum
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    const double t = block_sum(s[c], sh);
-    if (threadIdx.x == 0) out[c] = sqrt(t);
+  for (int o = 16, h = 2; h >= 1; o >>= 1, h >>= 1) {
+    const bool upper = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double send = upper ? s[i] : s[i + h];
+      s[i] = (upper ? s[i + h] : s[i]) + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (int o = 4; o >= 1; o >>= 1) s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+  if ((lane & 7) == 0) sh[lane >> 3][warp] = s[0];
+  __syncthreads();
+  if (warp < 4) {
+    const double t = warp_sum(lane < kNormThreads / 32 ? sh[warp][lane] : 0.0);
+    if (lane == 0) ((rows ? nAblk : nBblk) + 4 * I)[warp] = sqrt(t);
   }
 }
 
@@ -387,8 +400,8 @@ cudaError_t encode_f64_into(const Plan& P, const double* A, const double* B, voi
   a.n_arows = cdiv(d.m, kWarps);
   k_enc64<<<(unsigned)(a.n_acols + a.n_brows + a.n_ablk + a.n_bsq + a.n_arows), kThreads, 0, st>>>(
       a);
-  k_enc64_norms<<<(unsigned)(P.nvr + P.nvc), kThreads, 0, st>>>(a, at(P.L.nAblk), at(P.L.nBcol),
-                                                                at(P.L.nBblk));
+  k_enc64_norms<<<(unsigned)(P.nvr + P.nvc + cdiv(d.n, kNormThreads)), kNormThreads, 0, st>>>(
+      a, at(P.L.nAblk), at(P.L.nBcol), at(P.L.nBblk));
   count_launches(2);
   return cudaGetLastError();
 }

@@ -117,12 +117,25 @@ __device__ __forceinline__ double fma_t<double>(double a, double b, double c) { 
 template <>
 __device__ __forceinline__ float fma_t<float>(float a, float b, float c) { return fmaf(a, b, c); }
 
+// 1 for NaN and infinities, from the exponent bits (a binary64 comparison would take
+// another slot of the FP64 pipe per element).
+__device__ __forceinline__ int nonfinite(double x) {
+  return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000 ? 1 : 0;
+}
+__device__ __forceinline__ int nonfinite(float x) {
+  return (__float_as_int(x) & 0x7f800000) == 0x7f800000 ? 1 : 0;
+}
+
 template <typename TC>
 __device__ __forceinline__ TC warp_sum_t(TC v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+
+// Loads a lane has in flight when one warp walks a line (locate and correct are bound
+// by latency: a few warps of one CTA).
+constexpr int kLineLoads = 8;
 
 // Residuals of column line (I, j), computed by one warp (lanes split the rows;
 // sums in the element type, then added across the lanes); residuals and
@@ -137,11 +150,17 @@ __device__ int col_line_warp(const CheckArgs& a, int64_t I, int64_t j, double& r
   TC se = 0, sw = 0;
   int nf = 0;
   const int len = (int)(i1 - i0);
-  for (int t = lane; t < len; t += 32) {
-    const TC x = C[(i0 + t) * a.ldc + j];
-    se += x;
-    sw = fma_t<TC>((TC)(t + 1) * sc, x, sw);
-    nf += isfinite(x) ? 0 : 1;
+  for (int t0 = lane; t0 < len; t0 += 32 * kLineLoads) {
+    TC x[kLineLoads];
+#pragma unroll
+    for (int r = 0; r < kLineLoads; ++r)
+      x[r] = t0 + 32 * r < len ? C[(i0 + t0 + 32 * r) * a.ldc + j] : (TC)0;
+#pragma unroll
+    for (int r = 0; r < kLineLoads; ++r) {
+      se += x[r];
+      sw = fma_t<TC>((TC)(t0 + 32 * r + 1) * sc, x[r], sw);
+      nf += nonfinite(x[r]);
+    }
   }
   se = warp_sum_t<TC>(se);
   sw = warp_sum_t<TC>(sw);
@@ -166,11 +185,16 @@ __device__ int row_line_warp(const CheckArgs& a, int64_t i, int64_t J, double& r
   int nf = 0;
   const TC* p = C + i * a.ldc + j0;
   const int len = (int)(j1 - j0);
-  for (int t = lane; t < len; t += 32) {
-    const TC x = p[t];
-    se += x;
-    sw = fma_t<TC>((TC)(t + 1) * sc, x, sw);
-    nf += isfinite(x) ? 0 : 1;
+  for (int t0 = lane; t0 < len; t0 += 32 * kLineLoads) {
+    TC x[kLineLoads];
+#pragma unroll
+    for (int r = 0; r < kLineLoads; ++r) x[r] = t0 + 32 * r < len ? p[t0 + 32 * r] : (TC)0;
+#pragma unroll
+    for (int r = 0; r < kLineLoads; ++r) {
+      se += x[r];
+      sw = fma_t<TC>((TC)(t0 + 32 * r + 1) * sc, x[r], sw);
+      nf += nonfinite(x[r]);
+    }
   }
   se = warp_sum_t<TC>(se);
   sw = warp_sum_t<TC>(sw);
@@ -240,14 +264,14 @@ __device__ __forceinline__ void col_lines(const CheckArgs& a, const ColLines& c)
         for (int r = 0; r < 8; ++r) {
           e += x[r];
           w = fma_t<TC>(wtab[t + r], x[r], w);
-          nf |= isfinite(x[r]) ? 0 : 1;
+          nf |= nonfinite(x[r]);
         }
       }
       for (; t < nr; ++t) {
         const TC x = q[t * a.ldc];
         e += x;
         w = fma_t<TC>(wtab[t], x, w);
-        nf |= isfinite(x) ? 0 : 1;
+        nf |= nonfinite(x);
       }
       sw = fma_t<TC>((TC)(s0 - i0) * sc, e, sw + w);
       se += e;
@@ -325,7 +349,7 @@ __device__ __forceinline__ void row_lines(const CheckArgs& a, int64_t block) {
       const TC x = r < nr ? q[r * a.ldc + t] : (TC)0;
       v[r] += x;
       v[R + r] = fma_t<TC>(w, x, v[R + r]);
-      nfb |= isfinite(x) ? 0u : 1u << r;
+      nfb |= (uint32_t)nonfinite(x) << r;
     }
     w += (TC)32 * sc;
   }
@@ -782,13 +806,25 @@ __device__ __forceinline__ void locate_body(const Pol& A, int32_t* cnt, const Fl
     double s = 0.0, expect;
     if (how[t] == 0) {
       const int64_t I = r / G.vb_r, i0 = I * G.vb_r, i1 = min(i0 + G.vb_r, G.m);
-      for (int64_t i = i0 + lane; i < i1; i += 32)
-        if (i != r) s += A.ldc(p, i, c);
+      for (int64_t i = i0 + lane; i < i1; i += 32 * kLineLoads) {
+        double x[kLineLoads];
+#pragma unroll
+        for (int u = 0; u < kLineLoads; ++u)
+          x[u] = i + 32 * u < i1 && i + 32 * u != r ? A.ldc(p, i + 32 * u, c) : 0.0;
+#pragma unroll
+        for (int u = 0; u < kLineLoads; ++u) s += x[u];
+      }
       expect = A.expect_col(p, I, c);
     } else {
       const int64_t J = c / G.vb_c, j0 = J * G.vb_c, j1 = min(j0 + G.vb_c, G.n);
-      for (int64_t j = j0 + lane; j < j1; j += 32)
-        if (j != c) s += A.ldc(p, r, j);
+      for (int64_t j = j0 + lane; j < j1; j += 32 * kLineLoads) {
+        double x[kLineLoads];
+#pragma unroll
+        for (int u = 0; u < kLineLoads; ++u)
+          x[u] = j + 32 * u < j1 && j + 32 * u != c ? A.ldc(p, r, j + 32 * u) : 0.0;
+#pragma unroll
+        for (int u = 0; u < kLineLoads; ++u) s += x[u];
+      }
       expect = A.expect_row(p, r, J);
     }
     s = warp_sum(s);
@@ -1139,6 +1175,17 @@ __global__ void __launch_bounds__(kThreads) k_recover(TC* C, int64_t ldc, const 
   if (jj >= bc) return;
   if (timeout && *timeout) return;  // block checksums of an incomplete product
   const int64_t j = (int64_t)bj * bc + jj;
+  if (rs.t == 1) {  // the first checksum's coefficients are 1
+    for (int64_t r = blockIdx.y; r < bs; r += gridDim.y) {
+      const TC* q = C + r * ldc + j;
+      double s = 0.0;
+#pragma unroll 8
+      for (int I = 0; I < p; ++I)
+        if (I != rs.rows[0]) s += (double)q[I * bs * ldc];
+      C[((int64_t)rs.rows[0] * bs + r) * ldc + j] = (TC)(S[r * n + j] - s);
+    }
+    return;
+  }
   int e = 0;
   while ((1 << e) <= p) ++e;
   for (int64_t r = blockIdx.y; r < bs; r += gridDim.y) {
