@@ -460,7 +460,6 @@ struct ProdArgs {
   F64Args g;
   TileGrid T;
   int nkb, bpt;                  // k-steps of a panel; boxes per tile
-  int sweep;                     // k-steps of a sweep through the moduli
   int kpad, rows_a, row_cs, col_cs;
   const int2* a_row;
   const int2* b_col;
@@ -609,9 +608,7 @@ __device__ __forceinline__ TileView64 view_tile(const ProdArgs& p, int64_t t, in
 // CTAs of a cluster, each takes them like a whole tile, the residues meet in the
 // cluster's scratch and every CTA puts a share of the columns together: a small
 // product then occupies p.split times as many SMs.
-// kSweep: the moduli are taken once per p.sweep k-steps; a later sweep starts from the
-// residues that the one before left in the scratch.
-template <bool kPair, bool kSplit, bool kSweep>
+template <bool kPair, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_f64_tc(const __grid_constant__ Maps M, const ProdArgs p) {
   extern __shared__ uint8_t smem_raw[];
@@ -625,20 +622,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int rank = kPair ? (int)tc::cluster_ctarank() : 0;
   const int part = kSplit ? (int)tc::cluster_ctarank() : 0, nparts = kSplit ? p.split : 1;
   const int plane0 = kPlanes64 * part / nparts, plane1 = kPlanes64 * (part + 1) / nparts;
-  // Pass i over k-steps [k0, k1) of a plane: the magnitudes, then the moduli, these once per
-  // sweep of p.sweep k-steps.
-  struct Pass {
-    int plane, k0, k1;
-  };
-  const int passes = kSweep ? 1 + kModuli * ((p.nkb + p.sweep - 1) / p.sweep) : plane1;
-  auto pass = [&](int i) -> Pass {
-    if (i == 0) return {kMagPlane, 0, p.nkb};
-    if constexpr (kSweep) {
-      const int k0 = (i - 1) / kModuli * p.sweep;
-      return {(i - 1) % kModuli, k0, min(k0 + p.sweep, p.nkb)};
-    }
-    return {i - 1, 0, p.nkb};
-  };
   const bool issuer = rank == 0;  // its MMA warp issues for both CTAs of a pair
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + NS * stage);
   // full [8], empty [8], tmem full [2], tmem empty [2], drain, residues done
@@ -704,10 +687,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         // a pair's bytes (both CTAs') land on the issuer's barrier, which the
         // issuer's producers expect
         const uint32_t tx = (pA ? kABytes : (uint32_t)V.nbox * kBoxBytes) * (kPair ? 2 : 1);
-        for (int i = plane0; i < passes && ok; ++i) {
-          const Pass P = pass(i);
-          const int arow = P.plane * p.rows_a + V.arow, brow = P.plane * p.kpad;
-          for (int kb = P.k0; kb < P.k1; ++kb) {
+        // a plane of A and of B: the magnitudes, then the residues
+        for (int i = plane0; i < plane1 && ok; ++i) {
+          const int plane = i == 0 ? kMagPlane : i - 1;
+          const int arow = plane * p.rows_a + V.arow, brow = plane * p.kpad;
+          for (int kb = 0; kb < nkb; ++kb) {
             if (!tc::wait(empty(s), ph ^ 1, abort)) { ok = false; break; }
             const uint32_t sa = tc::smem_addr(smem + s * stage);
             if (issuer) tc::mbar_arrive_expect_tx(full(s), tx);
@@ -777,10 +761,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           return true;
         };
-        for (int i = plane0; i < passes && ok; ++i) {
-          const Pass P = pass(i);
-          ok = level(P.k1 - P.k0, i == 0 ? nkb : kGroupSteps);  // magnitudes: one accumulator
-        }
+        for (int i = plane0; i < plane1 && ok; ++i)
+          ok = level(nkb, i == 0 ? nkb : kGroupSteps);  // magnitudes: one accumulator
       }
       // every MMA has completed before TMEM is freed
       if constexpr (kPair)
@@ -855,34 +837,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane < nch) bad[lane] = (uint8_t)((leave >> lane) & 1);
         if (leave && lane == 0) atomicExch(&p.hdr[1], 1);
       }
-      // ---- residues (a later sweep adds to those before it)
-      for (int i = max(plane0, 1); i < passes; ++i) {
-        const Pass P = pass(i);
-        const int t = P.plane;
+      // ---- residues
+      for (int t = max(plane0, 1) - 1; t < plane1 - 1; ++t) {
         const float pm = kModulus.m[t].x, inv = kModulus.m[t].y;
         float sum[4][32];
 #pragma unroll
         for (int ci = 0; ci < 4; ++ci)
 #pragma unroll
           for (int u = 0; u < 32; ++u) sum[ci][u] = 0.0f;
-        if (kSweep && P.k0 > 0) {  // in flight until the first accumulator is full
-#pragma unroll
-          for (int ci = 0; ci < 4; ++ci)
-            if (ci < nch && c_lo + 32 * ci < c_hi) {
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                // a signed byte + 128 in the low byte of 2^23
-                const uint32_t old =
-                    scr[(int64_t)((t * nch + ci) * 8 + j) * 256] ^ 0x80808080u;
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                  sum[ci][4 * j + u] =
-                      __uint_as_float(__byte_perm(old, 0x4B000000u, 0x7440u | (uint32_t)u)) -
-                      8388736.0f;
-              }
-            }
-        }
-        for (int k0 = P.k0; k0 < P.k1; k0 += kGroupSteps) {
+        for (int k0 = 0; k0 < nkb; k0 += kGroupSteps) {
           if (!wait_all(tfull(acc), aph)) { ok = false; break; }
           tc::fence_after_sync();
           const uint32_t base = tmem + lanes + acc * 256 + c_lo;
@@ -1077,30 +1040,15 @@ bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, si
   return true;
 }
 
-// k-steps that a CTA pair takes through all moduli before the next ones.  A wave of tiles
-// shares 2048 rows of A and about 2400 columns of B, 101 MB per plane at k = 11264, so
-// pairs that have drifted a plane apart evict each other's panels from L2: 186 GB read per
-// launch of 11264^3 on a 22 x 22 grid where 50 would do.  Two sweeps of 88 k-steps there:
-// product in the step 43.8 -> 38.0 ms where DRAM is slow to answer, 38.5 -> 37.3 on another
-// chip; in three sweeps 37.6.  Below, a plane's share stays in L2: 8192^3 encode + product
-// in one sweep 15.82 ms, in two 16.03.
-constexpr int kSweepSteps = 128;
-static int sweep_steps(int nkb) {
-  const int sweeps = (int)cdiv(nkb, kSweepSteps);
-  return (int)cdiv(nkb, sweeps);
-}
-
 cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaStream_t st) {
   const F64TcRegions& r = P.f64tc;
   char* w = static_cast<char*>(ws) + P.f64tc_base;
   int* hdr = reinterpret_cast<int*>(static_cast<char*>(ws) + P.f64tc_hdr);
   const TileGrid T = tile_grid(g.m, g.n, g.R, g.Cc, r.bpt, r.pair);
   const char* stall = getenv("ABFT_TEST_STALL_PRODUCER");
-  const int nkb = (int)cdiv(std::min(g.k, r.kp), BK), sweep = sweep_steps(nkb);
-  const auto kernel = r.split > 1   ? k_gemm_f64_tc<false, true, false>
-                      : !r.pair     ? k_gemm_f64_tc<false, false, false>
-                      : nkb > sweep ? k_gemm_f64_tc<true, false, true>
-                                    : k_gemm_f64_tc<true, false, false>;
+  const auto kernel = r.pair      ? k_gemm_f64_tc<true, false>
+                      : r.split > 1 ? k_gemm_f64_tc<false, true>
+                                    : k_gemm_f64_tc<false, false>;
   const int boxes = cta_boxes(r.bpt, r.pair);
   const size_t smem = smem_bytes(boxes);
   cudaError_t e =
@@ -1158,7 +1106,6 @@ cudaError_t launch_gemm_f64_tc(const Plan& P, const F64Args& g, void* ws, cudaSt
     p.g = gp;
     p.T = T;
     p.nkb = (int)(kpad / BK);
-    p.sweep = sweep;
     p.bpt = r.bpt;
     p.kpad = (int)kpad; p.rows_a = (int)r.rows_a; p.row_cs = (int)r.row_cs;
     p.col_cs = (int)r.col_cs;

@@ -108,13 +108,6 @@ def test_edges(shape):
     assert np.array_equal(product(A, B, pad=1)[0], A @ B)
 
 
-# CTA pairs with more than 128 k-steps: two sweeps through the moduli, the last one shorter;
-# a panel of 255 k-steps and a last one of one
-@pytest.mark.parametrize("shape", [(2500, 2600, 8193), (2500, 2600, 16321)])
-def test_sweeps(shape):
-    test_edges(shape)
-
-
 @pytest.mark.parametrize("kind", ["rows", "graded", "outlier", "eye", "sparse", "equal", "wide",
                                   "zero"])
 def test_operand_kinds(kind):
