@@ -46,8 +46,10 @@
  *                         promotion (default: 256 rows when m > 128 and the K
  *                         loop has at least 32 k-steps).
  *  - ABFT_PAIR_TILES      1: single products run 256 x 256 tiles on CTA pairs
- *                         (clusters of two, one cta_group::2 MMA per K step;
- *                         default 0: one-CTA tiles, see ABFT_TALL_TILES).
+ *                         (clusters of two, one cta_group::2 MMA per K step);
+ *                         0: one-CTA tiles, see ABFT_TALL_TILES (default: pairs
+ *                         for bf16x6 with k >= 5120, bf16x3 with k >= 8192 and
+ *                         native FP8 with k >= 9216 that fill their waves).
  *  - ABFT_GROUP_M         raster group height in tile rows of single products
  *                         (default 2048 rows).
  *  - ABFT_GRP_SWAP        0: grouped products compute checksum rows in regular

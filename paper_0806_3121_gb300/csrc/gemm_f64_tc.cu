@@ -604,30 +604,15 @@ __device__ __forceinline__ TileView64 view_tile(const ProdArgs& p, int64_t t, in
   return V;
 }
 
-// Holds a worker (CTA pair) back until the others have come as far: called by one thread
-// of each before every kStepPlanes-th plane of its `round`-th tile, the n-th call of the
-// tile with call = n.  The workers of a wave share 2048 rows of A and about 2400 columns of
-// B, 73 MB per plane at k = 8192 and 101 MB at 11264; left alone they drift planes apart
-// (checksum tiles are narrower) and every one reads its panels from DRAM again.  11264^3 on
-// a 22 x 22 grid: 186 to 246 GB read per launch -> 61, product in the step 43.8 -> 31.3 ms;
-// 8192^3 encode + product 17.1 -> 14.7; 4096^3, where a plane is 37 MB, 2.88 either way.
-// Before every plane 11264^3 takes 31.4 ms and 4096^3 2.89, before each tile only nothing is
-// gained (the drift is within a tile).
-// It only orders the reads, so a worker whose fellows are not running (another stream's
-// kernel holds their SMs) gives up after the time of two such calls and stops waiting.
+// tc::keep_step before every kStepPlanes-th plane of a pair's tile.  The pairs of a wave
+// share 2048 rows of A and about 2400 columns of B, 73 MB per plane at k = 8192 and 101 MB
+// at 11264; left alone they drift planes apart (checksum tiles are narrower) and every one
+// reads its panels from DRAM again.  11264^3 on a 22 x 22 grid: 186 to 246 GB read per
+// launch -> 61, product in the step 43.8 -> 31.3 ms; 8192^3 encode + product 17.1 -> 14.7;
+// 4096^3, where a plane is 37 MB, 2.88 either way.  Before every plane 11264^3 takes 31.3
+// ms too and 4096^3 2.89; once per tile gains nothing (the drift is within a tile).
 constexpr int kStepPlanes = 3;
 constexpr int kStepCalls = (kPlanes64 + kStepPlanes - 1) / kStepPlanes;  // of a tile
-__device__ __forceinline__ bool keep_step(uint32_t* arrivals, uint32_t workers, int64_t total,
-                                          uint32_t round, uint32_t call, uint64_t limit_ns) {
-  const int64_t in_round = min((int64_t)workers, total - (int64_t)round * workers);
-  const uint32_t target = round * workers * kStepCalls + call * (uint32_t)in_round;
-  if ((int32_t)(atomicAdd(arrivals, 1u) + 1 - target) >= 0) return true;
-  const uint64_t t0 = tc::globaltimer();
-  while ((int32_t)(*(volatile uint32_t*)arrivals - target) < 0)
-    if (tc::globaltimer() - t0 > limit_ns) return false;
-  return true;
-}
-
 // kSplit: the planes of a tile (magnitudes, then the moduli) are dealt to the p.split
 // CTAs of a cluster, each takes them like a whole tile, the residues meet in the
 // cluster's scratch and every CTA puts a share of the columns together: a small
@@ -719,8 +704,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!together)
               atomicAdd(arr, 1u);
             else  // a k-step takes about 320 ns
-              together = keep_step(arr, (uint32_t)tstep, total, (uint32_t)((t - tfirst) / tstep),
-                                   i / kStepPlanes + 1, 640ull * kStepPlanes * nkb);
+              together = tc::keep_step(arr, (uint32_t)tstep, total, (uint32_t)((t - tfirst) / tstep),
+                                   i / kStepPlanes + 1, kStepCalls, 640ull * kStepPlanes * nkb);
           }
           const int arow = plane * p.rows_a + V.arow, brow = plane * p.kpad;
           for (int kb = 0; kb < nkb; ++kb) {

@@ -157,6 +157,8 @@ struct TcArgs {
   const uint32_t* f8grp;
   int64_t f8words;
   int64_t cs_stride;         // FP8 tile order: checksum tile c at position c * cs_stride
+  uint32_t* arrivals;        // tc::keep_step of the pair tiles (nullptr: off), its calls per
+  int calls;                 // tile
 };
 
 // The product kernel's parameters (tensor maps and arguments, passed by value
@@ -489,7 +491,8 @@ __device__ __forceinline__ void store_staged(const float* stg, int lane, float* 
 template <bool kPromote, bool kTall, bool kF8, bool kPair, class Sched>
 __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wait_ns,
                                         int stall_test, const int32_t* inj_hdr,
-                                        const InjectEntry* inj) {
+                                        const InjectEntry* inj, uint32_t* arrivals = nullptr,
+                                        int calls = 0) {
   using G = Geo<kTall, kPair>;
   static_assert(!(kPromote && kTall), "promotion runs on regular or pair tiles");
   static_assert(!kF8 || kPromote, "FP8 data tiles promote every k-step");
@@ -563,6 +566,7 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
       int s = 0;
       uint32_t ph = 0;
       int64_t issued = 0;  // stages filled and not known to be consumed
+      bool together = true;
       for (int64_t t = tfirst; t < total && !*abort; t += tstep) {
         const TileView T = S.view(t);
         if (stall_test && t == 0) continue;  // nothing will fill these stages
@@ -620,7 +624,22 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
         // incremental (no division per stage)
         int seg = 0, pa = (int)(T.seg_a & 3u), pb = (int)(T.seg_b & 3u);
         int64_t kb = 0, kc0 = 0, kc1 = min(T.chunk, nkb);
+        // pair tiles: the pairs of a wave stay within a few k-steps (kStepKsteps)
+        const bool stepper = kPair && pA && issuer && arrivals;
+        const int itv = stepper ? (int)((nkt + calls - 1) / calls) : 0;
+        int call = 0;
+        int64_t kstep = 0;
         for (int64_t kt = 0; kt < nkt; ++kt) {
+          if (stepper && kt == kstep) {
+            kstep += itv;
+            ++call;
+            if (together)
+              together = tc::keep_step(arrivals, (uint32_t)tstep, total,
+                                       (uint32_t)((t - tfirst) / tstep), call, calls,
+                                       1000ull * itv);
+            else
+              atomicAdd(arrivals, 1u);
+          }
           const int32_t kx = (int32_t)(kb * bkx);
           if (!tc::wait(empty(s), ph ^ 1, abort)) break;
           const uint32_t sa = tc::smem_addr(smem + s * G::kStageBytes);
@@ -697,6 +716,8 @@ __device__ __forceinline__ void tc_body(const Sched& S, int* status, uint64_t wa
             pb = (int)((T.seg_b >> (2 * seg)) & 3u);
           }
         }
+        if (stepper && call < calls)  // a K loop that fewer calls cover
+          atomicAdd(arrivals, (uint32_t)(calls - call));
       }
       // Do not leave copies in flight: wait for the last fills (bounded).  A
       // pair's copies complete on the issuer's barriers, so its CTAs wait
@@ -1177,7 +1198,8 @@ template <bool kPromote, bool kTall, bool kF8, bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_bf16(const __grid_constant__ TcMaps M, const TcArgs g) {
   const SingleSched<Geo<kTall, kPair>::kBM> S{&M, &g};
-  tc_body<kPromote, kTall, kF8, kPair>(S, g.status, g.wait_ns, g.stall_test, g.inj_hdr, g.inj);
+  tc_body<kPromote, kTall, kF8, kPair>(S, g.status, g.wait_ns, g.stall_test, g.inj_hdr, g.inj, g.arrivals,
+                                       g.calls);
 }
 
 // Many problems (grouped product).  The flattened tile list is a table of
@@ -1488,25 +1510,34 @@ bool use_tall(int64_t m, int64_t nkt, int chunk) {
   return m > BM && nkt >= 32;
 }
 
-// Pair tiles (256 x 256 on a CTA pair, see Geo).  Measured at 16384^3 against
-// the one-CTA schedules: FP8 (native data tiles) no faster (the MMA warp waits
-// on stage data 10 % of the time instead of 17 %, but a pair MMA that does not
-// wait runs about 5 % slower per SM than a one-CTA MMA); bf16 10 % slower than
-// tall tiles and the promoted bf16x3 / bf16x6 12-20 % slower than regular
-// tiles: a pair tile takes half as long as a tall one, so the same drift
-// between CTAs puts the tiles that share an operand panel twice as far apart
-// in K, and the product reads 17.8 GB from DRAM instead of 7.0; the promoted
-// products also wait twice as long for a free accumulator (both CTAs'
-// epilogues must release it).  FP8 with pair tiles: 4.097 ms per step against
-// 4.099 with regular tiles (the checksum-free product 3.12 against 3.04 ms).  So
-// no product uses them unless ABFT_PAIR_TILES=1 asks for them (0 or unset:
-// tall or regular tiles).
-bool use_pair(int64_t m, bool f8) {
+// Pair tiles (256 x 256 on a CTA pair, see Geo) for promoted and FP8 products with long
+// K: a pair stages two thirds of the bytes per flop of two regular tiles.  Left alone the
+// pairs of a wave drift apart in K and read their panels from DRAM again (bf16 16384^3:
+// 17.8 GB instead of 7.0); kept in step (kStepKsteps) they do not.  Whole steps, regular ->
+// pair: bf16x6 16384^3 33.55 -> 31.5 ms, bf16x3 8192^3 2.47 -> 2.40, FP8 16384^3 4.02 ->
+// 3.85; products alone: bf16x6 10000 x 9008 x 11120 8.84 -> 7.68 ms, FP8 1.20 -> 0.96,
+// bf16x3 2500 x 9008 x 12304 1.41 -> 1.24.  With short K the pairs' accumulators wait for
+// both CTAs' epilogues (bf16x6 16384 x 16384 x 2048 4.21 -> 4.31 ms, 4096^3 0.557 either
+// way, 5120^3 1.064 -> 1.050; bf16x3 5120^3 0.565 -> 0.570; FP8 8192^3 0.498 -> 0.508, 16384
+// x 16384 x 8192 1.84 -> 1.76), and few tiles fill their last wave less (2048 x 2048 x
+// 8192 bf16x6 0.27 -> 0.46 ms): the pairs may take as many waves as the regular tiles, or
+// 3 % more.  bf16 keeps its tall tiles (16384^3 step 5.56 -> 5.82 ms).  ABFT_PAIR_TILES=0
+// or 1 forces the choice.
+bool use_pair(const abft_desc& d, int64_t R, int64_t Cc, bool f8, int chunk) {
   const char* env = getenv("ABFT_PAIR_TILES");
-  (void)m;
-  (void)f8;
-  return env && env[0] == '1';
+  if (env && *env) return env[0] == '1';
+  if (d.k < (f8 ? 9216 : d.dtype == ABFT_BF16X6 ? 5120 : 8192) || !(f8 || chunk > 0)) return false;
+  auto waves = [&](int bm, int64_t workers) {
+    const int64_t tm = cdiv(d.m, bm), tn = cdiv(d.n, BN);
+    return cdiv(tm * tn + cdiv(R, bm) * tn + tm * cdiv(Cc, BN), workers);
+  };
+  const int64_t sms = num_sms();
+  return 100 * waves(2 * BM, sms / 2) <= 103 * waves(BM, sms);
 }
+
+// k-steps between two calls of tc::keep_step: bf16x6 16384^3 with 16 / 48 / 144 31.85 /
+// 31.57 / 31.45 ms per step, bf16x3 8192^3 2.44 / 2.40 / 2.41, FP8 16384^3 3.95 / 3.87 / 3.87.
+constexpr int kStepKsteps = 96;
 
 // Stride of the checksum tiles in the FP8 tile order.  Measured at FP8 16384^3:
 // all checksum tiles first (S = 1) 3.18 ms per ABFT product, S = 2 / 3 / 5
@@ -1592,8 +1623,10 @@ cudaError_t launch_gemm_bf16(const Plan& P, const TcOperands& op, float* C, void
   const char* w = static_cast<const char*>(ws);
   const int64_t R16 = checksums ? P.L.acs_rows : 0, C16 = checksums ? P.L.bcs_cols : 0;
   TcMaps M;
+  const int kpg = promote_ksteps(d.dtype);
+  const int chunk = kpg > 0 ? std::max(1, kpg / op.nseg) : 0;
   // pair tiles: each CTA of a pair copies half of a full tile's B boxes
-  const bool pair = use_pair(d.m, op.a8 != nullptr);
+  const bool pair = use_pair(d, R16, C16, op.a8 != nullptr, chunk);
   const int bdepth = pair ? 2 : 4;
   for (int pl = 0; pl < kPlanes; ++pl) {
     const int cpl = pl < P.L.planes ? pl : 0;  // checksum planes beyond the dtype's repeat plane 0
@@ -1621,8 +1654,7 @@ cudaError_t launch_gemm_bf16(const Plan& P, const TcOperands& op, float* C, void
   g.nseg = op.nseg;
   g.seg_a = op.seg_a;
   g.seg_b = op.seg_b;
-  const int kpg = promote_ksteps(d.dtype);
-  g.chunk = kpg > 0 ? std::max(1, kpg / op.nseg) : 0;
+  g.chunk = chunk;
   if (op.a8) {  // native FP8 data tiles on the e4m3 codes (promoted every k-step)
     if (!make_map_u8(&M.a[kF8Slot], op.a8, d.m, d.k, op.lda8, 128, BM / 2) ||
         !make_map_u8(&M.a128[kF8Slot], op.a8, d.m, d.k, op.lda8, 128, BM) ||
@@ -1690,7 +1722,16 @@ cudaError_t launch_gemm_bf16(const Plan& P, const TcOperands& op, float* C, void
                       : num_sms());
   if (workers == 0) return cudaSuccess;
   if (g.f8) g.cs_stride = cs_stride(g.t_total - g.t_data, g.t_total, workers);  // 1 unless set
-  e = cudaMemsetAsync(status, 0, sizeof(int), st);  // the status of this product
+  // the status of this product; in a workspace the arrivals' word lies before it
+  static_assert(kCntArrivals + 1 == kCntTimeout, "cleared together");
+  if (pair && ws) {
+    g.arrivals = reinterpret_cast<uint32_t*>(status) - 1;
+    const int64_t nkt = g.f8 ? cdiv(d.k, BK8) : cdiv(d.k, BK) * op.nseg;
+    g.calls = (int)cdiv(nkt, kStepKsteps);
+    e = cudaMemsetAsync(g.arrivals, 0, 2 * sizeof(int), st);
+  } else {
+    e = cudaMemsetAsync(status, 0, sizeof(int), st);
+  }
   if (e != cudaSuccess) return e;
   if (pair) {
     cudaLaunchConfig_t cfg = {};

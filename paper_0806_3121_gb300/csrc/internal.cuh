@@ -50,6 +50,7 @@ enum Counter : int {
   kCntOverflow = 3,
   kCntRecoverFlagged = 4,
   kCntCands = 5,
+  kCntArrivals = 7,       // of the product's pairs (tc::keep_step)
   kNumCleared = 8,
   kCntTimeout = 8,
   kCntFp8Inexact = 9,

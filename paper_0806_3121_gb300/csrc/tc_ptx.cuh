@@ -92,6 +92,23 @@ __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, volatile int
   }
 }
 
+// Holds a worker (CTA pair) of a persistent kernel back until the others have come as far:
+// one thread of each calls this `calls` times per tile, the n-th time in its `round`-th
+// tile with call = n.  It only orders reads, so that workers find each other's panels in
+// L2: a worker whose fellows are not running (another stream's kernel holds their SMs)
+// gets false after limit_ns, stops waiting and only counts itself in.
+__device__ __forceinline__ bool keep_step(uint32_t* arrivals, uint32_t workers, int64_t total,
+                                          uint32_t round, uint32_t call, uint32_t calls,
+                                          uint64_t limit_ns) {
+  const int64_t in_round = min((int64_t)workers, total - (int64_t)round * workers);
+  const uint32_t target = round * workers * calls + call * (uint32_t)in_round;
+  if ((int32_t)(atomicAdd(arrivals, 1u) + 1 - target) >= 0) return true;
+  const uint64_t t0 = globaltimer();
+  while ((int32_t)(*(volatile uint32_t*)arrivals - target) < 0)
+    if (globaltimer() - t0 > limit_ns) return false;
+  return true;
+}
+
 // 2-D tiled TMA load of the box at element coordinates (x inner, y outer)
 // into shared memory, completing on barrier `bar` (transaction bytes).
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
