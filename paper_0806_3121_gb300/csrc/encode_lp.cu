@@ -1177,10 +1177,19 @@ __device__ __forceinline__ void store_split8(const Planes& P, int64_t off, const
 
 // Rows of binary32 loads a thread of the split passes issues ahead.
 constexpr int kSplitRows = 8;
+// The split passes' CTA: 256 columns, eight per lane; the warps share the rows, batches of
+// kSplitRows in turn, and put their column sums together in shared memory.  Bound by
+// memory (4 bytes read and 2 per plane written per element) once the grid fills the chip;
+// with eight columns per thread of the whole CTA (2048 columns, every warp all the rows)
+// a 512^2 pass was a few CTAs that walked 128 rows each.  Whole encode, verify blocks 128 x
+// 256, bf16x3 / bf16x6: 512^2 138 / 147 -> 42 / 46 us, 2048^2 144 / 148 -> 40 / 42, 4096^2
+// 151 / 155 -> 79 / 83, 8192^2 207 / 247 -> 213 / 239 (blocks of 256 rows 245 / 268 -> 217 /
+// 242), 16384^2 739 / 885 -> 732 / 843.
+constexpr int kSplitCols = 256;
 
 // A: planes (m x ldk), column checksums of A per verify block from the
 // binary32 values (rows 2I, 2I+1 of the acs planes), per-row partial sums of
-// squares and checksum-norm partials.  CTA = 2048 columns x a block.
+// squares and checksum-norm partials (one per CTA column).
 __global__ void __launch_bounds__(kThreads) k_x3A_cols(const float* __restrict__ A, int64_t lda,
                                                        int64_t m, int64_t k, int vb, int e,
                                                        const Planes op, const Planes cs,
@@ -1188,8 +1197,10 @@ __global__ void __launch_bounds__(kThreads) k_x3A_cols(const float* __restrict__
                                                        int64_t nchr, double* __restrict__ part,
                                                        int64_t nch, int cs_on) {
   __shared__ float sh[kThreads / 32];
+  __shared__ float4 red[kThreads / 32][2][kSplitCols / 4];  // per warp: sums, weighted sums
+  static_assert(kSplitCols == kThreads, "a thread per column");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t c0 = (int64_t)blockIdx.x * kColsPerCta + 8 * threadIdx.x;
+  const int64_t c0 = (int64_t)blockIdx.x * kSplitCols + 8 * lane;
   const int64_t nvb = cdiv(m, vb);
   const float sc = scalbnf(1.0f, -e);
   for (int64_t I = blockIdx.y; I < nvb; I += gridDim.y) {
@@ -1199,7 +1210,7 @@ __global__ void __launch_bounds__(kThreads) k_x3A_cols(const float* __restrict__
     for (int q = 0; q < 8; ++q) se[q] = sw[q] = 0.f;
     // kSplitRows rows' loads in flight per thread before the first of them is used
     // (the plane stores would otherwise hold each next row's loads back)
-    for (int64_t ib = i0; ib < i1; ib += kSplitRows) {
+    for (int64_t ib = i0 + warp * kSplitRows; ib < i1; ib += kThreads / 32 * kSplitRows) {
       float vb8[kSplitRows][8];
 #pragma unroll
       for (int r = 0; r < kSplitRows; ++r)
@@ -1219,24 +1230,30 @@ __global__ void __launch_bounds__(kThreads) k_x3A_cols(const float* __restrict__
           sq = fmaf(v[q], v[q], sq);
         }
         sq = warp_sumf(sq);
-        const int64_t rc = (int64_t)blockIdx.x * (kThreads / 32) + warp;
-        if (lane == 0 && rc < nchr) rowpart[i * nchr + rc] = sq;
+        if (lane == 0 && blockIdx.x < nchr) rowpart[i * nchr + blockIdx.x] = sq;
       }
     }
     if (!cs_on) continue;  // chained: the checksum rows are carried, not formed
-    float q0 = 0.f, q1 = 0.f;
-    if (c0 < ldk) {
-      store_split8(cs, (2 * I) * ldk + c0, se);
-      store_split8(cs, (2 * I + 1) * ldk + c0, sw);
+    red[warp][0][2 * lane] = make_float4(se[0], se[1], se[2], se[3]);
+    red[warp][0][2 * lane + 1] = make_float4(se[4], se[5], se[6], se[7]);
+    red[warp][1][2 * lane] = make_float4(sw[0], sw[1], sw[2], sw[3]);
+    red[warp][1][2 * lane + 1] = make_float4(sw[4], sw[5], sw[6], sw[7]);
+    __syncthreads();
+    float te = 0.f, tw = 0.f;  // this thread's column
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        q0 = fmaf(se[q], se[q], q0);
-        q1 = fmaf(sw[q], sw[q], q1);
-      }
+    for (int w = 0; w < kThreads / 32; ++w) {
+      te += reinterpret_cast<const float*>(red[w][0])[threadIdx.x];
+      tw += reinterpret_cast<const float*>(red[w][1])[threadIdx.x];
     }
-    const float t0 = block_sumf(q0, sh);
+    const int64_t c = (int64_t)blockIdx.x * kSplitCols + threadIdx.x;
+    if (c < ldk) {
+      store_split1(cs, (2 * I) * ldk + c, te);
+      store_split1(cs, (2 * I + 1) * ldk + c, tw);
+    }
+    // (block_sumf: every thread has read red before the next block's sums go there)
+    const float t0 = block_sumf(te * te, sh);
     if (threadIdx.x == 0) part[(2 * I) * nch + blockIdx.x] = (double)t0;
-    const float t1 = block_sumf(q1, sh);
+    const float t1 = block_sumf(tw * tw, sh);
     if (threadIdx.x == 0) part[(2 * I + 1) * nch + blockIdx.x] = (double)t1;
   }
 }
@@ -1266,8 +1283,10 @@ __global__ void __launch_bounds__(kThreads) k_x3B_rows(const float* __restrict__
                                                        const Planes cs, int64_t ldcs,
                                                        float* __restrict__ colpart,
                                                        double* __restrict__ part, int64_t nch) {
-  const int lane = threadIdx.x & 31;
-  const int64_t c0 = (int64_t)blockIdx.x * kColsPerCta + 8 * threadIdx.x;
+  __shared__ float4 red[kThreads / 32][kSplitCols / 4];  // per warp: squares of the columns
+  __shared__ float2 redq[kThreads / 32][32];              // ... of the checksums
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t c0 = (int64_t)blockIdx.x * kSplitCols + 8 * lane;
   const int64_t l0 = (int64_t)blockIdx.y * kRowsPerCtaB, l1 = min(l0 + kRowsPerCtaB, k);
   const int seg = vb / 8;
   const bool leader = (lane % seg) == 0 && c0 < n;
@@ -1280,7 +1299,7 @@ __global__ void __launch_bounds__(kThreads) k_x3B_rows(const float* __restrict__
 #pragma unroll
   for (int q = 0; q < 8; ++q) cs2[q] = 0.f;
   float q0 = 0.f, q1 = 0.f;
-  for (int64_t lb = l0; lb < l1; lb += kSplitRows) {
+  for (int64_t lb = l0 + warp * kSplitRows; lb < l1; lb += kThreads / 32 * kSplitRows) {
     float vb8[kSplitRows][8];  // the rows' loads in flight before the first is used
 #pragma unroll
     for (int r = 0; r < kSplitRows; ++r)
@@ -1310,13 +1329,26 @@ __global__ void __launch_bounds__(kThreads) k_x3B_rows(const float* __restrict__
       }
     }
   }
-  if (leader) {
+  red[warp][2 * lane] = make_float4(cs2[0], cs2[1], cs2[2], cs2[3]);
+  red[warp][2 * lane + 1] = make_float4(cs2[4], cs2[5], cs2[6], cs2[7]);
+  redq[warp][lane] = make_float2(q0, q1);
+  __syncthreads();
+  float t = 0.f;  // this thread's column
+#pragma unroll
+  for (int w = 0; w < kThreads / 32; ++w)
+    t += reinterpret_cast<const float*>(red[w])[threadIdx.x];
+  const int64_t c = (int64_t)blockIdx.x * kSplitCols + threadIdx.x;
+  if (c < n) colpart[blockIdx.y * n + c] = t;
+  if (warp == 0 && leader) {
+    q0 = q1 = 0.f;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) {
+      q0 += redq[w][lane].x;
+      q1 += redq[w][lane].y;
+    }
     part[(2 * J) * nch + blockIdx.y] = q0;
     part[(2 * J + 1) * nch + blockIdx.y] = q1;
   }
-#pragma unroll
-  for (int q = 0; q < 8; ++q)
-    if (c0 + q < n) colpart[blockIdx.y * n + c0 + q] = cs2[q];
 }
 
 // Any verify block size: planes and column partials by one kernel, row
@@ -1700,9 +1732,9 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
     cudaMemsetAsync(nBblk, 0, sizeof(double) * 4 * P.nvc, st);
     return cudaGetLastError();
   }
-  const int64_t nchA = cdiv(d.k, kColsPerCta);
   const int64_t nchB = cdiv(d.k, kRowsPerCtaB);
   const int64_t nchr = cdiv(d.k, 256);
+  static_assert(kSplitCols == 256, "the split passes' columns of partials");
   double* partA = S.part;
   double* partB = partA + 2 * P.nvr * nchr;  // room for the bf16 pass's ceil(k/256) partials
   float* rowpart = reinterpret_cast<float*>(partB + 2 * P.nvc * nchB);
@@ -1730,8 +1762,8 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
       acsp.p[i] = reinterpret_cast<__nv_bfloat16*>(w + P.L.acs + i * P.L.acs_plane);
       bcsp.p[i] = reinterpret_cast<__nv_bfloat16*>(w + P.L.bcs + i * P.L.bcs_plane);
     }
-    k_x3A_cols<<<dim3((unsigned)nchA, gy(P.nvr)), kThreads, 0, st>>>(
-        Af, d.lda, d.m, d.k, d.vb_rows, P.er, opa, acsp, P.L.acs_ld, rowpart, nchr, partA, nchA,
+    k_x3A_cols<<<dim3((unsigned)nchr, gy(P.nvr)), kThreads, 0, st>>>(
+        Af, d.lda, d.m, d.k, d.vb_rows, P.er, opa, acsp, P.L.acs_ld, rowpart, nchr, partA, nchr,
         1);
     if (P.bs > 0) {
       Planes sp = acsp;
@@ -1740,7 +1772,7 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
           Af, d.lda, d.k, d.grid_p, P.bs, P.f, sp, P.L.acs_ld);
     }
     if (fastB) {
-      k_x3B_rows<<<dim3((unsigned)cdiv(P.L.op_b_ld, kColsPerCta), (unsigned)nchB), kThreads, 0,
+      k_x3B_rows<<<dim3((unsigned)cdiv(P.L.op_b_ld, kSplitCols), (unsigned)nchB), kThreads, 0,
                    st>>>(
           Bf, d.ldb, d.k, d.n, d.vb_cols, P.ec, opb, P.L.op_b_ld, bcsp, P.L.bcs_ld, colpart,
           partB, nchB);
@@ -1750,7 +1782,7 @@ cudaError_t launch_encode_lp(const Plan& P, const void* Av, const void* Bv, cons
       k_x3B_rows_any<<<dim3((unsigned)cdiv(nchB, kThreads / 32), gy(P.nvc)), kThreads, 0, st>>>(
           Bf, d.ldb, d.k, d.n, d.vb_cols, P.ec, bcsp, P.L.bcs_ld, partB, nchB);
     }
-    norms(nchA);
+    norms(nchr);
     count_launches(3 + (P.bs > 0 ? 1 : 0) + (fastB ? 0 : 1));
     return cudaGetLastError();
   }
@@ -1901,8 +1933,8 @@ cudaError_t launch_encode_lp_chained(const Plan& P, const void* Av, const void* 
   cudaError_t e = cudaSuccess;
   // A: operand planes and row norms from A; checksum rows carried (E of the
   // earlier product: verify rows, then block checksum rows) or formed
-  k_x3A_cols<<<dim3((unsigned)nchA, gy(P.nvr)), kThreads, 0, st>>>(
-      Af, d.lda, d.m, d.k, d.vb_rows, P.er, opa, acsp, P.L.acs_ld, rowpart, nchr, partA, nchA,
+  k_x3A_cols<<<dim3((unsigned)nchr, gy(P.nvr)), kThreads, 0, st>>>(
+      Af, d.lda, d.m, d.k, d.vb_rows, P.er, opa, acsp, P.L.acs_ld, rowpart, nchr, partA, nchr,
       PL ? 0 : 1);
   ++launches;
   if (PL) {
@@ -1929,7 +1961,7 @@ cudaError_t launch_encode_lp_chained(const Plan& P, const void* Av, const void* 
     if ((e = launch_carry_cols(*PR, wsR, carB, st)) != cudaSuccess) return e;
     launches += 3;
   } else if (fastB) {
-    k_x3B_rows<<<dim3((unsigned)cdiv(P.L.op_b_ld, kColsPerCta), (unsigned)nchB), kThreads, 0,
+    k_x3B_rows<<<dim3((unsigned)cdiv(P.L.op_b_ld, kSplitCols), (unsigned)nchB), kThreads, 0,
                  st>>>(Bf, d.ldb, d.k, d.n, d.vb_cols, P.ec, opb, P.L.op_b_ld, bcsp, P.L.bcs_ld,
                        colpart, partB, nchB);
     ++launches;
@@ -1940,7 +1972,7 @@ cudaError_t launch_encode_lp_chained(const Plan& P, const void* Av, const void* 
         Bf, d.ldb, d.k, d.n, d.vb_cols, P.ec, bcsp, P.L.bcs_ld, partB, nchB);
     launches += 2;
   }
-  norms(nchA);
+  norms(PL ? nchA : nchr);
   ++launches;
   count_launches(launches);
   return cudaGetLastError();

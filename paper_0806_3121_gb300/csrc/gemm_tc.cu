@@ -1198,8 +1198,8 @@ template <bool kPromote, bool kTall, bool kF8, bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
     k_gemm_bf16(const __grid_constant__ TcMaps M, const TcArgs g) {
   const SingleSched<Geo<kTall, kPair>::kBM> S{&M, &g};
-  tc_body<kPromote, kTall, kF8, kPair>(S, g.status, g.wait_ns, g.stall_test, g.inj_hdr, g.inj, g.arrivals,
-                                       g.calls);
+  tc_body<kPromote, kTall, kF8, kPair>(S, g.status, g.wait_ns, g.stall_test, g.inj_hdr, g.inj,
+                                       g.arrivals, g.calls);
 }
 
 // Many problems (grouped product).  The flattened tile list is a table of
