@@ -43,8 +43,9 @@
  *                         default 24 for ABFT_BF16X6 and ABFT_BF16X3, shared
  *                         by their six or three products, 0 else).
  *  - ABFT_TALL_TILES      0 / 1: 128- or 256-row tiles for products without
- *                         promotion (default: 256 rows when m > 128 and the K
- *                         loop has at least 32 k-steps).
+ *                         promotion (default: 256 rows when m > 128, the K
+ *                         loop has at least 32 k-steps and the tiles take at
+ *                         most 5/8 as many waves).
  *  - ABFT_PAIR_TILES      1: single products run 256 x 256 tiles on CTA pairs
  *                         (clusters of two, one cta_group::2 MMA per K step);
  *                         0: one-CTA tiles, see ABFT_TALL_TILES (default: pairs

@@ -124,6 +124,7 @@ struct TcArgs {
   int nseg;
   uint32_t seg_a, seg_b;
   int ntm, ntn, ntr, ntc;  // data tile rows/cols, checksum tile rows/cols (0 in plain mode)
+  int fit_h, fit_b;        // checksum halves / boxes in the last data tiles' padding (Grid)
   int64_t t_data, t_total;
   float* C;
   int64_t ldc;
@@ -391,13 +392,22 @@ struct SingleSched {
     V.hcnt = hrows;
     V.bsplit = T.kind == 2 ? 0 : bcols;
     V.nbox = bcols;
-    V.nmma = mma_cols(V.nbox, V.bsplit, T.col0, g.C16);
+    if (T.kind == 0 && g.fit_h > 0 && T.row0 + kBM >= g.m) {
+      V.hcnt += g.fit_h;
+      V.rowC = 0;
+    }
+    if (T.kind == 0 && g.fit_b > 0 && T.col0 + BN >= g.n) {
+      V.nbox += g.fit_b;
+      V.colC = 0;
+    }
+    V.nmma = mma_cols(V.nbox, V.bsplit, V.colC, g.C16);
     V.swap = V.nsw_h = V.nsw_n = 0;
     V.k2 = 1;
     V.maW = V.mbW = nullptr;
     V.rowW = (int32_t)T.row0;
     V.colW = (int32_t)T.col0;
-    V.nA128 = hrows % 2 == 0 ? hrows / 2 : 0;  // whole 128-row boxes, else per half
+    // whole 128-row boxes, else per half
+    V.nA128 = hrows % 2 == 0 && V.hcnt == hrows ? hrows / 2 : 0;
     if (V.nA128) V.maW = T.kind == 1 ? &M->acs128[0] : &M->a128[0];
     V.nW = 4;
     if (bcols == 4 && T.col0 + 256 <= ((T.kind == 2 ? g.C16 : g.n) / 64) * 64) {
@@ -1499,15 +1509,45 @@ int raster_group_rows(int bm) {
   return 2048 / bm;
 }
 
+// The tile grid of a product with bm-row tiles on `workers` CTAs (pairs).  Checksum rows
+// (columns) that fit the padding of the last data tile row (column) ride in it, as in the
+// grouped product, where that saves a wave: bf16 3001 x 2999 x 1112 324 -> 300 tiles on 152
+// SMs, 54 -> 44 us, x 4096 107 -> 82; bf16x3 3000 x 3000 x 8192 401 -> 290.  Otherwise they
+// are tiles of their own: a tile of both kinds copies its boxes one by one (bf16x3 6000 x
+// 5000 x 4096, seven waves either way, 667 us against 690).
+struct Grid {
+  int64_t ntm, ntn, ntr, ntc, waves;
+  int fit_h, fit_b;
+  int64_t total() const { return ntm * ntn + ntr * ntn + ntm * ntc; }
+};
+Grid tile_grid(int64_t m, int64_t n, int64_t R16, int64_t C16, bool f8, int bm, int64_t workers) {
+  Grid G{cdiv(m, bm), cdiv(n, BN), cdiv(R16, bm), cdiv(C16, BN), 0, 0, 0};
+  G.waves = cdiv(G.total(), workers);
+  if (f8) return G;  // data tiles on e4m3 codes, checksum tiles on bf16 planes
+  Grid H = G;
+  const int64_t h = cdiv(R16, 64), b = cdiv(C16, 64);
+  if (h > 0 && cdiv(m, 64) + h <= G.ntm * (bm / 64)) { H.fit_h = (int)h; H.ntr = 0; }
+  if (b > 0 && cdiv(n, 64) + b <= G.ntn * (BN / 64)) { H.fit_b = (int)b; H.ntc = 0; }
+  H.waves = cdiv(H.total(), workers);
+  return H.waves < G.waves ? H : G;
+}
+
 // Tall (256-row) tiles for products without promotion whose K loop is long
 // enough (at least 32 k-steps) that the tile's epilogue, which no longer
-// overlaps the next tile's MMAs, is a small share of it.  ABFT_TALL_TILES=0
-// or 1 forces the choice.
-bool use_tall(int64_t m, int64_t nkt, int chunk) {
+// overlaps the next tile's MMAs, is a small share of it, and that do not take
+// more than 5/8 of the waves of regular tiles: a wave of tall tiles takes 1.3 to 1.9 times
+// as long (regular / tall, bf16: 3001 x 2999 x 4096, two waves each, 82 / 115 us; 2048^3,
+// one each, 26 / 38; 4100 x 4000 x 4096, four and two, 117 / 110; 6000 x 5000 x 4096, seven
+// and four, 240 / 206; 700 x 10001 x 3000, two and one, 78 / 64).  ABFT_TALL_TILES=0 or 1
+// forces the choice.
+bool use_tall(const abft_desc& d, int64_t R16, int64_t C16, int chunk) {
   if (chunk > 0) return false;
   const char* env = getenv("ABFT_TALL_TILES");
   if (env && *env) return env[0] == '1';
-  return m > BM && nkt >= 32;
+  if (d.m <= BM || cdiv(d.k, BK) < 32) return false;
+  const int64_t sms = num_sms();
+  return 8 * tile_grid(d.m, d.n, R16, C16, false, 2 * BM, sms).waves <=
+         5 * tile_grid(d.m, d.n, R16, C16, false, BM, sms).waves;
 }
 
 // Pair tiles (256 x 256 on a CTA pair, see Geo) for promoted and FP8 products with long
@@ -1523,16 +1563,13 @@ bool use_tall(int64_t m, int64_t nkt, int chunk) {
 // 8192 bf16x6 0.27 -> 0.46 ms): the pairs may take as many waves as the regular tiles, or
 // 3 % more.  bf16 keeps its tall tiles (16384^3 step 5.56 -> 5.82 ms).  ABFT_PAIR_TILES=0
 // or 1 forces the choice.
-bool use_pair(const abft_desc& d, int64_t R, int64_t Cc, bool f8, int chunk) {
+bool use_pair(const abft_desc& d, int64_t R16, int64_t C16, bool f8, int chunk) {
   const char* env = getenv("ABFT_PAIR_TILES");
   if (env && *env) return env[0] == '1';
   if (d.k < (f8 ? 9216 : d.dtype == ABFT_BF16X6 ? 5120 : 8192) || !(f8 || chunk > 0)) return false;
-  auto waves = [&](int bm, int64_t workers) {
-    const int64_t tm = cdiv(d.m, bm), tn = cdiv(d.n, BN);
-    return cdiv(tm * tn + cdiv(R, bm) * tn + tm * cdiv(Cc, BN), workers);
-  };
   const int64_t sms = num_sms();
-  return 100 * waves(2 * BM, sms / 2) <= 103 * waves(BM, sms);
+  return 100 * tile_grid(d.m, d.n, R16, C16, f8, 2 * BM, sms / 2).waves <=
+         103 * tile_grid(d.m, d.n, R16, C16, f8, BM, sms).waves;
 }
 
 // k-steps between two calls of tc::keep_step: bf16x6 16384^3 with 16 / 48 / 144 31.85 /
@@ -1670,14 +1707,17 @@ cudaError_t launch_gemm_bf16(const Plan& P, const TcOperands& op, float* C, void
     g.f8grp = op.f8grp;
     g.f8words = cdiv(cdiv(d.k, 128), 32);
   }
-  const bool tall = !pair && !g.f8 && use_tall(d.m, cdiv(d.k, BK) * op.nseg, g.chunk);
+  const bool tall = !pair && !g.f8 && use_tall(d, R16, C16, g.chunk);
   const int bm = (tall || pair) ? 256 : BM;
-  g.ntm = (int)cdiv(d.m, bm);
-  g.ntn = (int)cdiv(d.n, BN);
-  g.ntr = checksums ? (int)cdiv(R16, bm) : 0;
-  g.ntc = checksums ? (int)cdiv(C16, BN) : 0;
-  g.t_data = (int64_t)g.ntm * g.ntn;
-  g.t_total = g.t_data + (int64_t)g.ntr * g.ntn + (int64_t)g.ntm * g.ntc;
+  const Grid G = tile_grid(d.m, d.n, R16, C16, g.f8 != 0, bm, num_sms() / (pair ? 2 : 1));
+  g.ntm = (int)G.ntm;
+  g.ntn = (int)G.ntn;
+  g.ntr = (int)G.ntr;
+  g.ntc = (int)G.ntc;
+  g.fit_h = G.fit_h;
+  g.fit_b = G.fit_b;
+  g.t_data = G.ntm * G.ntn;
+  g.t_total = G.total();
   g.C = C;
   g.ldc = d.ldc;
   g.E16 = checksums ? reinterpret_cast<float*>(const_cast<char*>(w) + P.L.E16) : nullptr;
