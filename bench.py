@@ -46,14 +46,17 @@ METRIC = "ABFT GEMM TFLOPS (useful 2mnk) and % overhead vs checksum-free GEMM, s
 # FP64 peak of GB300 (the DFMA pipe, no FP64 tensor path): 152 SMs x 2 DFMA/clk/SM
 # (measured rate) x 2 flop x 2070 MHz maximum SM clock.
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
+RESIDUE_PRODUCTS = 18  # bf16 products of one binary64 product on the tensor cores
 # Measured DRAM read + write per launch of the product kernel at the bench workloads (ncu
 # dram__bytes_read.sum + dram__bytes_write.sum, one launch after three warm-up products; the
 # counters take one pass, see profiles/), or None when the kernel changed since it was
-# captured.  f64: 34.22 + 1.10 GB; bf16 (256-row tiles): 6.77 + 1.17 GB; fp8 (e4m3 data
-# tiles): 5.72 + 1.63 GB; bf16x6: 59.96 + 1.58 GB; grouped 4096 (ABFT product after the
-# autotuner, default tuning): 19.06 + 20.58 GB.
-TRAFFIC_BYTES = {"f64_11264_grid22": 35.32e9, "bf16_16384": 7.95e9, "fp8_16384": 7.35e9,
-                 "bf16x6_16384": 61.54e9, "bf16_grouped_4096": 39.64e9}
+# captured.  f64 (residue product): 60.93 + 3.36 GB; bf16 (256-row tiles): 6.78 + 1.19 GB;
+# fp8 (e4m3 data tiles, CTA pairs): 5.47 + 1.57 GB; bf16x3 (pairs): 17.85 + 1.71 GB; bf16x6
+# (pairs): 26.66 + 1.71 GB; grouped 4096 (ABFT product after the autotuner, default tuning):
+# 18.94 + 20.55 GB.
+TRAFFIC_BYTES = {"f64_11264_grid22": 64.29e9, "bf16_16384": 7.96e9, "fp8_16384": 7.05e9,
+                 "bf16x3_16384": 19.56e9, "bf16x6_16384": 28.38e9,
+                 "bf16_grouped_4096": 39.49e9}
 
 
 def bf16_peak():
@@ -511,9 +514,14 @@ def run_workload(w, args, dev, rank, world, secondary=False):
         peak, peak_src = fp8_peak() if w.dtype == "fp8" else bf16_peak()
         roof = {"kernel": "k_gemm_bf16", "bound": "tensor", "peak_source": peak_src}
     else:
-        kernel_flops = 2.0 * w.k * ((w.m + L.R) * w.n + w.m * L.Cc)
-        peak, peak_src = FP64_PEAK_TFLOPS, "152 SMs x 2 DFMA/clk/SM (measured) x 2 flop x 2070 MHz"
-        roof = {"kernel": "k_gemm_f64", "bound": "alu", "peak_source": peak_src}
+        # the binary64 product: 17 residue products and the magnitude product, in bf16
+        kernel_flops = RESIDUE_PRODUCTS * 2.0 * w.k * ((w.m + L.R) * w.n + w.m * L.Cc)
+        peak, peak_src = bf16_peak()
+        roof = {"kernel": "k_gemm_f64_tc", "bound": "tensor", "peak_source": peak_src,
+                "note": f"{RESIDUE_PRODUCTS} bf16 products per binary64 product; the time "
+                        "includes the passes that form the residues",
+                "useful_over_fp64_pipe_peak": 2.0 * w.m * w.n * w.k / (gemm_avg * 1e-3) / 1e12 /
+                                              FP64_PEAK_TFLOPS}
     achieved = kernel_flops / (gemm_avg * 1e-3) / 1e12
     roof.update({"achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                  "traffic": TRAFFIC_BYTES.get(w.name), "algorithmic_flops_per_launch": kernel_flops})
