@@ -179,7 +179,15 @@ typedef struct {
  * invalid descriptor (abft_last_error() says why).  Every call that takes a
  * workspace requires its base to be 256-byte aligned (cudaMalloc and the
  * PyTorch caching allocator give at least that) and returns ABFT_ERR_INVALID
- * with nothing launched otherwise. */
+ * with nothing launched otherwise.
+ * ABFT_F64: where the product runs on the tensor cores (see abft_gemm) the
+ * workspace also holds the residue planes of one panel of K: 36 bytes per element
+ * of the panel of [A; acs] and [B, bcs] with K rounded up to 64 and each side to 256,
+ * for instance 1.4 GB at 4096^3 on an 8 x 8 grid and 9.6 GB at 11264^3 on a 22 x 22 grid.  The
+ * panels are chosen so that the planes take at most 12 GiB, five times the bytes of
+ * A, B and C plus 256 MiB, and half of what A, B, C and the checksums leave of
+ * 284208 MiB; where one panel of 64 does not fit, no planes are kept and the product
+ * runs on the FP64 pipe.  Beside them lie per-CTA residues (at most 162 MiB). */
 size_t abft_workspace_bytes(const abft_desc* desc);
 
 /* Fill *out (host) with the workspace layout.  ABFT_ERR_INVALID on a bad desc. */
@@ -264,8 +272,9 @@ abft_status abft_encode_chained(const abft_desc* desc, const void* A, const void
 
 /* The ABFT product (Eq. (1)): [A; C_C^T A] [B, B C_R] on the GPU.  Writes the
  * data block A B into C and the checksum blocks into ws (E and F).  Requires a
- * preceding abft_encode on the same ws and operands.  ABFT_F64 with m n k of at
- * least 2^21: the operands become integers whose residues modulo 17 small
+ * preceding abft_encode on the same ws and operands.  ABFT_F64 with k of at least
+ * 48, m n k of at least 2^21 and room for the planes (see abft_workspace_bytes):
+ * the operands become integers whose residues modulo 17 small
  * numbers (bf16, in ws below layout.scratch) are multiplied on the tensor cores;
  * the elements that would lose accuracy that way (NaN, infinities, exponents
  * outside [-440, 500], terms far below their row's and column's scales) run on

@@ -1,6 +1,6 @@
 // Binary64 ABFT product (Eq. (1)): [A; acs] [B, bcs] on the FP64 FMA pipe, for
-// products below 128^3, checksum-free products without a workspace and the
-// chunks that the product on the tensor cores (gemm_f64_tc.cu) leaves out.
+// products below 128^3 or with k < 48, products whose planes have no room
+// (plan_f64_tc), checksum-free products without a workspace and the chunks that the product on the tensor cores (gemm_f64_tc.cu) leaves out.
 //
 // On GB300 the FP64 FMA pipe issues 2 DFMA per clock per SM (measured
 // 1.20 TFLOP/s over 152 SMs); mma.sync f64 runs slower (1.05 TFLOP/s) and

@@ -67,7 +67,10 @@ constexpr uint32_t kABytes = BM * BK * 2, kBoxBytes = 64 * BK * 2;
 constexpr int kMaxStages = 8;
 constexpr int kMinExp = -440, kMaxExp = 500;
 constexpr int kCut = 1, kRefused = 2;  // operand lines that were rounded / cannot be held
-constexpr size_t kPlaneBudget = size_t(12) << 30;
+constexpr int kMinK = 48;         // shorter K loops run on the FP64 pipe (plan_f64_tc)
+constexpr double kMiB = 1048576.0;
+constexpr double kPlaneBudget = 12288 * kMiB;
+constexpr double kDeviceBytes = 284208 * kMiB;  // of a GB300's memory
 constexpr int kSms = 152;  // persistent CTAs the workspace is laid out for
 
 // Tile kinds.  One CTA: 128 rows x bpt 64-column boxes.  CTA pair (bpt = 4): 256
@@ -988,19 +991,33 @@ static int64_t split_workers(int split) {
 }
 
 bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, size_t* bytes) {
-  // 128^3: 136 us on the FP64 pipe (one 64 x 64 tile's chain of k), 59 here; below,
+  // 128^3: 136 us on the FP64 pipe (one 64 x 64 tile's chain of k), 32 here; below,
   // both are bound by latency and the FP64 pipe needs one launch instead of four
-  // (1024 x 1024 x 64: 134 and 64 us, 100000 x 3 x 300: 3.34 and 0.65 ms).
-  if (d.k < 1 || (double)d.m * (double)d.n * (double)d.k < 2097152.0) return false;
+  // (1024 x 1024 x 64: 134 and 64 us, 100000 x 3 x 300: 3.34 and 0.65 ms).  A K loop is
+  // padded to 64: from k = 48 on every shape measured is faster here (FP64 pipe / here,
+  // plain products: 2048 x 2048 x 48 342 / 138 us, 64 x 65536 x 48 342 / 309, 2^20 x 1 x 48
+  // 5.82 / 3.86 ms), at 32 some are slower (2048 x 2048 231 / 138 us, 64 x 65536 231 / 306)
+  // and at 16 and below all are (2048 x 2048 x 16 119 / 136, 64 x 65536 x 2 119 / 493: with
+  // so few terms many elements fail the magnitude check and run on both).
+  if (d.k < kMinK || (double)d.m * (double)d.n * (double)d.k < 2097152.0) return false;
   F64TcRegions& r = *rg;
   r.row_cs = cdiv(d.m, 2 * BM) * 2 * BM;
   r.rows_a = r.row_cs + cdiv(R, 2 * BM) * 2 * BM;
   r.col_cs = cdiv(d.n, 256) * 256;
   r.cols_b = r.col_cs + cdiv(Cc, 256) * 256;
-  // Panels of K: the planes stay within a budget.
+  // Panels of K: the planes take at most kPlaneBudget, five times what the operands and
+  // the result take (36 bytes per element of A and B instead of 8, before padding) and
+  // 256 MiB, and half of what these and the checksums leave of the device.  A product that has no room for
+  // a panel of one k-step runs on the FP64 pipe: short K under very long sides, whose
+  // planes are mostly padding, and operands that nearly fill the device.
   const int64_t per_k = (r.rows_a + r.cols_b) * kPlanes64 * 2;
-  const int64_t fit = (int64_t)(kPlaneBudget / per_k) / BK * BK;
-  r.kp = std::min<int64_t>({cdiv(d.k, BK) * BK, kMaxPanel, std::max<int64_t>(fit, BK)});
+  const double held = 8.0 * ((double)d.m * d.k + (double)d.k * d.n + (double)d.m * d.n);
+  const double sums = 8.0 * ((double)R * (d.n + d.k) + (double)Cc * (d.m + d.k));
+  const double budget =
+      std::min({kPlaneBudget, 5.0 * held + 256 * kMiB, 0.5 * (kDeviceBytes - held - sums)});
+  if (budget < (double)per_k * BK) return false;
+  const int64_t fit = (int64_t)(budget / (double)per_k) / BK * BK;
+  r.kp = std::min<int64_t>({cdiv(d.k, BK) * BK, kMaxPanel, fit});
   // Tile kind: clocks per k-step times waves.  The copies bind the one-CTA tiles
   // (L2 delivers about 75 bytes per clock and SM; a k-step of four, two, one boxes
   // is 48, 32, 24 KiB: 640, 420, 360 clocks at 4096^3, where the MMAs take 512,
