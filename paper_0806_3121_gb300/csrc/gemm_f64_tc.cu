@@ -184,8 +184,11 @@ constexpr ModulusTable make_table() {
 }
 __constant__ ModulusTable kModulus = make_table();
 
-// x 2^(bits - e) rounded to the nearest integer (|x| < 2^e, e = efield - 1022 with
-// efield the biased exponent of the line's largest element; bits <= 59).
+// x 2^(bits - e) rounded to the nearest integer, ties to even (|x| < 2^e, e = efield -
+// 1022 with efield the biased exponent of the line's largest element; bits <= 59).
+// Values whose last bit is the half (a line of elements 2^6 .. 2^7 below its largest
+// one) would all err the same way if ties left zero: the error of a sum of k of them
+// grew like k, where it grows like sqrt(k) now.
 __device__ __forceinline__ int64_t scaled(double x, int efield, int bits, bool& cut) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
   const int E = (int)(b >> 52) & 0x7ff;
@@ -194,7 +197,9 @@ __device__ __forceinline__ int64_t scaled(double x, int efield, int bits, bool& 
   const int r = efield - max(E, 1) + (63 - bits);
   uint64_t v = 0;
   if (r < 64) {
-    v = (m + ((1ull << r) >> 1)) >> r;
+    const uint64_t half = (1ull << r) >> 1, up = m + half;
+    v = up >> r;
+    if (half != 0 && (v << r) == up) v &= ~1ull;
     cut |= (v << r) != m;
   } else {
     cut |= m != 0;
