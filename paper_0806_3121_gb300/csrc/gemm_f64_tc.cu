@@ -197,10 +197,12 @@ __device__ __forceinline__ int64_t scaled(double x, int efield, int bits, bool& 
   const int r = efield - max(E, 1) + (63 - bits);
   uint64_t v = 0;
   if (r < 64) {
-    const uint64_t half = (1ull << r) >> 1, up = m + half;
+    const uint64_t up = m + ((1ull << r) >> 1);
     v = up >> r;
-    if (half != 0 && (v << r) == up) v &= ~1ull;
-    cut |= (v << r) != m;
+    const uint64_t t = v << r;
+    const bool c = t != m;
+    cut |= c;
+    v &= ~(uint64_t)(c & (t == up));  // a half, rounded up: to the even one
   } else {
     cut |= m != 0;
   }
