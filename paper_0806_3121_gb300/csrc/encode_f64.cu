@@ -92,7 +92,8 @@ __device__ __forceinline__ void enc_acols(const EncArgs& a, int64_t blk, double*
         e += x;
         w = fma(wtab[t], x, w);
       }
-      sw = fma((double)(s0 - i0) * sc, e, sw + w);
+      sw += w;
+      if (s0 > i0) sw = fma((double)(s0 - i0) * sc, e, sw);  // (0 Inf would be NaN)
       se += e;
     }
   }

@@ -273,7 +273,8 @@ __device__ __forceinline__ void col_lines(const CheckArgs& a, const ColLines& c)
         w = fma_t<TC>(wtab[t], x, w);
         nf |= nonfinite(x);
       }
-      sw = fma_t<TC>((TC)(s0 - i0) * sc, e, sw + w);
+      sw += w;
+      if (s0 > i0) sw = fma_t<TC>((TC)(s0 - i0) * sc, e, sw);  // (0 Inf would be NaN)
       se += e;
     }
   }
