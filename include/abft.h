@@ -87,9 +87,8 @@ typedef enum {
 
 typedef enum {
   ABFT_F64 = 0,     /* A, B, C binary64, binary64 checksums; the product runs on
-                       the tensor cores in exact bf16 residues (from 128^3 up, with
-                       a workspace) or on the FP64 pipe: never less accurate than a
-                       chain of binary64 multiply-adds                              */
+                       the tensor cores in exact bf16 residues or on the FP64 pipe
+                       (abft_gemm says when, and how accurate each is)              */
   ABFT_BF16 = 1,    /* A, B bfloat16; C binary32; tensor-core product, fp32 accum.  */
   ABFT_BF16X3 = 2,  /* A, B binary32 split into bf16 hi+lo planes by abft_encode;
                        product A_hi B_hi + A_hi B_lo + A_lo B_hi; C binary32        */
@@ -276,9 +275,17 @@ abft_status abft_encode_chained(const abft_desc* desc, const void* A, const void
  * 48, m n k of at least 2^21 and room for the planes (see abft_workspace_bytes):
  * the operands become integers whose residues modulo 17 small
  * numbers (bf16, in ws below layout.scratch) are multiplied on the tensor cores;
- * the elements that would lose accuracy that way (NaN, infinities, exponents
+ * 32 x 32 chunks with an element that does not qualify (NaN, infinities, exponents
  * outside [-440, 500], terms far below their row's and column's scales) run on
- * the FP64 pipe, as all smaller products do.  ABFT_BF16X3 and
+ * the FP64 pipe, as all smaller products do.  Accuracy, with u = 2^-53: on the tensor
+ * cores an element errs by at most 0.7 sqrt(k) u (|A||B|)_ij (the operands are rounded
+ * to 58 or 59 bits below their row's or column's largest element) plus a rounding
+ * of the result, two per panel of K where K takes several (longer than 16320, or see
+ * abft_workspace_bytes); on the FP64 pipe, a chain of k multiply-adds, by at most k u
+ * (|A||B|)_ij.  On generic data the former is far below the latter; where neighbouring
+ * terms cancel a chain can be closer.  The time depends on the operands: chunks that do not
+ * qualify are computed on both (all of them: 570 us instead of 50 at 512^3, 117 ms
+ * instead of 2 at 4096^3; the FP64 pipe alone takes 527 us and 110 ms).  ABFT_BF16X3 and
  * ABFT_BF16X6 multiply the bf16 operand planes that encode wrote.
  * ABFT_FP8_E4M3: the data block multiplies the e4m3 codes of A and the
  * transposed codes of B that encode wrote, on the 8-bit tensor path

@@ -15,18 +15,28 @@
 // C_ij = 2^(eA_i + eB_j - 2 b) C' is rounded to nearest once: all in integer and
 // exact binary32 arithmetic.
 //
-// Accuracy.  What is lost is the rounding of a and b to 59 bits below their row's
-// and column's scale: a rms error of at most 2^-60.3 (b = 59) per term in units of
-// 2^(eA_i + eB_j).  A DFMA chain's rounding errors are about 0.38 2^-53 sqrt(k / 2)
-// times the rms of the terms' sum, at least 0.27 2^-53 M_ij with M_ij = sum_l |a_il
-// b_lj| in the same units.  So the product is as accurate as the chain where M_ij >=
-// 2^(53 - b - 1.3) / 0.27 sqrt(k) = 0.0235 sqrt(k) (b = 59).  M is one more product
-// (plane 17: the magnitudes as bf16, rounded towards zero), and every tile computes
-// it first: each element is checked, so rows of mixed scales, graded operands whose
-// large rows meet small columns, and sparse operands never lose accuracy.  Elements
-// of rows and columns that are integers as they are need no check.  The 32 x 32
-// chunks that hold an element below the line, NaN or infinite operands or exponents
-// outside [-440, 500] are left to the DFMA kernel (k_gemm_f64_bad).
+// Accuracy.  What is lost is the rounding of a and b to b bits below their row's and
+// column's scale: each term errs by at most 2^-b in units of 2^(eA_i + eB_j), so an
+// element by at most k 2^-b.  With M_ij = sum_l |a_il b_lj| in the same units, an element
+// is taken only where M_ij >= 1.52 2^(53 - b) sqrt(k): its error is then at most 0.66
+// sqrt(k) u M_ij (u = 2^-53), plus one rounding of the result (of each panel's, when K
+// takes several).  That is the bound that holds for every operand; it is no statement
+// about a chain of multiply-adds on the same data.  On generic data (independent
+// roundings, partial sums that grow) the errors are far below the chain's, whose
+// roundings come to about 0.38 u sqrt(k / 2) times the rms of the terms' sum, at least
+// 0.27 u M_ij; but where neighbours nearly cancel the chain's partial sums stay small and
+// it can be the closer one (pairs that agree to 1e-3 in a row whose largest element meets
+// a zero: errors of 4 to 7 times the chain's at k = 1024 to 12000, 0.1 u M_ij).  M is one
+// more product (plane 17: the magnitudes as bf16, rounded towards zero), and every tile
+// computes it first: each element is checked, so rows of mixed scales, graded operands
+// whose large rows meet small columns, and sparse operands keep that bound.  Elements of
+// rows and columns that are integers as they are need no check.  The 32 x 32 chunks that
+// hold an element below the line, NaN or infinite operands or exponents outside [-440,
+// 500] are left to the DFMA kernel (k_gemm_f64_bad).
+//
+// Those chunks cost both products: where all of them are left out (columns of A and rows
+// of B graded over 16 decades, or rows below 2^-440) 128^3 takes 164 us (the FP64 pipe
+// alone 135), 512^3 570 (527), 2048^3 14.63 ms (14.29), 4096^3 116.8 (110.0).
 //
 // The tensor cores bound it: 18 products of 2 m n k bf16 flops each.  (Exact digits
 // in radix 256 instead of residues take 29 to 37 products for the same accuracy,
