@@ -224,7 +224,9 @@ cudaError_t clear_carry(const Plan& P, void* ws, cudaStream_t st) {
   return e;
 }
 
-// Partial-reduction sizes used by the encode kernels (in doubles).
+// Doubles of scratch set aside for the encode kernels' partial sums.  Binary64: they use
+// the last term (the column squares of B); the whole sum stays the limit of
+// abft_encode_noalloc, whose refusals callers know.
 size_t part_elems(const Plan& P) {
   const int64_t k = std::max<int64_t>(P.d.k, 1);
   if (P.d.dtype != ABFT_F64) return (lp_part_bytes(P) + 7) / 8;
