@@ -284,8 +284,8 @@ abft_status abft_encode_chained(const abft_desc* desc, const void* A, const void
  * abft_workspace_bytes); on the FP64 pipe, a chain of k multiply-adds, by at most k u
  * (|A||B|)_ij.  On generic data the former is far below the latter; where neighbouring
  * terms cancel a chain can be closer.  The time depends on the operands: chunks that do not
- * qualify are computed on both (all of them: 570 us instead of 50 at 512^3, 117 ms
- * instead of 2 at 4096^3; the FP64 pipe alone takes 527 us and 110 ms).  ABFT_BF16X3 and
+ * qualify are computed on both (all of them: 570 us instead of 47 at 512^3, 117 ms
+ * instead of 1.9 at 4096^3; the FP64 pipe alone takes 526 us and 110 ms).  ABFT_BF16X3 and
  * ABFT_BF16X6 multiply the bf16 operand planes that encode wrote.
  * ABFT_FP8_E4M3: the data block multiplies the e4m3 codes of A and the
  * transposed codes of B that encode wrote, on the 8-bit tensor path

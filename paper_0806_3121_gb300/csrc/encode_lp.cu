@@ -1183,8 +1183,9 @@ constexpr int kSplitRows = 8;
 // with eight columns per thread of the whole CTA (2048 columns, every warp all the rows)
 // a 512^2 pass was a few CTAs that walked 128 rows each.  Whole encode, verify blocks 128 x
 // 256, bf16x3 / bf16x6: 512^2 138 / 147 -> 42 / 46 us, 2048^2 144 / 148 -> 40 / 42, 4096^2
-// 151 / 155 -> 79 / 83, 8192^2 207 / 247 -> 213 / 239 (blocks of 256 rows 245 / 268 -> 217 /
-// 242), 16384^2 739 / 885 -> 732 / 843.
+// 151 / 155 -> 79 / 83, 5000^2 162 / 170 -> 105 / 113, 8192^2 212 / 255 -> 209 / 237 (blocks of
+// 256 rows 252 / 276 -> 213 / 241), 12000^2 433 / 524 -> 436 / 500, 16384^2 741 / 892 -> 729 /
+// 840.
 constexpr int kSplitCols = 256;
 
 // A: planes (m x ldk), column checksums of A per verify block from the

@@ -48,8 +48,8 @@
 // a finished modulus, one byte each, in a per-CTA scratch (coalesced, mostly L2).
 //
 // Measured, product kernels alone: 8192^3 on a 16 x 16 grid 949 ms on the FP64 pipe,
-// 11.7 .. 15 here (with the clock); 4096^3 on an 8 x 8 grid 130 -> 1.95; 2048^3 16.3 ->
-// 0.28; 1000 x 1501 x 777 2.36 -> 0.093; 512^3 0.53 -> 0.053.  Relative Frobenius error
+// 11.6 .. 15 here (with the clock); 4096^3 on an 8 x 8 grid 130 -> 1.98; 2048^3 16.3 ->
+// 0.28; 1000 x 1501 x 777 2.36 -> 0.088; 512^3 0.53 -> 0.026.  Relative Frobenius error
 // against the exact product, N(0,1): 4.5e-17 (DFMA 7.7e-16) at k = 512, 4.7e-17 (2.0e-15)
 // at k = 4096, 7.0e-17 (4.9e-15) at k = 20000 in two panels of K.
 #include <cuda.h>
@@ -327,7 +327,7 @@ constexpr int kSliceRows = 16;    // 4 where 16 would leave SMs idle
 // (32 columns x 256 rows per CTA).  Two passes over the operands in two launches
 // (here and k_f64_slice) instead of one CTA that walks a strip of columns twice:
 // 512^3 31 -> 21 us, 8192^3 1.60 -> 0.82 ms with nine planes of radix-256 digits.  The
-// 18 planes are 36 bytes per element: 1.07 ms at 8192^3 for 6.3 GB, 0.87 of the copy
+// 18 planes are 36 bytes per element: 1.09 ms at 8192^3 for 6.3 GB, 0.85 of the copy
 // rate.
 __device__ __forceinline__ void max_rows(const SliceArgs& a, const double* src, int64_t ld,
                                          int64_t rows, int64_t row_out, int64_t blk,
@@ -1041,8 +1041,11 @@ bool plan_f64_tc(const abft_desc& d, int64_t R, int64_t Cc, F64TcRegions* rg, si
   // 256, 192); a pair's CTAs copy 32 KiB per 512-clock k-step (590).  Whole steps
   // with pairs / four / two / one boxes: 512^3 241 / 237 / 190 / 170 us, 1000 x 1501
   // x 777 313 / 327 / 265 / 300, 2048 chain 1.32 / 1.16 / 1.25 / 1.58 ms, 4096^3
-  // 3.03 / 3.11 / 3.24 / 4.61, 8192^3 encode + product 16.7 / 17.0 / 19.8 / 28.4:
-  // the rule takes the best of each.
+  // 3.03 / 3.11 / 3.24 / 4.61, 8192^3 encode + product 16.7 / 17.0 / 19.8 / 28.4.  The
+  // model was fitted there; elsewhere (18 shapes from 256^3 to 8192^2 x 1024, ragged and
+  // narrow ones, each kind and split forced in turn) its choice is within 1 % of the best
+  // but for 4000 x 4000 x 500 (pairs 616 us, four boxes 586) and 6000 x 6000 x 2000 (four
+  // boxes 2437, pairs 2343).
   // Few tiles leave SMs idle: their planes are split over clusters of 2, 3 or 6 CTAs
   // (the residues are put together in about 8000 clocks per box).  512^3 step with one /
   // two / three / six CTAs per tile of one box 171 / 157 / 149 / 156 us, of two boxes 193 /

@@ -1561,8 +1561,14 @@ bool use_tall(const abft_desc& d, int64_t R16, int64_t C16, int chunk) {
 // way, 5120^3 1.064 -> 1.050; bf16x3 5120^3 0.565 -> 0.570; FP8 8192^3 0.498 -> 0.508, 16384
 // x 16384 x 8192 1.84 -> 1.76), and few tiles fill their last wave less (2048 x 2048 x
 // 8192 bf16x6 0.27 -> 0.46 ms): the pairs may take as many waves as the regular tiles, or
-// 3 % more.  bf16 keeps its tall tiles (16384^3 step 5.56 -> 5.82 ms).  ABFT_PAIR_TILES=0
-// or 1 forces the choice.
+// 3 % more.  bf16 keeps its tall tiles (16384^3 step 5.56 -> 5.82 ms).  Between the lines
+// (bf16x3 with encode, 8192^2 x 6144 / 7168 / 8192 / 12288: 1.80 -> 1.81, 2.10 -> 2.14, 2.36
+// -> 2.40, 3.52 -> 3.49 ms; bf16x6 8192^2 x 4608 / 5120 2.53 -> 2.47, 2.77 -> 2.79) the two
+// differ by less than two runs of one side (2 - 4 %, under the power cap) where the waves
+// are full; with part-filled waves pairs gain below the line too (bf16x3 6000 x 7000 x 6500
+// 1.85 -> 1.43, 4096^2 x 7000 0.63 -> 0.60, 12000 x 10000 x 7168 3.81 -> 3.61), so for
+// bf16x3 the line is a safe one, not the crossover.  ABFT_PAIR_TILES=0 or 1 forces the
+// choice.
 bool use_pair(const abft_desc& d, int64_t R16, int64_t C16, bool f8, int chunk) {
   const char* env = getenv("ABFT_PAIR_TILES");
   if (env && *env) return env[0] == '1';
